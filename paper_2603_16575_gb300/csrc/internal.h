@@ -269,9 +269,9 @@ struct GradContrib {       // one fragment's amplitude of a pair and the fragmen
 void launch_pm_localize(const double* C, int n_ao, int n, const int* atom_ao, int n_atom, double l_loc, int max_sweeps,
                         double* P, double* U, double* out, int* status, int num_sms, cudaStream_t st);
 // The same sweeps over a cooperative grid (atoms spread over the CTAs, one bounded grid
-// barrier per rotation); false when the grid cannot be co-resident (nothing launched
-// then).  part: 4 * min(n_atom, num_sms) doubles; bar: 2 unsigned; err |= ERR_TIMEOUT
-// if a barrier wait gave up.
+// barrier per step of disjoint rotations); false when the grid cannot be co-resident
+// (nothing launched then).  P: n_atom n (n | 1) doubles; part: 4 * min(n_atom, num_sms) *
+// (n / 2 + 1) doubles; bar: 2 unsigned; err |= ERR_TIMEOUT if a barrier wait gave up.
 bool launch_pm_localize_grid(const double* C, int n, const int* atom_ao, int n_atom, double l_loc, int max_sweeps,
                              double* P, double* U, double* out, int* status, double* part, unsigned* bar, int* err,
                              int num_sms, cudaStream_t st);

@@ -1,0 +1,241 @@
+// Operands and launches of the FP64 tensor-core contraction (tc_oz.cuh).
+#include "internal.h"
+#include "oz_split.cuh"
+#include "tc_oz.cuh"
+
+namespace osv {
+
+// Rows already contiguous in k (stored or generated B with k = aux, dense row-major matrices): one warp per
+// (row, chunk), lanes along k in pairs.
+struct OzSrcB {            // row a of slot u: B[i0 + u][a][.]
+  BSrc src;
+  int i0;
+  __device__ __forceinline__ double get(int u, int r, int k) const { return src.get(i0 + u, r, k); }
+};
+struct OzSrcBT {           // row P of slot u: B[xs[u]][.][P]
+  BSrc src;
+  const int* xs;
+  __device__ __forceinline__ double get(int u, int r, int k) const { return src.get(xs[u], k, r); }
+};
+
+template <class Src>
+__global__ void __launch_bounds__(256) k_oz_rows(Src src, int rows, int K, int ld, uint16_t* __restrict__ D,
+                                                 int* __restrict__ ex) {
+  const int u = blockIdx.y, lane = threadIdx.x & 31;
+  const int nch = (K + oz::CHUNK - 1) / oz::CHUNK;
+  const long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (w >= (long long)rows * nch) return;   // warp-uniform
+  const int r = (int)(w / nch), c = (int)(w % nch), k0 = c * oz::CHUNK;
+  double x[8];
+#pragma unroll
+  for (int v = 0; v < 8; v++) {
+    const int k = k0 + 64 * (v >> 1) + 2 * lane + (v & 1);
+    x[v] = k < K ? src.get(u, r, k) : 0.0;
+  }
+  const size_t slice = (size_t)rows * ld;
+  const int e = oz::warp_slices(x, min(oz::CHUNK, K - k0), D + ((size_t)u * oz::NSL * rows + r) * ld + k0, slice, lane);
+  if (lane == 0) ex[((size_t)u * rows + r) * nch + c] = e;
+}
+
+// Rows strided in k (their index innermost): one CTA per 16 rows x one chunk, transposed through shared memory so
+// that both the reads (rows innermost) and the digit writes (k innermost) are coalesced.
+template <class Src>
+__global__ void __launch_bounds__(256) k_oz_cols(Src src, int rows, int K, int ld, uint16_t* __restrict__ D,
+                                                 int* __restrict__ ex) {
+  __shared__ double tile[oz::CHUNK][17];
+  const int u = blockIdx.z, r0 = blockIdx.x * 16, c = blockIdx.y, k0 = c * oz::CHUNK;
+  const int nch = (K + oz::CHUNK - 1) / oz::CHUNK;
+  for (int t = threadIdx.x; t < oz::CHUNK * 16; t += 256) {
+    const int k = t >> 4, r = t & 15;
+    tile[k][r] = (k0 + k < K && r0 + r < rows) ? src.get(u, r0 + r, k0 + k) : 0.0;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const size_t slice = (size_t)rows * ld;
+  for (int dr = threadIdx.x >> 5; dr < 16 && r0 + dr < rows; dr += 8) {   // warp-uniform
+    double x[8];
+#pragma unroll
+    for (int v = 0; v < 8; v++) x[v] = tile[64 * (v >> 1) + 2 * lane + (v & 1)][dr];
+    const int r = r0 + dr;
+    const int e = oz::warp_slices(x, min(oz::CHUNK, K - k0), D + ((size_t)u * oz::NSL * rows + r) * ld + k0, slice, lane);
+    if (lane == 0) ex[((size_t)u * rows + r) * nch + c] = e;
+  }
+}
+
+// A list of dense matrices with the row index innermost ([K][rows], row stride ldm), optionally scaled by w[k];
+// digits zero up to kpad.
+__global__ void __launch_bounds__(256) k_oz_mats(const OzMat* __restrict__ mats, const double* __restrict__ w,
+                                                 int ld, uint16_t* __restrict__ D, int* __restrict__ ex) {
+  __shared__ double tile[oz::CHUNK][17];
+  const OzMat mt = mats[blockIdx.z];
+  const int r0 = blockIdx.x * 16, c = blockIdx.y, k0 = c * oz::CHUNK, K = mt.K;
+  if (r0 >= mt.rows || k0 >= K) return;
+  for (int t = threadIdx.x; t < oz::CHUNK * 16; t += 256) {
+    const int k = t >> 4, r = t & 15;
+    double v = 0.0;
+    if (k0 + k < K && r0 + r < mt.rows) {
+      v = mt.p[(size_t)(k0 + k) * mt.ldm + r0 + r];
+      if (w) v *= w[k0 + k];
+    }
+    tile[k][r] = v;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const size_t slice = (size_t)mt.m.ss * ld;
+  for (int dr = threadIdx.x >> 5; dr < 16 && r0 + dr < mt.rows; dr += 8) {
+    double x[8];
+#pragma unroll
+    for (int v = 0; v < 8; v++) x[v] = tile[64 * (v >> 1) + 2 * lane + (v & 1)][dr];
+    const int r = r0 + dr;
+    const int e = oz::warp_slices(x, min(oz::CHUNK, mt.kpad - k0), D + ((size_t)mt.m.row + r) * ld + k0, slice, lane);
+    if (lane == 0) ex[mt.m.eb + (size_t)r * mt.m.es + c] = e;
+  }
+}
+// The same for matrices with k innermost ([rows][K], row stride ldm): a warp per (row, chunk).
+__global__ void __launch_bounds__(256) k_oz_rmats(const OzMat* __restrict__ mats, int ld, uint16_t* __restrict__ D,
+                                                  int* __restrict__ ex) {
+  const OzMat mt = mats[blockIdx.z];
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5), c = blockIdx.y, k0 = c * oz::CHUNK, lane = threadIdx.x & 31;
+  if (r >= mt.rows || k0 >= mt.K) return;
+  double x[8];
+#pragma unroll
+  for (int v = 0; v < 8; v++) {
+    const int k = k0 + 64 * (v >> 1) + 2 * lane + (v & 1);
+    x[v] = k < mt.K ? mt.p[(size_t)r * mt.ldm + k] : 0.0;
+  }
+  const int e = oz::warp_slices(x, min(oz::CHUNK, mt.kpad - k0), D + ((size_t)mt.m.row + r) * ld + k0,
+                                (size_t)mt.m.ss * ld, lane);
+  if (lane == 0) ex[mt.m.eb + (size_t)r * mt.m.es + c] = e;
+}
+
+void launch_oz_rows(const BSrc& src, int i0, int nb, uint16_t* D, int* ex, cudaStream_t st) {
+  if (!nb) return;
+  const long long warps = (long long)src.n_vir * oz::n_chunks(src.n_aux);
+  k_oz_rows<<<dim3((unsigned)((warps + 7) / 8), nb), 256, 0, st>>>(OzSrcB{src, i0}, src.n_vir, src.n_aux,
+                                                                   oz::ld_of(src.n_aux), D, ex);
+  note_launch(1);
+}
+void launch_oz_cols(const BSrc& src, const int* xs, int nb, uint16_t* D, int* ex, cudaStream_t st) {
+  if (!nb) return;
+  k_oz_cols<<<dim3((src.n_aux + 15) / 16, oz::n_chunks(src.n_vir), nb), 256, 0, st>>>(
+      OzSrcBT{src, xs}, src.n_aux, src.n_vir, oz::ld_of(src.n_vir), D, ex);
+  note_launch(1);
+}
+void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const double* w, bool k_inner, int ld,
+                    uint16_t* D, int* ex, cudaStream_t st) {
+  if (!n) return;
+  for (int q = 0; q < n; q += 65535) {     // grid z limit
+    const int nq = n - q < 65535 ? n - q : 65535;
+    if (k_inner)
+      k_oz_rmats<<<dim3((max_rows + 7) / 8, oz::n_chunks(max_K), nq), 256, 0, st>>>(mats + q, ld, D, ex);
+    else
+      k_oz_mats<<<dim3((max_rows + 15) / 16, oz::n_chunks(max_K), nq), 256, 0, st>>>(mats + q, w, ld, D, ex);
+    note_launch(1);
+  }
+}
+
+// out[row][col] (row-major)
+struct OzEpiRow {
+  __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
+    double* o = static_cast<double*>(jb.out) + (size_t)(jb.m0 + r) * jb.ld_out + jb.n0 + c0;
+#pragma unroll
+    for (int u = 0; u < oz::DCOL; u++)
+      if (c0 + u < jb.n_valid) o[u] = v[u];
+  }
+};
+// T[a][b] = T[b][a] = v / (e_a + e_b - s) for a >= b; out = T_i, s = 2 f_ii
+struct OzEpiT {
+  const double* e_vir;
+  __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
+    const int a = jb.m0 + r;
+    const double ea = e_vir[a] - jb.s;
+    double* T = static_cast<double*>(jb.out);
+#pragma unroll
+    for (int u = 0; u < oz::DCOL; u++) {
+      const int b = jb.n0 + c0 + u;
+      if (c0 + u < jb.n_valid && a >= b) {
+        const double t = v[u] / (ea + e_vir[b]);
+        T[(size_t)a * jb.ld_out + b] = t;
+        T[(size_t)b * jb.ld_out + a] = t;
+      }
+    }
+  }
+};
+
+// Digits of the output instead of its values: row m0 + r, k = n0 + c of the matrix at store row o_row (o_ss
+// rows per slice), under the exponent code exW[o_e] (a bound of the whole matrix); columns past n_valid up to the
+// next multiple of 16 are written as zeros (up to 32 by the lanes of the last column group).
+struct OzEpiDigits {
+  uint16_t* D;
+  int ld;
+  const int* exW;
+  __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
+    const int e = exW[jb.o_e];
+    const bool live = e > oz::EX_ZERO / 2 && e < oz::EX_NAN / 2;
+    uint16_t* o = D + ((size_t)jb.o_row + jb.m0 + r) * ld + jb.n0 + c0;
+    const size_t slice = (size_t)jb.o_ss * ld;
+    // the last column group also clears the group after it when that completes a 32-wide k-block
+    const bool tail = c0 + oz::DCOL >= jb.n_valid && ((jb.n0 + c0) & 16) == 0;
+#pragma unroll
+    for (int h = 0; h < oz::DCOL / 8; h++) {
+      long long f[8];
+#pragma unroll
+      for (int u = 0; u < 8; u++)
+        f[u] = (live && c0 + 8 * h + u < jb.n_valid) ? oz::fixed63(v[8 * h + u], (unsigned)(e + 1022)) : 0;
+#pragma unroll
+      for (int s = oz::NSL - 1; s >= 0; s--) {
+        uint4 w;
+        w.x = oz::digit_pair(f[0], f[1], s);
+        w.y = oz::digit_pair(f[2], f[3], s);
+        w.z = oz::digit_pair(f[4], f[5], s);
+        w.w = oz::digit_pair(f[6], f[7], s);
+        *reinterpret_cast<uint4*>(o + s * slice + 8 * h) = w;
+        if (tail) *reinterpret_cast<uint4*>(o + s * slice + 16 + 8 * h) = make_uint4(0, 0, 0, 0);
+      }
+    }
+  }
+};
+
+namespace {
+// 2-D BF16 map over rows x ld, 64-byte swizzle, box 32 x box_rows.  K < ld: k past K reads as 0.
+bool make_digit_map(CUtensorMap* m, const OzOperand& A, int box_rows) {
+  auto enc = tensor_map_encoder();
+  if (!enc) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)A.K, (cuuint64_t)A.rows};
+  cuuint64_t strides[1] = {(cuuint64_t)A.ld * 2};
+  cuuint32_t box[2] = {(cuuint32_t)oz::BK, (cuuint32_t)box_rows};
+  cuuint32_t es[2] = {1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(A.D), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <class Epi>
+int run(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const int* skip,
+        int* err, Epi epi, cudaStream_t st) {
+  if (!n_jobs) return 0;
+  if (cudaFuncSetAttribute(oz::k_oz<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM) != cudaSuccess)
+    return -1;
+  CUtensorMap ma, mb;
+  if (!make_digit_map(&ma, A, oz::AROWS) || !make_digit_map(&mb, B, oz::BROWS)) return -1;
+  oz::k_oz<Epi><<<tc::persistent_grid(n_jobs), oz::NTHREADS, oz::SMEM, st>>>(ma, mb, A.ex, B.ex, jobs, n_jobs, segs, skip,
+                                                                             err, epi);
+  note_launch(1);
+  return 0;
+}
+}  // namespace
+
+int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                   const int* skip, int* err, cudaStream_t st) {
+  return run(A, B, jobs, n_jobs, segs, skip, err, OzEpiRow{}, st);
+}
+int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                     const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st) {
+  return run(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits{D, ld, exW}, st);
+}
+int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int* err,
+                  cudaStream_t st) {
+  return run(A, A, jobs, n_jobs, segs, nullptr, err, OzEpiT{e_vir}, st);
+}
+
+}  // namespace osv

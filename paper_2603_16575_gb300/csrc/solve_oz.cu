@@ -1,0 +1,203 @@
+// FP64 form, A3-A4 on the tensor cores: every pair's preconditioner basis polished to FP64
+// accuracy, and the amplitude iterations of many fragments at once in that basis.
+//
+// With T_p = X_p Y_p X_p^T (T starts at 0 and every update of Algorithm 7 lies in the span of X_p),
+// U_p = P_p X_p orthonormal and F diagonal in it, Eq. (res_close) reads
+//   R~_p = K~_p - D_p o Y_p + C_p,   C_p = sum_terms c_t Sigma_pq op(Y_q) Sigma_pq^T,
+// K~_p = X_p^T K_p X_p, Sigma_pq = U_p^T U_q, and the update is Y_p <- (K~_p + C_p) / D_p: the
+// products of the pair with itself (half of the operations of the raw-basis residual) are gone.
+// The rest are two products per coupling term, both FP64 contractions of tc_oz.cuh:
+//   W_t^T = Sigma_pq op(Y_q)^T    digits written by the epilogue, one exponent per matrix
+//   C_p   = sum_t c_t Sigma_pq W_t
+// A sweep is four launches over all fragments: W, C, the element-wise update with the digits of
+// the new Y, and the convergence test, whose flags make the next sweep leave finished fragments out.
+//
+// The exponents are bounds, so no pass over W is needed for its largest element: |W_t| <= the norm
+// of op(Y_q), since the rows of Sigma_pq are no longer than 1.  The slices hold 63 bits below the
+// bound, ten more than the mantissa.
+#include "oz_split.cuh"
+#include "pairview.cuh"
+
+namespace osv {
+
+// ---------------------------------------------------------------- basis polish
+// One step of the refinement of Ogita and Aishima (Japan J. Indust. Appl. Math. 35 (2018) 1007) on
+// the basis U0 = P X: with S1 = U0^T U0 and F1 = U0^T e U0 formed from U0 itself (entries of order 1;
+// X^T S X would carry eps |X|^2, X reaching lambda_min(S)^(-1/2)),
+//   R = 1 - S1, lambda_a = F1_aa / S1_aa, E_ab = (F1_ab + lambda_b R_ab) / (lambda_b - lambda_a)
+// (R_ab / 2 where that is not small: equal or nearly equal lambda, and a = b), X <- X (1 + E),
+// e~ = lambda.  U = U0 (1 + E) is then orthonormal and F diagonal in it to FP64 rounding.
+__global__ void __launch_bounds__(NT) k_oz_polish(const OzPolish* __restrict__ jobs, int n_jobs, int max_m,
+                                                  double* scratch) {
+  __shared__ double sm[GEMM_SMEM_WIDE];
+  double* XE = scratch + (size_t)blockIdx.x * max_m * max_m;
+  for (int q = blockIdx.x; q < n_jobs; q += gridDim.x) {
+    const OzPolish jb = jobs[q];
+    const int m = jb.m, r = jb.r;
+    for (int idx = threadIdx.x; idx < r * r; idx += NT) {
+      const int a = idx / r, b = idx % r;
+      const double R = (a == b ? 1.0 : 0.0) - 0.5 * (jb.S1[idx] + jb.S1[b * r + a]);
+      double e = 0.5 * R;
+      if (a != b) {
+        const double la = jb.F1[a * r + a] / jb.S1[a * r + a], lb = jb.F1[b * r + b] / jb.S1[b * r + b];
+        const double num = 0.5 * (jb.F1[idx] + jb.F1[b * r + a]) + lb * R, gap = lb - la;
+        if (fabs(num) < 0.1 * fabs(gap)) e = num / gap;
+      }
+      jb.IE[idx] = e;
+    }
+    __syncthreads();
+    cta_gemm_a(m, r, r, 1.0, dense_view(jb.X, m, r, m), dense_view(jb.IE, r, r, r), 0.0, XE, r, sm);
+    for (int idx = threadIdx.x; idx < m * r; idx += NT) jb.X[(size_t)(idx / r) * m + idx % r] += XE[idx];
+    for (int a = threadIdx.x; a < r; a += NT) {
+      jb.et[a] = jb.F1[(size_t)a * r + a] / jb.S1[(size_t)a * r + a];
+      jb.IE[(size_t)a * r + a] += 1.0;
+    }
+    __syncthreads();
+  }
+}
+void launch_oz_polish(const OzPolish* jobs, int n_jobs, int max_m, double* scratch, int n_cta, cudaStream_t st) {
+  if (!n_jobs) return;
+  k_oz_polish<<<n_cta, NT, 0, st>>>(jobs, n_jobs, max_m, scratch);
+  note_launch(1);
+}
+
+// ---------------------------------------------------------------- update
+// Exponent code of a bound |x| < 2^e.
+__device__ __forceinline__ int bound_exp(double x) {
+  if (!(x > 0.0)) return oz::EX_ZERO;
+  return oz::chunk_exp(oz::exp_field(x));
+}
+
+// Digits of row m of op(Y) (r x r; v: 0 Y, 1 Y^T, 2 Y + Y^T) under the exponent code e, one warp.
+__device__ __forceinline__ void row_digits(const double* Y, int r, int m, int v, int e, int kpad, uint16_t* dst,
+                                           size_t slice, int lane) {
+  const bool live = e > oz::EX_ZERO / 2 && e < oz::EX_NAN / 2;
+  for (int k = 2 * lane; k < kpad; k += 64) {
+    double x[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const int kk = k + u;
+      x[u] = 0.0;
+      if (kk < r) {
+        if (v != 1) x[u] = Y[(size_t)m * r + kk];
+        if (v != 0) x[u] += Y[(size_t)kk * r + m];
+      }
+    }
+    long long f0 = live ? oz::fixed63(x[0], (unsigned)(e + 1022)) : 0, f1 = live ? oz::fixed63(x[1], (unsigned)(e + 1022)) : 0;
+#pragma unroll
+    for (int s = oz::NSL - 1; s >= 0; s--)
+      *reinterpret_cast<uint32_t*>(dst + s * slice + k) = oz::digit_pair(f0, f1, s);
+  }
+}
+
+__global__ void __launch_bounds__(NT) k_oz_update(const OzPair* __restrict__ pairs, int n_pairs,
+                                                  const int* __restrict__ done, int first, int ld, int nch,
+                                                  uint16_t* __restrict__ D, int* __restrict__ ex,
+                                                  int* __restrict__ exW, double* __restrict__ pe,
+                                                  double* __restrict__ pu) {
+  __shared__ double red[40];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int q = blockIdx.x; q < n_pairs; q += gridDim.x) {
+    const OzPair p = pairs[q];
+    if (done[p.frag]) continue;
+    const int r = p.r;
+    double du = 0.0, am = 0.0, ss = 0.0;
+    bool bad = false;
+    for (int idx = threadIdx.x; idx < r * r; idx += NT) {
+      const int a = idx / r, b = idx % r;
+      const double y = (p.Kt[idx] + (first ? 0.0 : p.C[idx])) / (p.fij - p.et[a] - p.et[b]);
+      du = fmax(du, fabs(y - (first ? 0.0 : p.Y[idx])));
+      p.Y[idx] = y;
+      am = fmax(am, fabs(y));
+      ss += y * y;
+      bad |= !isfinite(y);
+    }
+    bad = __syncthreads_or(bad);
+    du = cta_max(du, red);
+    am = cta_max(am, red);
+    ss = cta_sum(ss, red);       // ends with a barrier: Y is complete
+    double e = 0.0;
+    for (int idx = threadIdx.x; idx < r * r; idx += NT) {
+      const int a = idx / r, b = idx % r;
+      e += p.Kt[idx] * (2.0 * p.Y[idx] - p.Y[(size_t)b * r + a]);
+    }
+    e = cta_sum(e, red);
+    if (threadIdx.x == 0) {
+      pe[q] = p.diag ? e : 2.0 * e;
+      pu[q] = bad ? __longlong_as_double(0x7FF8000000000000ll) : du;
+    }
+    const double nrm = bad ? 0.0 : sqrt(ss) * (1.0 + 1e-3);
+    const int eY = bound_exp(bad ? 0.0 : am), eW = bound_exp(nrm);
+    for (int v = 0; v < 3; v++) {
+      const int id = p.ver[v];
+      if (id < 0) continue;
+      const int up = (v == 2), ey = eY == oz::EX_ZERO ? eY : eY + up, ew = eW == oz::EX_ZERO ? eW : eW + up;
+      if (threadIdx.x < nch) {
+        ex[(size_t)id * nch + threadIdx.x] = ey;
+        exW[(size_t)id * nch + threadIdx.x] = ew;
+      }
+      uint16_t* base = D + (size_t)p.vrow[v] * ld;
+      for (int m = warp; m < r; m += NT / 32)
+        row_digits(p.Y, r, m, v, ey, p.kpad, base + (size_t)m * ld, (size_t)r * ld, lane);
+    }
+    __syncthreads();
+  }
+}
+
+// One thread per fragment: its energy and largest update from its pairs (in order), the test of
+// Algorithm 7, the result record and the flag that stops it.
+__global__ void k_oz_converge(const int* __restrict__ pair0, int n_frag, const double* __restrict__ pe,
+                              const double* __restrict__ pu, SolveOpts o, double ulps, int it, double* __restrict__ e_prev,
+                              int* __restrict__ done, int* __restrict__ left, FragOut* __restrict__ out,
+                              const int* __restrict__ out_id) {
+  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+  if (f >= n_frag || done[f]) return;
+  double e = 0.0, um = 0.0;
+  bool nan = false;
+  for (int q = pair0[f]; q < pair0[f + 1]; q++) {
+    e += pe[q];
+    um = fmax(um, pu[q]);
+    nan |= isnan(pu[q]);
+  }
+  int status = ERR_NOCONV;
+  if (nan || !isfinite(e) || !isfinite(um)) status = ERR_NONFINITE;
+  else if (um < o.tol_update && fabs(e - e_prev[f]) < fmax(o.tol_energy, ulps * fabs(e))) status = 0;
+  e_prev[f] = e;
+  out[out_id[f]] = FragOut{e, nan ? __longlong_as_double(0x7FF8000000000000ll) : um, it, status};
+  if (status != ERR_NOCONV || it == o.max_iter) done[f] = 1;
+  else atomicAdd(left, 1);
+}
+
+void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, int nch, uint16_t* D,
+                      int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st) {
+  if (!n_pairs) return;
+  k_oz_update<<<n_cta, NT, 0, st>>>(pairs, n_pairs, done, first ? 1 : 0, ld, nch, D, ex, exW, pe, pu);
+  note_launch(1);
+}
+void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
+                        double* e_prev, int* done, int* left, FragOut* out, const int* out_id, cudaStream_t st) {
+  if (!n_frag) return;
+  cudaMemsetAsync(left, 0, sizeof(int), st);
+  k_oz_converge<<<(n_frag + 127) / 128, 128, 0, st>>>(pair0, n_frag, pe, pu, o, ulps, it, e_prev, done, left, out, out_id);
+  note_launch(1);
+}
+
+// T_p = X_p Y_p X_p^T of the listed pairs (the gradient and the weak pairs use the raw OSV basis).
+__global__ void __launch_bounds__(NT) k_oz_raw(const OzPair* __restrict__ pairs, int n_pairs, int max_m,
+                                               double* scratch) {
+  __shared__ double sm[GEMM_SMEM_WIDE];
+  double* W = scratch + (size_t)blockIdx.x * max_m * max_m;
+  for (int q = blockIdx.x; q < n_pairs; q += gridDim.x) {
+    const OzPair p = pairs[q];
+    const View Xv = dense_view(p.X, p.m, p.r, p.m);
+    cta_gemm_a(p.m, p.r, p.r, 1.0, Xv, dense_view(p.Y, p.r, p.r, p.r), 0.0, W, p.r, sm);
+    cta_gemm_a(p.m, p.m, p.r, 1.0, dense_view(W, p.m, p.r, p.r), transpose(Xv), 0.0, p.T, p.m, sm);
+  }
+}
+void launch_oz_raw(const OzPair* pairs, int n_pairs, int max_m, double* scratch, int n_cta, cudaStream_t st) {
+  if (!n_pairs) return;
+  k_oz_raw<<<n_cta, NT, 0, st>>>(pairs, n_pairs, max_m, scratch);
+  note_launch(1);
+}
+
+}  // namespace osv

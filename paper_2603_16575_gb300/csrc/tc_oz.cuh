@@ -1,0 +1,270 @@
+// FP64 contraction on the tcgen05 tensor cores (sm_103a) by exact integer slices.
+//
+//   D[m][n] = sum_seg coef_seg sum_k A_seg[m][k] B_seg[n][k]      A, B, D in FP64
+//
+// FP64 runs at 2 FMAs a clock and SM on this part, BF16 tensor products at 4096: a
+// product of integers cut small enough for the tensor core to sum them exactly gives an
+// FP64 result from BF16 products (the splitting of Ozaki, Ogita, Oishi and Rump, Numer.
+// Algorithms 59 (2012) 95; integer form: Ootomo, Ozaki and Yokota, 2024).
+//
+//  * Within a chunk of CHUNK = 256 consecutive k, row m of A is
+//      A[m][k] = 2^(e_m - 7) sum_{s=1..8} a_s 2^(-8 (s-1)),  a_s integer, |a_s| <= 128,
+//    e_m the smallest exponent with max_k |A[m][k]| < 2^e_m (oz_split.cuh): 63 fractional
+//    bits, ten more than the mantissa, so a value keeps its full mantissa down to 2^-10 of
+//    the row's largest in the chunk and an absolute 2^(e_m - 64) below that.
+//  * A product a_s b_t of level l = s + t is at most 2^14, a chunk sum of one slice pair at
+//    most 2^22, and a sum of up to four pairs (levels 2-5) stays an exact FP32 integer
+//    whatever the accumulator's rounding; levels 6-9 have 5 to 8 pairs, whose sums pass 2^24
+//    only if every digit is extreme, and are 2^-32 and less of the result's scale then.
+//    Levels above 9 (below 2^-64 of the chunk scale) are dropped: 36 products.
+//  * The drain warps join the level sums of a chunk into one 64-bit integer (levels 2-7 by
+//    shifts, 8 and 9 in full where it has room for them and rounded in otherwise), convert it once and add it to the FP64 sum of the element
+//    with one FMA: K / 256 roundings per element where an FP64 dot product makes K.
+//
+// Bound: the shared-memory reads of the MMAs.  An M = 128, N = 64, K = 16 MMA reads 6 KB
+// (48 cycles) for 32 cycles of multiplication; the eight 64-column level accumulators fill
+// the 512 TMEM columns, so N = 64 is the widest tile.  36 products make 128 x 64 x 256
+// cost ~28k cycles an SM; the drain (about 15k, FP64 and integer pipes) runs under the next
+// chunk's MMAs: every level has its own full / empty barrier, so level l of the next chunk
+// starts as soon as level l of this one has been read.
+//
+// Persistent CTAs (one per SM) over output tiles of 128 rows (TMEM lanes) x up to 64 columns:
+//   warp 0     TMA producer: the 8 + 8 slice tiles of a 32-wide k-block per stage (64-byte
+//              swizzle, K-major), two stages of 96 KB
+//   warp 1     TMEM allocation and the single MMA-issuing thread
+//   warps 2-17 drain and epilogue: four warps per TMEM lane quarter, 16 columns each (the 64-bit
+//              integers, the FP64 sums and the level being read of 32 columns do not fit the registers)
+// Every mbarrier wait is bounded; a timeout sets ERR_TIMEOUT in *err, the roles leave their
+// loops, the producer waits (bounded) for its copies in flight and the MMA thread for its
+// last commit, and the CTA frees its tensor memory and returns without hanging.
+#pragma once
+#include <cuda.h>
+#include <stdint.h>
+
+#include "oz_job.h"
+#include "oz_split.cuh"
+#include "tc_ptx.cuh"
+
+namespace osv {
+namespace oz {
+
+constexpr int A_TILE = BM * BK * 2;          // 8 KB per A slice tile (filled up to m rows)
+constexpr int B_TILE = BN * BK * 2;          // 4 KB per B slice tile (filled up to n rows)
+constexpr int STAGE = NSL * (A_TILE + B_TILE);
+constexpr int NSTAGE = 2;
+constexpr int SMEM = NSTAGE * STAGE + 1024;  // + slack for 1024-byte alignment
+constexpr int AROWS = 64, BROWS = 32;        // rows of one TMA box of the A and B operands
+constexpr int NDRAIN = 16;                   // drain warps
+constexpr int DCOL = BN * 4 / NDRAIN;        // columns of one: four warps share a TMEM lane quarter
+constexpr int NTHREADS = 64 + 32 * NDRAIN;
+constexpr int NLEV = 8;                      // levels 2 .. 9
+constexpr int KBC = CHUNK / BK;              // k-blocks of a full chunk
+constexpr int TMEM_COLS = 512;
+constexpr int ERR_TC_TIMEOUT = 16;           // same bit as ERR_TIMEOUT of the library
+
+// acc + coef * v * 2^x for the sum x of two chunk exponents less the integer's unit; out of the
+// normal range: zero rows (EX_ZERO) add 0, non-finite rows (EX_NAN) give NaN, the rest through ldexp.
+__device__ __forceinline__ double oz_fma(long long v, int x, double coef, double acc) {
+  if (x >= -1022 && x <= 1023)
+    return fma((double)v, coef * __longlong_as_double((long long)(x + 1023) << 52), acc);
+  if (x >= EX_NAN / 2) return __longlong_as_double(0x7FF8000000000000ll);
+  if (x <= EX_ZERO / 2) return acc;
+  return fma(coef, ldexp((double)v, x), acc);
+}
+
+// Epi: epi(job, row, col0, acc) stores columns col0 .. col0 + 15 of the tile's row (row < m_valid).
+template <class Epi>
+__global__ void __launch_bounds__(NTHREADS, 1)
+    k_oz(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const int* __restrict__ exA,
+         const int* __restrict__ exB, const Job* __restrict__ jobs, int n_jobs, const Seg* __restrict__ segs,
+         const int* __restrict__ skip, int* err, Epi epi) {
+  extern __shared__ uint8_t dsm[];
+  __shared__ __align__(8) uint64_t bar_full[NSTAGE], bar_empty[NSTAGE], bar_accf[NLEV], bar_acce[NLEV];
+  __shared__ uint32_t s_tmem;
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~(uintptr_t)1023);
+  const uint32_t sbase = tc::su32(sm);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::su32(&s_tmem)),
+                 "r"(TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NSTAGE; s++) {
+      tc::mbar_init(&bar_full[s], 1);
+      tc::mbar_init(&bar_empty[s], 1);
+    }
+    for (int l = 0; l < NLEV; l++) {
+      tc::mbar_init(&bar_accf[l], 1);
+      tc::mbar_init(&bar_acce[l], NDRAIN);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = s_tmem;
+  bool ok = true;
+  // The CTA takes tiles blockIdx.x, + gridDim.x, ...; g counts its k-blocks and ch its
+  // chunks, so all barrier phases carry over from tile to tile.  Every role walks the same
+  // (tile, segment, chunk, k-block) sequence.
+  if (warp == 0) {
+    if (lane == 0) {                                             // ---- TMA producer
+      long long g = 0;
+      for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
+        const Job jb = jobs[tile];
+        if (jb.skip >= 0 && skip[jb.skip]) continue;
+        const int nbox = (jb.n_valid + BROWS - 1) / BROWS, mbox = (jb.m_valid + AROWS - 1) / AROWS;
+        const uint32_t bytes = NSL * (mbox * AROWS + nbox * BROWS) * BK * 2;
+        for (int q = 0; ok && q < jb.nseg; q++) {
+          const Seg sg = segs[jb.seg0 + q];
+          const int nkb = (sg.K + BK - 1) / BK, ra = sg.a.row + jb.m0, rb = sg.b.row + jb.n0;
+          for (int c = 0; c < nkb; c++, g++) {
+            const int s = (int)(g % NSTAGE);
+            if (g >= NSTAGE) ok = tc::mbar_wait(tc::su32(&bar_empty[s]), (uint32_t)(((g / NSTAGE) - 1) & 1));
+            if (!ok) break;
+            const uint32_t fb = tc::su32(&bar_full[s]);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(bytes) : "memory");
+            const uint32_t st = sbase + s * STAGE;
+            for (int sl = 0; sl < NSL; sl++) {
+              for (int bx = 0; bx < mbox; bx++)
+                tc::tma_load_2d(st + sl * A_TILE + bx * AROWS * BK * 2, &tmA, fb, c * BK, ra + sl * sg.a.ss + bx * AROWS);
+              for (int bx = 0; bx < nbox; bx++)
+                tc::tma_load_2d(st + NSL * A_TILE + sl * B_TILE + bx * BROWS * BK * 2, &tmB, fb, c * BK,
+                                rb + sl * sg.b.ss + bx * BROWS);
+            }
+          }
+        }
+      }
+      if (!ok) {
+        // leaving early: let the copies already issued land first (bounded waits); only the
+        // last armed k-block of each stage can be outstanding
+        for (long long gg = g - 1; gg >= 0 && gg >= g - NSTAGE; gg--)
+          tc::mbar_wait(tc::su32(&bar_full[gg % NSTAGE]), (uint32_t)((gg / NSTAGE) & 1));
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {                                             // ---- MMA issuer
+      long long g = 0, ch = 0;
+      for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
+        const Job jb = jobs[tile];
+        if (jb.skip >= 0 && skip[jb.skip]) continue;
+        const int npad = (jb.n_valid + 15) & ~15;
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(npad >> 3) << 17) |
+                               ((uint32_t)(BM >> 4) << 24);
+        for (int q = 0; ok && q < jb.nseg; q++) {
+          const int nkb = (segs[jb.seg0 + q].K + BK - 1) / BK;
+          for (int c = 0; c < nkb; c++, g++) {
+            const int s = (int)(g % NSTAGE);
+            const bool first = (c % KBC) == 0, last = (c % KBC) == KBC - 1 || c == nkb - 1;
+            ok = tc::mbar_wait(tc::su32(&bar_full[s]), (uint32_t)((g / NSTAGE) & 1));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t st = sbase + s * STAGE;
+            for (int l = 0; l < NLEV; l++) {
+              if (first && ch > 0) {
+                ok = tc::mbar_wait(tc::su32(&bar_acce[l]), (uint32_t)((ch - 1) & 1));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+              }
+              const uint32_t dacc = tmem + (uint32_t)(l * BN);
+              for (int sa = 0; sa <= l; sa++)                    // slices sa + sb = l (counted from 0)
+                for (int ks = 0; ks < BK / 16; ks++)
+                  tc::mma_f16(dacc, tc::desc_sw64(st + sa * A_TILE + ks * 32),
+                              tc::desc_sw64(st + NSL * A_TILE + (l - sa) * B_TILE + ks * 32), idesc,
+                              (first && sa == 0 && ks == 0) ? 0u : 1u);
+              if (last) tc::commit(&bar_accf[l]);
+            }
+            if (!ok) break;
+            tc::commit(&bar_empty[s]);
+            if (last) ch++;
+          }
+        }
+      }
+      // wait (bounded) for the last commit of each stage: every MMA issued has then completed
+      // and no arrival is in flight when the CTA exits
+      if (!ok) {
+        tc::commit(&bar_empty[g % NSTAGE]);
+        g++;
+      }
+      for (long long gg = g - 1; gg >= 0 && gg >= g - NSTAGE; gg--)
+        tc::mbar_wait(tc::su32(&bar_empty[gg % NSTAGE]), (uint32_t)((gg / NSTAGE) & 1));
+    }
+  } else {                                                       // ---- drain + epilogue
+    const int quad = warp & 3;                                   // TMEM lane quarter of this warp
+    const int col0 = ((warp - 2) >> 2) * DCOL;                   // and its columns
+    const uint32_t lcol = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)col0;
+    const int row = 32 * quad + lane;
+    long long ch = 0;
+    for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
+      const Job jb = jobs[tile];
+      if (jb.skip >= 0 && skip[jb.skip]) continue;
+      const bool live = col0 < jb.n_valid;                       // warp-uniform
+      double acc[DCOL];
+#pragma unroll
+      for (int u = 0; u < DCOL; u++) acc[u] = 0.0;
+      for (int q = 0; ok && q < jb.nseg; q++) {
+        const Seg* sg = segs + jb.seg0 + q;
+        const int nch = (sg->K + CHUNK - 1) / CHUNK;
+        const int* ea_p = exA + sg->a.eb + (long long)(jb.m0 + min(row, jb.m_valid - 1)) * sg->a.es;
+        const int* eb_p = exB + sg->b.eb + (long long)(jb.n0 + min(col0 + (lane & (DCOL - 1)), jb.n_valid - 1)) * sg->b.es;
+        const double coef = sg->coef;
+        for (int c = 0; ok && c < nch; c++, ch++) {
+          const int ea = ea_p[c] - 54, eb = eb_p[c];
+          long long v[DCOL];
+          int lo[DCOL];
+#pragma unroll
+          for (int u = 0; u < DCOL; u++) {
+            v[u] = 0;
+            lo[u] = 0;
+          }
+#pragma unroll
+          for (int l = 0; l < NLEV; l++) {
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::su32(&bar_accf[l]), (uint32_t)(ch & 1)));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            uint32_t x[DCOL];
+            if (live) {
+              OSV_TMEM_LD16(lcol + l * BN, x);
+              asm volatile("tcgen05.wait::ld.sync.aligned;");
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&bar_acce[l]);
+            if (!live) continue;
+#pragma unroll
+            for (int u = 0; u < DCOL; u++) {
+              const int d = __float2int_rn(__uint_as_float(x[u]));
+              if (l < 6) v[u] = (v[u] << 8) + d;                   // levels 2 .. 7
+              else if (l == 6) lo[u] = d;                          // level 8, unit 2^-8
+              else {                                               // level 9, unit 2^-16: the chunk is complete
+                int e = ea + __shfl_sync(0xffffffffu, eb, u);
+                const long long w = ((long long)lo[u] << 8) + d;
+                long long t;
+                if ((unsigned long long)(v[u] + (1ll << 45)) >> 46) t = v[u] + ((w + 32768) >> 16);
+                else {                                             // room below: levels 8 and 9 in full
+                  t = (v[u] << 16) + w;
+                  e -= 16;
+                }
+                acc[u] = oz_fma(t, e, coef, acc[u]);
+              }
+            }
+          }
+        }
+      }
+      if (!ok) break;
+      if (row < jb.m_valid && live) epi(jb, row, col0, acc);
+    }
+  }
+  if (!ok) atomicOr(err, ERR_TC_TIMEOUT);
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
+}
+
+}  // namespace oz
+}  // namespace osv
