@@ -76,7 +76,7 @@ __device__ inline void sign_vectors(double* V, int n, int k) {
   for (int t = warp; t < k; t += NT_EIG / 32) {
     double* x = V + (size_t)t * n;
     double best = -1.0;
-    int bi = 0x7fffffff;
+    int bi = n - 1;   // in range when no entry compares (NaN)
     for (int r = lane; r < n; r += 32) {
       const double a = fabs(x[r]);
       if (a > best) { best = a; bi = r; }
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(EB_WARPS * 32) k_eig_back_df(const double* T, 
   }
   __syncwarp();
   double best = -1.0;
-  int bi = 0x7fffffff;
+  int bi = n - 1;   // in range when no entry compares (NaN)
   for (int r = lane; r < n; r += 32) {
     const double a = fabs(x[r]);
     if (a > best) { best = a; bi = r; }
@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(EB_WARPS * 32) k_eig_back(const double* T, int
     __syncwarp();
   }
   double best = -1.0;
-  int bi = 0x7fffffff;
+  int bi = n - 1;   // in range when no entry compares (NaN)
   for (int r = lane; r < n; r += 32) {
     const double a = fabs(x[r]);
     if (a > best) { best = a; bi = r; }
