@@ -644,6 +644,218 @@ int gproj_tensor(osvmp2_ctx* c, const std::vector<GJob>& gj, const std::vector<l
   return 0;
 }
 
+// ---- FP64 contractions on the tensor cores (tc_oz.cuh) --------------------------------
+// Digit stores are temporaries of a call.  A call that has no room for them (a device-memory
+// cap, a full device) runs the CUDA-core kernels, which need none: the helpers return
+// OZ_NO_ROOM then, with nothing launched that the caller would have to undo.
+constexpr int OZ_NO_ROOM = -100;
+
+// Bytes of the digits of `rows` operand rows with K elements each, and of their exponents.
+size_t oz_digit_bytes(size_t rows, int K) { return rows * oz::NSL * oz::ld_of(K) * sizeof(uint16_t); }
+size_t oz_exp_bytes(size_t rows, int K) { return rows * oz::n_chunks(K) * sizeof(int); }
+
+int oz_room(osvmp2_ctx* c, Tmp& t, size_t bytes) {
+  if (!tmp_alloc(c, t, bytes)) return 0;
+  c->err.clear();
+  return OZ_NO_ROOM;
+}
+
+// A list of tiles and of the segments they sum.
+struct OzList {
+  std::vector<oz::Job> jobs;
+  std::vector<oz::Seg> segs;
+  void seg(const oz::Mat& a, const oz::Mat& b, int K, double coef = 1.0) { segs.push_back(oz::Seg{a, b, K, 0, coef}); }
+  // tiles of a rows x cols output that sums the segments added since first
+  void tiles(int first, int rows, int cols, void* out, int ld_out, oz::Job proto = oz::Job{}) {
+    for (int m0 = 0; m0 < rows; m0 += oz::BM)
+      for (int n0 = 0; n0 < cols; n0 += oz::BN) {
+        oz::Job jb = proto;
+        jb.seg0 = first;
+        jb.nseg = (int)segs.size() - first;
+        jb.m0 = m0;
+        jb.n0 = n0;
+        jb.m_valid = std::min(oz::BM, rows - m0);
+        jb.n_valid = std::min(oz::BN, cols - n0);
+        jb.ld_out = ld_out;
+        jb.out = out;
+        jobs.push_back(jb);
+      }
+  }
+  // out = A B^T
+  void product(const oz::Mat& a, int ra, const oz::Mat& b, int rb, int K, double* out, int ld_out) {
+    oz::Job p{};
+    p.skip = -1;
+    const int first = (int)segs.size();
+    seg(a, b, K);
+    tiles(first, ra, rb, out, ld_out, p);
+  }
+};
+// Device copies of a list.
+struct OzDev {
+  Tmp j, s;
+  int n = 0;
+};
+int oz_upload(osvmp2_ctx* c, const OzList& l, OzDev& d) {
+  d.n = (int)l.jobs.size();
+  if (!d.n) return 0;
+  TRY(tmp_alloc(c, d.j, l.jobs.size() * sizeof(oz::Job)));
+  TRY(tmp_alloc(c, d.s, l.segs.size() * sizeof(oz::Seg)));
+  CK(cudaMemcpyAsync(d.j.p, l.jobs.data(), l.jobs.size() * sizeof(oz::Job), cudaMemcpyHostToDevice, c->st));
+  CK(cudaMemcpyAsync(d.s.p, l.segs.data(), l.segs.size() * sizeof(oz::Seg), cudaMemcpyHostToDevice, c->st));
+  return 0;
+}
+int oz_run(osvmp2_ctx* c, const OzOperand& A, const OzOperand& B, const OzList& l) {
+  if (l.jobs.empty()) return 0;
+  OzDev d;
+  TRY(oz_upload(c, l, d));
+  if (launch_oz_gemm(A, B, (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, nullptr, c->err_d, c->st))
+    return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for an FP64 contraction failed");
+  CK(cudaGetLastError());
+  return 0;
+}
+
+// Digits of a set of dense matrices in one store of row length K.
+struct OzMats {
+  Tmp D, ex, md;
+  OzOperand op{};
+  std::vector<OzMat> mats;
+  int max_rows = 0, K;
+  long long rows = 0;      // rows of the matrices (the store has NSL times as many)
+  explicit OzMats(int K_) : K(K_) {}
+  // matrix of r rows and k <= K elements a row at p (row stride ldm); the digits past k are zero up to
+  // the next multiple of 32, as far as a tile of K = k reads
+  int add(const double* p, int r, int ldm, int k) {
+    const int nch = oz::n_chunks(K);
+    OzMat m{p, r, k, std::min(oz::ld_of(K), (k + oz::BK - 1) / oz::BK * oz::BK), ldm,
+            oz::Mat{(int)(rows * oz::NSL), r, (int)(rows * nch), nch}};
+    mats.push_back(m);
+    rows += r;
+    max_rows = std::max(max_rows, r);
+    return (int)mats.size() - 1;
+  }
+  const oz::Mat& mat(int id) const { return mats[id].m; }
+};
+// Room for the digits of s (OZ_NO_ROOM without), then the digits, scaled by w[k] unless NULL.
+int oz_mats_room(osvmp2_ctx* c, OzMats& s) {
+  if (s.rows * oz::NSL + oz::BM >= (long long)INT32_MAX || s.rows * oz::n_chunks(s.K) >= (long long)INT32_MAX)
+    return OZ_NO_ROOM;
+  TRY(oz_room(c, s.D, oz_digit_bytes((size_t)s.rows, s.K)));
+  TRY(oz_room(c, s.ex, oz_exp_bytes((size_t)s.rows, s.K)));
+  TRY(oz_room(c, s.md, s.mats.size() * sizeof(OzMat)));
+  s.op = OzOperand{(const uint16_t*)s.D.p, s.rows * oz::NSL, s.K, oz::ld_of(s.K), (const int*)s.ex.p};
+  return 0;
+}
+int oz_mats_fill(osvmp2_ctx* c, OzMats& s, const double* w, bool k_inner) {
+  if (s.mats.empty()) return 0;
+  CK(cudaMemcpyAsync(s.md.p, s.mats.data(), s.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
+  launch_oz_mats((const OzMat*)s.md.p, (int)s.mats.size(), s.max_rows, s.K, w, k_inner, oz::ld_of(s.K), (uint16_t*)s.D.p,
+                 (int*)s.ex.p, c->st);
+  CK(cudaGetLastError());
+  return 0;
+}
+
+// S_(x,y) = Q_x^T Q_y and F_(x,y) = (e Q_x)^T Q_y of every listed block.
+int oz_sf(osvmp2_ctx* c, const std::vector<SFJob>& sfj) {
+  const int n = c->sys.n_occ, nv = c->sys.n_vir;
+  std::vector<int> at(n, -1);
+  OzMats q(nv), eq(nv);
+  for (const SFJob& j : sfj)
+    for (int x : {j.x, j.y})
+      if (at[x] < 0) {
+        const int k = c->n_osv[x];
+        at[x] = q.add(c->Qp[x], k, k, nv);
+        eq.add(c->Qp[x], k, k, nv);
+      }
+  TRY(oz_mats_room(c, q));
+  TRY(oz_mats_room(c, eq));
+  TRY(oz_mats_fill(c, q, nullptr, false));
+  TRY(oz_mats_fill(c, eq, c->sys.e_vir, false));
+  OzList ls, lf;
+  for (const SFJob& j : sfj) {
+    const oz::Mat &a = q.mat(at[j.x]), &b = q.mat(at[j.y]);
+    const int ka = c->n_osv[j.x], kb = c->n_osv[j.y];
+    ls.product(a, ka, b, kb, nv, j.S, kb);
+    lf.product(a, ka, b, kb, nv, j.F, kb);
+  }
+  TRY(oz_run(c, q.op, q.op, ls));
+  return oz_run(c, eq.op, q.op, lf);
+}
+
+// B~_i^(x) = B_i^T Q_x of every listed job; the orbitals i in batches whose digits fit a fixed budget.
+int oz_project(osvmp2_ctx* c, const std::vector<ProjJob>& pj) {
+  const int n = c->sys.n_occ, nv = c->sys.n_vir, nx = c->sys.n_aux, nch = oz::n_chunks(nv);
+  std::vector<std::vector<int>> by_i(n);
+  std::vector<int> at(n, -1), is;
+  OzMats q(nv);
+  for (size_t t = 0; t < pj.size(); t++) {
+    const int x = pj[t].x, k = c->n_osv[x];
+    by_i[pj[t].i].push_back((int)t);
+    if (at[x] < 0) at[x] = q.add(c->Qp[x], k, k, nv);
+  }
+  for (int i = 0; i < n; i++)
+    if (!by_i[i].empty()) is.push_back(i);
+  if (is.empty()) return 0;
+  const size_t slot = oz_digit_bytes(nx, nv), budget = (size_t)4 << 30;
+  const size_t per = std::max<size_t>(1, std::min<size_t>(is.size(), budget / slot));
+  if ((double)per * oz::NSL * nx + oz::BM >= (double)INT32_MAX) return OZ_NO_ROOM;
+  Tmp D, ex, xd;
+  TRY(oz_mats_room(c, q));
+  TRY(oz_room(c, D, per * slot));
+  TRY(oz_room(c, ex, oz_exp_bytes(per * nx, nv)));
+  TRY(oz_room(c, xd, is.size() * sizeof(int)));
+  CK(cudaMemcpyAsync(xd.p, is.data(), is.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+  TRY(oz_mats_fill(c, q, nullptr, false));
+  const OzOperand A{(const uint16_t*)D.p, (long long)(per * oz::NSL * nx), nv, oz::ld_of(nv), (const int*)ex.p};
+  for (size_t b0 = 0; b0 < is.size(); b0 += per) {
+    const int nb = (int)std::min(per, is.size() - b0);
+    launch_oz_cols(bsrc(c), (const int*)xd.p + b0, nb, (uint16_t*)D.p, (int*)ex.p, c->st);
+    CK(cudaGetLastError());
+    OzList l;
+    for (int u = 0; u < nb; u++)
+      for (int t : by_i[is[b0 + u]]) {
+        const int k = c->n_osv[pj[t].x];
+        l.product(oz::Mat{u * oz::NSL * nx, nx, u * nx * nch, nch}, nx, q.mat(at[pj[t].x]), k, nv, pj[t].out, k);
+      }
+    TRY(oz_run(c, A, q.op, l));
+  }
+  return 0;
+}
+
+// K_(ij,ij) of every listed job from the projections, in batches whose digits fit a fixed budget.
+int oz_exchange(osvmp2_ctx* c, const std::vector<KJob>& kj) {
+  const int nx = c->sys.n_aux;
+  const size_t budget = (size_t)8 << 30;
+  size_t k0 = 0;
+  while (k0 < kj.size()) {
+    OzMats s(nx);
+    std::unordered_map<const double*, int> at;
+    auto add = [&](const double* p, int r) {
+      auto it = at.find(p);
+      if (it != at.end()) return it->second;
+      const int id = s.add(p, r, r, nx);
+      at[p] = id;
+      return id;
+    };
+    OzList l;
+    size_t k1 = k0;
+    for (; k1 < kj.size() && (k1 == k0 || oz_digit_bytes((size_t)s.rows, nx) < budget); k1++) {
+      const KJob& j = kj[k1];
+      const int ni = c->n_osv[j.i], nj = j.i == j.j ? 0 : c->n_osv[j.j], m = ni + nj;
+      const int lh[2] = {add(j.Bii, ni), nj ? add(j.Bij, nj) : -1};
+      const int rh[2] = {nj ? add(j.Bji, ni) : lh[0], nj ? add(j.Bjj, nj) : -1};
+      for (int a = 0; a < (nj ? 2 : 1); a++)
+        for (int b = 0; b < (nj ? 2 : 1); b++)
+          l.product(s.mat(lh[a]), a ? nj : ni, s.mat(rh[b]), b ? nj : ni, nx,
+                    j.out + (size_t)(a ? ni : 0) * m + (b ? ni : 0), m);
+    }
+    TRY(oz_mats_room(c, s));
+    TRY(oz_mats_fill(c, s, nullptr, false));
+    TRY(oz_run(c, s.op, s.op, l));
+    k0 = k1;
+  }
+  return 0;
+}
+
 int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req, osvmp2_prec prec);
 
 // A failure part-way through leaves pairs marked as pending and blocks only
@@ -835,16 +1047,22 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
   for (auto& j : pj) f_pj += 2.0 * nx * (double)nv * c->n_osv[j.x];
   for (auto& j : kj) { const double m = pair_dim_h(c, j.i, j.j); f_k += 2.0 * nx * m * m; }
   ph_begin(c, OSVMP2_PH_SF);
-  launch_sf(t, c->sys.e_vir, (const SFJob*)jsf.p, (int)sfj.size(), max_n, c->st);
+  int oz = oz_sf(c, sfj);
+  if (oz == OZ_NO_ROOM) launch_sf(t, c->sys.e_vir, (const SFJob*)jsf.p, (int)sfj.size(), max_n, c->st);
+  else TRY(oz);
   ph_end(c, OSVMP2_PH_SF, f_sf);
   CK(cudaGetLastError());
   if (!mixed) {   // raw-basis projection and exchange blocks (FP64 form only)
     ph_begin(c, OSVMP2_PH_PROJECT);
-    launch_project(bsrc(c), t, (const ProjJob*)jpj.p, (int)pj.size(), max_nx, 0, c->st);
+    oz = oz_project(c, pj);
+    if (oz == OZ_NO_ROOM) launch_project(bsrc(c), t, (const ProjJob*)jpj.p, (int)pj.size(), max_nx, 0, c->st);
+    else TRY(oz);
     ph_end(c, OSVMP2_PH_PROJECT, f_pj, c->sys.B ? 8.0 * (double)pj.size() * nx * nv : 0.0);
     CK(cudaGetLastError());
     ph_begin(c, OSVMP2_PH_EXCHANGE);
-    launch_exchange(t, nx, (const KJob*)jk.p, (int)kj.size(), max_m, 0, c->st);
+    oz = oz_exchange(c, kj);
+    if (oz == OZ_NO_ROOM) launch_exchange(t, nx, (const KJob*)jk.p, (int)kj.size(), max_m, 0, c->st);
+    else TRY(oz);
     ph_end(c, OSVMP2_PH_EXCHANGE, f_k);
     CK(cudaGetLastError());
   }
@@ -1075,7 +1293,9 @@ int ensure_sf_blocks_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>&
   TRY(tmp_alloc(c, jd, sfj.size() * sizeof(SFJob)));
   CK(cudaMemcpyAsync(jd.p, sfj.data(), sfj.size() * sizeof(SFJob), cudaMemcpyHostToDevice, c->st));
   ph_begin(c, OSVMP2_PH_SF);
-  launch_sf(tables(c), c->sys.e_vir, (const SFJob*)jd.p, (int)sfj.size(), 0, c->st);
+  const int oz = oz_sf(c, sfj);
+  if (oz == OZ_NO_ROOM) launch_sf(tables(c), c->sys.e_vir, (const SFJob*)jd.p, (int)sfj.size(), 0, c->st);
+  else TRY(oz);
   ph_end(c, OSVMP2_PH_SF, fl);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->st));
@@ -1243,6 +1463,36 @@ int tii_tensor(osvmp2_ctx* c, int i0, int b, double* T, float* Bt, int nsl, int 
     CK(cudaMemcpyAsync(jd.p, jobs.data(), jobs.size() * sizeof(tc::Job), cudaMemcpyHostToDevice, c->st));
     if (launch_tii_tc(Bt, (long long)nu * tc::NSL * nv, nx, ldx, (const tc::Job*)jd.p, (int)jobs.size(),
                       c->sys.e_vir, c->err_d, c->st))
+      return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for T_ii failed");
+    CK(cudaGetLastError());
+  }
+  return 0;
+}
+
+// FP64 T_i of orbitals [i0, i0+b) on the tensor cores, up to nsl orbitals' digits (D, ex) at a time.
+int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int nsl) {
+  const int nv = c->sys.n_vir, nx = c->sys.n_aux, n = c->sys.n_occ, nch = oz::n_chunks(nx);
+  for (int u0 = 0; u0 < b; u0 += nsl) {
+    const int nu = std::min(nsl, b - u0);
+    launch_oz_rows(bsrc(c), i0 + u0, nu, D, ex, c->st);
+    CK(cudaGetLastError());
+    OzList all, l;
+    for (int u = 0; u < nu; u++) {
+      const int i = i0 + u0 + u;
+      const oz::Mat m{u * oz::NSL * nv, nv, u * nv * nch, nch};
+      all.product(m, nv, m, nv, nx, T + (size_t)(u0 + u) * nv * nv, nv);
+      for (oz::Job& jb : all.jobs)
+        if (jb.n0 < jb.m0 + oz::BM) {          // tiles that touch the lower triangle
+          jb.s = 2.0 * c->f_h[(size_t)i * n + i];
+          l.jobs.push_back(jb);
+        }
+      all.jobs.clear();
+    }
+    l.segs = all.segs;
+    OzDev d;
+    TRY(oz_upload(c, l, d));
+    if (launch_oz_tii(OzOperand{D, (long long)nu * oz::NSL * nv, nx, oz::ld_of(nx), ex}, (const oz::Job*)d.j.p, d.n,
+                      (const oz::Seg*)d.s.p, c->sys.e_vir, c->err_d, c->st))
       return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for T_ii failed");
     CK(cudaGetLastError());
   }
@@ -1432,6 +1682,11 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
   const size_t slot_bytes = (size_t)tc::NSL * nv * ldx * sizeof(float);
   const int nsl = tii_tc ? (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, ((size_t)1 << 30) / slot_bytes)) : 0;
   Tmp Tm, Vm, wm, km, sm, Bt;
+  // FP64 form: digits of B for up to 2 GB of orbitals at a time; without room for one orbital's, the
+  // CUDA-core kernel
+  const size_t ozslot = oz_digit_bytes(nv, s->n_aux);
+  const int noz = tii_tc ? 0 : (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, ((size_t)2 << 30) / ozslot));
+  Tmp ozD, ozE;
   if (tii_tc) TRY(tmp_alloc(c, Bt, (size_t)nsl * slot_bytes));
   TRY(tmp_alloc(c, Tm, (size_t)nb * nv * nv * sizeof(double)));
   TRY(tmp_alloc(c, Vm, (size_t)nb * nv * kmax * sizeof(double)));
@@ -1447,6 +1702,8 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
   } else {
     TRY(tmp_alloc(c, sm, (size_t)nb * eig_osv_scratch_doubles(nv, kmax) * sizeof(double)));
   }
+  const bool tii_digits = !tii_tc && (double)noz * oz::NSL * nv + oz::BM < (double)INT32_MAX &&
+                          !oz_room(c, ozD, noz * ozslot) && !oz_room(c, ozE, oz_exp_bytes((size_t)noz * nv, s->n_aux));
   std::vector<int> nrows_h(nb);
   const uint64_t rosv_key = mix64((uint64_t)s->seed ^ (7ull * STREAM_MUL));
   Tmp qtab;
@@ -1461,6 +1718,8 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
     ph_begin(c, OSVMP2_PH_TII);
     if (tii_tc)
       TRY(tii_tensor(c, i0, b, (double*)Tm.p, (float*)Bt.p, nsl, ldx));
+    else if (tii_digits)
+      TRY(tii_oz(c, i0, b, (double*)Tm.p, (uint16_t*)ozD.p, (int*)ozE.p, noz));
     else
       launch_tii(bsrc(c), s->e_vir, s->f_occ, n, i0, b, (double*)Tm.p, c->st);
     ph_end(c, OSVMP2_PH_TII, (double)b * nv * (double)nv * s->n_aux, s->B ? 8.0 * b * (double)nv * s->n_aux : 0.0);

@@ -22,7 +22,6 @@
 #include "internal.h"
 #include "tc_tf32x3.cuh"
 
-#include <cudaTypedefs.h>
 
 namespace osv {
 
@@ -119,8 +118,7 @@ struct EpiRow64 {
   }
 };
 
-namespace {
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
     void* p = nullptr;
@@ -132,11 +130,10 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   }
   return fn;
 }
-}  // namespace
 
 // 2-D FP32 map over rows x n_k (row stride ldk floats), 128-byte swizzle, box 32 x box_rows.
 bool make_slice_map(CUtensorMap* m, const float* base, int n_k, int ldk, long long rows, int box_rows) {
-  auto enc = encode_fn();
+  auto enc = tensor_map_encoder();
   if (!enc) return false;
   cuuint64_t dims[2] = {(cuuint64_t)n_k, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ldk * 4};

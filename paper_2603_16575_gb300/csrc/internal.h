@@ -2,9 +2,11 @@
 // translation units of libosvmp2.  Not part of the C ABI.
 #pragma once
 #include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include "common.cuh"
+#include "oz_job.h"
 #include "tc_job.h"
 
 namespace osv {
@@ -108,6 +110,67 @@ void launch_rosv_backq(const double* Vs, const double* ws, const int* ks, const 
 // Copy V[b][:, :k_b] into the packed Q store (Q[i0+b] as [nv][k]).
 void launch_pack_q(const double* V, const double* w, int nb, int nv, int kmax, const int* k,
                    double* const* Qdst, double* const* wdst, cudaStream_t st);
+
+// ---- FP64 contractions on the tensor cores (oz_gemm.cu, tc_oz.cuh)
+// Digit store of an operand: rows of K BF16 digits with stride ld (a multiple of 8), and chunk exponents.
+struct OzOperand {
+  const uint16_t* D;
+  long long rows;
+  int K, ld;
+  const int* ex;
+};
+struct OzMat {           // dense matrix whose digits go to m; row stride ldm (see launch_oz_mats)
+  const double* p;
+  int rows, K, kpad, ldm;  // kpad >= K: digits of k in [K, kpad) are written as zeros
+  oz::Mat m;
+};
+// Digits of B: rows B[i0 + u][a][.] (K = aux) or B[xs[u]][.][P] (K = vir); slot u, slice s, row r at
+// row (u NSL + s) rows + r of the store, exponent row u rows + r.
+void launch_oz_rows(const BSrc& src, int i0, int nb, uint16_t* D, int* ex, cudaStream_t st);
+void launch_oz_cols(const BSrc& src, const int* xs, int nb, uint16_t* D, int* ex, cudaStream_t st);
+// Digits of dense matrices: [K][rows] (row index innermost), scaled by w[k] unless NULL; or, k_inner, [rows][K].
+void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const double* w, bool k_inner, int ld,
+                    uint16_t* D, int* ex, cudaStream_t st);
+// out[row][col] per job (row-major); T_ii tiles of the lower triangle (mirrored, with denominators).
+// Return 0, or -1 if a tensor map could not be encoded.
+int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                   const int* skip, int* err, cudaStream_t st);
+int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int* err,
+                  cudaStream_t st);
+// The digits of the output (jobs' o_row, o_ss, o_e) into the store D with row stride ld (a multiple of 32).
+int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                     const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st);
+// ---- FP64 amplitude iterations on the tensor cores (solve_oz.cu)
+struct OzPolish {        // pair basis refinement
+  int m, r;
+  const double* S1;      // U0^T U0 [r][r]
+  const double* F1;      // U0^T e U0
+  double* IE;            // out: 1 + E [r][r]
+  double* X;             // [m][m], first r columns; in place
+  double* et;            // out
+};
+void launch_oz_polish(const OzPolish* jobs, int n_jobs, int max_m, double* scratch, int n_cta, cudaStream_t st);
+struct OzPair {          // a pair of a fragment
+  int frag, r, m, diag;
+  int kpad;              // r rounded up to 32
+  int ver[3];            // matrix id of the digits of Y, Y^T, Y + Y^T, -1 where no term uses them
+  int vrow[3];           // their store rows
+  int pad;
+  double fij;            // f_ii + f_jj
+  const double* Kt;      // [r][r]
+  const double* et;      // [r]
+  const double* X;       // [m][m]
+  double* Y;             // [r][r]
+  double* C;             // [r][r]
+  double* T;             // [m][m] raw-basis amplitude (launch_oz_raw) or NULL
+};
+void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, int nch, uint16_t* D,
+                      int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st);
+void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
+                        double* e_prev, int* done, int* left, FragOut* out, const int* out_id, cudaStream_t st);
+void launch_oz_raw(const OzPair* pairs, int n_pairs, int max_m, double* scratch, int n_cta, cudaStream_t st);
+// cuTensorMapEncodeTiled (NULL if the driver has none)
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
 // ---- A1-A2 (pair_integrals.cu)
 struct ProjJob {         // B~_{i}^{(x)} = B[i]^T Q_x  -> out [n_aux][n_x]
