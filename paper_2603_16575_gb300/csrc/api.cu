@@ -2,6 +2,7 @@
 // device-resident OSV / pair store, job lists for the kernels, and the MBE(3)
 // fragment enumeration.  All arithmetic of the method runs in the kernels.
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -117,6 +118,11 @@ struct osvmp2_ctx {
   std::vector<float*> us_base_h;
   std::vector<long long> us_alloc_rows_h, us_row_h;
   int us_ldv = 0;
+  // FP64 form: digits of U_p (polished basis) of each pair: store of its build and matrix in it (-1: none)
+  std::vector<void*> ud_alloc;
+  std::vector<OzOperand> ud_store;
+  std::vector<int> ud_of;
+  std::vector<oz::Mat> ud_mat;
   std::vector<int> m_h;
   std::vector<int> pi_h, pj_h;       // pair id -> (i, j)
   // last MBE call
@@ -258,15 +264,32 @@ struct Tmp {
     if (p) pool_put(c, p);
   }
 };
-int tmp_alloc(osvmp2_ctx* c, Tmp& t, size_t bytes) {
+// The digits of the pair bases (FP64 form) are kept for later solves as long as nothing else needs
+// their memory: give them up (the pairs then count as having none).  True if there were any.
+bool drop_basis_digits(osvmp2_ctx* c) {
+  if (c->ud_alloc.empty()) return false;
+  for (void* p : c->ud_alloc) pool_put(c, p);
+  c->ud_alloc.clear();
+  c->ud_store.clear();
+  std::fill(c->ud_of.begin(), c->ud_of.end(), -1);
+  return true;
+}
+// keep: the caller is using the basis digits
+int tmp_alloc(osvmp2_ctx* c, Tmp& t, size_t bytes, bool keep = false) {
   if (t.p) pool_put(t.c, t.p);
   t.c = c;
   cudaError_t e = pool_get(c, &t.p, bytes);
+  if (e != cudaSuccess && !keep && drop_basis_digits(c)) e = pool_get(c, &t.p, bytes);
   if (e != cudaSuccess) {
     t.p = nullptr;
     return fail(c, OSVMP2_E_NOMEM, "cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
   }
   return 0;
+}
+
+void tmp_free(Tmp& t) {
+  if (t.p) pool_put(t.c, t.p);
+  t.p = nullptr;
 }
 
 void free_system(osvmp2_ctx* c) {
@@ -275,6 +298,7 @@ void free_system(osvmp2_ctx* c) {
   c->sys_allocs.clear();
   for (void* p : c->pair_allocs) pool_put(c, p);
   c->pair_allocs.clear();
+  drop_basis_digits(c);
   c->pair_prec = -1;
   c->have_sys = c->have_osv = false;
   c->n_osv.clear(); c->Qp.clear(); c->Wp.clear();
@@ -282,6 +306,7 @@ void free_system(osvmp2_ctx* c) {
   c->S_h.clear(); c->F_h.clear(); c->K_h.clear(); c->X_h.clear(); c->et_h.clear(); c->bt_h.clear(); c->Kt_h.clear();
   c->U_h.clear(); c->Gi_h.clear(); c->Gj_h.clear(); c->Sh_h.clear(); c->Gh_h.clear();
   c->us_base_h.clear(); c->us_alloc_rows_h.clear(); c->us_row_h.clear();
+  c->ud_store.clear(); c->ud_of.clear(); c->ud_mat.clear();
   c->m_h.clear(); c->pi_h.clear(); c->pj_h.clear();
   c->frags.clear(); c->frag_out.clear(); c->weak.clear(); c->weak_e.clear();
   c->n_osv_d = nullptr; c->Q_d = nullptr; c->sf_id_d = nullptr; c->S_d = c->F_d = nullptr;
@@ -471,6 +496,7 @@ int palloc(osvmp2_ctx* c, double** p, size_t n) {
   *p = nullptr;
   const size_t bytes = std::max<size_t>(16, n * sizeof(double));
   cudaError_t e = pool_get(c, reinterpret_cast<void**>(p), bytes);
+  if (e != cudaSuccess && drop_basis_digits(c)) e = pool_get(c, reinterpret_cast<void**>(p), bytes);
   if (e != cudaSuccess)
     return fail(c, OSVMP2_E_NOMEM, "cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
   c->pair_allocs.push_back(*p);
@@ -482,6 +508,7 @@ int reset_pairs(osvmp2_ctx* c) {
   CK(cudaStreamSynchronize(c->st));
   for (void* p : c->pair_allocs) pool_put(c, p);
   c->pair_allocs.clear();
+  drop_basis_digits(c);
   const size_t nn = (size_t)c->sys.n_occ * c->sys.n_occ;
   c->sf_id.assign(nn, -1);
   c->pair_id.assign(nn, -1);
@@ -489,6 +516,7 @@ int reset_pairs(osvmp2_ctx* c) {
   c->S_h.clear(); c->F_h.clear(); c->K_h.clear(); c->X_h.clear(); c->et_h.clear(); c->bt_h.clear(); c->Kt_h.clear();
   c->U_h.clear(); c->Gi_h.clear(); c->Gj_h.clear(); c->Sh_h.clear(); c->Gh_h.clear();
   c->us_base_h.clear(); c->us_alloc_rows_h.clear(); c->us_row_h.clear();
+  c->ud_store.clear(); c->ud_of.clear(); c->ud_mat.clear();
   c->m_h.clear(); c->pi_h.clear(); c->pj_h.clear(); c->r_h.clear();
   TRY(upload(c, c->sf_id_d, c->sf_id));
   TRY(upload(c, c->pair_id_d, c->pair_id));
@@ -655,7 +683,7 @@ size_t oz_digit_bytes(size_t rows, int K) { return rows * oz::NSL * oz::ld_of(K)
 size_t oz_exp_bytes(size_t rows, int K) { return rows * oz::n_chunks(K) * sizeof(int); }
 
 int oz_room(osvmp2_ctx* c, Tmp& t, size_t bytes) {
-  if (!tmp_alloc(c, t, bytes)) return 0;
+  if (!tmp_alloc(c, t, bytes, true)) return 0;
   c->err.clear();
   return OZ_NO_ROOM;
 }
@@ -698,8 +726,8 @@ struct OzDev {
 int oz_upload(osvmp2_ctx* c, const OzList& l, OzDev& d) {
   d.n = (int)l.jobs.size();
   if (!d.n) return 0;
-  TRY(tmp_alloc(c, d.j, l.jobs.size() * sizeof(oz::Job)));
-  TRY(tmp_alloc(c, d.s, l.segs.size() * sizeof(oz::Seg)));
+  TRY(oz_room(c, d.j, l.jobs.size() * sizeof(oz::Job)));
+  TRY(oz_room(c, d.s, l.segs.size() * sizeof(oz::Seg)));
   CK(cudaMemcpyAsync(d.j.p, l.jobs.data(), l.jobs.size() * sizeof(oz::Job), cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(d.s.p, l.segs.data(), l.segs.size() * sizeof(oz::Seg), cudaMemcpyHostToDevice, c->st));
   return 0;
@@ -852,6 +880,525 @@ int oz_exchange(osvmp2_ctx* c, const std::vector<KJob>& kj) {
     TRY(oz_mats_fill(c, s, nullptr, false));
     TRY(oz_run(c, s.op, s.op, l));
     k0 = k1;
+  }
+  return 0;
+}
+
+// FP64 form: U_p = P_p X_p of the new pairs with the basis polished (solve_oz.cu), kept as digits for the
+// pair-couple overlaps.  X and e~ become those of the polished basis.  Pairs in batches whose temporaries
+// fit a fixed budget.
+int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, int max_m) {
+  const int n = c->sys.n_occ, nv = c->sys.n_vir;
+  c->ud_of.resize(c->K_h.size(), -1);
+  c->ud_mat.resize(c->K_h.size());
+  int max_n = 1, max_r = 1;
+  long long rows = 0;
+  std::vector<int> pid;
+  for (auto& p : newp) {
+    const int id = c->pair_id[(size_t)p.first * n + p.second];
+    pid.push_back(id);
+    rows += c->r_h[id];
+    max_r = std::max(max_r, c->r_h[id]);
+    max_n = std::max({max_n, c->n_osv[p.first], c->n_osv[p.second]});
+    if (c->r_h[id] < 1) return OZ_NO_ROOM;
+  }
+  const int nch = oz::n_chunks(nv), ld = oz::ld_of(nv);
+  if (rows * oz::NSL + oz::BM >= (long long)INT32_MAX || rows * nch >= (long long)INT32_MAX) return OZ_NO_ROOM;
+  // digits of the Q_i with the OSV index innermost (rows of P)
+  OzMats q(max_n);
+  std::vector<int> at(n, -1);
+  for (auto& p : newp)
+    for (int x : {p.first, p.second})
+      if (at[x] < 0) at[x] = q.add(c->Qp[x], nv, c->n_osv[x], c->n_osv[x]);
+  TRY(oz_mats_room(c, q));
+  Tmp dmem, emem;          // kept at the end
+  TRY(oz_room(c, dmem, oz_digit_bytes((size_t)rows, nv)));
+  TRY(oz_room(c, emem, oz_exp_bytes((size_t)rows, nv)));
+  TRY(oz_mats_fill(c, q, nullptr, true));
+  const OzOperand store{(const uint16_t*)dmem.p, rows * oz::NSL, nv, ld, (const int*)emem.p};
+  const int sid = (int)c->ud_store.size();
+  const double budget = 3e9;
+  long long row = 0;
+  const int n_cta = 2 * c->num_sms;
+  for (size_t b0 = 0; b0 < newp.size();) {
+    size_t b1 = b0;
+    size_t u0sz = 0, sqsz = 0;
+    for (double held = 0.0; b1 < newp.size() && (b1 == b0 || held < budget); b1++) {
+      const size_t r = c->r_h[pid[b1]];
+      held += 56.0 * r * nv + 56.0 * r * max_r;
+      u0sz += r * nv;
+      sqsz += r * r;
+    }
+    Tmp u0, sq, scr, pj, mj;
+    TRY(oz_room(c, u0, u0sz * sizeof(double)));
+    TRY(oz_room(c, sq, 3 * sqsz * sizeof(double)));
+    TRY(oz_room(c, scr, (size_t)n_cta * max_m * max_m * sizeof(double)));
+    TRY(oz_room(c, pj, (b1 - b0) * sizeof(OzPolish)));
+    TRY(oz_room(c, mj, (b1 - b0) * sizeof(OzMat)));
+    OzMats xs(max_n), uc(nv), ue(nv), ur(max_r), ie(max_r);
+    OzList lu, ls, lf, lo;
+    std::vector<OzPolish> pol;
+    std::vector<OzMat> fin;
+    size_t uo = 0, so = 0;
+    int mr = 0;
+    for (size_t t = b0; t < b1; t++) {
+      const int i = newp[t].first, j = newp[t].second, id = pid[t], r = c->r_h[id], m = c->m_h[id];
+      const int ni = c->n_osv[i], nj = i == j ? 0 : c->n_osv[j];
+      double* X = c->X_h[id];
+      double* U0 = (double*)u0.p + uo;
+      double* S1 = (double*)sq.p + so;
+      double *F1 = S1 + sqsz, *IE = F1 + sqsz;
+      uo += (size_t)r * nv;
+      so += (size_t)r * r;
+      mr = std::max(mr, r);
+      oz::Job proto{};
+      proto.skip = -1;
+      const int first = (int)lu.segs.size(), xt = xs.add(X, r, m, ni);
+      lu.seg(q.mat(at[i]), xs.mat(xt), ni);
+      if (nj) {
+        const int xb = xs.add(X + (size_t)ni * m, r, m, nj);
+        lu.seg(q.mat(at[j]), xs.mat(xb), nj);
+      }
+      lu.tiles(first, nv, r, U0, r, proto);
+      const int a = uc.add(U0, r, r, nv);
+      ue.add(U0, r, r, nv);
+      ls.product(uc.mat(a), r, uc.mat(a), r, nv, S1, r);
+      lf.product(ue.mat(a), r, uc.mat(a), r, nv, F1, r);
+      pol.push_back(OzPolish{m, r, S1, F1, IE, X, c->et_h[id]});
+      lo.product(ur.mat(ur.add(U0, nv, r, r)), nv, ie.mat(ie.add(IE, r, r, r)), r, r, U0, r);
+      const oz::Mat um{(int)(row * oz::NSL), r, (int)(row * nch), nch};
+      fin.push_back(OzMat{U0, r, nv, nv, r, um});
+      c->ud_mat[id] = um;
+      row += r;
+    }
+    TRY(oz_mats_room(c, xs));
+    TRY(oz_mats_room(c, uc));
+    TRY(oz_mats_room(c, ue));
+    TRY(oz_mats_room(c, ur));
+    TRY(oz_mats_room(c, ie));
+    TRY(oz_mats_fill(c, xs, nullptr, false));
+    TRY(oz_run(c, q.op, xs.op, lu));
+    TRY(oz_mats_fill(c, uc, nullptr, false));
+    TRY(oz_mats_fill(c, ue, c->sys.e_vir, false));
+    TRY(oz_mats_fill(c, ur, nullptr, true));
+    TRY(oz_run(c, uc.op, uc.op, ls));
+    TRY(oz_run(c, ue.op, uc.op, lf));
+    CK(cudaMemcpyAsync(pj.p, pol.data(), pol.size() * sizeof(OzPolish), cudaMemcpyHostToDevice, c->st));
+    launch_oz_polish((const OzPolish*)pj.p, (int)pol.size(), max_m, (double*)scr.p, n_cta, c->st);
+    CK(cudaGetLastError());
+    TRY(oz_mats_fill(c, ie, nullptr, false));
+    TRY(oz_run(c, ur.op, ie.op, lo));
+    CK(cudaMemcpyAsync(mj.p, fin.data(), fin.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
+    launch_oz_mats((const OzMat*)mj.p, (int)fin.size(), mr, nv, nullptr, false, ld, (uint16_t*)dmem.p, (int*)emem.p,
+                   c->st);
+    CK(cudaGetLastError());
+    b0 = b1;
+  }
+  c->ud_store.push_back(store);
+  for (int id : pid) c->ud_of[id] = sid;
+  for (Tmp* t : {&dmem, &emem}) {
+    c->ud_alloc.push_back(t->p);
+    t->p = nullptr;
+  }
+  return 0;
+}
+
+// Amplitude iterations of a list of fragments in the FP64 form (solve_oz.cu).  orbs: ascending orbitals of
+// each; results to out[out_id[f]]; raw-basis amplitudes (pairs a <= b in order, m^2 each) to tdst + toff[out_id[f]]
+// unless tdst is NULL; pair_e (host, may be NULL; one fragment): the pair energies.  Fragments in batches that
+// fit the device; OZ_NO_ROOM when one does not, or when a pair has no polished basis.
+// raw: whether the stored amplitudes are those of the raw basis; otherwise Y (r^2) is left in the slot.
+// df: dE/df of each fragment times its weight (launch_oz_df), NULL if not wanted.
+struct OzWant {
+  bool raw = true;
+  double* df = nullptr;             // device [n][9], by out_id
+  const std::vector<Frag>* frags = nullptr;   // by out_id
+};
+int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, const std::vector<int>& out_id, size_t f0,
+                   size_t f1, const SolveOpts& so, double ulps, FragOut* out, double* tdst, const long long* toff,
+                   double* pair_e, const OzWant& want) {
+  const int n = c->sys.n_occ, nv = c->sys.n_vir;
+  struct Term { int p, q, ver; double coef; };     // pairs by index in the batch
+  std::vector<OzPair> pairs;
+  std::vector<int> pid, pair0{0}, oid;
+  std::vector<Term> terms;
+  std::vector<int> term0{0};
+  int max_r = 1, max_m = 1;
+  size_t ysz = 0;
+  for (size_t f = f0; f < f1; f++) {
+    const std::vector<int>& o = orbs[f];
+    const int nc = (int)o.size(), base = (int)pairs.size();
+    auto lp = [&](int a, int b) { return base + a * nc - a * (a - 1) / 2 + (b - a); };
+    size_t toff_p = 0;
+    for (int a = 0; a < nc; a++)
+      for (int b = a; b < nc; b++) {
+        const int i = o[a], j = o[b], id = c->pair_id[(size_t)i * n + j];
+        if (id < 0 || id >= (int)c->ud_of.size() || c->ud_of[id] < 0) return OZ_NO_ROOM;
+        OzPair p{};
+        p.frag = (int)(f - f0);
+        p.r = c->r_h[id];
+        p.m = c->m_h[id];
+        p.diag = a == b;
+        p.kpad = (p.r + oz::BK - 1) / oz::BK * oz::BK;
+        p.ver[0] = p.ver[1] = p.ver[2] = -1;
+        p.fij = c->f_h[(size_t)i * n + i] + c->f_h[(size_t)j * n + j];
+        p.Kt = c->Kt_h[id];
+        p.et = c->et_h[id];
+        p.X = c->X_h[id];
+        p.T = tdst ? tdst + toff[out_id[f]] + toff_p : nullptr;
+        toff_p += (size_t)p.m * p.m;
+        ysz += (size_t)p.r * p.r;
+        max_r = std::max(max_r, p.r);
+        max_m = std::max(max_m, p.m);
+        pairs.push_back(p);
+        pid.push_back(id);
+      }
+    for (int a = 0; a < nc; a++)
+      for (int b = a; b < nc; b++) {
+        const int P = lp(a, b), i = o[a], j = o[b];
+        std::vector<std::array<double, 3>> tq;   // pair, coefficient of Y_q, of Y_q^T
+        auto put = [&](int x, int y, double coef) {
+          if (coef == 0.0) return;
+          const int Q = lp(std::min(x, y), std::max(x, y));
+          for (auto& t : tq)
+            if ((int)t[0] == Q) {
+              t[x > y ? 2 : 1] += coef;
+              return;
+            }
+          tq.push_back({(double)Q, x > y ? 0.0 : coef, x > y ? coef : 0.0});
+        };
+        for (int k = 0; k < nc; k++) {
+          if (k != b) put(a, k, -c->f_h[(size_t)o[k] * n + j]);
+          if (k != a) put(k, b, -c->f_h[(size_t)i * n + o[k]]);
+        }
+        for (auto& t : tq) {
+          const int Q = (int)t[0];
+          if (pairs[Q].diag || t[1] == t[2] || t[1] == 0.0 || t[2] == 0.0) {
+            // one matrix: Y (diagonal pairs: both orders are Y's own), Y^T or Y + Y^T
+            const int v = t[2] == 0.0 ? 0 : (t[1] == 0.0 ? 1 : 2);
+            terms.push_back(Term{P, Q, v, v == 1 ? t[2] : t[1]});
+          } else {
+            terms.push_back(Term{P, Q, 0, t[1]});
+            terms.push_back(Term{P, Q, 1, t[2]});
+          }
+        }
+        term0.push_back((int)terms.size());
+      }
+    pair0.push_back((int)pairs.size());
+    oid.push_back(out_id[f]);
+  }
+  // dE/df: the products of every (k < l, j) of a fragment, as further terms
+  const int nts = (int)terms.size();
+  std::vector<OzDf> dfs;
+  if (want.df)
+    for (size_t f = f0; f < f1; f++) {
+      const int nc = (int)orbs[f].size(), base = pair0[f - f0];
+      auto lp = [&](int x, int y) {
+        const int a = std::min(x, y), b = std::max(x, y);
+        return base + a * nc - a * (a - 1) / 2 + (b - a);
+      };
+      OzDf d{};
+      d.nc = nc;
+      d.pair0 = base;
+      d.out = out_id[f];
+      d.weight = (*want.frags)[out_id[f]].weight;
+      dfs.push_back(d);
+      for (int k = 0; k < nc; k++)
+        for (int l = k + 1; l < nc; l++)
+          for (int j = 0; j < nc; j++) {
+            const int Q = lp(l, j);
+            // <op1(T~_p), op2(T_q)>: one transposition when exactly one of (k, j), (l, j) is reversed
+            const int v = pairs[Q].diag ? 0 : ((k > j) != (l > j) ? 1 : 0);
+            terms.push_back(Term{lp(k, j), Q, v, 1.0});
+          }
+    }
+  const int np = (int)pairs.size(), nfb = (int)(f1 - f0), nt = (int)terms.size();
+  const int LD = (max_r + oz::BK - 1) / oz::BK * oz::BK, nch = oz::n_chunks(max_r);
+  // digit matrices of the amplitudes
+  int nver = 0;
+  long long yrows = 0;
+  for (const Term& t : terms) {
+    OzPair& q = pairs[t.q];
+    if (q.ver[t.ver] < 0) {
+      q.ver[t.ver] = nver++;
+      q.vrow[t.ver] = (int)(yrows * oz::NSL);
+      yrows += q.r;
+    }
+  }
+  // pair-couple overlaps Sigma_(lo,hi), in both orientations
+  struct Couple { int lo, hi; };
+  std::vector<Couple> cps;
+  std::unordered_map<uint64_t, int> cid;
+  std::vector<int> tc(nt);
+  size_t sgsz = 0;
+  std::vector<size_t> sgo;
+  for (int t = 0; t < nt; t++) {
+    const int P = pid[terms[t].p], Q = pid[terms[t].q];
+    const int lo = std::min(P, Q), hi = std::max(P, Q);
+    const uint64_t key = ((uint64_t)lo << 32) | (unsigned)hi;
+    auto it = cid.find(key);
+    if (it == cid.end()) {
+      it = cid.emplace(key, (int)cps.size()).first;
+      cps.push_back(Couple{lo, hi});
+      sgo.push_back(sgsz);
+      sgsz += (size_t)c->r_h[lo] * c->r_h[hi];
+    }
+    tc[t] = it->second;
+  }
+  long long srows = 0;
+  for (const Couple& k : cps) srows += c->r_h[k.lo] + c->r_h[k.hi];
+  if (yrows * oz::NSL + oz::BM >= (long long)INT32_MAX || srows * oz::NSL + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
+  // W: pairs in groups whose digits fit a fixed budget
+  const double wbudget = 8e9;
+  std::vector<int> grp{0};
+  long long wrows = 0, wcur = 0;
+  for (int p = 0; p < np; p++) {
+    const long long w = (long long)(term0[p + 1] - term0[p]) * pairs[p].r;
+    if (p > grp.back() && (double)(wcur + w) * oz::NSL * LD * 2 > wbudget) {
+      grp.push_back(p);
+      wcur = 0;
+    }
+    wcur += w;
+    wrows = std::max(wrows, wcur);
+  }
+  grp.push_back(np);
+  std::vector<int> dgrp{nts};       // the dE/df terms, in groups of their own
+  wcur = 0;
+  for (int t = nts; t < nt; t++) {
+    const long long w = pairs[terms[t].p].r;
+    if (t > dgrp.back() && (double)(wcur + w) * oz::NSL * LD * 2 > wbudget) {
+      dgrp.push_back(t);
+      wcur = 0;
+    }
+    wcur += w;
+    wrows = std::max(wrows, wcur);
+  }
+  dgrp.push_back(nt);
+  if (wrows * oz::NSL + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
+  Tmp yc, yd, yx, wx, wd, sd, sx, sgm, pr, p0, pe, pu, ep, dn, lf, oi, smj;
+  TRY(oz_room(c, yc, 2 * ysz * sizeof(double)));
+  TRY(oz_room(c, yd, (size_t)yrows * oz::NSL * LD * 2));
+  TRY(oz_room(c, yx, (size_t)std::max(1, nver) * nch * sizeof(int)));
+  TRY(oz_room(c, wx, (size_t)std::max(1, nver) * nch * sizeof(int)));
+  TRY(oz_room(c, wd, (size_t)wrows * oz::NSL * LD * 2));
+  TRY(oz_room(c, sd, (size_t)srows * oz::NSL * LD * 2));
+  TRY(oz_room(c, sx, (size_t)srows * nch * sizeof(int)));
+  TRY(oz_room(c, sgm, sgsz * sizeof(double)));
+  TRY(oz_room(c, pr, np * sizeof(OzPair)));
+  TRY(oz_room(c, p0, pair0.size() * sizeof(int)));
+  TRY(oz_room(c, pe, np * sizeof(double)));
+  TRY(oz_room(c, pu, np * sizeof(double)));
+  TRY(oz_room(c, ep, nfb * sizeof(double)));
+  TRY(oz_room(c, dn, nfb * sizeof(int)));
+  TRY(oz_room(c, lf, sizeof(int)));
+  TRY(oz_room(c, oi, nfb * sizeof(int)));
+  TRY(oz_room(c, smj, 2 * std::max<size_t>(1, cps.size()) * sizeof(OzMat)));
+  {
+    size_t off = 0;
+    for (OzPair& p : pairs) {
+      p.Y = p.T && !want.raw ? p.T : (double*)yc.p + off;
+      p.C = (double*)yc.p + ysz + off;
+      off += (size_t)p.r * p.r;
+    }
+  }
+  CK(cudaMemcpyAsync(pr.p, pairs.data(), np * sizeof(OzPair), cudaMemcpyHostToDevice, c->st));
+  CK(cudaMemcpyAsync(p0.p, pair0.data(), pair0.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+  CK(cudaMemcpyAsync(oi.p, oid.data(), nfb * sizeof(int), cudaMemcpyHostToDevice, c->st));
+  CK(cudaMemsetAsync(ep.p, 0, nfb * sizeof(double), c->st));
+  CK(cudaMemsetAsync(dn.p, 0, nfb * sizeof(int), c->st));
+  // overlaps, grouped by the stores of the two bases, then their digits
+  std::vector<oz::Mat> slo(cps.size()), shi(cps.size());
+  if (!cps.empty()) {
+    std::map<std::pair<int, int>, OzList> groups;
+    std::vector<OzMat> m1, m2;
+    long long row = 0;
+    for (size_t u = 0; u < cps.size(); u++) {
+      const int lo = cps[u].lo, hi = cps[u].hi, rl = c->r_h[lo], rh = c->r_h[hi];
+      double* S = (double*)sgm.p + sgo[u];
+      groups[{c->ud_of[lo], c->ud_of[hi]}].product(c->ud_mat[lo], rl, c->ud_mat[hi], rh, nv, S, rh);
+      slo[u] = oz::Mat{(int)(row * oz::NSL), rl, (int)(row * nch), nch};
+      m1.push_back(OzMat{S, rl, rh, (rh + oz::BK - 1) / oz::BK * oz::BK, rh, slo[u]});
+      row += rl;
+      shi[u] = oz::Mat{(int)(row * oz::NSL), rh, (int)(row * nch), nch};
+      m2.push_back(OzMat{S, rh, rl, (rl + oz::BK - 1) / oz::BK * oz::BK, rh, shi[u]});
+      row += rh;
+    }
+    for (auto& g : groups) TRY(oz_run(c, c->ud_store[g.first.first], c->ud_store[g.first.second], g.second));
+    CK(cudaMemcpyAsync(smj.p, m1.data(), m1.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemcpyAsync((OzMat*)smj.p + m1.size(), m2.data(), m2.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
+    launch_oz_mats((const OzMat*)smj.p, (int)m1.size(), max_r, max_r, nullptr, true, LD, (uint16_t*)sd.p, (int*)sx.p, c->st);
+    launch_oz_mats((const OzMat*)smj.p + m1.size(), (int)m2.size(), max_r, max_r, nullptr, false, LD, (uint16_t*)sd.p,
+                   (int*)sx.p, c->st);
+    CK(cudaGetLastError());
+  }
+  const OzOperand So{(const uint16_t*)sd.p, srows * oz::NSL, LD, LD, (const int*)sx.p};
+  const OzOperand Yo{(const uint16_t*)yd.p, std::max<long long>(1, yrows) * oz::NSL, LD, LD, (const int*)yx.p};
+  const OzOperand Wo{(const uint16_t*)wd.p, std::max<long long>(1, wrows) * oz::NSL, LD, LD, (const int*)wx.p};
+  // the two products of every group of pairs
+  const size_t ng = grp.size() - 1;
+  std::vector<OzDev> d1(ng), d2(ng);
+  for (size_t g = 0; g < ng; g++) {
+    OzList l1, l2;
+    long long wrow = 0;
+    for (int p = grp[g]; p < grp[g + 1]; p++) {
+      const OzPair& P = pairs[p];
+      const int first = (int)l2.segs.size();
+      for (int t = term0[p]; t < term0[p + 1]; t++) {
+        const Term& tm = terms[t];
+        const OzPair& Q = pairs[tm.q];
+        const oz::Mat S = pid[p] == cps[tc[t]].lo ? slo[tc[t]] : shi[tc[t]];
+        const int ve = Q.ver[tm.ver] * nch;
+        oz::Job proto{};
+        proto.skip = P.frag;
+        proto.o_row = (int)(wrow * oz::NSL);
+        proto.o_ss = P.r;
+        proto.o_e = ve;
+        const int f1s = (int)l1.segs.size();
+        l1.seg(S, oz::Mat{Q.vrow[tm.ver], Q.r, ve, 0}, Q.r);
+        l1.tiles(f1s, P.r, Q.r, nullptr, 0, proto);
+        l2.seg(S, oz::Mat{(int)(wrow * oz::NSL), P.r, ve, 0}, Q.r, tm.coef);
+        wrow += P.r;
+      }
+      if ((int)l2.segs.size() > first) {
+        oz::Job proto{};
+        proto.skip = P.frag;
+        l2.tiles(first, P.r, P.r, P.C, P.r, proto);
+      }
+    }
+    TRY(oz_upload(c, l1, d1[g]));
+    TRY(oz_upload(c, l2, d2[g]));
+  }
+  CK(cudaMemsetAsync((double*)yc.p + ysz, 0, ysz * sizeof(double), c->st));   // pairs without couplings keep C = 0
+  const int n_cta = std::min(np, 4 * c->num_sms);
+  for (int it = 1; it <= so.max_iter; it++) {
+    if (it > 1)
+      for (size_t g = 0; g < ng; g++) {
+        if (d1[g].n && launch_oz_digits(So, Yo, (const oz::Job*)d1[g].j.p, d1[g].n, (const oz::Seg*)d1[g].s.p,
+                                        (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, c->err_d, c->st))
+          return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
+        if (d2[g].n && launch_oz_gemm(So, Wo, (const oz::Job*)d2[g].j.p, d2[g].n, (const oz::Seg*)d2[g].s.p,
+                                      (const int*)dn.p, c->err_d, c->st))
+          return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
+      }
+    launch_oz_update((const OzPair*)pr.p, np, (const int*)dn.p, it == 1, LD, nch, (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p,
+                     (double*)pe.p, (double*)pu.p, n_cta, c->st);
+    launch_oz_converge((const int*)p0.p, nfb, (const double*)pe.p, (const double*)pu.p, so, ulps, it, (double*)ep.p,
+                       (int*)dn.p, (int*)lf.p, out, (const int*)oi.p, c->st);
+    CK(cudaGetLastError());
+    if (it >= 4 || it == so.max_iter) {      // (a finished fragment's sweeps are skipped on the device, few finish before the fourth)
+      int left = 0;
+      CK(cudaMemcpyAsync(&left, lf.p, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+      CK(cudaStreamSynchronize(c->st));
+      if (!left) break;
+    }
+  }
+  if (want.df) {
+    // W of the dE/df terms, then their dots
+    Tmp parts, dfd;
+    OzList l1, l2;
+    std::vector<std::array<int, 4>> cut;    // first job of l1 and l2 per group
+    long long wrow = 0;
+    int ntile = 0;
+    size_t g = 0;
+    int df = -1, dot = 0, left_dots = 0;
+    for (int t = nts; t < nt; t++) {
+      if (t == dgrp[g]) {
+        cut.push_back({(int)l1.jobs.size(), (int)l2.jobs.size(), 0, 0});
+        wrow = 0;
+        g++;
+      }
+      while (left_dots == 0) {               // next fragment that has dots
+        df++;
+        dot = 0;
+        left_dots = dfs[df].nc * dfs[df].nc * (dfs[df].nc - 1) / 2;
+      }
+      const Term& tm = terms[t];
+      const OzPair &P = pairs[tm.p], &Q = pairs[tm.q];
+      const int ve = Q.ver[tm.ver] * nch;
+      const bool same = pid[tm.p] == pid[tm.q];
+      if (same) return fail(c, OSVMP2_E_STATE, "dE/df: a pair met itself");
+      const oz::Mat S = pid[tm.p] == cps[tc[t]].lo ? slo[tc[t]] : shi[tc[t]];
+      oz::Job proto{};
+      proto.skip = -1;
+      proto.o_row = (int)(wrow * oz::NSL);
+      proto.o_ss = P.r;
+      proto.o_e = ve;
+      const int f1s = (int)l1.segs.size(), f2s = (int)l2.segs.size();
+      l1.seg(S, oz::Mat{Q.vrow[tm.ver], Q.r, ve, 0}, Q.r);
+      l1.tiles(f1s, P.r, Q.r, nullptr, 0, proto);
+      l2.seg(S, oz::Mat{(int)(wrow * oz::NSL), P.r, ve, 0}, Q.r);
+      const size_t j0 = l2.jobs.size();
+      l2.tiles(f2s, P.r, P.r, P.Y, P.r, proto);
+      dfs[df].tile0[dot] = ntile;
+      for (size_t j = j0; j < l2.jobs.size(); j++) l2.jobs[j].o_row = ntile++;
+      dfs[df].tile0[++dot] = ntile;
+      left_dots--;
+      wrow += P.r;
+    }
+    cut.push_back({(int)l1.jobs.size(), (int)l2.jobs.size(), 0, 0});
+    TRY(oz_room(c, parts, (size_t)std::max(1, ntile) * 16 * sizeof(double)));
+    TRY(oz_room(c, dfd, dfs.size() * sizeof(OzDf)));
+    OzDev u1, u2;
+    TRY(oz_upload(c, l1, u1));
+    TRY(oz_upload(c, l2, u2));
+    CK(cudaMemcpyAsync(dfd.p, dfs.data(), dfs.size() * sizeof(OzDf), cudaMemcpyHostToDevice, c->st));
+    for (size_t q = 0; q + 1 < cut.size(); q++) {
+      if (launch_oz_digits(So, Yo, (const oz::Job*)u1.j.p + cut[q][0], cut[q + 1][0] - cut[q][0], (const oz::Seg*)u1.s.p,
+                           (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, c->err_d, c->st) ||
+          launch_oz_dots(So, Wo, (const oz::Job*)u2.j.p + cut[q][1], cut[q + 1][1] - cut[q][1], (const oz::Seg*)u2.s.p,
+                         (double*)parts.p, c->err_d, c->st))
+        return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for dE/df failed");
+    }
+    launch_oz_df((const OzDf*)dfd.p, nfb, (const OzPair*)pr.p, (const double*)parts.p, want.df, std::min(nfb, 4 * c->num_sms),
+                 c->st);
+    CK(cudaGetLastError());
+  }
+  if (tdst && want.raw) {
+    Tmp scr;
+    TRY(oz_room(c, scr, (size_t)n_cta * max_m * max_m * sizeof(double)));
+    launch_oz_raw((const OzPair*)pr.p, np, max_m, (double*)scr.p, n_cta, c->st);
+    CK(cudaGetLastError());
+  }
+  if (pair_e) {
+    CK(cudaMemcpyAsync(pair_e, pe.p, np * sizeof(double), cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+  }
+  return 0;
+}
+
+int oz_solve(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, const std::vector<int>& out_id, const SolveOpts& so,
+             double ulps, FragOut* out, double* tdst, const long long* toff, double* pair_e,
+             const OzWant& want = OzWant{}) {
+  const int n = c->sys.n_occ;
+  // device memory of a fragment: amplitudes and their digits, W and the overlaps
+  std::vector<double> mem(orbs.size(), 0.0);
+  for (size_t f = 0; f < orbs.size(); f++) {
+    const std::vector<int>& o = orbs[f];
+    for (size_t a = 0; a < o.size(); a++)
+      for (size_t b = a; b < o.size(); b++) {
+        const double m = pair_dim_h(c, o[a], o[b]);
+        mem[f] += m * (m + 32.0) * 16.0 * (4.0 + 3.0 * 4.0 * (o.size() - 1) / 2.0);
+      }
+  }
+  (void)n;
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+    cudaGetLastError();
+    fr = (size_t)8 << 30;
+  }
+  double budget = std::min(std::max((double)fr / 3.0, 1e9), 4e10);
+  if (c->opts.mem_cap_mib > 0) budget = std::min(budget, (double)c->opts.mem_cap_mib * 1048576.0 / 2.0);
+  size_t f0 = 0;
+  while (f0 < orbs.size()) {
+    size_t f1 = f0;
+    for (double held = 0.0; f1 < orbs.size() && (f1 == f0 || held + mem[f1] <= budget); f1++) held += mem[f1];
+    const int rc = oz_solve_batch(c, orbs, out_id, f0, f1, so, ulps, out, tdst, toff, pair_e, want);
+    if (rc == OZ_NO_ROOM && f1 - f0 > 1) {     // a smaller batch
+      budget *= 0.5;
+      continue;
+    }
+    if (rc) return rc;
+    f0 = f1;
   }
   return 0;
 }
@@ -1070,12 +1617,11 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
   const int n_warps = std::min<int>((int)pjb.size(), 16 * c->num_sms);
   const int n_cta_pm = std::min<int>((int)pjb.size(), 3 * c->num_sms);
   const bool warp_pc = max_m <= PW_MAX_ORDER;
-  TRY(tmp_alloc(c, scr, std::max({(size_t)n_cta * precond_scratch_doubles(max_m),
-                                  warp_pc ? precond_w_scratch_doubles(max_m, n_warps) : (size_t)0,
-                                  mixed_pc ? precond_mixed_scratch_doubles(max_m, n_cta_pm) : (size_t)0}) *
-                                     sizeof(double)));
+  // Batched preconditioner (precond_mixed.cu): always in the mixed form; in the FP64 form when its work
+  // areas fit, followed by the polish below.  Without room, one warp or CTA per pair in FP64.
   Tmp pm_slots, pm_off, pm_m, pm_order;
-  if (mixed_pc) {
+  bool pm = mixed_pc;
+  {
     std::vector<long long> off(pjb.size());
     std::vector<int> md(pjb.size()), ord(pjb.size());
     long long tot = 0;
@@ -1086,14 +1632,38 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
       ord[q] = (int)q;
     }
     std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return md[a] > md[b]; });
-    TRY(tmp_alloc(c, pm_slots, (size_t)tot * sizeof(double)));
-    TRY(tmp_alloc(c, pm_off, off.size() * sizeof(long long)));
-    TRY(tmp_alloc(c, pm_m, md.size() * sizeof(int)));
-    TRY(tmp_alloc(c, pm_order, ord.size() * sizeof(int)));
-    CK(cudaMemcpyAsync(pm_off.p, off.data(), off.size() * sizeof(long long), cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(pm_m.p, md.data(), md.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(pm_order.p, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+    if (mixed_pc) {
+      TRY(tmp_alloc(c, pm_slots, (size_t)tot * sizeof(double)));
+      TRY(tmp_alloc(c, pm_off, off.size() * sizeof(long long)));
+      TRY(tmp_alloc(c, pm_m, md.size() * sizeof(int)));
+      TRY(tmp_alloc(c, pm_order, ord.size() * sizeof(int)));
+    } else {
+      pm = !oz_room(c, pm_slots, (size_t)tot * sizeof(double)) && !oz_room(c, pm_off, off.size() * sizeof(long long)) &&
+           !oz_room(c, pm_m, md.size() * sizeof(int)) && !oz_room(c, pm_order, ord.size() * sizeof(int));
+    }
+    if (pm) {
+      CK(cudaMemcpyAsync(pm_off.p, off.data(), off.size() * sizeof(long long), cudaMemcpyHostToDevice, c->st));
+      CK(cudaMemcpyAsync(pm_m.p, md.data(), md.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+      CK(cudaMemcpyAsync(pm_order.p, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+    }
   }
+  const size_t scr_pm = precond_mixed_scratch_doubles(max_m, n_cta_pm);
+  const size_t scr_old = std::max((size_t)n_cta * precond_scratch_doubles(max_m),
+                                  warp_pc ? precond_w_scratch_doubles(max_m, n_warps) : (size_t)0);
+  if (mixed_pc || !pm) TRY(tmp_alloc(c, scr, std::max(scr_old, mixed_pc ? scr_pm : (size_t)0) * sizeof(double)));
+  else if (oz_room(c, scr, std::max(scr_pm, (size_t)n_cta * max_m * max_m) * sizeof(double))) {
+    pm = false;
+    TRY(tmp_alloc(c, scr, scr_old * sizeof(double)));
+  }
+  // the FP64 preconditioner without the batched one's work areas
+  auto precond64 = [&]() {
+    if (warp_pc)
+      launch_precond_w(t, c->opts.tau_s, (const PJob*)jp.p, (int)pjb.size(), max_m, (double*)scr.p, n_warps, c->err_d,
+                       c->st);
+    else
+      launch_precond(t, c->opts.tau_s, (const PJob*)jp.p, (int)pjb.size(), max_m, (double*)scr.p, n_cta, c->err_d,
+                     c->st);
+  };
   double f_pc = 0.0;
   for (auto& j : pjb) {
     const double m = pair_dim_h(c, j.i, j.j);
@@ -1106,17 +1676,18 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     }
   }
   ph_begin(c, OSVMP2_PH_PRECOND);
-  if (mixed_pc) {
-    if (launch_precond_mixed(t, c->opts.tau_s, (const PJob*)jp.p, (const int*)pm_order.p, (int)pjb.size(), max_m,
-                             (double*)pm_slots.p, (const long long*)pm_off.p, (const int*)pm_m.p, (double*)scr.p,
-                             n_cta_pm, c->err_d, c->st))
+  if (pm) {
+    const int rc = launch_precond_mixed(t, c->opts.tau_s, (const PJob*)jp.p, (const int*)pm_order.p, (int)pjb.size(), max_m,
+                                        (double*)pm_slots.p, (const long long*)pm_off.p, (const int*)pm_m.p,
+                                        (double*)scr.p, n_cta_pm, c->err_d, !mixed, c->st);
+    if (rc && mixed_pc)
       return fail(c, OSVMP2_E_ARG, "pair order %d exceeds the mixed preconditioner's shared scratch", max_m);
-  } else if (warp_pc)
-    launch_precond_w(t, c->opts.tau_s, (const PJob*)jp.p, (int)pjb.size(), max_m, (double*)scr.p, n_warps, c->err_d,
-                     c->st);
-  else
-    launch_precond(t, c->opts.tau_s, (const PJob*)jp.p, (int)pjb.size(), max_m, (double*)scr.p, n_cta, c->err_d,
-                   c->st);
+    if (rc) pm = false;
+  }
+  if (!pm) {
+    if (!mixed_pc) TRY(tmp_alloc(c, scr, scr_old * sizeof(double)));
+    precond64();
+  }
   ph_end(c, OSVMP2_PH_PRECOND, f_pc);
   CK(cudaGetLastError());
   TRY(check_err_flag(c, "pair integrals"));
@@ -1241,7 +1812,20 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     ph_end(c, OSVMP2_PH_EXCHANGE, f_kg);
     CK(cudaGetLastError());
     TRY(check_err_flag(c, "mixed pair build"));
-  } else {   // K~ = X^T K X (used by the preconditioner-basis solver)
+  } else {   // polished basis, K~ = X^T K X (used by the preconditioner-basis solver)
+    ph_begin(c, OSVMP2_PH_PRECOND);
+    oz = oz_pair_basis(c, newp, max_m);
+    if (oz && oz != OZ_NO_ROOM) return oz;
+    if (oz == OZ_NO_ROOM && pm) {   // no room to polish: bases accurate to FP64 without it
+      tmp_free(pm_slots);
+      TRY(tmp_alloc(c, scr, scr_old * sizeof(double)));
+      precond64();
+      CK(cudaGetLastError());
+      TRY(check_err_flag(c, "pair integrals"));
+      CK(cudaMemcpyAsync(c->r_h.data(), c->r_d, c->r_h.size() * sizeof(int), cudaMemcpyDeviceToHost, c->st));
+      CK(cudaStreamSynchronize(c->st));
+    }
+    ph_end(c, OSVMP2_PH_PRECOND, 0.0);
     std::vector<KtJob> ktj;
     for (size_t q = 0; q < kj.size(); q++) ktj.push_back(KtJob{kj[q].i, kj[q].j, c->Kt_h[c->pair_id[(size_t)kj[q].i * n + kj[q].j]]});
     Tmp jkt;
@@ -1490,7 +2074,7 @@ int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int ns
     }
     l.segs = all.segs;
     OzDev d;
-    TRY(oz_upload(c, l, d));
+    if (int rc = oz_upload(c, l, d)) return rc;
     if (launch_oz_tii(OzOperand{D, (long long)nu * oz::NSL * nv, nx, oz::ld_of(nx), ex}, (const oz::Job*)d.j.p, d.n,
                       (const oz::Seg*)d.s.p, c->sys.e_vir, c->err_d, c->st))
       return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for T_ii failed");
@@ -1718,10 +2302,10 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
     ph_begin(c, OSVMP2_PH_TII);
     if (tii_tc)
       TRY(tii_tensor(c, i0, b, (double*)Tm.p, (float*)Bt.p, nsl, ldx));
-    else if (tii_digits)
-      TRY(tii_oz(c, i0, b, (double*)Tm.p, (uint16_t*)ozD.p, (int*)ozE.p, noz));
-    else
+    else if (int rc = tii_digits ? tii_oz(c, i0, b, (double*)Tm.p, (uint16_t*)ozD.p, (int*)ozE.p, noz) : OZ_NO_ROOM) {
+      if (rc != OZ_NO_ROOM) return rc;
       launch_tii(bsrc(c), s->e_vir, s->f_occ, n, i0, b, (double*)Tm.p, c->st);
+    }
     ph_end(c, OSVMP2_PH_TII, (double)b * nv * (double)nv * s->n_aux, s->B ? 8.0 * b * (double)nv * s->n_aux : 0.0);
     CK(cudaGetLastError());
     ph_begin(c, OSVMP2_PH_EIG);
@@ -1738,7 +2322,7 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
                     "(raise opts.rosv_max_rows)", n_max, i0, i0 + b);
     } else {
       const double nd = nv;
-      const bool full = (nv <= 160) || (l_osv <= 0.0);
+      const bool full = (nv <= 16) || (l_osv <= 0.0);
       const double fl = (double)b * (full ? 9.0 * nd * nd * nd : (4.0 / 3.0) * nd * nd * nd);
       ph_begin(c, OSVMP2_PH_K_EIG);
       launch_eig_osv((double*)Tm.p, b, nv, l_osv, kmax, (double*)Vm.p, (double*)wm.p, (int*)km.p, (double*)sm.p,
@@ -1882,6 +2466,31 @@ int osvmp2_solve(osvmp2_ctx* c, const int32_t* orbs, int32_t n_orbs, osvmp2_prec
     for (int b = a; b < n_orbs; b++) req.push_back({orbs[a], orbs[b]});
   TRY(ensure_pairs(c, req, prec));
   const int np = (int)req.size();
+  if (prec == OSVMP2_FP64) {   // in the preconditioner basis on the tensor cores, when its buffers fit
+    Tmp fo;
+    TRY(tmp_alloc(c, fo, sizeof(FragOut)));
+    CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
+    const SolveOpts so{c->opts.tol_update, c->opts.tol_energy, c->opts.max_iter, 0};
+    std::vector<double> pair_e(np);
+    ph_begin(c, OSVMP2_PH_SUBSOLVE);
+    const int oz = oz_solve(c, {std::vector<int>(orbs, orbs + n_orbs)}, {0}, so, 0.0, (FragOut*)fo.p, nullptr, nullptr,
+                            pair_e.data());
+    ph_end(c, OSVMP2_PH_SUBSOLVE, 0.0);
+    if (oz && oz != OZ_NO_ROOM) return oz;
+    if (!oz) {
+      FragOut h;
+      CK(cudaMemcpyAsync(&h, fo.p, sizeof h, cudaMemcpyDeviceToHost, c->st));
+      TRY(check_err_flag(c, "solve"));
+      if (h.status == ERR_NONFINITE) return fail(c, OSVMP2_E_NUMERIC, "non-finite energy in solve");
+      *e_out = h.energy;
+      if (iters_out) *iters_out = h.iters;
+      if (pair_e_out) std::copy(pair_e.begin(), pair_e.end(), pair_e_out);
+      if (h.status)
+        return fail(c, OSVMP2_E_NOCONV, "solve did not converge in %d iterations (max|update| %.3e)", c->opts.max_iter,
+                    h.umax);
+      return OSVMP2_OK;
+    }
+  }
   size_t tot = 0;
   int max_m = 0;
   for (auto& p : req) {
@@ -2069,8 +2678,10 @@ static int distance_fragments(osvmp2_ctx* c, double r2, double r3, double* e_out
 // MBE(3) energy of the fragments in c->frags; with tstore != NULL the converged
 // amplitudes of every fragment are kept (fragment f at tstore + toff[f], local
 // pairs a<=b in order).
+// y_form (FP64 form, may be NULL): the caller takes the amplitudes as Y in the preconditioner basis; *y_form says
+// whether they are, and dE/df is then in *df.
 static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_stats* stats, Tmp* tstore,
-                     std::vector<long long>* toff) {
+                     std::vector<long long>* toff, bool* y_form = nullptr, Tmp* df = nullptr) {
   const int n = c->sys.n_occ;
   const int nf = (int)c->frags.size();
   std::vector<std::pair<int, int>> req;
@@ -2112,7 +2723,7 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
   TRY(tmp_alloc(c, d_out, nf * sizeof(FragOut)));
   TRY(tmp_alloc(c, d_cnt, sizeof(int)));
   const size_t per_cta = (prec == OSVMP2_MIXED) ? frag_mixed_scratch_doubles(max_m) : frag_scratch_doubles(max_m);
-  TRY(tmp_alloc(c, d_scr, (size_t)n_cta * per_cta * sizeof(double)));
+  if (prec == OSVMP2_MIXED) TRY(tmp_alloc(c, d_scr, (size_t)n_cta * per_cta * sizeof(double)));
   CK(cudaMemcpyAsync(d_orbs.p, orbs_h.data(), orbs_h.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(d_order.p, order.data(), nf * sizeof(int), cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(d_w.p, w_h.data(), nf * sizeof(int), cudaMemcpyHostToDevice, c->st));
@@ -2225,8 +2836,29 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
     ph_end(c, OSVMP2_PH_K_FRAGSOLVE, 0.0);
   } else {
     ph_begin(c, OSVMP2_PH_K_FRAGSOLVE);
-    launch_frag_solve(tables(c), (const int*)d_orbs.p, (const int*)d_order.p, nf, max_m, so, (double*)d_scr.p, n_cta,
-                      (int*)d_cnt.p, (FragOut*)d_out.p, tdst, (const long long*)d_toff.p, c->st);
+    std::vector<std::vector<int>> fo(nf);
+    for (int f = 0; f < nf; f++)
+      for (int u = 0; u < 3; u++)
+        if (c->frags[order[f]].orbs[u] >= 0) fo[f].push_back(c->frags[order[f]].orbs[u]);
+    CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
+    OzWant want;
+    if (y_form) {
+      want.raw = false;
+      if (df) {
+        TRY(tmp_alloc(c, *df, (size_t)nf * 9 * sizeof(double)));
+        want.df = (double*)df->p;
+        want.frags = &c->frags;
+      }
+    }
+    const int oz = oz_solve(c, fo, order, so, 3.5527136788005009e-15, (FragOut*)d_out.p, tdst, tstore ? toff->data() : nullptr,
+                            nullptr, want);
+    if (y_form) *y_form = !oz;
+    if (oz && oz != OZ_NO_ROOM) return oz;
+    if (oz == OZ_NO_ROOM) {   // raw-basis residual, one CTA per fragment on the CUDA cores
+      TRY(tmp_alloc(c, d_scr, (size_t)n_cta * per_cta * sizeof(double)));
+      launch_frag_solve(tables(c), (const int*)d_orbs.p, (const int*)d_order.p, nf, max_m, so, (double*)d_scr.p, n_cta,
+                        (int*)d_cnt.p, (FragOut*)d_out.p, tdst, (const long long*)d_toff.p, c->st);
+    }
     launch_weighted_sum((const FragOut*)d_out.p, (const int*)d_w.p, nf, c->scal_d, c->st);
     ph_end(c, OSVMP2_PH_K_FRAGSOLVE, 0.0);
   }
@@ -2239,7 +2871,7 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
   CK(cudaMemcpyAsync(e_out, c->scal_d, sizeof(double), cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
   ph_collect(c);
-  if (prec == OSVMP2_MIXED) TRY(check_err_flag(c, "mixed fragment solve"));
+  TRY(check_err_flag(c, prec == OSVMP2_MIXED ? "mixed fragment solve" : "fragment solve"));
   double f_solve = 0.0;
   for (int f = 0; f < nf; f++)
     f_solve += (prec == OSVMP2_MIXED) ? fragment_mixed_flops(c, c->frags[f], c->frag_out[f].iters)
@@ -2744,13 +3376,251 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
   return OSVMP2_OK;
 }
 
+// FP64 adjoint on the tensor cores.  W_p = sum_C c T~ and H_p = sum_C c (T~ T^T + [i != j] T~^T T) of every pair in its
+// preconditioner basis (S = 1 there): with T~ = 2 Y - Y^T, H is a sum of products of Y and Y^T over the contributions, one
+// segment each; then both go to the raw OSV basis.  Pairs in batches whose digits fit a fixed budget.
+static int oz_grad_pairs(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plist, const std::vector<GradPairJob>& pjobs,
+                         const std::vector<GradContrib>& con, const GradContrib* d_con, int max_m, double* scr, int n_cta) {
+  const int n = c->sys.n_occ, np = (int)plist.size();
+  int max_r = 1;
+  size_t sz = 0;
+  std::vector<OzGradPair> gp(np);
+  for (int q = 0; q < np; q++) {
+    const int id = c->pair_id[(size_t)plist[q].first * n + plist[q].second], r = c->r_h[id];
+    gp[q] = OzGradPair{r, c->m_h[id], pjobs[q].c0, pjobs[q].c1, c->X_h[id], nullptr, nullptr, pjobs[q].W, pjobs[q].H};
+    max_r = std::max(max_r, r);
+    sz += 2 * (size_t)r * r;
+  }
+  Tmp wh, gd;
+  TRY(oz_room(c, wh, sz * sizeof(double)));
+  TRY(oz_room(c, gd, np * sizeof(OzGradPair)));
+  size_t off = 0;
+  for (OzGradPair& g : gp) {
+    g.Wy = (double*)wh.p + off;
+    g.Hy = g.Wy + (size_t)g.r * g.r;
+    off += 2 * (size_t)g.r * g.r;
+  }
+  CK(cudaMemsetAsync(wh.p, 0, sz * sizeof(double), c->st));     // H of a pair without contributions
+  CK(cudaMemcpyAsync(gd.p, gp.data(), np * sizeof(OzGradPair), cudaMemcpyHostToDevice, c->st));
+  for (int q0 = 0; q0 < np;) {
+    OzMats yn(max_r), yt(max_r);      // rows of Y, rows of Y^T
+    OzList l;
+    int q1 = q0;
+    for (; q1 < np && (q1 == q0 || oz_digit_bytes((size_t)yn.rows, max_r) < ((size_t)2 << 30)); q1++) {
+      const OzGradPair& g = gp[q1];
+      for (int k = g.c0; k < g.c1; k++) {
+        yn.add(con[k].T, g.r, g.r, g.r);
+        yt.add(con[k].T, g.r, g.r, g.r);
+      }
+    }
+    if (yn.mats.empty()) {
+      q0 = q1;
+      continue;
+    }
+    // one store for both, the rows of Y^T after those of Y
+    Tmp D, ex, md;
+    const int nch = oz::n_chunks(max_r), ld = oz::ld_of(max_r);
+    const long long rows = 2 * yn.rows;
+    if (rows * oz::NSL + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
+    TRY(oz_room(c, D, oz_digit_bytes((size_t)rows, max_r)));
+    TRY(oz_room(c, ex, oz_exp_bytes((size_t)rows, max_r)));
+    TRY(oz_room(c, md, 2 * yn.mats.size() * sizeof(OzMat)));
+    for (OzMat& m : yt.mats) {
+      m.m.row += (int)(yn.rows * oz::NSL);
+      m.m.eb += (int)(yn.rows * nch);
+    }
+    CK(cudaMemcpyAsync(md.p, yn.mats.data(), yn.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemcpyAsync((OzMat*)md.p + yn.mats.size(), yt.mats.data(), yt.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice,
+                       c->st));
+    launch_oz_mats((const OzMat*)md.p, (int)yn.mats.size(), max_r, max_r, nullptr, true, ld, (uint16_t*)D.p, (int*)ex.p, c->st);
+    launch_oz_mats((const OzMat*)md.p + yn.mats.size(), (int)yt.mats.size(), max_r, max_r, nullptr, false, ld,
+                   (uint16_t*)D.p, (int*)ex.p, c->st);
+    CK(cudaGetLastError());
+    size_t k0 = 0;
+    for (int q = q0; q < q1; q++) {
+      const OzGradPair& g = gp[q];
+      const int first = (int)l.segs.size();
+      for (int k = g.c0; k < g.c1; k++, k0++) {
+        const oz::Mat &N = yn.mat((int)k0), &T = yt.mat((int)k0);
+        const double w = con[k].weight;
+        l.seg(N, N, g.r, 2.0 * w);                         // 2 Y Y^T - Y^T Y^T
+        l.seg(T, N, g.r, -w);
+        if (plist[q].first != plist[q].second) {           // 2 Y^T Y - Y Y
+          l.seg(T, T, g.r, 2.0 * w);
+          l.seg(N, T, g.r, -w);
+        }
+      }
+      if ((int)l.segs.size() == first) continue;
+      oz::Job proto{};
+      proto.skip = -1;
+      l.tiles(first, g.r, g.r, g.Hy, g.r, proto);
+    }
+    const OzOperand op{(const uint16_t*)D.p, rows * oz::NSL, max_r, ld, (const int*)ex.p};
+    TRY(oz_run(c, op, op, l));
+    q0 = q1;
+  }
+  launch_oz_gsum((const OzGradPair*)gd.p, np, d_con, c->st);
+  launch_oz_graw((const OzGradPair*)gd.p, np, max_m, scr, n_cta, c->st);
+  CK(cudaGetLastError());
+  return 0;
+}
+
+// Y -> T = X Y X^T in place in the amplitude store of all fragments.
+static int raw_amplitudes(osvmp2_ctx* c, double* tstore, const std::vector<long long>& toff, int max_m, double* scr, int n_cta) {
+  const int n = c->sys.n_occ;
+  std::vector<OzPair> pr;
+  for (size_t f = 0; f < c->frags.size(); f++) {
+    double* p = tstore + toff[f];
+    for (int a = 0; a < 3; a++)
+      for (int b = a; b < 3; b++) {
+        const int i = c->frags[f].orbs[a], j = c->frags[f].orbs[b];
+        if (i < 0 || j < 0) continue;
+        const int id = c->pair_id[(size_t)i * n + j];
+        OzPair q{};
+        q.r = c->r_h[id];
+        q.m = c->m_h[id];
+        q.X = c->X_h[id];
+        q.Y = q.T = p;
+        p += (size_t)q.m * q.m;
+        pr.push_back(q);
+      }
+  }
+  Tmp d;
+  TRY(tmp_alloc(c, d, pr.size() * sizeof(OzPair)));
+  CK(cudaMemcpyAsync(d.p, pr.data(), pr.size() * sizeof(OzPair), cudaMemcpyHostToDevice, c->st));
+  launch_oz_raw((const OzPair*)d.p, (int)pr.size(), max_m, scr, n_cta, c->st);
+  CK(cudaGetLastError());
+  return 0;
+}
+
+// dE/dB_o = 4 sum_x Q_x Y_o^(x), Y_o^(x) = rows of W'_p (W or W^T) times P_p^T B_partner, summed over the pairs: the
+// orbitals o in batches whose digits fit a fixed budget.
+static int oz_grad_dB(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plist, const std::vector<GradPairJob>& pjobs,
+                      double* dB) {
+  const int n = c->sys.n_occ, nv = c->sys.n_vir, nx = c->sys.n_aux;
+  int max_n = 1;
+  std::vector<std::vector<int>> of(n);      // pairs of each orbital
+  std::vector<int> at(n, -1);
+  for (size_t q = 0; q < plist.size(); q++) {
+    const int i = plist[q].first, j = plist[q].second;
+    of[i].push_back((int)q);
+    if (i != j) of[j].push_back((int)q);
+    max_n = std::max({max_n, c->n_osv[i], c->n_osv[j]});
+  }
+  // digits of Q (rows a) and of the blocks W_ab (rows of W, rows of W^T)
+  OzMats qd(max_n), wr(max_n), wc(max_n);
+  for (int o = 0; o < n; o++)
+    if (!of[o].empty()) at[o] = qd.add(c->Qp[o], nv, c->n_osv[o], c->n_osv[o]);
+  std::vector<std::array<int, 4>> wid(plist.size());     // [a][b]: rows of block a, k of block b
+  for (size_t q = 0; q < plist.size(); q++) {
+    const int i = plist[q].first, j = plist[q].second, ni = c->n_osv[i], nj = i == j ? 0 : c->n_osv[j], m = ni + nj;
+    for (int a = 0; a < (nj ? 2 : 1); a++)
+      for (int b = 0; b < (nj ? 2 : 1); b++) {
+        const int ra = a ? nj : ni, kb = b ? nj : ni;
+        wid[q][2 * a + b] = wr.add(pjobs[q].W + (size_t)(a ? ni : 0) * m + (b ? ni : 0), ra, m, kb);   // W[a][b]
+        wc.add(pjobs[q].W + (size_t)(b ? ni : 0) * m + (a ? ni : 0), ra, m, kb);                       // W^T[a][b] = W[b][a]^T
+      }
+  }
+  TRY(oz_mats_room(c, qd));
+  TRY(oz_mats_room(c, wr));
+  TRY(oz_mats_room(c, wc));
+  TRY(oz_mats_fill(c, qd, nullptr, true));
+  TRY(oz_mats_fill(c, wr, nullptr, true));
+  TRY(oz_mats_fill(c, wc, nullptr, false));
+  CK(cudaMemsetAsync(dB, 0, (size_t)n * nv * nx * sizeof(double), c->st));
+  auto bt = [&](int a, int x) { return c->bt_h[c->bt_id[(size_t)a * n + x]]; };
+  const size_t budget = (size_t)6 << 30;
+  for (int o0 = 0; o0 < n;) {
+    OzMats bd(max_n), yd(max_n);
+    std::unordered_map<const double*, int> bid;
+    auto badd = [&](const double* p, int k) {
+      auto it = bid.find(p);
+      if (it != bid.end()) return it->second;
+      const int id = bd.add(p, nx, k, k);
+      bid[p] = id;
+      return id;
+    };
+    struct Seg2 { bool tr; int w, b, k; };
+    struct Out { int o, x; std::vector<Seg2> segs; };
+    std::vector<Out> outs;
+    int o1 = o0;
+    for (; o1 < n && (o1 == o0 || oz_digit_bytes((size_t)(bd.rows + (long long)outs.size() * nx), max_n) < budget); o1++) {
+      std::map<int, Out> by_x;
+      for (int q : of[o1]) {
+        const int i = plist[q].first, j = plist[q].second, ni = c->n_osv[i];
+        const int nj = i == j ? 0 : c->n_osv[j];
+        // W' = W for (o, partner) = (i, j), W^T for (j, i); its k blocks meet P_p^T B_partner = [Bt(pt, i) Bt(pt, j)]
+        const bool tr = o1 != i;
+        const int pt = o1 == i ? j : i;
+        for (int a = 0; a < (nj ? 2 : 1); a++) {
+          const int x = a ? j : i;
+          Out& t = by_x[x];
+          t.o = o1;
+          t.x = x;
+          t.segs.push_back(Seg2{tr, wid[q][2 * a], badd(bt(pt, i), ni), ni});
+          if (nj) t.segs.push_back(Seg2{tr, wid[q][2 * a + 1], badd(bt(pt, j), nj), nj});
+        }
+      }
+      for (auto& kv : by_x) outs.push_back(std::move(kv.second));
+    }
+    if (!outs.empty()) {
+      size_t ysz = 0;
+      for (const Out& t : outs) ysz += (size_t)nx * c->n_osv[t.x];
+      Tmp ym;
+      TRY(oz_room(c, ym, ysz * sizeof(double)));
+      TRY(oz_mats_room(c, bd));
+      TRY(oz_mats_fill(c, bd, nullptr, true));
+      // Y^T [aux][n_x], the terms with W and with W^T in one launch each (the second adds)
+      OzList ln, lt, lb;
+      size_t yo = 0;
+      std::vector<double*> yp;
+      for (const Out& t : outs) {
+        double* Y = (double*)ym.p + yo;
+        yo += (size_t)nx * c->n_osv[t.x];
+        yp.push_back(Y);
+        yd.add(Y, nx, c->n_osv[t.x], c->n_osv[t.x]);
+      }
+      CK(cudaMemsetAsync(ym.p, 0, ysz * sizeof(double), c->st));
+      for (size_t u = 0; u < outs.size(); u++)
+        for (int tr = 0; tr < 2; tr++) {
+          OzList& l = tr ? lt : ln;
+          const int first = (int)l.segs.size();
+          for (const Seg2& s : outs[u].segs)
+            if (s.tr == (bool)tr) l.seg(bd.mat(s.b), (tr ? wc : wr).mat(s.w), s.k);
+          if ((int)l.segs.size() == first) continue;
+          oz::Job proto{};
+          proto.skip = -1;
+          proto.s = 1.0;                                   // add to the output
+          l.tiles(first, nx, c->n_osv[outs[u].x], yp[u], c->n_osv[outs[u].x], proto);
+        }
+      TRY(oz_run(c, bd.op, wr.op, ln));
+      TRY(oz_run(c, bd.op, wc.op, lt));
+      TRY(oz_mats_room(c, yd));
+      TRY(oz_mats_fill(c, yd, nullptr, true));
+      for (size_t u = 0; u < outs.size();) {
+        const int o = outs[u].o, first = (int)lb.segs.size();
+        for (; u < outs.size() && outs[u].o == o; u++)
+          lb.seg(qd.mat(at[outs[u].x]), yd.mat((int)u), c->n_osv[outs[u].x], 4.0);
+        oz::Job proto{};
+        proto.skip = -1;
+        lb.tiles(first, nv, nx, dB + (size_t)o * nv * nx, nx, proto);
+      }
+      TRY(oz_run(c, qd.op, yd.op, lb));
+    }
+    o0 = o1;
+  }
+  return 0;
+}
+
 static int energy_grad_impl(osvmp2_ctx* c, double r2, double r3, osvmp2_prec prec, double* e_out, double* dE_dB,
                             double* dE_df, double* dE_de, osvmp2_mbe_stats* stats, bool relaxed, double* gap_out) {
   if (!c) return OSVMP2_E_ARG;
   Tmp tstore;
   std::vector<long long> toff;
   TRY(distance_fragments(c, r2, r3, e_out));
-  TRY(mbe3_core(c, prec, e_out, stats, &tstore, &toff));
+  bool y_form = false;
+  Tmp gfrag;
+  TRY(mbe3_core(c, prec, e_out, stats, &tstore, &toff, prec == OSVMP2_FP64 ? &y_form : nullptr, dE_df ? &gfrag : nullptr));
   const int n = c->sys.n_occ, nv = c->sys.n_vir, nx = c->sys.n_aux;
   const int nf = (int)c->frags.size();
   // unique pairs of the fragment list, each with its (fragment-ordered) contributions
@@ -2800,6 +3670,7 @@ static int energy_grad_impl(osvmp2_ctx* c, double r2, double r3, osvmp2_prec pre
     }
   }
   const Tables t = tables(c);
+  const bool df_done = y_form;      // dE/df per fragment came with the amplitudes
   const int n_cta = std::max(1, std::min(np, 2 * c->num_sms));
   Tmp d_pj, d_cf, scr;
   TRY(tmp_alloc(c, d_pj, pjobs.size() * sizeof(GradPairJob)));
@@ -2816,7 +3687,17 @@ static int energy_grad_impl(osvmp2_ctx* c, double r2, double r3, osvmp2_prec pre
   }
   const bool mixed = prec == OSVMP2_MIXED;
   ph_begin(c, OSVMP2_PH_GRAD);
-  if (mixed)
+  if (y_form) {   // W and H from the amplitudes in the preconditioner basis
+    const int oz = oz_grad_pairs(c, plist, pjobs, cflat, (const GradContrib*)d_cf.p, max_m, (double*)scr.p, n_cta);
+    if (oz && oz != OZ_NO_ROOM) return oz;
+    if (oz == OZ_NO_ROOM || relaxed) {
+      // raw-basis amplitudes (in place) for the CUDA-core adjoint or the OSV response
+      TRY(raw_amplitudes(c, (double*)tstore.p, toff, max_m, (double*)scr.p, n_cta));
+      if (oz) y_form = false;
+    }
+  }
+  if (y_form) {
+  } else if (mixed)
     launch_gradm_pair(t, (const GradPairJob*)d_pj.p, np, (const GradContrib*)d_cf.p, (double*)scr.p, n_cta, max_m,
                       c->st);
   else
@@ -2832,7 +3713,8 @@ static int energy_grad_impl(osvmp2_ctx* c, double r2, double r3, osvmp2_prec pre
       launch_grad_de(t, (const GradPairJob*)d_pj.p, np, (double*)scr.p, n_cta, max_m, (double*)dpair.p, dE_de, c->st);
     CK(cudaGetLastError());
   }
-  Tmp gfrag, d_fptr, d_flist, d_orbs, d_w, d_toff;
+  const bool have_df = !mixed && gfrag.p && df_done;
+  Tmp d_fptr, d_flist, d_orbs, d_w, d_toff;
   if (dE_df) {
     std::vector<int> fptr(n + 1, 0), flist, orbs_h(3 * (size_t)nf), w_h(nf);
     std::vector<std::vector<int>> per(n);
@@ -2847,7 +3729,7 @@ static int energy_grad_impl(osvmp2_ctx* c, double r2, double r3, osvmp2_prec pre
       fptr[k + 1] = fptr[k] + (int)per[k].size();
       for (int f : per[k]) flist.push_back(f);
     }
-    TRY(tmp_alloc(c, gfrag, (size_t)nf * 9 * sizeof(double)));
+    if (!gfrag.p) TRY(tmp_alloc(c, gfrag, (size_t)nf * 9 * sizeof(double)));
     TRY(tmp_alloc(c, d_fptr, fptr.size() * sizeof(int)));
     TRY(tmp_alloc(c, d_flist, std::max<size_t>(1, flist.size()) * sizeof(int)));
     TRY(tmp_alloc(c, d_orbs, orbs_h.size() * sizeof(int)));
@@ -2861,8 +3743,11 @@ static int energy_grad_impl(osvmp2_ctx* c, double r2, double r3, osvmp2_prec pre
     CK(cudaMemcpyAsync(d_toff.p, toff.data(), toff.size() * sizeof(long long), cudaMemcpyHostToDevice, c->st));
     const int n_cta_f = std::max(1, std::min(nf, 2 * c->num_sms));
     Tmp scr_f;
-    TRY(tmp_alloc(c, scr_f, (size_t)n_cta_f * 2 * max_m * max_m * sizeof(double)));
-    if (mixed)
+    if (!have_df) TRY(tmp_alloc(c, scr_f, (size_t)n_cta_f * 2 * max_m * max_m * sizeof(double)));
+    if (have_df)
+      launch_grad_df_reduce(t, (const int*)d_orbs.p, (const double*)gfrag.p, nf, (const int*)d_fptr.p,
+                            (const int*)d_flist.p, dE_df, c->st);
+    else if (mixed)
       launch_gradm_df(t, (const int*)d_orbs.p, (const int*)d_w.p, (const double*)tstore.p,
                       (const long long*)d_toff.p, nf, max_m, (double*)scr_f.p, n_cta_f, (double*)gfrag.p,
                       (const int*)d_fptr.p, (const int*)d_flist.p, dE_df, c->st);
@@ -2925,7 +3810,12 @@ static int energy_grad_impl(osvmp2_ctx* c, double r2, double r3, osvmp2_prec pre
     launch_gradm_dB(nv, nx, (const GradBJob*)d_bj.p, (int)bj.size(), (const GradMBTerm*)d_bt.p, dE_dB, c->st);
     CK(cudaGetLastError());
   }
+  int oz_db = OZ_NO_ROOM;
   if (dE_dB && !mixed) {
+    oz_db = oz_grad_dB(c, plist, pjobs, dE_dB);
+    if (oz_db && oz_db != OZ_NO_ROOM) return oz_db;
+  }
+  if (dE_dB && !mixed && oz_db) {
     // combos (o, x): x = o and every partner of o in the pair list
     std::vector<std::vector<int>> partners(n);
     for (auto& p : plist)

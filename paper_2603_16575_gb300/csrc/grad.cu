@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(NT) k_grad_pair(Tables t, const GradPairJob* _
 // ---- per pair: d_p[a] = (P H_p P^T)_aa
 __global__ void __launch_bounds__(NT) k_grad_de_pair(Tables t, const GradPairJob* __restrict__ jobs, int n_jobs,
                                                      double* scratch, int max_m, double* dpair) {
-  __shared__ double sm[GEMM_SMEM_DOUBLES];
+  __shared__ double sm[GEMM_SMEM_WIDE];
   const int nv = t.n_vir;
   double* M = scratch + (size_t)blockIdx.x * (size_t)nv * max_m;   // P H  [nv][m]
   for (int jid = blockIdx.x; jid < n_jobs; jid += gridDim.x) {
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(NT) k_grad_de_pair(Tables t, const GradPairJob
     P.rows = nv; P.cols = m; P.rs = nv; P.cs = ni;
     P.b[0][0] = P.b[1][0] = Blk{t.Q[jb.i], ni, 0};
     P.b[0][1] = P.b[1][1] = Blk{nj ? t.Q[jb.j] : t.Q[jb.i], nj ? nj : ni, 0};
-    cta_gemm(nv, m, m, 1.0, P, dense_view(jb.H, m, m, m), 0.0, M, m, sm);
+    cta_gemm_a(nv, m, m, 1.0, P, dense_view(jb.H, m, m, m), 0.0, M, m, sm);
     for (int a = threadIdx.x; a < nv; a += NT) {
       double s = 0.0;
       for (int c = 0; c < m; c++) s += M[(size_t)a * m + c] * P.get(a, c);

@@ -140,6 +140,9 @@ int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz:
 // The digits of the output (jobs' o_row, o_ss, o_e) into the store D with row stride ld (a multiple of 32).
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                      const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st);
+// Dot products of (2 Y - Y^T) with the product of every job (see OzEpiDot), 16 partial sums per job.
+int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                   double* parts, int* err, cudaStream_t st);
 // ---- FP64 amplitude iterations on the tensor cores (solve_oz.cu)
 struct OzPolish {        // pair basis refinement
   int m, r;
@@ -169,6 +172,23 @@ void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool fi
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
                         double* e_prev, int* done, int* left, FragOut* out, const int* out_id, cudaStream_t st);
 void launch_oz_raw(const OzPair* pairs, int n_pairs, int max_m, double* scratch, int n_cta, cudaStream_t st);
+struct OzDf {            // dE/df of a fragment of nc <= 3 orbitals
+  int nc, pair0, out;    // its pairs; fragment index of the result
+  int pad;
+  double weight;
+  int tile0[10];         // tiles of dot t: [tile0[t], tile0[t + 1])
+};
+void launch_oz_df(const OzDf* frags, int n_frag, const OzPair* pairs, const double* parts, double* g, int n_cta,
+                  cudaStream_t st);
+struct OzGradPair {      // adjoint of a pair
+  int r, m, c0, c1;      // contributions [c0, c1) (Y of a fragment, its weight)
+  const double* X;
+  double *Wy, *Hy;       // [r][r]
+  double *W, *H;         // [m][m] raw basis
+};
+struct GradContrib;
+void launch_oz_gsum(const OzGradPair* jobs, int n_jobs, const GradContrib* con, cudaStream_t st);
+void launch_oz_graw(const OzGradPair* jobs, int n_jobs, int max_m, double* scratch, int n_cta, cudaStream_t st);
 // cuTensorMapEncodeTiled (NULL if the driver has none)
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
@@ -214,8 +234,9 @@ void launch_precond(const Tables& t, double tau_s, const PJob* jobs, int n_jobs,
 size_t precond_w_scratch_doubles(int max_m, int n_warps);
 int launch_precond_w(const Tables& t, double tau_s, const PJob* jobs, int n_jobs, int max_m, double* scratch,
                      int n_warps, int* err, cudaStream_t st);
-// Mixed form (precond_mixed.cu): block-structured canonical orthogonalisation in
-// FP64, F' diagonalised in FP32, exact leftovers Sh/Gh; -1 if max_m is too large.
+// precond_mixed.cu: block-structured canonical orthogonalisation in FP64, F' diagonalised
+// in FP32 with exact leftovers Sh/Gh (mixed form) or in FP64 (fp64: jobs without Sh; the basis
+// is to be polished afterwards); -1 if max_m is too large.
 // Per-pair intermediates: one slot of precond_mixed_slot_doubles(m) at slots + off[job];
 // mdim[job] = pair order m; order: the jobs in the order the CTAs take them
 // (grid-stride; descending m balances the launch).
@@ -223,7 +244,7 @@ size_t precond_mixed_slot_doubles(int m);
 size_t precond_mixed_scratch_doubles(int max_m, int n_cta);
 int launch_precond_mixed(const Tables& t, double tau_s, const PJob* jobs, const int* order, int n_jobs, int max_m,
                          double* slots, const long long* off, const int* mdim, double* scratch, int n_cta, int* err,
-                         cudaStream_t st);
+                         bool fp64, cudaStream_t st);
 
 // ---- A4-A5 (solve.cu)
 // Fragments: orbs [n][3] (-1 padded, ascending), order[] = processing order.

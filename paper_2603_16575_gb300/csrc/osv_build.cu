@@ -65,6 +65,12 @@ void launch_tii(const BSrc& src, const double* e_vir, const double* f_occ, int n
 
 // ---------------------------------------------------------------- eigen
 constexpr int ZSMEM_MAX = 160;   // Z kept in shared memory up to this order
+// Orders up to this take the full decomposition also when only the eigenpairs above a threshold are wanted:
+// below it the fixed costs of the top-k path (multisection, inverse iteration) are the larger ones.
+constexpr int EIG_FULL_MAX = 16;
+// Full decomposition with Z in shared memory: every eigenpair is wanted and Z fits, or the matrix is tiny.  (One
+// thread chases the bulge there: 46 ms at order 160 against 6 ms for the top-k path.)
+static bool eig_in_smem(int nv, double thr) { return thr > 0.0 ? nv <= EIG_FULL_MAX : nv <= ZSMEM_MAX; }
 constexpr int NT_EIG = 1024;     // threads of the OSV eigen kernel (more loads in flight)
 constexpr int INV_GROUPS = 4;    // warps running the lane-batched inverse iteration (176 n doubles each)
 constexpr int EB_DF_MAXN = 1536; // double-float back-transformation: the vector in registers up to this order
@@ -552,8 +558,8 @@ __global__ void __launch_bounds__(NT_EIG) k_eig_osv(double* T, int nv, double th
 // double-float (whose sweep stages each tile in two halves).
 static int eig_tile_rows(bool dfl_tridiag) { return dfl_tridiag ? 16 : 32; }
 static int eig_tile_warps(int nv, double thr, int rows) {
-  (void)thr;   // the top-k path and the full path with Z in global memory both sweep in tiles
-  if (nv <= ZSMEM_MAX) return 0;
+  // the top-k path and the full path with Z in global memory both sweep in tiles
+  if (eig_in_smem(nv, thr)) return 0;
   const size_t cap = (size_t)224 * 1024 / sizeof(double), base = (size_t)4 * nv + 64, tile = (size_t)rows * 33;
   const int ntw = cap > base ? (int)std::min<size_t>(NT_EIG / 32, (cap - base) / tile) : 0;
   return ntw >= 2 ? ntw : 0;
@@ -561,7 +567,8 @@ static int eig_tile_warps(int nv, double thr, int rows) {
 
 void launch_eig_osv(double* T, int nb, int nv, double thr, int kmax, double* V, double* w, int* k,
                     double* scratch, int* err, bool dfl_tridiag, cudaStream_t st) {
-  const int zsmem = nv <= ZSMEM_MAX;
+  const int zsmem = eig_in_smem(nv, thr);
+  if (nv <= ZSMEM_MAX) dfl_tridiag = false;   // FP64 in both forms at these orders
   size_t smem = (size_t)(4 * nv + 64) * sizeof(double);
   // the full path (thr <= 0) sweeps in FP64 tiles whatever dfl_tridiag says
   const int rows = (thr > 0.0) ? eig_tile_rows(dfl_tridiag) : eig_tile_rows(false);
@@ -575,7 +582,8 @@ void launch_eig_osv(double* T, int nb, int nv, double thr, int kmax, double* V, 
 
 void launch_eig_back(double* T, int nb, int nv, double thr, int kmax, double* V, const int* k, double* scratch,
                      bool dfl_tridiag, cudaStream_t st) {
-  if (nv <= ZSMEM_MAX || !(thr > 0.0)) return;   // the other paths form the eigenvectors in k_eig_osv
+  if (eig_in_smem(nv, thr) || !(thr > 0.0)) return;   // the other paths form the eigenvectors in k_eig_osv
+  if (nv <= ZSMEM_MAX) dfl_tridiag = false;
   const int ntw = eig_tile_warps(nv, thr, eig_tile_rows(dfl_tridiag));
   dim3 grid(nb, (std::min(kmax, nv) + EB_WARPS - 1) / EB_WARPS);
   const size_t ss = eig_osv_scratch_doubles(nv, kmax);

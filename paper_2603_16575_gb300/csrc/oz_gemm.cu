@@ -134,17 +134,19 @@ void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const dou
   }
 }
 
-// out[row][col] (row-major)
+// out[row][col] (row-major), added to what is there when job.s = 1
 struct OzEpiRow {
+  static constexpr bool kWarp = false;
   __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     double* o = static_cast<double*>(jb.out) + (size_t)(jb.m0 + r) * jb.ld_out + jb.n0 + c0;
 #pragma unroll
     for (int u = 0; u < oz::DCOL; u++)
-      if (c0 + u < jb.n_valid) o[u] = v[u];
+      if (c0 + u < jb.n_valid) o[u] = jb.s == 0.0 ? v[u] : o[u] + v[u];
   }
 };
 // T[a][b] = T[b][a] = v / (e_a + e_b - s) for a >= b; out = T_i, s = 2 f_ii
 struct OzEpiT {
+  static constexpr bool kWarp = false;
   const double* e_vir;
   __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     const int a = jb.m0 + r;
@@ -166,6 +168,7 @@ struct OzEpiT {
 // rows per slice), under the exponent code exW[o_e] (a bound of the whole matrix); columns past n_valid up to the
 // next multiple of 16 are written as zeros (up to 32 by the lanes of the last column group).
 struct OzEpiDigits {
+  static constexpr bool kWarp = false;
   uint16_t* D;
   int ld;
   const int* exW;
@@ -193,6 +196,27 @@ struct OzEpiDigits {
         if (tail) *reinterpret_cast<uint4*>(o + s * slice + 16 + 8 * h) = make_uint4(0, 0, 0, 0);
       }
     }
+  }
+};
+
+// <2 Y - Y^T, D> of the tile's part of D (never stored): Y = the r x r matrix at job.out (r = ld_out), one
+// partial sum per drain warp at parts + 16 job.o_row.
+struct OzEpiDot {
+  static constexpr bool kWarp = true;
+  double* parts;
+  __device__ __forceinline__ void warp(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
+    const double* Y = static_cast<const double*>(jb.out);
+    double s = 0.0;
+    if (r < jb.m_valid) {
+      const int a = jb.m0 + r;
+#pragma unroll
+      for (int u = 0; u < oz::DCOL; u++) {
+        const int b = jb.n0 + c0 + u;
+        if (c0 + u < jb.n_valid) s += (2.0 * Y[(size_t)a * jb.ld_out + b] - Y[(size_t)b * jb.ld_out + a]) * v[u];
+      }
+    }
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) parts[(size_t)oz::NDRAIN * jb.o_row + (threadIdx.x >> 5) - 2] = s;
   }
 };
 
@@ -232,6 +256,10 @@ int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, 
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                      const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st) {
   return run(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits{D, ld, exW}, st);
+}
+int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                   double* parts, int* err, cudaStream_t st) {
+  return run(A, B, jobs, n_jobs, segs, nullptr, err, OzEpiDot{parts}, st);
 }
 int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int* err,
                   cudaStream_t st) {

@@ -1,4 +1,5 @@
-// A3 for the mixed form: a basis X of the pair space with X^T F X ~ diag(e~) and
+// A3 of both forms (the FP64 form diagonalises F' in FP64, skips the leftovers and polishes the
+// basis afterwards, solve_oz.cu): a basis X of the pair space with X^T F X ~ diag(e~) and
 // X^T S X ~ 1 (Eq. prec_eig), plus the exact leftovers
 //   S^ = X^T S X - 1,   G^ = (X^T F X - diag(e~)) - (f_ii + f_jj)/2 S^
 // (double-float products, stored FP32: they are ~1e-7) that the mixed fragment solver
@@ -14,7 +15,7 @@
 // the canonical orthogonalisation drops the eigenvalue 1 - sigma_k =
 // mu_k / (1 + sigma_k) below tau_s (1 + sigma_max).  Then F' = Y^T F Y (double-float,
 // entries bounded by the virtual energies whatever the conditioning of Y) is
-// diagonalised in FP32 (F' = W diag(e~) W^T) and X = Y W.  A diagonal pair has
+// diagonalised in FP32 (mixed form) (F' = W diag(e~) W^T) and X = Y W.  A diagonal pair has
 // S_(ii,ii) = Q_i^T Q_i = 1: Y = 1, F' = F_(i,i).
 //
 // Launches (CTA kernels take one pair per CTA, grid-stride over the pairs in
@@ -24,7 +25,7 @@
 //   (1c) recorded rotations applied to Z, kept directions, Y, Z^T C Z (CTA; the
 //        products with Z in double-float);
 //   (2)  F' = Y^T F Y (tiled double-float GEMMs, CTA);
-//   (3a-c) the same three steps for the FP32 eigen-decomposition of F';
+//   (3a-c) the same three steps for the eigen-decomposition of F' (FP32, or FP64);
 //   (4)  X = Y W and the leftovers (tiled double-float GEMMs, CTA).
 // C and its eigen-decomposition stay FP64: C = 1 - M^T M cancels, and its small
 // eigenvalues set both the kept directions and Z.  The products with Z, Y and W
@@ -260,15 +261,16 @@ __global__ void __launch_bounds__(NT, 2) k_pm_fprime(Tables t, const PJob* __res
   }
 }
 
-// (3a) F' symmetrised in FP32, tridiagonalised, Z of the reflectors
-__global__ void __launch_bounds__(NT, 3) k_pm_eig32_a(const PJob* __restrict__ jobs, const int* __restrict__ order,
-                                                      int n_jobs, double* slots, const long long* off,
-                                                      const int* mdim, int max_m, double* scratch) {
-  extern __shared__ float esmf[];   // eigen-solver scratch: 4 max_m + 33 floats
-  float* esm = esmf;
+// (3a) F' symmetrised (in FP32 for the mixed form), tridiagonalised, Z of the reflectors
+template <class T>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2)
+    k_pm_eig_a(const PJob* __restrict__ jobs, const int* __restrict__ order, int n_jobs, double* slots,
+               const long long* off, const int* mdim, int max_m, double* scratch) {
+  extern __shared__ double esm_raw[];   // eigen-solver scratch: 4 max_m + 33 elements
+  T* esm = reinterpret_cast<T*>(esm_raw);
   const size_t M2 = (size_t)max_m * max_m;
-  float* A32 = reinterpret_cast<float*>(scratch + (size_t)blockIdx.x * pm_cta_doubles(max_m));
-  float* tau32 = A32 + M2;
+  T* A = reinterpret_cast<T*>(scratch + (size_t)blockIdx.x * pm_cta_doubles(max_m));
+  T* tau = A + M2;
   for (int q = blockIdx.x; q < n_jobs; q += gridDim.x) {
     const int jid = order[q];
     const PJob jb = jobs[jid];
@@ -276,39 +278,40 @@ __global__ void __launch_bounds__(NT, 3) k_pm_eig32_a(const PJob* __restrict__ j
     const PmPair pp = pm_pair(slots, off, jid, m);
     for (int idx = threadIdx.x; idx < r * r; idx += NT) {
       const int a = idx / r, b = idx % r;
-      A32[idx] = (float)(0.5 * (pp.Fp[idx] + pp.Fp[(size_t)b * r + a]));
+      A[idx] = (T)(0.5 * (pp.Fp[idx] + pp.Fp[(size_t)b * r + a]));
     }
     __syncthreads();
-    pm_tridiag(A32, r, pm_eig<float>(pp.wk, m), tau32, esm);
+    pm_tridiag(A, r, pm_eig<T>(pp.wk, m), tau, esm);
   }
 }
 
 // (3c) eig(F') completed: W, e~
-__global__ void __launch_bounds__(NT, 3) k_pm_eig32_c(const PJob* __restrict__ jobs, const int* __restrict__ order,
-                                                      int n_jobs, double* slots, const long long* off,
-                                                      const int* mdim, int max_m, double* scratch, int* err) {
-  extern __shared__ float esmf[];   // eigen-solver scratch: 4 max_m + 33 floats
-  float* esm = esmf;
+template <class T>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2)
+    k_pm_eig_c(const PJob* __restrict__ jobs, const int* __restrict__ order, int n_jobs, double* slots,
+               const long long* off, const int* mdim, int max_m, double* scratch, int* err) {
+  extern __shared__ double esm_raw[];   // eigen-solver scratch: 4 max_m + 33 elements
+  T* esm = reinterpret_cast<T*>(esm_raw);
   const size_t M2 = (size_t)max_m * max_m;
-  float* A32 = reinterpret_cast<float*>(scratch + (size_t)blockIdx.x * pm_cta_doubles(max_m));
-  float* e32 = A32 + M2;        // in-CTA solve of a pair whose chase record overflowed
-  float* eb = e32 + max_m;
-  float* tau32 = eb + max_m;
+  T* A = reinterpret_cast<T*>(scratch + (size_t)blockIdx.x * pm_cta_doubles(max_m));
+  T* ew = A + M2;               // in-CTA solve of a pair whose chase record overflowed
+  T* eb = ew + max_m;
+  T* tau = eb + max_m;
   for (int q = blockIdx.x; q < n_jobs; q += gridDim.x) {
     const int jid = order[q];
     const PJob jb = jobs[jid];
     const int m = mdim[jid], r = *jb.r;
     const PmPair pp = pm_pair(slots, off, jid, m);
-    const PmEig<float> w = pm_eig<float>(pp.wk, m);
-    const float* ev = w.d;
+    const PmEig<T> w = pm_eig<T>(pp.wk, m);
+    const T* ev = w.d;
     if (w.hdr[0] == 2) {
       for (int idx = threadIdx.x; idx < r * r; idx += NT) {
         const int a = idx / r, b = idx % r;
-        A32[idx] = (float)(0.5 * (pp.Fp[idx] + pp.Fp[(size_t)b * r + a]));
+        A[idx] = (T)(0.5 * (pp.Fp[idx] + pp.Fp[(size_t)b * r + a]));
       }
       __syncthreads();
-      if (cta_syev_cm(A32, r, r, e32, w.Z, r, eb, tau32, esm) && threadIdx.x == 0) atomicOr(err, ERR_EIG);
-      ev = e32;
+      if (cta_syev_cm(A, r, r, ew, w.Z, r, eb, tau, esm) && threadIdx.x == 0) atomicOr(err, ERR_EIG);
+      ev = ew;
     } else {
       apply_qr_record_cm(w.Z, r, r, w.swp, w.hdr[1], w.rot);
     }
@@ -316,7 +319,10 @@ __global__ void __launch_bounds__(NT, 3) k_pm_eig32_c(const PJob* __restrict__ j
       const int tv = idx / r, a = idx % r;
       pp.W[(size_t)a * r + tv] = (double)w.Z[idx];
     }
-    for (int c = threadIdx.x; c < r; c += NT) pp.et[c] = (double)ev[c];
+    for (int c = threadIdx.x; c < r; c += NT) {
+      pp.et[c] = (double)ev[c];
+      if (!isfinite((double)ev[c])) atomicOr(err, ERR_NONFINITE);
+    }
     __syncthreads();
   }
 }
@@ -346,12 +352,19 @@ __global__ void __launch_bounds__(NT, 2) k_pm_final(Tables t, const PJob* __rest
     const View Wv = dense_view(pp.W, r, r, r);
     if (i != j) {
       cta_gemm_df(m, r, r, 1.0, dense_view(pp.Y, m, r, r), Wv, 0.0, jb.X, m, sm);       // X = Y W
-      for (int idx = threadIdx.x; idx < ni * r; idx += NT) T1[idx] = pp.W[idx];        // (Y^T S Y) W, top rows
-      cta_gemm_df(nk, r, nk, 1.0, dense_view(pp.ZCZ, nk, nk, nk), dense_view(pp.W + (size_t)ni * r, nk, r, r), 0.0,
-               T1 + (size_t)ni * r, r, sm);
+      if (jb.Sh) {
+        for (int idx = threadIdx.x; idx < ni * r; idx += NT) T1[idx] = pp.W[idx];      // (Y^T S Y) W, top rows
+        cta_gemm_df(nk, r, nk, 1.0, dense_view(pp.ZCZ, nk, nk, nk), dense_view(pp.W + (size_t)ni * r, nk, r, r), 0.0,
+                    T1 + (size_t)ni * r, r, sm);
+      }
     } else {
       for (int idx = threadIdx.x; idx < m * r; idx += NT) jb.X[(size_t)(idx / r) * m + idx % r] = pp.W[idx];
-      cta_gemm_df(r, r, r, 1.0, dense_view(t.S[t.sf_id[i * n + i]], ni, ni, ni), Wv, 0.0, T1, r, sm);
+      if (jb.Sh) cta_gemm_df(r, r, r, 1.0, dense_view(t.S[t.sf_id[i * n + i]], ni, ni, ni), Wv, 0.0, T1, r, sm);
+    }
+    for (int c = threadIdx.x; c < r; c += NT) jb.et[c] = pp.et[c];
+    if (!jb.Sh) {               // FP64 form: the basis is polished afterwards (solve_oz.cu)
+      __syncthreads();
+      continue;
     }
     cta_gemm_df(r, r, r, 1.0, transpose(Wv), dense_view(T1, r, r, r), 0.0, St, r, sm);      // S~
     cta_gemm_df(r, r, r, 1.0, dense_view(pp.Fp, r, r, r), Wv, 0.0, T1, r, sm);
@@ -365,7 +378,6 @@ __global__ void __launch_bounds__(NT, 2) k_pm_final(Tables t, const PJob* __rest
       jb.Gh[idx] = (float)gh;
       if (!isfinite(sh) || !isfinite(gh)) atomicOr(err, ERR_NONFINITE);
     }
-    for (int c = threadIdx.x; c < r; c += NT) jb.et[c] = pp.et[c];
     __syncthreads();
   }
 }
@@ -374,29 +386,37 @@ size_t precond_mixed_slot_doubles(int m) { return pm_slot_doubles(m); }
 
 size_t precond_mixed_scratch_doubles(int max_m, int n_cta) { return (size_t)n_cta * pm_cta_doubles(max_m); }
 
-int launch_precond_mixed(const Tables& t, double tau_s, const PJob* jobs, const int* order, int n_jobs, int max_m,
-                         double* slots, const long long* off, const int* mdim, double* scratch, int n_cta, int* err,
-                         cudaStream_t st) {
-  if (!n_jobs) return 0;
+template <class T>
+static int run_precond(const Tables& t, double tau_s, const PJob* jobs, const int* order, int n_jobs, int max_m,
+                       double* slots, const long long* off, const int* mdim, double* scratch, int n_cta, int* err,
+                       cudaStream_t st) {
   const size_t sm_d = ((size_t)4 * max_m + 33) * sizeof(double) + (size_t)max_m * sizeof(int);
-  const size_t sm_f = ((size_t)4 * max_m + 33) * sizeof(float);
+  const size_t sm_t = ((size_t)4 * max_m + 33) * sizeof(T);
   if (sm_d > 160 * 1024) return -1;
   if (cudaFuncSetAttribute(k_pm_overlap_a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_d) != cudaSuccess ||
       cudaFuncSetAttribute(k_pm_overlap_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_d) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_eig32_a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_f) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_eig32_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_f) != cudaSuccess)
+      cudaFuncSetAttribute(k_pm_eig_a<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_t) != cudaSuccess ||
+      cudaFuncSetAttribute(k_pm_eig_c<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_t) != cudaSuccess)
     return -1;
   const int n_chase = (n_jobs + 31) / 32;
   k_pm_overlap_a<<<n_cta, NT, sm_d, st>>>(t, jobs, order, n_jobs, slots, off, max_m, scratch);
   k_pm_chase<double><<<n_chase, 32, 0, st>>>(t, jobs, order, n_jobs, slots, off, mdim, 0, err);
   k_pm_overlap_c<<<n_cta, NT, sm_d, st>>>(t, tau_s, jobs, order, n_jobs, slots, off, max_m, scratch, err);
   k_pm_fprime<<<n_cta, NT, 0, st>>>(t, jobs, order, n_jobs, slots, off, max_m, scratch);
-  k_pm_eig32_a<<<n_cta, NT, sm_f, st>>>(jobs, order, n_jobs, slots, off, mdim, max_m, scratch);
-  k_pm_chase<float><<<n_chase, 32, 0, st>>>(t, jobs, order, n_jobs, slots, off, mdim, 1, err);
-  k_pm_eig32_c<<<n_cta, NT, sm_f, st>>>(jobs, order, n_jobs, slots, off, mdim, max_m, scratch, err);
+  k_pm_eig_a<T><<<n_cta, NT, sm_t, st>>>(jobs, order, n_jobs, slots, off, mdim, max_m, scratch);
+  k_pm_chase<T><<<n_chase, 32, 0, st>>>(t, jobs, order, n_jobs, slots, off, mdim, 1, err);
+  k_pm_eig_c<T><<<n_cta, NT, sm_t, st>>>(jobs, order, n_jobs, slots, off, mdim, max_m, scratch, err);
   k_pm_final<<<n_cta, NT, 0, st>>>(t, jobs, order, n_jobs, slots, off, max_m, scratch, err);
   note_launch(8);
   return 0;
+}
+
+int launch_precond_mixed(const Tables& t, double tau_s, const PJob* jobs, const int* order, int n_jobs, int max_m,
+                         double* slots, const long long* off, const int* mdim, double* scratch, int n_cta, int* err,
+                         bool fp64, cudaStream_t st) {
+  if (!n_jobs) return 0;
+  return fp64 ? run_precond<double>(t, tau_s, jobs, order, n_jobs, max_m, slots, off, mdim, scratch, n_cta, err, st)
+              : run_precond<float>(t, tau_s, jobs, order, n_jobs, max_m, slots, off, mdim, scratch, n_cta, err, st);
 }
 
 }  // namespace osv

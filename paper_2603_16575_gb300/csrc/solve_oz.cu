@@ -182,7 +182,8 @@ void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const do
   note_launch(1);
 }
 
-// T_p = X_p Y_p X_p^T of the listed pairs (the gradient and the weak pairs use the raw OSV basis).
+// T_p = X_p Y_p X_p^T of the listed pairs (the weak pairs and the OSV response use the raw OSV basis); T may
+// be Y's own storage.
 __global__ void __launch_bounds__(NT) k_oz_raw(const OzPair* __restrict__ pairs, int n_pairs, int max_m,
                                                double* scratch) {
   __shared__ double sm[GEMM_SMEM_WIDE];
@@ -197,6 +198,91 @@ __global__ void __launch_bounds__(NT) k_oz_raw(const OzPair* __restrict__ pairs,
 void launch_oz_raw(const OzPair* pairs, int n_pairs, int max_m, double* scratch, int n_cta, cudaStream_t st) {
   if (!n_pairs) return;
   k_oz_raw<<<n_cta, NT, 0, st>>>(pairs, n_pairs, max_m, scratch);
+  note_launch(1);
+}
+
+// ---------------------------------------------------------------- adjoint in the preconditioner basis
+// dE/df of a fragment, -sum_j <T~_kj, T_lj> - sum_i <T~_il, T_ik> = -2 sum_j <T~_kj, T_lj> (the second sum is the
+// transpose of the first): for k != l the products Sigma_pq op(Y_q) Sigma_pq^T of a coupling, dotted with
+// 2 Y_p - Y_p^T by the contraction's epilogue (each of a fragment's nine (k < l, j) once); for k = l the dots of the
+// pairs with themselves, formed here.  One CTA per fragment.
+__global__ void __launch_bounds__(NT) k_oz_df(const OzDf* __restrict__ frags, int n_frag,
+                                              const OzPair* __restrict__ pairs, const double* __restrict__ parts,
+                                              double* __restrict__ g) {
+  __shared__ double red[40];
+  __shared__ double self[6];
+  for (int f = blockIdx.x; f < n_frag; f += gridDim.x) {
+    const OzDf d = frags[f];
+    const int np = d.nc * (d.nc + 1) / 2;
+    for (int p = 0; p < np; p++) {
+      const OzPair pr = pairs[d.pair0 + p];
+      double s = 0.0;
+      for (int idx = threadIdx.x; idx < pr.r * pr.r; idx += NT)
+        s += (2.0 * pr.Y[idx] - pr.Y[(size_t)(idx % pr.r) * pr.r + idx / pr.r]) * pr.Y[idx];
+      s = cta_sum(s, red);
+      if (threadIdx.x == 0) self[p] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double* out = g + (size_t)d.out * 9;
+      int t = 0;   // dots in the order (k < l), j
+      for (int k = 0; k < d.nc; k++)
+        for (int l = k; l < d.nc; l++) {
+          double s = 0.0;
+          for (int j = 0; j < d.nc; j++) {
+            if (k == l) {
+              const int a = min(k, j), b = max(k, j);
+              s += self[a * d.nc - a * (a - 1) / 2 + (b - a)];
+            } else {
+              for (int q = d.tile0[t]; q < d.tile0[t + 1]; q++)
+                for (int u = 0; u < 16; u++) s += parts[(size_t)16 * q + u];
+              t++;
+            }
+          }
+          out[k * 3 + l] = out[l * 3 + k] = -2.0 * d.weight * s;
+        }
+    }
+    __syncthreads();
+  }
+}
+void launch_oz_df(const OzDf* frags, int n_frag, const OzPair* pairs, const double* parts, double* g, int n_cta,
+                  cudaStream_t st) {
+  if (!n_frag) return;
+  k_oz_df<<<n_cta, NT, 0, st>>>(frags, n_frag, pairs, parts, g);
+  note_launch(1);
+}
+
+// W_p = sum_C c_C (2 Y - Y^T) over the contributions of each pair.
+__global__ void __launch_bounds__(NT) k_oz_gsum(const OzGradPair* __restrict__ jobs, const GradContrib* __restrict__ con) {
+  const OzGradPair jb = jobs[blockIdx.x];
+  const int r = jb.r;
+  for (int idx = blockIdx.y * NT + threadIdx.x; idx < r * r; idx += gridDim.y * NT) {
+    const int tr = (idx % r) * r + idx / r;
+    double s = 0.0;
+    for (int q = jb.c0; q < jb.c1; q++) s += con[q].weight * (2.0 * con[q].T[idx] - con[q].T[tr]);
+    jb.Wy[idx] = s;
+  }
+}
+void launch_oz_gsum(const OzGradPair* jobs, int n_jobs, const GradContrib* con, cudaStream_t st) {
+  if (!n_jobs) return;
+  k_oz_gsum<<<dim3(n_jobs, 8), NT, 0, st>>>(jobs, con);
+  note_launch(1);
+}
+// W = X W_y X^T and H = X H_y X^T.
+__global__ void __launch_bounds__(NT) k_oz_graw(const OzGradPair* __restrict__ jobs, int n_jobs, int max_m,
+                                                double* scratch) {
+  __shared__ double sm[GEMM_SMEM_WIDE];
+  double* A = scratch + (size_t)blockIdx.x * max_m * max_m;
+  for (int q = blockIdx.x; q < 2 * n_jobs; q += gridDim.x) {
+    const OzGradPair p = jobs[q >> 1];
+    const View Xv = dense_view(p.X, p.m, p.r, p.m);
+    cta_gemm_a(p.m, p.r, p.r, 1.0, Xv, dense_view((q & 1) ? p.Hy : p.Wy, p.r, p.r, p.r), 0.0, A, p.r, sm);
+    cta_gemm_a(p.m, p.m, p.r, 1.0, dense_view(A, p.m, p.r, p.r), transpose(Xv), 0.0, (q & 1) ? p.H : p.W, p.m, sm);
+  }
+}
+void launch_oz_graw(const OzGradPair* jobs, int n_jobs, int max_m, double* scratch, int n_cta, cudaStream_t st) {
+  if (!n_jobs) return;
+  k_oz_graw<<<n_cta, NT, 0, st>>>(jobs, n_jobs, max_m, scratch);
   note_launch(1);
 }
 

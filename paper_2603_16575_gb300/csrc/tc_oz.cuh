@@ -77,7 +77,9 @@ __device__ __forceinline__ double oz_fma(long long v, int x, double coef, double
   return fma(coef, ldexp((double)v, x), acc);
 }
 
-// Epi: epi(job, row, col0, acc) stores columns col0 .. col0 + 15 of the tile's row (row < m_valid).
+// Epi: epi(job, row, col0, acc) stores columns col0 .. col0 + 15 of the tile's row (row < m_valid); or, when
+// Epi::kWarp, epi.warp(job, row, col0, acc) called by every lane of a drain warp, tiles without rows or columns
+// for it included.
 template <class Epi>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_oz(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const int* __restrict__ exA,
@@ -261,7 +263,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
       }
       if (!ok) break;
-      if (row < jb.m_valid && live) epi(jb, row, col0, acc);
+      if constexpr (Epi::kWarp) epi.warp(jb, row, col0, acc);
+      else if (row < jb.m_valid && live) epi(jb, row, col0, acc);
     }
   }
   if (!ok) atomicOr(err, ERR_TC_TIMEOUT);
