@@ -120,6 +120,7 @@ struct osvmp2_ctx {
   int us_ldv = 0;
   // FP64 form: digits of U_p (polished basis) of each pair: store of its build and matrix in it (-1: none)
   std::vector<void*> ud_alloc;
+  std::vector<char> pm_basis;        // FP64 form: pair bases from the batched preconditioner
   std::vector<OzOperand> ud_store;
   std::vector<int> ud_of;
   std::vector<oz::Mat> ud_mat;
@@ -299,6 +300,7 @@ void free_system(osvmp2_ctx* c) {
   for (void* p : c->pair_allocs) pool_put(c, p);
   c->pair_allocs.clear();
   drop_basis_digits(c);
+  c->pm_basis.clear();
   c->pair_prec = -1;
   c->have_sys = c->have_osv = false;
   c->n_osv.clear(); c->Qp.clear(); c->Wp.clear();
@@ -509,6 +511,7 @@ int reset_pairs(osvmp2_ctx* c) {
   for (void* p : c->pair_allocs) pool_put(c, p);
   c->pair_allocs.clear();
   drop_basis_digits(c);
+  c->pm_basis.clear();
   const size_t nn = (size_t)c->sys.n_occ * c->sys.n_occ;
   c->sf_id.assign(nn, -1);
   c->pair_id.assign(nn, -1);
@@ -1816,6 +1819,10 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     ph_begin(c, OSVMP2_PH_PRECOND);
     oz = oz_pair_basis(c, newp, max_m);
     if (oz && oz != OZ_NO_ROOM) return oz;
+    if (pm && oz != OZ_NO_ROOM) {
+      c->pm_basis.resize(c->K_h.size(), 0);
+      for (auto& p : newp) c->pm_basis[c->pair_id[(size_t)p.first * n + p.second]] = 1;
+    }
     if (oz == OZ_NO_ROOM && pm) {   // no room to polish: bases accurate to FP64 without it
       tmp_free(pm_slots);
       TRY(tmp_alloc(c, scr, scr_old * sizeof(double)));
@@ -2442,6 +2449,28 @@ int osvmp2_get_precond(osvmp2_ctx* c, int32_t i, int32_t j, double* X, double* e
   const int pid = c->pair_id[(size_t)i * n + j];
   if (pid < 0) return fail(c, OSVMP2_E_STATE, "pair (%d,%d) not built", i, j);
   const int m = c->m_h[pid];
+  if (c->pair_prec == OSVMP2_FP64 && c->r_h[pid] < m && pid < (int)c->pm_basis.size() && c->pm_basis[pid]) {
+    // A dependent pair space: the coefficients of a basis are not unique, and the batched preconditioner's are
+    // not the shortest ones.  Hand out those of the canonical orthogonalisation of S.
+    Tmp xb, scr, jd;
+    TRY(tmp_alloc(c, xb, ((size_t)m * m + m + 1) * sizeof(double)));
+    TRY(tmp_alloc(c, scr, precond_scratch_doubles(m) * sizeof(double)));
+    TRY(tmp_alloc(c, jd, sizeof(PJob)));
+    double* xp = (double*)xb.p;
+    const PJob job{i, j, xp, xp + (size_t)m * m, (int*)(xp + (size_t)m * m + m), nullptr, nullptr};
+    CK(cudaMemcpyAsync(jd.p, &job, sizeof job, cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
+    CK(cudaMemsetAsync(xb.p, 0, ((size_t)m * m + m + 1) * sizeof(double), c->st));
+    launch_precond(tables(c), c->opts.tau_s, (const PJob*)jd.p, 1, m, (double*)scr.p, 1, c->err_d, c->st);
+    CK(cudaGetLastError());
+    int r = 0;
+    CK(cudaMemcpyAsync(&r, job.r, sizeof r, cudaMemcpyDeviceToHost, c->st));
+    if (X) CK(cudaMemcpyAsync(X, job.X, (size_t)m * m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
+    if (et) CK(cudaMemcpyAsync(et, job.et, (size_t)m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
+    TRY(check_err_flag(c, "preconditioner"));
+    if (r_out) *r_out = r;
+    return OSVMP2_OK;
+  }
   if (X) CK(cudaMemcpyAsync(X, c->X_h[pid], (size_t)m * m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
   if (et) CK(cudaMemcpyAsync(et, c->et_h[pid], (size_t)m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
   CK(cudaStreamSynchronize(c->st));
