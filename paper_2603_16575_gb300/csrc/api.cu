@@ -981,16 +981,18 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
     TRY(oz_mats_room(c, ie));
     TRY(oz_mats_fill(c, xs, nullptr, false));
     TRY(oz_run(c, q.op, xs.op, lu));
-    TRY(oz_mats_fill(c, uc, nullptr, false));
-    TRY(oz_mats_fill(c, ue, c->sys.e_vir, false));
-    TRY(oz_mats_fill(c, ur, nullptr, true));
-    TRY(oz_run(c, uc.op, uc.op, ls));
-    TRY(oz_run(c, ue.op, uc.op, lf));
     CK(cudaMemcpyAsync(pj.p, pol.data(), pol.size() * sizeof(OzPolish), cudaMemcpyHostToDevice, c->st));
-    launch_oz_polish((const OzPolish*)pj.p, (int)pol.size(), max_m, (double*)scr.p, n_cta, c->st);
-    CK(cudaGetLastError());
-    TRY(oz_mats_fill(c, ie, nullptr, false));
-    TRY(oz_run(c, ur.op, ie.op, lo));
+    for (int step = 0; step < 3; step++) {
+      TRY(oz_mats_fill(c, uc, nullptr, false));
+      TRY(oz_mats_fill(c, ue, c->sys.e_vir, false));
+      TRY(oz_mats_fill(c, ur, nullptr, true));
+      TRY(oz_run(c, uc.op, uc.op, ls));
+      TRY(oz_run(c, ue.op, uc.op, lf));
+      launch_oz_polish((const OzPolish*)pj.p, (int)pol.size(), max_m, (double*)scr.p, n_cta, c->st);
+      CK(cudaGetLastError());
+      TRY(oz_mats_fill(c, ie, nullptr, false));
+      TRY(oz_run(c, ur.op, ie.op, lo));
+    }
     CK(cudaMemcpyAsync(mj.p, fin.data(), fin.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
     launch_oz_mats((const OzMat*)mj.p, (int)fin.size(), mr, nv, nullptr, false, ld, (uint16_t*)dmem.p, (int*)emem.p,
                    c->st);
@@ -1623,6 +1625,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
   // Batched preconditioner (precond_mixed.cu): always in the mixed form; in the FP64 form when its work
   // areas fit, followed by the polish below.  Without room, one warp or CTA per pair in FP64.
   Tmp pm_slots, pm_off, pm_m, pm_order;
+  std::vector<int> pm_sorted;       // pair orders as the kernels take them
   bool pm = mixed_pc;
   {
     std::vector<long long> off(pjb.size());
@@ -1635,6 +1638,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
       ord[q] = (int)q;
     }
     std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return md[a] > md[b]; });
+    for (int q : ord) pm_sorted.push_back(md[q]);
     if (mixed_pc) {
       TRY(tmp_alloc(c, pm_slots, (size_t)tot * sizeof(double)));
       TRY(tmp_alloc(c, pm_off, off.size() * sizeof(long long)));
@@ -1681,8 +1685,8 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
   ph_begin(c, OSVMP2_PH_PRECOND);
   if (pm) {
     const int rc = launch_precond_mixed(t, c->opts.tau_s, (const PJob*)jp.p, (const int*)pm_order.p, (int)pjb.size(), max_m,
-                                        (double*)pm_slots.p, (const long long*)pm_off.p, (const int*)pm_m.p,
-                                        (double*)scr.p, n_cta_pm, c->err_d, !mixed, c->st);
+                                        max_n, pm_sorted.data(), (double*)pm_slots.p, (const long long*)pm_off.p, (const int*)pm_m.p,
+                                        (double*)scr.p, n_cta_pm, c->num_sms, c->err_d, c->st);
     if (rc && mixed_pc)
       return fail(c, OSVMP2_E_ARG, "pair order %d exceeds the mixed preconditioner's shared scratch", max_m);
     if (rc) pm = false;

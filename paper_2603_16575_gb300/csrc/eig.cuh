@@ -798,7 +798,8 @@ __device__ __forceinline__ void chase_rotation(float x, float z, float& c, float
   }
 }
 
-template <class T>
+// S: stride of d and e (one tridiagonal per lane, interleaved in shared memory).
+template <int S = 1, class T>
 __device__ inline int tridiag_qr_record(T* __restrict__ d, T* __restrict__ e, int n, int* __restrict__ swp, int cap_s,
                                         T* __restrict__ rot, int cap_r, int* n_sw, bool partial = false) {
   const T eps = sizeof(T) == 8 ? T(2.220446049250313e-16) : T(1.1920929e-07);
@@ -808,14 +809,14 @@ __device__ inline int tridiag_qr_record(T* __restrict__ d, T* __restrict__ e, in
   for (int sweeps = 0;; sweeps++) {
     int h = n - 1;
     while (h > 0) {
-      if (fabs(e[h - 1]) <= eps * (fabs(d[h - 1]) + fabs(d[h]))) { e[h - 1] = T(0.0); h--; }
+      if (fabs(e[(h - 1) * S]) <= eps * (fabs(d[(h - 1) * S]) + fabs(d[(h) * S]))) { e[(h - 1) * S] = T(0.0); h--; }
       else break;
     }
     if (h == 0) { *n_sw = ns; return 0; }
     if (sweeps >= max_sweeps) return 1;
     int l = h - 1;
     while (l > 0) {
-      if (fabs(e[l - 1]) <= eps * (fabs(d[l - 1]) + fabs(d[l]))) { e[l - 1] = T(0.0); break; }
+      if (fabs(e[(l - 1) * S]) <= eps * (fabs(d[(l - 1) * S]) + fabs(d[(l) * S]))) { e[(l - 1) * S] = T(0.0); break; }
       l--;
     }
     if (ns >= cap_s || nr + (h - l) > cap_r) {
@@ -827,24 +828,24 @@ __device__ inline int tridiag_qr_record(T* __restrict__ d, T* __restrict__ e, in
     ns++;
     T* cs = rot + 2 * (size_t)nr;
     nr += h - l;
-    const T delta = T(0.5) * (d[h - 1] - d[h]);
-    const T eh = e[h - 1];
+    const T delta = T(0.5) * (d[(h - 1) * S] - d[(h) * S]);
+    const T eh = e[(h - 1) * S];
     const T den = delta + copysign(hypot(delta, eh), delta);
-    const T mu = d[h] - (den != T(0.0) ? eh * eh / den : T(0.0));
-    // d[k] and e[k] as updated by the previous rotation stay in registers
-    T dk = d[l], ek = e[l];
+    const T mu = d[(h) * S] - (den != T(0.0) ? eh * eh / den : T(0.0));
+    // d[(k) * S] and e[(k) * S] as updated by the previous rotation stay in registers
+    T dk = d[(l) * S], ek = e[(l) * S];
     T x = dk - mu, z = ek;
     for (int k = l; k < h; k++) {
-      const T cc = d[k + 1];
-      const T en = (k + 1 < h) ? e[k + 1] : T(0.0);
+      const T cc = d[(k + 1) * S];
+      const T en = (k + 1 < h) ? e[(k + 1) * S] : T(0.0);
       T c, s, r;
       chase_rotation(x, z, c, s, r);
-      if (k > l) e[k - 1] = r;
+      if (k > l) e[(k - 1) * S] = r;
       const T a = dk, b = ek;
-      d[k] = c * c * a + T(2.0) * c * s * b + s * s * cc;
+      d[(k) * S] = c * c * a + T(2.0) * c * s * b + s * s * cc;
       dk = s * s * a - T(2.0) * c * s * b + c * c * cc;
       const T ekn = c * s * (cc - a) + (c * c - s * s) * b;
-      e[k] = ekn;
+      e[(k) * S] = ekn;
       if (k + 1 < h) {
         x = ekn;
         z = s * en;
@@ -853,7 +854,7 @@ __device__ inline int tridiag_qr_record(T* __restrict__ d, T* __restrict__ e, in
       cs[2 * (k - l)] = c;
       cs[2 * (k - l) + 1] = s;
     }
-    d[h] = dk;
+    d[(h) * S] = dk;
   }
 }
 

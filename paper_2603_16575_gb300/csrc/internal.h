@@ -147,8 +147,8 @@ int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, 
 struct OzPolish {        // pair basis refinement
   int m, r;
   const double* S1;      // U0^T U0 [r][r]
-  const double* F1;      // U0^T e U0
-  double* IE;            // out: 1 + E [r][r]
+  double* F1;            // U0^T e U0 (overwritten)
+  double* IE;            // out: the change of basis, U = U0 IE [r][r]
   double* X;             // [m][m], first r columns; in place
   double* et;            // out
 };
@@ -234,17 +234,17 @@ void launch_precond(const Tables& t, double tau_s, const PJob* jobs, int n_jobs,
 size_t precond_w_scratch_doubles(int max_m, int n_warps);
 int launch_precond_w(const Tables& t, double tau_s, const PJob* jobs, int n_jobs, int max_m, double* scratch,
                      int n_warps, int* err, cudaStream_t st);
-// precond_mixed.cu: block-structured canonical orthogonalisation in FP64, F' diagonalised
-// in FP32 with exact leftovers Sh/Gh (mixed form) or in FP64 (fp64: jobs without Sh; the basis
-// is to be polished afterwards); -1 if max_m is too large.
+// precond_mixed.cu: block-structured orthogonalisation in FP64, F' diagonalised in FP32, with exact
+// leftovers Sh/Gh for the jobs that have them (mixed form; in the FP64 form the basis is polished
+// afterwards); max_n: the largest OSV count; -1 if max_m is too large.
 // Per-pair intermediates: one slot of precond_mixed_slot_doubles(m) at slots + off[job];
 // mdim[job] = pair order m; order: the jobs in the order the CTAs take them
 // (grid-stride; descending m balances the launch).
 size_t precond_mixed_slot_doubles(int m);
 size_t precond_mixed_scratch_doubles(int max_m, int n_cta);
-int launch_precond_mixed(const Tables& t, double tau_s, const PJob* jobs, const int* order, int n_jobs, int max_m,
-                         double* slots, const long long* off, const int* mdim, double* scratch, int n_cta, int* err,
-                         bool fp64, cudaStream_t st);
+int launch_precond_mixed(const Tables& t, double tau_s, const PJob* jobs, const int* order, int n_jobs, int max_m, int max_n,
+                         const int* m_sorted, double* slots, const long long* off, const int* mdim, double* scratch,
+                         int n_cta, int num_sms, int* err, cudaStream_t st);
 
 // ---- A4-A5 (solve.cu)
 // Fragments: orbs [n][3] (-1 padded, ascending), order[] = processing order.

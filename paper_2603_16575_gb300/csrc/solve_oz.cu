@@ -21,37 +21,114 @@
 namespace osv {
 
 // ---------------------------------------------------------------- basis polish
-// One step of the refinement of Ogita and Aishima (Japan J. Indust. Appl. Math. 35 (2018) 1007) on
-// the basis U0 = P X: with S1 = U0^T U0 and F1 = U0^T e U0 formed from U0 itself (entries of order 1;
-// X^T S X would carry eps |X|^2, X reaching lambda_min(S)^(-1/2)),
-//   R = 1 - S1, lambda_a = F1_aa / S1_aa, E_ab = (F1_ab + lambda_b R_ab) / (lambda_b - lambda_a)
-// (R_ab / 2 where that is not small: equal or nearly equal lambda, and a = b), X <- X (1 + E),
-// e~ = lambda.  U = U0 (1 + E) is then orthonormal and F diagonal in it to FP64 rounding.
+// Steps of the refinement of Ogita and Aishima (Japan J. Indust. Appl. Math. 35 (2018) 1007) on the basis
+// U0 = P X: with S1 = U0^T U0 and F1 = U0^T e U0 formed from U0 itself (entries of order 1; X^T S X would carry
+// eps |X|^2, X reaching lambda_min(S)^(-1/2)) and R = 1 - S1,
+//   A = F1 + (R F1 + F1 R) / 2 to first order in R, the Fock matrix of the orthonormalised basis U0 (1 + R / 2);
+//   E_ab = A_ab / (A_bb - A_aa),  U <- U0 (1 + R / 2)(1 + E), X likewise, e~ = diag(A).
+// Each step squares the errors, so three take the FP32 Jacobi basis (R and the off-diagonal A ~ 1e-6) to FP64 rounding,
+// unless a pair of eigenvalues is close: pairs with |A_ab| > 1e-3 |A_bb - A_aa| are first diagonalised by Jacobi
+// rotations G among themselves (a handful at most), and 1 + E is that of the rotated A.
+constexpr int POL_MAX = 256;      // close pairs handled by rotations in one step
+constexpr int POL_SWEEPS = 4;
 __global__ void __launch_bounds__(NT) k_oz_polish(const OzPolish* __restrict__ jobs, int n_jobs, int max_m,
                                                   double* scratch) {
   __shared__ double sm[GEMM_SMEM_WIDE];
-  double* XE = scratch + (size_t)blockIdx.x * max_m * max_m;
-  for (int q = blockIdx.x; q < n_jobs; q += gridDim.x) {
-    const OzPolish jb = jobs[q];
+  __shared__ int s_n, s_rec;
+  __shared__ unsigned key[POL_MAX], list[POL_MAX];
+  __shared__ unsigned short rec[POL_MAX * POL_SWEEPS];
+  double* rcs = sm;               // (c, s) of the recorded rotations; the GEMM tiles come later
+  static_assert(2 * POL_MAX * POL_SWEEPS <= GEMM_SMEM_WIDE, "rotation record");
+  double* A = scratch + (size_t)blockIdx.x * max_m * max_m;
+  const int tid = threadIdx.x;
+  for (int jq = blockIdx.x; jq < n_jobs; jq += gridDim.x) {
+    const OzPolish jb = jobs[jq];
     const int m = jb.m, r = jb.r;
-    for (int idx = threadIdx.x; idx < r * r; idx += NT) {
+    double* RG = jb.F1;           // R / 2, then R G / 2
+    if (tid == 0) s_n = s_rec = 0;
+    for (int idx = tid; idx < r * r; idx += NT) {
       const int a = idx / r, b = idx % r;
       const double R = (a == b ? 1.0 : 0.0) - 0.5 * (jb.S1[idx] + jb.S1[b * r + a]);
-      double e = 0.5 * R;
+      A[idx] = 0.5 * (jb.F1[idx] + jb.F1[b * r + a]) + 0.5 * R * (jb.F1[(size_t)a * r + a] + jb.F1[(size_t)b * r + b]);
+    }
+    __syncthreads();
+    for (int idx = tid; idx < r * r; idx += NT) {
+      const int a = idx / r, b = idx % r;
+      RG[idx] = 0.5 * ((a == b ? 1.0 : 0.0) - 0.5 * (jb.S1[idx] + jb.S1[b * r + a]));
+      if (a < b) {
+        const double x = fabs(A[idx]), da = A[(size_t)a * r + a], db = A[(size_t)b * r + b];
+        if (x > 1e-3 * fabs(db - da) && x > 1e-15 * (fabs(da) + fabs(db))) {
+          const int k = atomicAdd(&s_n, 1);
+          if (k < POL_MAX) key[k] = (unsigned)idx;
+        }
+      }
+    }
+    __syncthreads();
+    const int n = min(s_n, POL_MAX);
+    for (int k = tid; k < n; k += NT) {            // in index order, whatever order they were found in
+      int rank = 0;
+      for (int u = 0; u < n; u++) rank += key[u] < key[k];
+      list[rank] = key[k];
+    }
+    __syncthreads();
+    for (int sw = 0; sw < POL_SWEEPS && n > 0; sw++)
+      for (int k = 0; k < n; k++) {
+        const int p = list[k] / r, q = list[k] % r;
+        const double app = A[(size_t)p * r + p], aqq = A[(size_t)q * r + q], apq = A[(size_t)p * r + q];
+        __syncthreads();
+        if (!(fabs(apq) > 1e-6 * fabs(aqq - app) && fabs(apq) > 1e-16 * (fabs(app) + fabs(aqq)))) continue;   // uniform
+        const double th = (aqq - app) / (2.0 * apq);
+        const double tt = copysign(1.0, th) / (fabs(th) + sqrt(1.0 + th * th));
+        const double c = 1.0 / sqrt(1.0 + tt * tt), s = tt * c;
+        for (int u = tid; u < r; u += NT) {
+          if (u != p && u != q) {
+            const double x = A[(size_t)p * r + u], y = A[(size_t)q * r + u];
+            const double nx = c * x - s * y, ny = s * x + c * y;
+            A[(size_t)p * r + u] = A[(size_t)u * r + p] = nx;
+            A[(size_t)q * r + u] = A[(size_t)u * r + q] = ny;
+          }
+          const double x = RG[(size_t)u * r + p], y = RG[(size_t)u * r + q];
+          RG[(size_t)u * r + p] = c * x - s * y;
+          RG[(size_t)u * r + q] = s * x + c * y;
+        }
+        if (tid == 0) {
+          A[(size_t)p * r + p] = app - tt * apq;
+          A[(size_t)q * r + q] = aqq + tt * apq;
+          A[(size_t)p * r + q] = A[(size_t)q * r + p] = 0.0;
+          rec[s_rec] = (unsigned short)k;
+          rcs[2 * s_rec] = c;
+          rcs[2 * s_rec + 1] = s;
+          s_rec++;
+        }
+        __syncthreads();
+      }
+    __syncthreads();
+    for (int idx = tid; idx < r * r; idx += NT) {
+      const int a = idx / r, b = idx % r;
+      double e = a == b ? 1.0 : 0.0;
       if (a != b) {
-        const double la = jb.F1[a * r + a] / jb.S1[a * r + a], lb = jb.F1[b * r + b] / jb.S1[b * r + b];
-        const double num = 0.5 * (jb.F1[idx] + jb.F1[b * r + a]) + lb * R, gap = lb - la;
-        if (fabs(num) < 0.1 * fabs(gap)) e = num / gap;
+        const double x = A[idx], gap = A[(size_t)b * r + b] - A[(size_t)a * r + a];
+        if (fabs(x) < 1e-2 * fabs(gap)) e = x / gap;
       }
       jb.IE[idx] = e;
     }
+    for (int a = tid; a < r; a += NT) jb.et[a] = A[(size_t)a * r + a];
     __syncthreads();
-    cta_gemm_a(m, r, r, 1.0, dense_view(jb.X, m, r, m), dense_view(jb.IE, r, r, r), 0.0, XE, r, sm);
-    for (int idx = threadIdx.x; idx < m * r; idx += NT) jb.X[(size_t)(idx / r) * m + idx % r] += XE[idx];
-    for (int a = threadIdx.x; a < r; a += NT) {
-      jb.et[a] = jb.F1[(size_t)a * r + a] / jb.S1[(size_t)a * r + a];
-      jb.IE[(size_t)a * r + a] += 1.0;
+    for (int k = s_rec - 1; k >= 0; k--) {         // G (1 + E): the rotations on the rows, last one first
+      const int p = list[rec[k]] / r, q = list[rec[k]] % r;
+      const double c = rcs[2 * k], s = rcs[2 * k + 1];
+      for (int u = tid; u < r; u += NT) {
+        const double x = jb.IE[(size_t)p * r + u], y = jb.IE[(size_t)q * r + u];
+        jb.IE[(size_t)p * r + u] = c * x + s * y;
+        jb.IE[(size_t)q * r + u] = c * y - s * x;
+      }
+      __syncthreads();
     }
+    __syncthreads();
+    for (int idx = tid; idx < r * r; idx += NT) jb.IE[idx] += RG[idx];
+    __syncthreads();
+    cta_gemm_a(m, r, r, 1.0, dense_view(jb.X, m, r, m), dense_view(jb.IE, r, r, r), 0.0, A, r, sm);
+    for (int idx = tid; idx < m * r; idx += NT) jb.X[(size_t)(idx / r) * m + idx % r] = A[idx];
     __syncthreads();
   }
 }
