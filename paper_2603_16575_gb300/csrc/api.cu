@@ -682,7 +682,7 @@ int gproj_tensor(osvmp2_ctx* c, const std::vector<GJob>& gj, const std::vector<l
 constexpr int OZ_NO_ROOM = -100;
 
 // Bytes of the digits of `rows` operand rows with K elements each, and of their exponents.
-size_t oz_digit_bytes(size_t rows, int K) { return rows * oz::NSL * oz::ld_of(K) * sizeof(uint16_t); }
+size_t oz_digit_bytes(size_t rows, int K, int ns = oz::NSL) { return rows * ns * oz::ld_of(K) * sizeof(uint16_t); }
 size_t oz_exp_bytes(size_t rows, int K) { return rows * oz::n_chunks(K) * sizeof(int); }
 
 int oz_room(osvmp2_ctx* c, Tmp& t, size_t bytes) {
@@ -735,11 +735,11 @@ int oz_upload(osvmp2_ctx* c, const OzList& l, OzDev& d) {
   CK(cudaMemcpyAsync(d.s.p, l.segs.data(), l.segs.size() * sizeof(oz::Seg), cudaMemcpyHostToDevice, c->st));
   return 0;
 }
-int oz_run(osvmp2_ctx* c, const OzOperand& A, const OzOperand& B, const OzList& l) {
+int oz_run(osvmp2_ctx* c, const OzOperand& A, const OzOperand& B, const OzList& l, int ns = oz::NSL) {
   if (l.jobs.empty()) return 0;
   OzDev d;
   TRY(oz_upload(c, l, d));
-  if (launch_oz_gemm(A, B, (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, nullptr, c->err_d, c->st))
+  if (launch_oz_gemm(A, B, (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, nullptr, ns, c->err_d, c->st))
     return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for an FP64 contraction failed");
   CK(cudaGetLastError());
   return 0;
@@ -750,15 +750,15 @@ struct OzMats {
   Tmp D, ex, md;
   OzOperand op{};
   std::vector<OzMat> mats;
-  int max_rows = 0, K;
-  long long rows = 0;      // rows of the matrices (the store has NSL times as many)
-  explicit OzMats(int K_) : K(K_) {}
+  int max_rows = 0, K, ns;
+  long long rows = 0;      // rows of the matrices (the store has ns times as many)
+  explicit OzMats(int K_, int ns_ = oz::NSL) : K(K_), ns(ns_) {}
   // matrix of r rows and k <= K elements a row at p (row stride ldm); the digits past k are zero up to
   // the next multiple of 32, as far as a tile of K = k reads
   int add(const double* p, int r, int ldm, int k) {
     const int nch = oz::n_chunks(K);
     OzMat m{p, r, k, std::min(oz::ld_of(K), (k + oz::BK - 1) / oz::BK * oz::BK), ldm,
-            oz::Mat{(int)(rows * oz::NSL), r, (int)(rows * nch), nch}};
+            oz::Mat{(int)(rows * ns), r, (int)(rows * nch), nch}};
     mats.push_back(m);
     rows += r;
     max_rows = std::max(max_rows, r);
@@ -768,18 +768,18 @@ struct OzMats {
 };
 // Room for the digits of s (OZ_NO_ROOM without), then the digits, scaled by w[k] unless NULL.
 int oz_mats_room(osvmp2_ctx* c, OzMats& s) {
-  if (s.rows * oz::NSL + oz::BM >= (long long)INT32_MAX || s.rows * oz::n_chunks(s.K) >= (long long)INT32_MAX)
+  if (s.rows * s.ns + oz::BM >= (long long)INT32_MAX || s.rows * oz::n_chunks(s.K) >= (long long)INT32_MAX)
     return OZ_NO_ROOM;
-  TRY(oz_room(c, s.D, oz_digit_bytes((size_t)s.rows, s.K)));
+  TRY(oz_room(c, s.D, oz_digit_bytes((size_t)s.rows, s.K, s.ns)));
   TRY(oz_room(c, s.ex, oz_exp_bytes((size_t)s.rows, s.K)));
   TRY(oz_room(c, s.md, s.mats.size() * sizeof(OzMat)));
-  s.op = OzOperand{(const uint16_t*)s.D.p, s.rows * oz::NSL, s.K, oz::ld_of(s.K), (const int*)s.ex.p};
+  s.op = OzOperand{(const uint16_t*)s.D.p, s.rows * s.ns, s.K, oz::ld_of(s.K), (const int*)s.ex.p};
   return 0;
 }
 int oz_mats_fill(osvmp2_ctx* c, OzMats& s, const double* w, bool k_inner) {
   if (s.mats.empty()) return 0;
   CK(cudaMemcpyAsync(s.md.p, s.mats.data(), s.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
-  launch_oz_mats((const OzMat*)s.md.p, (int)s.mats.size(), s.max_rows, s.K, w, k_inner, oz::ld_of(s.K), (uint16_t*)s.D.p,
+  launch_oz_mats((const OzMat*)s.md.p, (int)s.mats.size(), s.max_rows, s.K, w, k_inner, s.ns, oz::ld_of(s.K), (uint16_t*)s.D.p,
                  (int*)s.ex.p, c->st);
   CK(cudaGetLastError());
   return 0;
@@ -839,7 +839,7 @@ int oz_project(osvmp2_ctx* c, const std::vector<ProjJob>& pj) {
   const OzOperand A{(const uint16_t*)D.p, (long long)(per * oz::NSL * nx), nv, oz::ld_of(nv), (const int*)ex.p};
   for (size_t b0 = 0; b0 < is.size(); b0 += per) {
     const int nb = (int)std::min(per, is.size() - b0);
-    launch_oz_cols(bsrc(c), (const int*)xd.p + b0, nb, (uint16_t*)D.p, (int*)ex.p, c->st);
+    launch_oz_cols(bsrc(c), (const int*)xd.p + b0, nb, oz::NSL, (uint16_t*)D.p, (int*)ex.p, c->st);
     CK(cudaGetLastError());
     OzList l;
     for (int u = 0; u < nb; u++)
@@ -994,7 +994,7 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
       TRY(oz_run(c, ur.op, ie.op, lo));
     }
     CK(cudaMemcpyAsync(mj.p, fin.data(), fin.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
-    launch_oz_mats((const OzMat*)mj.p, (int)fin.size(), mr, nv, nullptr, false, ld, (uint16_t*)dmem.p, (int*)emem.p,
+    launch_oz_mats((const OzMat*)mj.p, (int)fin.size(), mr, nv, nullptr, false, oz::NSL, ld, (uint16_t*)dmem.p, (int*)emem.p,
                    c->st);
     CK(cudaGetLastError());
     b0 = b1;
@@ -1015,6 +1015,7 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
 // raw: whether the stored amplitudes are those of the raw basis; otherwise Y (r^2) is left in the slot.
 // df: dE/df of each fragment times its weight (launch_oz_df), NULL if not wanted.
 struct OzWant {
+  int ns = oz::NSL;                 // slices of the products (8: FP64)
   bool raw = true;
   double* df = nullptr;             // device [n][9], by out_id
   const std::vector<Frag>* frags = nullptr;   // by out_id
@@ -1022,6 +1023,7 @@ struct OzWant {
 int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, const std::vector<int>& out_id, size_t f0,
                    size_t f1, const SolveOpts& so, double ulps, FragOut* out, double* tdst, const long long* toff,
                    double* pair_e, const OzWant& want) {
+  const int NS = want.ns;
   const int n = c->sys.n_occ, nv = c->sys.n_vir;
   struct Term { int p, q, ver; double coef; };     // pairs by index in the batch
   std::vector<OzPair> pairs;
@@ -1126,7 +1128,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     OzPair& q = pairs[t.q];
     if (q.ver[t.ver] < 0) {
       q.ver[t.ver] = nver++;
-      q.vrow[t.ver] = (int)(yrows * oz::NSL);
+      q.vrow[t.ver] = (int)(yrows * NS);
       yrows += q.r;
     }
   }
@@ -1152,14 +1154,14 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   }
   long long srows = 0;
   for (const Couple& k : cps) srows += c->r_h[k.lo] + c->r_h[k.hi];
-  if (yrows * oz::NSL + oz::BM >= (long long)INT32_MAX || srows * oz::NSL + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
+  if (yrows * NS + oz::BM >= (long long)INT32_MAX || srows * NS + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
   // W: pairs in groups whose digits fit a fixed budget
   const double wbudget = 8e9;
   std::vector<int> grp{0};
   long long wrows = 0, wcur = 0;
   for (int p = 0; p < np; p++) {
     const long long w = (long long)(term0[p + 1] - term0[p]) * pairs[p].r;
-    if (p > grp.back() && (double)(wcur + w) * oz::NSL * LD * 2 > wbudget) {
+    if (p > grp.back() && (double)(wcur + w) * NS * LD * 2 > wbudget) {
       grp.push_back(p);
       wcur = 0;
     }
@@ -1171,7 +1173,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   wcur = 0;
   for (int t = nts; t < nt; t++) {
     const long long w = pairs[terms[t].p].r;
-    if (t > dgrp.back() && (double)(wcur + w) * oz::NSL * LD * 2 > wbudget) {
+    if (t > dgrp.back() && (double)(wcur + w) * NS * LD * 2 > wbudget) {
       dgrp.push_back(t);
       wcur = 0;
     }
@@ -1179,14 +1181,14 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     wrows = std::max(wrows, wcur);
   }
   dgrp.push_back(nt);
-  if (wrows * oz::NSL + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
+  if (wrows * NS + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
   Tmp yc, yd, yx, wx, wd, sd, sx, sgm, pr, p0, pe, pu, ep, dn, lf, oi, smj;
   TRY(oz_room(c, yc, 2 * ysz * sizeof(double)));
-  TRY(oz_room(c, yd, (size_t)yrows * oz::NSL * LD * 2));
+  TRY(oz_room(c, yd, (size_t)yrows * NS * LD * 2));
   TRY(oz_room(c, yx, (size_t)std::max(1, nver) * nch * sizeof(int)));
   TRY(oz_room(c, wx, (size_t)std::max(1, nver) * nch * sizeof(int)));
-  TRY(oz_room(c, wd, (size_t)wrows * oz::NSL * LD * 2));
-  TRY(oz_room(c, sd, (size_t)srows * oz::NSL * LD * 2));
+  TRY(oz_room(c, wd, (size_t)wrows * NS * LD * 2));
+  TRY(oz_room(c, sd, (size_t)srows * NS * LD * 2));
   TRY(oz_room(c, sx, (size_t)srows * nch * sizeof(int)));
   TRY(oz_room(c, sgm, sgsz * sizeof(double)));
   TRY(oz_room(c, pr, np * sizeof(OzPair)));
@@ -1221,24 +1223,24 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
       const int lo = cps[u].lo, hi = cps[u].hi, rl = c->r_h[lo], rh = c->r_h[hi];
       double* S = (double*)sgm.p + sgo[u];
       groups[{c->ud_of[lo], c->ud_of[hi]}].product(c->ud_mat[lo], rl, c->ud_mat[hi], rh, nv, S, rh);
-      slo[u] = oz::Mat{(int)(row * oz::NSL), rl, (int)(row * nch), nch};
+      slo[u] = oz::Mat{(int)(row * NS), rl, (int)(row * nch), nch};
       m1.push_back(OzMat{S, rl, rh, (rh + oz::BK - 1) / oz::BK * oz::BK, rh, slo[u]});
       row += rl;
-      shi[u] = oz::Mat{(int)(row * oz::NSL), rh, (int)(row * nch), nch};
+      shi[u] = oz::Mat{(int)(row * NS), rh, (int)(row * nch), nch};
       m2.push_back(OzMat{S, rh, rl, (rl + oz::BK - 1) / oz::BK * oz::BK, rh, shi[u]});
       row += rh;
     }
     for (auto& g : groups) TRY(oz_run(c, c->ud_store[g.first.first], c->ud_store[g.first.second], g.second));
     CK(cudaMemcpyAsync(smj.p, m1.data(), m1.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync((OzMat*)smj.p + m1.size(), m2.data(), m2.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
-    launch_oz_mats((const OzMat*)smj.p, (int)m1.size(), max_r, max_r, nullptr, true, LD, (uint16_t*)sd.p, (int*)sx.p, c->st);
-    launch_oz_mats((const OzMat*)smj.p + m1.size(), (int)m2.size(), max_r, max_r, nullptr, false, LD, (uint16_t*)sd.p,
+    launch_oz_mats((const OzMat*)smj.p, (int)m1.size(), max_r, max_r, nullptr, true, NS, LD, (uint16_t*)sd.p, (int*)sx.p, c->st);
+    launch_oz_mats((const OzMat*)smj.p + m1.size(), (int)m2.size(), max_r, max_r, nullptr, false, NS, LD, (uint16_t*)sd.p,
                    (int*)sx.p, c->st);
     CK(cudaGetLastError());
   }
-  const OzOperand So{(const uint16_t*)sd.p, srows * oz::NSL, LD, LD, (const int*)sx.p};
-  const OzOperand Yo{(const uint16_t*)yd.p, std::max<long long>(1, yrows) * oz::NSL, LD, LD, (const int*)yx.p};
-  const OzOperand Wo{(const uint16_t*)wd.p, std::max<long long>(1, wrows) * oz::NSL, LD, LD, (const int*)wx.p};
+  const OzOperand So{(const uint16_t*)sd.p, srows * NS, LD, LD, (const int*)sx.p};
+  const OzOperand Yo{(const uint16_t*)yd.p, std::max<long long>(1, yrows) * NS, LD, LD, (const int*)yx.p};
+  const OzOperand Wo{(const uint16_t*)wd.p, std::max<long long>(1, wrows) * NS, LD, LD, (const int*)wx.p};
   // the two products of every group of pairs
   const size_t ng = grp.size() - 1;
   std::vector<OzDev> d1(ng), d2(ng);
@@ -1255,13 +1257,13 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
         const int ve = Q.ver[tm.ver] * nch;
         oz::Job proto{};
         proto.skip = P.frag;
-        proto.o_row = (int)(wrow * oz::NSL);
+        proto.o_row = (int)(wrow * NS);
         proto.o_ss = P.r;
         proto.o_e = ve;
         const int f1s = (int)l1.segs.size();
         l1.seg(S, oz::Mat{Q.vrow[tm.ver], Q.r, ve, 0}, Q.r);
         l1.tiles(f1s, P.r, Q.r, nullptr, 0, proto);
-        l2.seg(S, oz::Mat{(int)(wrow * oz::NSL), P.r, ve, 0}, Q.r, tm.coef);
+        l2.seg(S, oz::Mat{(int)(wrow * NS), P.r, ve, 0}, Q.r, tm.coef);
         wrow += P.r;
       }
       if ((int)l2.segs.size() > first) {
@@ -1279,13 +1281,13 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     if (it > 1)
       for (size_t g = 0; g < ng; g++) {
         if (d1[g].n && launch_oz_digits(So, Yo, (const oz::Job*)d1[g].j.p, d1[g].n, (const oz::Seg*)d1[g].s.p,
-                                        (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, c->err_d, c->st))
+                                        (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, NS, c->err_d, c->st))
           return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
         if (d2[g].n && launch_oz_gemm(So, Wo, (const oz::Job*)d2[g].j.p, d2[g].n, (const oz::Seg*)d2[g].s.p,
-                                      (const int*)dn.p, c->err_d, c->st))
+                                      (const int*)dn.p, NS, c->err_d, c->st))
           return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
       }
-    launch_oz_update((const OzPair*)pr.p, np, (const int*)dn.p, it == 1, LD, nch, (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p,
+    launch_oz_update((const OzPair*)pr.p, np, (const int*)dn.p, it == 1, NS, LD, nch, (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p,
                      (double*)pe.p, (double*)pu.p, n_cta, c->st);
     launch_oz_converge((const int*)p0.p, nfb, (const double*)pe.p, (const double*)pu.p, so, ulps, it, (double*)ep.p,
                        (int*)dn.p, (int*)lf.p, out, (const int*)oi.p, c->st);
@@ -1325,13 +1327,13 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
       const oz::Mat S = pid[tm.p] == cps[tc[t]].lo ? slo[tc[t]] : shi[tc[t]];
       oz::Job proto{};
       proto.skip = -1;
-      proto.o_row = (int)(wrow * oz::NSL);
+      proto.o_row = (int)(wrow * NS);
       proto.o_ss = P.r;
       proto.o_e = ve;
       const int f1s = (int)l1.segs.size(), f2s = (int)l2.segs.size();
       l1.seg(S, oz::Mat{Q.vrow[tm.ver], Q.r, ve, 0}, Q.r);
       l1.tiles(f1s, P.r, Q.r, nullptr, 0, proto);
-      l2.seg(S, oz::Mat{(int)(wrow * oz::NSL), P.r, ve, 0}, Q.r);
+      l2.seg(S, oz::Mat{(int)(wrow * NS), P.r, ve, 0}, Q.r);
       const size_t j0 = l2.jobs.size();
       l2.tiles(f2s, P.r, P.r, P.Y, P.r, proto);
       dfs[df].tile0[dot] = ntile;
@@ -1349,7 +1351,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     CK(cudaMemcpyAsync(dfd.p, dfs.data(), dfs.size() * sizeof(OzDf), cudaMemcpyHostToDevice, c->st));
     for (size_t q = 0; q + 1 < cut.size(); q++) {
       if (launch_oz_digits(So, Yo, (const oz::Job*)u1.j.p + cut[q][0], cut[q + 1][0] - cut[q][0], (const oz::Seg*)u1.s.p,
-                           (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, c->err_d, c->st) ||
+                           (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, NS, c->err_d, c->st) ||
           launch_oz_dots(So, Wo, (const oz::Job*)u2.j.p + cut[q][1], cut[q + 1][1] - cut[q][1], (const oz::Seg*)u2.s.p,
                          (double*)parts.p, c->err_d, c->st))
         return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for dE/df failed");
@@ -2069,7 +2071,7 @@ int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int ns
   const int nv = c->sys.n_vir, nx = c->sys.n_aux, n = c->sys.n_occ, nch = oz::n_chunks(nx);
   for (int u0 = 0; u0 < b; u0 += nsl) {
     const int nu = std::min(nsl, b - u0);
-    launch_oz_rows(bsrc(c), i0 + u0, nu, D, ex, c->st);
+    launch_oz_rows(bsrc(c), i0 + u0, nu, oz::NSL, D, ex, c->st);
     CK(cudaGetLastError());
     OzList all, l;
     for (int u = 0; u < nu; u++) {
@@ -2087,7 +2089,7 @@ int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int ns
     OzDev d;
     if (int rc = oz_upload(c, l, d)) return rc;
     if (launch_oz_tii(OzOperand{D, (long long)nu * oz::NSL * nv, nx, oz::ld_of(nx), ex}, (const oz::Job*)d.j.p, d.n,
-                      (const oz::Seg*)d.s.p, c->sys.e_vir, c->err_d, c->st))
+                      (const oz::Seg*)d.s.p, c->sys.e_vir, oz::NSL, c->err_d, c->st))
       return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for T_ii failed");
     CK(cudaGetLastError());
   }
@@ -3465,8 +3467,8 @@ static int oz_grad_pairs(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& 
     CK(cudaMemcpyAsync(md.p, yn.mats.data(), yn.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync((OzMat*)md.p + yn.mats.size(), yt.mats.data(), yt.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice,
                        c->st));
-    launch_oz_mats((const OzMat*)md.p, (int)yn.mats.size(), max_r, max_r, nullptr, true, ld, (uint16_t*)D.p, (int*)ex.p, c->st);
-    launch_oz_mats((const OzMat*)md.p + yn.mats.size(), (int)yt.mats.size(), max_r, max_r, nullptr, false, ld,
+    launch_oz_mats((const OzMat*)md.p, (int)yn.mats.size(), max_r, max_r, nullptr, true, oz::NSL, ld, (uint16_t*)D.p, (int*)ex.p, c->st);
+    launch_oz_mats((const OzMat*)md.p + yn.mats.size(), (int)yt.mats.size(), max_r, max_r, nullptr, false, oz::NSL, ld,
                    (uint16_t*)D.p, (int*)ex.p, c->st);
     CK(cudaGetLastError());
     size_t k0 = 0;

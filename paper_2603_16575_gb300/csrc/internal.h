@@ -124,22 +124,23 @@ struct OzMat {           // dense matrix whose digits go to m; row stride ldm (s
   int rows, K, kpad, ldm;  // kpad >= K: digits of k in [K, kpad) are written as zeros
   oz::Mat m;
 };
+// ns: slices (8: FP64; 5 and 4: 39 and 31 bits for the mixed form); operands with more slices serve too.
 // Digits of B: rows B[i0 + u][a][.] (K = aux) or B[xs[u]][.][P] (K = vir); slot u, slice s, row r at
-// row (u NSL + s) rows + r of the store, exponent row u rows + r.
-void launch_oz_rows(const BSrc& src, int i0, int nb, uint16_t* D, int* ex, cudaStream_t st);
-void launch_oz_cols(const BSrc& src, const int* xs, int nb, uint16_t* D, int* ex, cudaStream_t st);
+// row (u ns + s) rows + r of the store, exponent row u rows + r.
+void launch_oz_rows(const BSrc& src, int i0, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st);
+void launch_oz_cols(const BSrc& src, const int* xs, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st);
 // Digits of dense matrices: [K][rows] (row index innermost), scaled by w[k] unless NULL; or, k_inner, [rows][K].
-void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const double* w, bool k_inner, int ld,
+void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const double* w, bool k_inner, int ns, int ld,
                     uint16_t* D, int* ex, cudaStream_t st);
 // out[row][col] per job (row-major); T_ii tiles of the lower triangle (mirrored, with denominators).
 // Return 0, or -1 if a tensor map could not be encoded.
 int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                   const int* skip, int* err, cudaStream_t st);
-int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int* err,
-                  cudaStream_t st);
+                   const int* skip, int ns, int* err, cudaStream_t st);
+int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int ns,
+                  int* err, cudaStream_t st);
 // The digits of the output (jobs' o_row, o_ss, o_e) into the store D with row stride ld (a multiple of 32).
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                     const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st);
+                     const int* skip, uint16_t* D, int ld, const int* exW, int ns, int* err, cudaStream_t st);
 // Dot products of (2 Y - Y^T) with the product of every job (see OzEpiDot), 16 partial sums per job.
 int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    double* parts, int* err, cudaStream_t st);
@@ -167,7 +168,7 @@ struct OzPair {          // a pair of a fragment
   double* C;             // [r][r]
   double* T;             // [m][m] raw-basis amplitude (launch_oz_raw) or NULL
 };
-void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, int nch, uint16_t* D,
+void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ns, int ld, int nch, uint16_t* D,
                       int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st);
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
                         double* e_prev, int* done, int* left, FragOut* out, const int* out_id, cudaStream_t st);

@@ -18,7 +18,7 @@ struct OzSrcBT {           // row P of slot u: B[xs[u]][.][P]
   __device__ __forceinline__ double get(int u, int r, int k) const { return src.get(xs[u], k, r); }
 };
 
-template <class Src>
+template <int NS, class Src>
 __global__ void __launch_bounds__(256) k_oz_rows(Src src, int rows, int K, int ld, uint16_t* __restrict__ D,
                                                  int* __restrict__ ex) {
   const int u = blockIdx.y, lane = threadIdx.x & 31;
@@ -33,13 +33,13 @@ __global__ void __launch_bounds__(256) k_oz_rows(Src src, int rows, int K, int l
     x[v] = k < K ? src.get(u, r, k) : 0.0;
   }
   const size_t slice = (size_t)rows * ld;
-  const int e = oz::warp_slices(x, min(oz::CHUNK, K - k0), D + ((size_t)u * oz::NSL * rows + r) * ld + k0, slice, lane);
+  const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, K - k0), D + ((size_t)u * NS * rows + r) * ld + k0, slice, lane);
   if (lane == 0) ex[((size_t)u * rows + r) * nch + c] = e;
 }
 
 // Rows strided in k (their index innermost): one CTA per 16 rows x one chunk, transposed through shared memory so
 // that both the reads (rows innermost) and the digit writes (k innermost) are coalesced.
-template <class Src>
+template <int NS, class Src>
 __global__ void __launch_bounds__(256) k_oz_cols(Src src, int rows, int K, int ld, uint16_t* __restrict__ D,
                                                  int* __restrict__ ex) {
   __shared__ double tile[oz::CHUNK][17];
@@ -57,13 +57,14 @@ __global__ void __launch_bounds__(256) k_oz_cols(Src src, int rows, int K, int l
 #pragma unroll
     for (int v = 0; v < 8; v++) x[v] = tile[64 * (v >> 1) + 2 * lane + (v & 1)][dr];
     const int r = r0 + dr;
-    const int e = oz::warp_slices(x, min(oz::CHUNK, K - k0), D + ((size_t)u * oz::NSL * rows + r) * ld + k0, slice, lane);
+    const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, K - k0), D + ((size_t)u * NS * rows + r) * ld + k0, slice, lane);
     if (lane == 0) ex[((size_t)u * rows + r) * nch + c] = e;
   }
 }
 
 // A list of dense matrices with the row index innermost ([K][rows], row stride ldm), optionally scaled by w[k];
 // digits zero up to kpad.
+template <int NS>
 __global__ void __launch_bounds__(256) k_oz_mats(const OzMat* __restrict__ mats, const double* __restrict__ w,
                                                  int ld, uint16_t* __restrict__ D, int* __restrict__ ex) {
   __shared__ double tile[oz::CHUNK][17];
@@ -87,11 +88,12 @@ __global__ void __launch_bounds__(256) k_oz_mats(const OzMat* __restrict__ mats,
 #pragma unroll
     for (int v = 0; v < 8; v++) x[v] = tile[64 * (v >> 1) + 2 * lane + (v & 1)][dr];
     const int r = r0 + dr;
-    const int e = oz::warp_slices(x, min(oz::CHUNK, mt.kpad - k0), D + ((size_t)mt.m.row + r) * ld + k0, slice, lane);
+    const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, mt.kpad - k0), D + ((size_t)mt.m.row + r) * ld + k0, slice, lane);
     if (lane == 0) ex[mt.m.eb + (size_t)r * mt.m.es + c] = e;
   }
 }
 // The same for matrices with k innermost ([rows][K], row stride ldm): a warp per (row, chunk).
+template <int NS>
 __global__ void __launch_bounds__(256) k_oz_rmats(const OzMat* __restrict__ mats, int ld, uint16_t* __restrict__ D,
                                                   int* __restrict__ ex) {
   const OzMat mt = mats[blockIdx.z];
@@ -103,40 +105,47 @@ __global__ void __launch_bounds__(256) k_oz_rmats(const OzMat* __restrict__ mats
     const int k = k0 + 64 * (v >> 1) + 2 * lane + (v & 1);
     x[v] = k < mt.K ? mt.p[(size_t)r * mt.ldm + k] : 0.0;
   }
-  const int e = oz::warp_slices(x, min(oz::CHUNK, mt.kpad - k0), D + ((size_t)mt.m.row + r) * ld + k0,
+  const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, mt.kpad - k0), D + ((size_t)mt.m.row + r) * ld + k0,
                                 (size_t)mt.m.ss * ld, lane);
   if (lane == 0) ex[mt.m.eb + (size_t)r * mt.m.es + c] = e;
 }
 
-void launch_oz_rows(const BSrc& src, int i0, int nb, uint16_t* D, int* ex, cudaStream_t st) {
+// One call of f<NS> for the slice counts in use.
+#define OZ_DISPATCH(ns, call)              \
+  do {                                     \
+    if ((ns) == 8) { constexpr int NS = 8; call; } \
+    else if ((ns) == 5) { constexpr int NS = 5; call; } \
+    else { constexpr int NS = 4; call; }   \
+  } while (0)
+
+void launch_oz_rows(const BSrc& src, int i0, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st) {
   if (!nb) return;
   const long long warps = (long long)src.n_vir * oz::n_chunks(src.n_aux);
-  k_oz_rows<<<dim3((unsigned)((warps + 7) / 8), nb), 256, 0, st>>>(OzSrcB{src, i0}, src.n_vir, src.n_aux,
-                                                                   oz::ld_of(src.n_aux), D, ex);
+  const dim3 grid((unsigned)((warps + 7) / 8), nb);
+  OZ_DISPATCH(ns, (k_oz_rows<NS><<<grid, 256, 0, st>>>(OzSrcB{src, i0}, src.n_vir, src.n_aux, oz::ld_of(src.n_aux), D, ex)));
   note_launch(1);
 }
-void launch_oz_cols(const BSrc& src, const int* xs, int nb, uint16_t* D, int* ex, cudaStream_t st) {
+void launch_oz_cols(const BSrc& src, const int* xs, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st) {
   if (!nb) return;
-  k_oz_cols<<<dim3((src.n_aux + 15) / 16, oz::n_chunks(src.n_vir), nb), 256, 0, st>>>(
-      OzSrcBT{src, xs}, src.n_aux, src.n_vir, oz::ld_of(src.n_vir), D, ex);
+  const dim3 grid((src.n_aux + 15) / 16, oz::n_chunks(src.n_vir), nb);
+  OZ_DISPATCH(ns, (k_oz_cols<NS><<<grid, 256, 0, st>>>(OzSrcBT{src, xs}, src.n_aux, src.n_vir, oz::ld_of(src.n_vir), D, ex)));
   note_launch(1);
 }
-void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const double* w, bool k_inner, int ld,
+void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const double* w, bool k_inner, int ns, int ld,
                     uint16_t* D, int* ex, cudaStream_t st) {
   if (!n) return;
   for (int q = 0; q < n; q += 65535) {     // grid z limit
     const int nq = n - q < 65535 ? n - q : 65535;
-    if (k_inner)
-      k_oz_rmats<<<dim3((max_rows + 7) / 8, oz::n_chunks(max_K), nq), 256, 0, st>>>(mats + q, ld, D, ex);
-    else
-      k_oz_mats<<<dim3((max_rows + 15) / 16, oz::n_chunks(max_K), nq), 256, 0, st>>>(mats + q, w, ld, D, ex);
+    const dim3 gr((max_rows + 7) / 8, oz::n_chunks(max_K), nq), gc((max_rows + 15) / 16, oz::n_chunks(max_K), nq);
+    if (k_inner) OZ_DISPATCH(ns, (k_oz_rmats<NS><<<gr, 256, 0, st>>>(mats + q, ld, D, ex)));
+    else OZ_DISPATCH(ns, (k_oz_mats<NS><<<gc, 256, 0, st>>>(mats + q, w, ld, D, ex)));
     note_launch(1);
   }
 }
 
 // out[row][col] (row-major), added to what is there when job.s = 1
 struct OzEpiRow {
-  static constexpr bool kWarp = false;
+  static constexpr bool kWarp = false, kDigits = false;
   __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     double* o = static_cast<double*>(jb.out) + (size_t)(jb.m0 + r) * jb.ld_out + jb.n0 + c0;
 #pragma unroll
@@ -146,7 +155,7 @@ struct OzEpiRow {
 };
 // T[a][b] = T[b][a] = v / (e_a + e_b - s) for a >= b; out = T_i, s = 2 f_ii
 struct OzEpiT {
-  static constexpr bool kWarp = false;
+  static constexpr bool kWarp = false, kDigits = false;
   const double* e_vir;
   __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     const int a = jb.m0 + r;
@@ -167,42 +176,41 @@ struct OzEpiT {
 // Digits of the output instead of its values: row m0 + r, k = n0 + c of the matrix at store row o_row (o_ss
 // rows per slice), under the exponent code exW[o_e] (a bound of the whole matrix); columns past n_valid up to the
 // next multiple of 16 are written as zeros (up to 32 by the lanes of the last column group).
+template <int NS>
 struct OzEpiDigits {
-  static constexpr bool kWarp = false;
+  static constexpr bool kWarp = false, kDigits = true;
+  static constexpr int T = 7 + 8 * (NS - 1);
   uint16_t* D;
   int ld;
   const int* exW;
-  __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
-    const int e = exW[jb.o_e];
-    const bool live = e > oz::EX_ZERO / 2 && e < oz::EX_NAN / 2;
+  __device__ __forceinline__ int exponent(const oz::Job& jb) const { return exW[jb.o_e]; }
+  __device__ __forceinline__ void digits(const oz::Job& jb, int r, int c0, long long (&f)[oz::DCOL]) const {
     uint16_t* o = D + ((size_t)jb.o_row + jb.m0 + r) * ld + jb.n0 + c0;
     const size_t slice = (size_t)jb.o_ss * ld;
     // the last column group also clears the group after it when that completes a 32-wide k-block
     const bool tail = c0 + oz::DCOL >= jb.n_valid && ((jb.n0 + c0) & 16) == 0;
 #pragma unroll
-    for (int h = 0; h < oz::DCOL / 8; h++) {
-      long long f[8];
+    for (int u = 0; u < oz::DCOL; u++)
+      if (c0 + u >= jb.n_valid) f[u] = 0;
 #pragma unroll
-      for (int u = 0; u < 8; u++)
-        f[u] = (live && c0 + 8 * h + u < jb.n_valid) ? oz::fixed63(v[8 * h + u], (unsigned)(e + 1022)) : 0;
+    for (int h = 0; h < oz::DCOL / 8; h++)
 #pragma unroll
-      for (int s = oz::NSL - 1; s >= 0; s--) {
+      for (int s = NS - 1; s >= 0; s--) {
         uint4 w;
-        w.x = oz::digit_pair(f[0], f[1], s);
-        w.y = oz::digit_pair(f[2], f[3], s);
-        w.z = oz::digit_pair(f[4], f[5], s);
-        w.w = oz::digit_pair(f[6], f[7], s);
+        w.x = oz::digit_pair(f[8 * h], f[8 * h + 1], s);
+        w.y = oz::digit_pair(f[8 * h + 2], f[8 * h + 3], s);
+        w.z = oz::digit_pair(f[8 * h + 4], f[8 * h + 5], s);
+        w.w = oz::digit_pair(f[8 * h + 6], f[8 * h + 7], s);
         *reinterpret_cast<uint4*>(o + s * slice + 8 * h) = w;
         if (tail) *reinterpret_cast<uint4*>(o + s * slice + 16 + 8 * h) = make_uint4(0, 0, 0, 0);
       }
-    }
   }
 };
 
 // <2 Y - Y^T, D> of the tile's part of D (never stored): Y = the r x r matrix at job.out (r = ld_out), one
 // partial sum per drain warp at parts + 16 job.o_row.
 struct OzEpiDot {
-  static constexpr bool kWarp = true;
+  static constexpr bool kWarp = true, kDigits = false;
   double* parts;
   __device__ __forceinline__ void warp(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     const double* Y = static_cast<const double*>(jb.out);
@@ -234,15 +242,15 @@ bool make_digit_map(CUtensorMap* m, const OzOperand& A, int box_rows) {
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <class Epi>
+template <int NS, class Epi>
 int run(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const int* skip,
         int* err, Epi epi, cudaStream_t st) {
   if (!n_jobs) return 0;
-  if (cudaFuncSetAttribute(oz::k_oz<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM) != cudaSuccess)
-    return -1;
+  constexpr int SMEM = oz::Cfg<NS>::SMEM;
+  if (cudaFuncSetAttribute(oz::k_oz<NS, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess) return -1;
   CUtensorMap ma, mb;
   if (!make_digit_map(&ma, A, oz::AROWS) || !make_digit_map(&mb, B, oz::BROWS)) return -1;
-  oz::k_oz<Epi><<<tc::persistent_grid(n_jobs), oz::NTHREADS, oz::SMEM, st>>>(ma, mb, A.ex, B.ex, jobs, n_jobs, segs, skip,
+  oz::k_oz<NS, Epi><<<tc::persistent_grid(n_jobs), oz::NTHREADS, SMEM, st>>>(ma, mb, A.ex, B.ex, jobs, n_jobs, segs, skip,
                                                                              err, epi);
   note_launch(1);
   return 0;
@@ -250,20 +258,26 @@ int run(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs,
 }  // namespace
 
 int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                   const int* skip, int* err, cudaStream_t st) {
-  return run(A, B, jobs, n_jobs, segs, skip, err, OzEpiRow{}, st);
+                   const int* skip, int ns, int* err, cudaStream_t st) {
+  int rc = 0;
+  OZ_DISPATCH(ns, (rc = run<NS>(A, B, jobs, n_jobs, segs, skip, err, OzEpiRow{}, st)));
+  return rc;
 }
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                     const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st) {
-  return run(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits{D, ld, exW}, st);
+                     const int* skip, uint16_t* D, int ld, const int* exW, int ns, int* err, cudaStream_t st) {
+  int rc = 0;
+  OZ_DISPATCH(ns, (rc = run<NS>(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits<NS>{D, ld, exW}, st)));
+  return rc;
 }
 int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    double* parts, int* err, cudaStream_t st) {
-  return run(A, B, jobs, n_jobs, segs, nullptr, err, OzEpiDot{parts}, st);
+  return run<8>(A, B, jobs, n_jobs, segs, nullptr, err, OzEpiDot{parts}, st);
 }
-int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int* err,
-                  cudaStream_t st) {
-  return run(A, A, jobs, n_jobs, segs, nullptr, err, OzEpiT{e_vir}, st);
+int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int ns,
+                  int* err, cudaStream_t st) {
+  int rc = 0;
+  OZ_DISPATCH(ns, (rc = run<NS>(A, A, jobs, n_jobs, segs, nullptr, err, OzEpiT{e_vir}, st)));
+  return rc;
 }
 
 }  // namespace osv

@@ -2,7 +2,7 @@
 //
 // The values of one operand row inside one chunk of 256 k share the scale 2^e, e the smallest
 // exponent with max|x| < 2^e.  Each is rounded to the integer F = round(x 2^(63 - e)) (exact down
-// to 2^-10 of the chunk's largest) and written in balanced base 256,
+// to 2^-10 of the chunk's largest; fewer bits with fewer than the eight slices) and written in balanced base 256,
 //   F = sum_{s=0..7} d_s 256^(7 - s),  |d_s| <= 128 (d_0: the remaining top part, |d_0| <= 128),
 // each digit a BF16 number (integers up to 256 are exact).  Integer arithmetic throughout.
 #pragma once
@@ -41,7 +41,15 @@ __device__ __forceinline__ int chunk_exp(unsigned emax) {
   return emax == 0 ? EX_ZERO : (emax == 2047 ? EX_NAN : (int)emax - 1022);
 }
 
-// Digit s (taken in the order s = 7 .. 0) of two values, as a BF16 pair.
+// round(x 2^(T - e)) for NS slices, T = 7 + 8 (NS - 1) (63 for eight).
+template <int NS>
+__device__ __forceinline__ long long fixedn(double x, unsigned emax) {
+  const long long F = fixed63(x, emax);
+  constexpr int D = 8 * (NSL - NS);
+  return D ? (F + (1ll << (D > 0 ? D - 1 : 0))) >> D : F;
+}
+
+// Digit s (taken in the order s = NS - 1 .. 0) of two values, as a BF16 pair.
 __device__ __forceinline__ uint32_t digit_pair(long long& f0, long long& f1, int s) {
   const int d0 = s ? (int)(signed char)(f0 & 255) : (int)f0, d1 = s ? (int)(signed char)(f1 & 255) : (int)f1;
   f0 = (f0 - d0) >> 8;
@@ -51,6 +59,7 @@ __device__ __forceinline__ uint32_t digit_pair(long long& f0, long long& f1, int
 
 // One row-chunk held by a warp: lane l has elements k = 64 u + 2 l + {0, 1}, u = 0 .. 3 (zero past the
 // end).  Writes the digits at dst + s * slice + k for k < kv and returns the exponent code.
+template <int NS>
 __device__ __forceinline__ int warp_slices(const double x[8], int kv, uint16_t* dst, size_t slice, int lane) {
   unsigned em = 0;
 #pragma unroll
@@ -61,9 +70,9 @@ __device__ __forceinline__ int warp_slices(const double x[8], int kv, uint16_t* 
   for (int u = 0; u < 4; u++) {
     const int k = 64 * u + 2 * lane;
     if (k >= kv) continue;
-    long long f0 = live ? fixed63(x[2 * u], em) : 0, f1 = live ? fixed63(x[2 * u + 1], em) : 0;
+    long long f0 = live ? fixedn<NS>(x[2 * u], em) : 0, f1 = live ? fixedn<NS>(x[2 * u + 1], em) : 0;
 #pragma unroll
-    for (int s = NSL - 1; s >= 0; s--)   // k + 1 may be one past an odd K: still inside the padded row
+    for (int s = NS - 1; s >= 0; s--)   // k + 1 may be one past an odd K: still inside the padded row
       *reinterpret_cast<uint32_t*>(dst + s * slice + k) = digit_pair(f0, f1, s);
   }
   return chunk_exp(em);

@@ -12,6 +12,8 @@
 //    e_m the smallest exponent with max_k |A[m][k]| < 2^e_m (oz_split.cuh): 63 fractional
 //    bits, ten more than the mantissa, so a value keeps its full mantissa down to 2^-10 of
 //    the row's largest in the chunk and an absolute 2^(e_m - 64) below that.
+//  * Callers that need less take fewer slices (NS = 5: 39 bits, 15 products; NS = 4: 31 bits, 10 products): the leading
+//    ones of the same digits.
 //  * A product a_s b_t of level l = s + t is at most 2^14, a chunk sum of one slice pair at
 //    most 2^22, and a sum of up to four pairs (levels 2-5) stays an exact FP32 integer
 //    whatever the accumulator's rounding; levels 6-9 have 5 to 8 pairs, whose sums pass 2^24
@@ -28,8 +30,14 @@
 // chunk's MMAs: every level has its own full / empty barrier, so level l of the next chunk
 // starts as soon as level l of this one has been read.
 //
+// The issuing thread's address arithmetic counts too: the 36 products of a K step are unrolled with
+// the slice offsets as constants added to one descriptor each (1.3x on the projections), K steps past
+// the end of a short chunk and quadrants without rows are skipped, and the digit epilogue requantises by
+// integer shifts.  Tensor pipe 50-71% active in the projections, 19-34% in contractions of a length of
+// ~56, which wait on their drain.
+//
 // Measured against the 64 x 64-tile FP64 CTA products (64 orbitals, 320 virtuals, 1200 aux): T_ii 8.5 ->
-// 0.95 ms, projections 53.4 -> 4.0 ms, exchange blocks 16.9 -> 3.2 ms, S and F 2.9 -> 0.53 ms, digits
+// 0.8 ms, projections 53.4 -> 3.2 ms, exchange blocks 16.9 -> 2.6 ms, S and F 2.9 -> 0.44 ms, digits
 // included; at 6 orbitals and 40 virtuals each is still faster or equal (T_ii 0.13 -> 0.05 ms), so there is
 // no size rule.  The CUDA-core kernels remain for calls without room for the digits.
 //
@@ -55,38 +63,46 @@ namespace oz {
 
 constexpr int A_TILE = BM * BK * 2;          // 8 KB per A slice tile (filled up to m rows)
 constexpr int B_TILE = BN * BK * 2;          // 4 KB per B slice tile (filled up to n rows)
-constexpr int STAGE = NSL * (A_TILE + B_TILE);
-constexpr int NSTAGE = 2;
-constexpr int SMEM = NSTAGE * STAGE + 1024;  // + slack for 1024-byte alignment
 constexpr int AROWS = 64, BROWS = 32;        // rows of one TMA box of the A and B operands
 constexpr int NDRAIN = 16;                   // drain warps
 constexpr int DCOL = BN * 4 / NDRAIN;        // columns of one: four warps share a TMEM lane quarter
 constexpr int NTHREADS = 64 + 32 * NDRAIN;
-constexpr int NLEV = 8;                      // levels 2 .. 9
 constexpr int KBC = CHUNK / BK;              // k-blocks of a full chunk
 constexpr int TMEM_COLS = 512;
 constexpr int ERR_TC_TIMEOUT = 16;           // same bit as ERR_TIMEOUT of the library
 
+template <int NS>
+struct Cfg {
+  static constexpr int STAGE = NS * (A_TILE + B_TILE);
+  static constexpr int NSTAGE = NS == 8 ? 2 : (NS == 5 ? 3 : 4);
+  static constexpr int SMEM = NSTAGE * STAGE + 1024;   // + slack for 1024-byte alignment
+  static constexpr int NBUF = NS <= 4 ? 2 : 1;         // sets of NS level accumulators in the 512 TMEM columns
+  static constexpr int UNIT = 14 + 8 * (NS < 6 ? NS - 1 : 5);   // the joined integer is in units of 2^(e_m + e_n - UNIT)
+};
+
 // acc + coef * v * 2^x for the sum x of two chunk exponents less the integer's unit; out of the
-// normal range: zero rows (EX_ZERO) add 0, non-finite rows (EX_NAN) give NaN, the rest through ldexp.
+// normal range: zero rows (EX_ZERO) add 0, non-finite rows (EX_NAN) give NaN, the rest in two factors.
+__device__ __forceinline__ double pow2(int x) { return __longlong_as_double((long long)(x + 1023) << 52); }
 __device__ __forceinline__ double oz_fma(long long v, int x, double coef, double acc) {
-  if (x >= -1022 && x <= 1023)
-    return fma((double)v, coef * __longlong_as_double((long long)(x + 1023) << 52), acc);
+  if (x >= -1022 && x <= 1023) return fma((double)v, coef * pow2(x), acc);
   if (x >= EX_NAN / 2) return __longlong_as_double(0x7FF8000000000000ll);
-  if (x <= EX_ZERO / 2) return acc;
-  return fma(coef, ldexp((double)v, x), acc);
+  if (x < -2040 || x > 2040) return x < 0 ? acc : acc + (double)v * __longlong_as_double(0x7FF0000000000000ll);
+  return fma(coef, (double)v * pow2(x / 2) * pow2(x - x / 2), acc);
 }
 
 // Epi: epi(job, row, col0, acc) stores columns col0 .. col0 + 15 of the tile's row (row < m_valid); or, when
 // Epi::kWarp, epi.warp(job, row, col0, acc) called by every lane of a drain warp, tiles without rows or columns
-// for it included.
-template <class Epi>
+// for it included; or, when Epi::kDigits, epi.digits(job, row, col0, F) with F = round(value 2^(T - e)),
+// T = epi.T, e = epi.exponent(job): a tile of one chunk comes there by an integer shift, never as an FP64 number.
+template <int NS, class Epi>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_oz(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const int* __restrict__ exA,
          const int* __restrict__ exB, const Job* __restrict__ jobs, int n_jobs, const Seg* __restrict__ segs,
          const int* __restrict__ skip, int* err, Epi epi) {
+  using C = Cfg<NS>;
+  constexpr int NST = C::NSTAGE, NB = C::NBUF;
   extern __shared__ uint8_t dsm[];
-  __shared__ __align__(8) uint64_t bar_full[NSTAGE], bar_empty[NSTAGE], bar_accf[NLEV], bar_acce[NLEV];
+  __shared__ __align__(8) uint64_t bar_full[NST], bar_empty[NST], bar_accf[NB * NS], bar_acce[NB * NS];
   __shared__ uint32_t s_tmem;
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = tc::su32(sm);
@@ -98,11 +114,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NSTAGE; s++) {
+    for (int s = 0; s < NST; s++) {
       tc::mbar_init(&bar_full[s], 1);
       tc::mbar_init(&bar_empty[s], 1);
     }
-    for (int l = 0; l < NLEV; l++) {
+    for (int l = 0; l < NB * NS; l++) {
       tc::mbar_init(&bar_accf[l], 1);
       tc::mbar_init(&bar_acce[l], NDRAIN);
     }
@@ -125,22 +141,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const Job jb = jobs[tile];
         if (jb.skip >= 0 && skip[jb.skip]) continue;
         const int nbox = (jb.n_valid + BROWS - 1) / BROWS, mbox = (jb.m_valid + AROWS - 1) / AROWS;
-        const uint32_t bytes = NSL * (mbox * AROWS + nbox * BROWS) * BK * 2;
+        const uint32_t bytes = NS * (mbox * AROWS + nbox * BROWS) * BK * 2;
         for (int q = 0; ok && q < jb.nseg; q++) {
           const Seg sg = segs[jb.seg0 + q];
           const int nkb = (sg.K + BK - 1) / BK, ra = sg.a.row + jb.m0, rb = sg.b.row + jb.n0;
           for (int c = 0; c < nkb; c++, g++) {
-            const int s = (int)(g % NSTAGE);
-            if (g >= NSTAGE) ok = tc::mbar_wait(tc::su32(&bar_empty[s]), (uint32_t)(((g / NSTAGE) - 1) & 1));
+            const int s = (int)(g % NST);
+            if (g >= NST) ok = tc::mbar_wait(tc::su32(&bar_empty[s]), (uint32_t)(((g / NST) - 1) & 1));
             if (!ok) break;
             const uint32_t fb = tc::su32(&bar_full[s]);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(bytes) : "memory");
-            const uint32_t st = sbase + s * STAGE;
-            for (int sl = 0; sl < NSL; sl++) {
+            const uint32_t st = sbase + s * C::STAGE;
+            for (int sl = 0; sl < NS; sl++) {
               for (int bx = 0; bx < mbox; bx++)
                 tc::tma_load_2d(st + sl * A_TILE + bx * AROWS * BK * 2, &tmA, fb, c * BK, ra + sl * sg.a.ss + bx * AROWS);
               for (int bx = 0; bx < nbox; bx++)
-                tc::tma_load_2d(st + NSL * A_TILE + sl * B_TILE + bx * BROWS * BK * 2, &tmB, fb, c * BK,
+                tc::tma_load_2d(st + NS * A_TILE + sl * B_TILE + bx * BROWS * BK * 2, &tmB, fb, c * BK,
                                 rb + sl * sg.b.ss + bx * BROWS);
             }
           }
@@ -149,8 +165,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (!ok) {
         // leaving early: let the copies already issued land first (bounded waits); only the
         // last armed k-block of each stage can be outstanding
-        for (long long gg = g - 1; gg >= 0 && gg >= g - NSTAGE; gg--)
-          tc::mbar_wait(tc::su32(&bar_full[gg % NSTAGE]), (uint32_t)((gg / NSTAGE) & 1));
+        for (long long gg = g - 1; gg >= 0 && gg >= g - NST; gg--)
+          tc::mbar_wait(tc::su32(&bar_full[gg % NST]), (uint32_t)((gg / NST) & 1));
       }
     }
   } else if (warp == 1) {
@@ -163,27 +179,37 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(npad >> 3) << 17) |
                                ((uint32_t)(BM >> 4) << 24);
         for (int q = 0; ok && q < jb.nseg; q++) {
-          const int nkb = (segs[jb.seg0 + q].K + BK - 1) / BK;
+          const int K = segs[jb.seg0 + q].K, nkb = (K + BK - 1) / BK;
           for (int c = 0; c < nkb; c++, g++) {
-            const int s = (int)(g % NSTAGE);
+            const int s = (int)(g % NST), b = (int)(ch % NB) * NS;
             const bool first = (c % KBC) == 0, last = (c % KBC) == KBC - 1 || c == nkb - 1;
-            ok = tc::mbar_wait(tc::su32(&bar_full[s]), (uint32_t)((g / NSTAGE) & 1));
+            const int nks = K - c * BK > 16 ? 2 : 1;             // 16-wide steps that hold elements
+            ok = tc::mbar_wait(tc::su32(&bar_full[s]), (uint32_t)((g / NST) & 1));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const uint32_t st = sbase + s * STAGE;
-            for (int l = 0; l < NLEV; l++) {
-              if (first && ch > 0) {
-                ok = tc::mbar_wait(tc::su32(&bar_acce[l]), (uint32_t)((ch - 1) & 1));
+            // one thread issues an MMA every ~50 cycles: descriptors by constant offsets from two bases
+            const uint32_t st = sbase + s * C::STAGE;
+            const uint64_t da = tc::desc_sw64(st), db = tc::desc_sw64(st + NS * A_TILE);
+            const uint32_t acc0 = first ? 0u : 1u;
+#pragma unroll
+            for (int l = 0; l < NS; l++) {
+              if (first && ch >= NB) {
+                ok = tc::mbar_wait(tc::su32(&bar_acce[b + l]), (uint32_t)((ch / NB - 1) & 1));
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;");
               }
-              const uint32_t dacc = tmem + (uint32_t)(l * BN);
+              const uint32_t dacc = tmem + (uint32_t)((b + l) * BN);
+#pragma unroll
               for (int sa = 0; sa <= l; sa++)                    // slices sa + sb = l (counted from 0)
-                for (int ks = 0; ks < BK / 16; ks++)
-                  tc::mma_f16(dacc, tc::desc_sw64(st + sa * A_TILE + ks * 32),
-                              tc::desc_sw64(st + NSL * A_TILE + (l - sa) * B_TILE + ks * 32), idesc,
-                              (first && sa == 0 && ks == 0) ? 0u : 1u);
-              if (last) tc::commit(&bar_accf[l]);
+                tc::mma_f16(dacc, da + (uint64_t)(sa * A_TILE >> 4), db + (uint64_t)((l - sa) * B_TILE >> 4), idesc,
+                            sa == 0 ? acc0 : 1u);
+              if (nks == 2) {
+#pragma unroll
+                for (int sa = 0; sa <= l; sa++)
+                  tc::mma_f16(dacc, da + (uint64_t)((sa * A_TILE + 32) >> 4),
+                              db + (uint64_t)(((l - sa) * B_TILE + 32) >> 4), idesc, 1u);
+              }
+              if (last) tc::commit(&bar_accf[b + l]);
             }
             if (!ok) break;
             tc::commit(&bar_empty[s]);
@@ -194,11 +220,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // wait (bounded) for the last commit of each stage: every MMA issued has then completed
       // and no arrival is in flight when the CTA exits
       if (!ok) {
-        tc::commit(&bar_empty[g % NSTAGE]);
+        tc::commit(&bar_empty[g % NST]);
         g++;
       }
-      for (long long gg = g - 1; gg >= 0 && gg >= g - NSTAGE; gg--)
-        tc::mbar_wait(tc::su32(&bar_empty[gg % NSTAGE]), (uint32_t)((gg / NSTAGE) & 1));
+      for (long long gg = g - 1; gg >= 0 && gg >= g - NST; gg--)
+        tc::mbar_wait(tc::su32(&bar_empty[gg % NST]), (uint32_t)((gg / NST) & 1));
     }
   } else {                                                       // ---- drain + epilogue
     const int quad = warp & 3;                                   // TMEM lane quarter of this warp
@@ -209,10 +235,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
       const Job jb = jobs[tile];
       if (jb.skip >= 0 && skip[jb.skip]) continue;
-      const bool live = col0 < jb.n_valid;                       // warp-uniform
-      double acc[DCOL];
+      const bool live = col0 < jb.n_valid && 32 * quad < jb.m_valid;   // warp-uniform
+      double acc[Epi::kDigits ? 1 : DCOL];
+      long long f[Epi::kDigits ? DCOL : 1];
+      int eout = 0;
+      if constexpr (Epi::kDigits) {
+        eout = epi.exponent(jb);
 #pragma unroll
-      for (int u = 0; u < DCOL; u++) acc[u] = 0.0;
+        for (int u = 0; u < DCOL; u++) f[u] = 0;
+      } else {
+#pragma unroll
+        for (int u = 0; u < DCOL; u++) acc[u] = 0.0;
+      }
       for (int q = 0; ok && q < jb.nseg; q++) {
         const Seg* sg = segs + jb.seg0 + q;
         const int nch = (sg->K + CHUNK - 1) / CHUNK;
@@ -220,51 +254,65 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int* eb_p = exB + sg->b.eb + (long long)(jb.n0 + min(col0 + (lane & (DCOL - 1)), jb.n_valid - 1)) * sg->b.es;
         const double coef = sg->coef;
         for (int c = 0; ok && c < nch; c++, ch++) {
-          const int ea = ea_p[c] - 54, eb = eb_p[c];
+          const int b = (int)(ch % NB) * NS;
+          const uint32_t ph = (uint32_t)((ch / NB) & 1);
+          const int ea = ea_p[c] - C::UNIT, eb = eb_p[c];
           long long v[DCOL];
-          int lo[DCOL];
+          int lo[NS > 6 ? DCOL : 1];
 #pragma unroll
-          for (int u = 0; u < DCOL; u++) {
-            v[u] = 0;
-            lo[u] = 0;
-          }
+          for (int u = 0; u < DCOL; u++) v[u] = 0;
 #pragma unroll
-          for (int l = 0; l < NLEV; l++) {
-            ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::su32(&bar_accf[l]), (uint32_t)(ch & 1)));
+          for (int l = 0; l < NS; l++) {
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::su32(&bar_accf[b + l]), ph));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
             uint32_t x[DCOL];
             if (live) {
-              OSV_TMEM_LD16(lcol + l * BN, x);
+              OSV_TMEM_LD16(lcol + (b + l) * BN, x);
               asm volatile("tcgen05.wait::ld.sync.aligned;");
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&bar_acce[l]);
+            if (lane == 0) tc::mbar_arrive(&bar_acce[b + l]);
             if (!live) continue;
 #pragma unroll
             for (int u = 0; u < DCOL; u++) {
               const int d = __float2int_rn(__uint_as_float(x[u]));
               if (l < 6) v[u] = (v[u] << 8) + d;                   // levels 2 .. 7
-              else if (l == 6) lo[u] = d;                          // level 8, unit 2^-8
-              else {                                               // level 9, unit 2^-16: the chunk is complete
+              if constexpr (NS > 6) {
+                if (l == 6) lo[u] = d;                             // level 8, unit 2^-8
+              }
+              if (l == NS - 1) {                                   // the chunk is complete
                 int e = ea + __shfl_sync(0xffffffffu, eb, u);
-                const long long w = ((long long)lo[u] << 8) + d;
-                long long t;
-                if ((unsigned long long)(v[u] + (1ll << 45)) >> 46) t = v[u] + ((w + 32768) >> 16);
-                else {                                             // room below: levels 8 and 9 in full
-                  t = (v[u] << 16) + w;
-                  e -= 16;
+                long long t = v[u];
+                if constexpr (NS > 6) {                            // level 9, unit 2^-16
+                  const long long w = ((long long)lo[u] << 8) + d;
+                  if ((unsigned long long)(t + (1ll << 45)) >> 46) t += (w + 32768) >> 16;
+                  else {                                           // room below: levels 8 and 9 in full
+                    t = (t << 16) + w;
+                    e -= 16;
+                  }
                 }
-                acc[u] = oz_fma(t, e, coef, acc[u]);
+                if constexpr (Epi::kDigits) {
+                  // F = t 2^(e + T - eout), rounded; |F| < 2^T since eout is a bound of the value
+                  const int sh = eout - Epi::T - e;
+                  f[u] += sh <= 0 ? (sh > -63 ? t << -sh : 0) : (sh < 63 ? (t + (1ll << (sh - 1))) >> sh : 0);
+                } else {
+                  acc[u] = oz_fma(t, e, coef, acc[u]);
+                }
               }
             }
           }
         }
       }
       if (!ok) break;
-      if constexpr (Epi::kWarp) epi.warp(jb, row, col0, acc);
-      else if (row < jb.m_valid && live) epi(jb, row, col0, acc);
+      if constexpr (Epi::kDigits) {
+        if (row < jb.m_valid && live) epi.digits(jb, row, col0, f);
+      } else if constexpr (Epi::kWarp) {
+        epi.warp(jb, row, col0, acc);
+      } else {
+        if (row < jb.m_valid && live) epi(jb, row, col0, acc);
+      }
     }
   }
   if (!ok) atomicOr(err, ERR_TC_TIMEOUT);
