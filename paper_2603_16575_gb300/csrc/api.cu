@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "osvmp2.h"
+#include "eig_topk.h"
 #include "internal.h"
 
 namespace {
@@ -78,6 +79,7 @@ struct osvmp2_ctx {
   osvmp2_opts opts{};
   std::string err;
   int num_sms = 148;
+  int eig_nclu[9] = {};              // resident clusters of the tridiagonalisation by size; [1] = 0: not yet asked
   std::vector<void*> sys_allocs;     // freed when a new system is set
   std::vector<void*> pair_allocs;    // pair store; freed with the system or on a precision change
   int pair_prec = -1;                // precision the pair store was built with
@@ -369,6 +371,11 @@ void ph_begin(osvmp2_ctx* c, int ph) {
   }
   cudaEventRecord(ev[c->ph_used[ph]], c->st);
 }
+const int* eig_nclu(osvmp2_ctx* c) {
+  if (c->eig_nclu[1] <= 0) eig_cluster_table(c->eig_nclu);
+  return c->eig_nclu;
+}
+
 void ph_end(osvmp2_ctx* c, int ph, double flops, double bytes = 0.0) {
   auto& ev = c->ph_ev[ph];
   if (ev.size() >= c->ph_used[ph] + 2) {
@@ -2201,7 +2208,7 @@ static int rosv_batch(osvmp2_ctx* c, double* T, int b, int i0, double l_osv, int
     CK(cudaGetLastError());
   }
   const double thr2 = l_osv * l_osv;
-  launch_eig_osv(M, b, ldm, thr2, ldm, Vs, ws, ks, es, c->err_d, false, c->st);
+  launch_eig_osv(M, b, ldm, thr2, ldm, Vs, ws, ks, es, c->err_d, false, eig_nclu(c), c->st);
   launch_eig_back(M, b, ldm, thr2, ldm, Vs, ks, es, false, c->st);
   launch_rosv_backq(Vs, ws, ks, Z, nrows, b, nv, n_max, ldm, kmax, V, w, k, c->st);
   CK(cudaGetLastError());
@@ -2339,7 +2346,7 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
       const double fl = (double)b * (full ? 9.0 * nd * nd * nd : (4.0 / 3.0) * nd * nd * nd);
       ph_begin(c, OSVMP2_PH_K_EIG);
       launch_eig_osv((double*)Tm.p, b, nv, l_osv, kmax, (double*)Vm.p, (double*)wm.p, (int*)km.p, (double*)sm.p,
-                     c->err_d, tii_tc, c->st);
+                     c->err_d, tii_tc, eig_nclu(c), c->st);
       ph_end(c, OSVMP2_PH_K_EIG, fl);
       launch_eig_back((double*)Tm.p, b, nv, l_osv, kmax, (double*)Vm.p, (const int*)km.p, (double*)sm.p, tii_tc,
                       c->st);
@@ -3373,7 +3380,7 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(Tc.p, Tm.p, (size_t)b * V2 * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
     launch_eig_osv((double*)Tm.p, b, nv, 0.0, nv, (double*)Vm.p, (double*)wm.p, (int*)km.p, (double*)em.p, c->err_d,
-                   false, c->st);
+                   false, eig_nclu(c), c->st);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(wh.data(), wm.p, (size_t)b * nv * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));

@@ -109,445 +109,6 @@ __device__ inline void cta_tridiag(T* A, int n, int lda, T* d, T* e, T* tau, T* 
   __syncthreads();
 }
 
-// Householder tridiagonalisation as cta_tridiag, for large n with A in global
-// memory: the symmetric matvec p = tau A' v is formed column-wise (thread c
-// owns column c and walks the rows, so every load instruction of a warp is
-// coalesced and a thread keeps many independent loads in flight), and the
-// rank-2 update is applied the same way.  Reflector k is also stored
-// contiguously in row k to the right of the diagonal (A[k][k+1+t] = v_t,
-// v_0 = 1; that part of the upper triangle is not read again), for the
-// back-transformation.
-template <int NTH = NT>
-__device__ inline void cta_tridiag_col(double* A, int n, int lda, double* d, double* e, double* tau, double* v,
-                                       double* p, double* red) {
-  const int tid = threadIdx.x;
-  __shared__ double s_tc, s_sc;
-  for (int k = 0; k + 2 < n; k++) {
-    const int L = n - k - 1;
-    double* Ak = A + (size_t)(k + 1) * lda + (k + 1);
-    double part = 0.0;
-    for (int t = tid; t < L; t += NTH) {
-      const double x = A[(size_t)(k + 1 + t) * lda + k];
-      v[t] = x;
-      if (t > 0) part += x * x;
-    }
-    const double sigma = cta_sum(part, red);
-    if (tid == 0) {
-      const double alpha = v[0];
-      double tu = 0.0, beta = alpha, sc = 0.0;
-      if (sigma > 0.0) {
-        const double mu = sqrt(alpha * alpha + sigma);
-        beta = alpha <= 0.0 ? mu : -mu;
-        tu = (beta - alpha) / beta;
-        sc = 1.0 / (alpha - beta);
-      }
-      s_tc = tu;
-      s_sc = sc;
-      d[k] = A[(size_t)k * lda + k];
-      e[k] = beta;
-      tau[k] = tu;
-    }
-    __syncthreads();
-    const double tk = s_tc;
-    if (tk != 0.0) {
-      const double sc = s_sc;
-      for (int t = tid; t < L; t += NTH) v[t] = (t == 0) ? 1.0 : v[t] * sc;
-      __syncthreads();
-      // p_c = tau sum_r A'[r][c] v_r   (A' symmetric)
-      for (int c = tid; c < L; c += NTH) {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        int r = 0;
-        for (; r + 3 < L; r += 4) {
-          const double a0 = Ak[(size_t)r * lda + c], a1 = Ak[(size_t)(r + 1) * lda + c];
-          const double a2 = Ak[(size_t)(r + 2) * lda + c], a3 = Ak[(size_t)(r + 3) * lda + c];
-          s0 = fma(a0, v[r], s0);
-          s1 = fma(a1, v[r + 1], s1);
-          s2 = fma(a2, v[r + 2], s2);
-          s3 = fma(a3, v[r + 3], s3);
-        }
-        for (; r < L; r++) s0 = fma(Ak[(size_t)r * lda + c], v[r], s0);
-        p[c] = tk * ((s0 + s1) + (s2 + s3));
-      }
-      __syncthreads();
-      double pv = 0.0;
-      for (int t = tid; t < L; t += NTH) pv += p[t] * v[t];
-      const double Kc = 0.5 * tk * cta_sum(pv, red);
-      for (int t = tid; t < L; t += NTH) p[t] -= Kc * v[t];
-      __syncthreads();
-      // A'[r][c] -= v_r w_c + w_r v_c
-      for (int c = tid; c < L; c += NTH) {
-        const double vc = v[c], wc = p[c];
-        int r = 0;
-        for (; r + 3 < L; r += 4) {
-          double* a = Ak + (size_t)r * lda + c;
-          const double a0 = a[0], a1 = a[lda], a2 = a[2 * (size_t)lda], a3 = a[3 * (size_t)lda];
-          a[0] = a0 - (v[r] * wc + p[r] * vc);
-          a[lda] = a1 - (v[r + 1] * wc + p[r + 1] * vc);
-          a[2 * (size_t)lda] = a2 - (v[r + 2] * wc + p[r + 2] * vc);
-          a[3 * (size_t)lda] = a3 - (v[r + 3] * wc + p[r + 3] * vc);
-        }
-        for (; r < L; r++) Ak[(size_t)r * lda + c] -= v[r] * wc + p[r] * vc;
-      }
-      for (int t = tid + 1; t < L; t += NTH) A[(size_t)(k + 1 + t) * lda + k] = v[t];
-      for (int t = tid; t < L; t += NTH) A[(size_t)k * lda + (k + 1 + t)] = v[t];
-    }
-    __syncthreads();
-  }
-  if (tid == 0) {
-    if (n >= 2) {
-      d[n - 2] = A[(size_t)(n - 2) * lda + (n - 2)];
-      e[n - 2] = A[(size_t)(n - 1) * lda + (n - 2)];
-      if (n >= 3) tau[n - 2] = 0.0;
-    }
-    d[n - 1] = A[(size_t)(n - 1) * lda + (n - 1)];
-    tau[n - 1] = 0.0;
-  }
-  __syncthreads();
-}
-
-// Householder tridiagonalisation of the symmetric A (row-major, lda, global
-// memory) keeping only its lower triangle, for the OSV eigenproblem.  Each
-// step fuses the rank-2 update of the previous reflector with the symmetric
-// matvec of the current one, in one pass over the lower triangle of the
-// trailing block: per stored element two FMAs of the update and two of the
-// matvec (its column sum and, through a shared-memory tile, its row sum),
-// against three FMAs per element of the full matrix and three passes over it
-// in cta_tridiag_col.  The trailing block is cut into 32 x 32 tiles, handled
-// by ntw warps in a fixed order; their partial sums go to gpart and are added
-// in a fixed order, so the result is deterministic.
-// Outputs as cta_tridiag_col: d, e, tau, and reflector k in row k to the right
-// of the diagonal (A[k][k+1+t] = v_t, v_0 = 1).
-// sm: 4 n + 64 doubles (vp, wp, vk, p, red) + ntw * 32 * 33 doubles of tiles;
-// gpart: nb (nb + 1) / 2 * 64 doubles, nb = ceil((n - 1) / 32).
-template <int NTH>
-__device__ inline void cta_tridiag_sym(double* A, int n, int lda, double* d, double* e, double* tau, double* sm,
-                                       int ntw, double* gpart) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double* vp = sm;            // previous reflector v_{k-1}, by global index (0 outside its range)
-  double* wp = vp + n;        // previous w_{k-1}
-  double* vk = wp + n;        // current reflector v_k
-  double* p = vk + n;         // A_k v_k, then w_k
-  double* red = p + n;        // 64
-  double* tiles = red + 64;   // ntw x 32 x 33
-  __shared__ double s_tc, s_sc;
-  for (int t = tid; t < n; t += NTH) { vp[t] = 0.0; wp[t] = 0.0; }
-  __syncthreads();
-  for (int k = 0; k + 2 < n; k++) {
-    const int L = n - k - 1, k1 = k + 1;
-    // (a) column k (rows k..n-1) receives the previous update
-    double part = 0.0;
-    for (int r = k + tid; r < n; r += NTH) {
-      double a = A[(size_t)r * lda + k];
-      if (k > 0) a = fma(-wp[r], vp[k], fma(-vp[r], wp[k], a));
-      if (r == k) d[k] = a;
-      else {
-        vk[r] = a;
-        if (r > k1) part += a * a;
-      }
-    }
-    // (b) Householder reflector of column k below the diagonal
-    const double sigma = cta_sum(part, red);
-    if (tid == 0) {
-      const double alpha = vk[k1];
-      double tu = 0.0, beta = alpha, sc = 0.0;
-      if (sigma > 0.0) {
-        const double mu = sqrt(alpha * alpha + sigma);
-        beta = alpha <= 0.0 ? mu : -mu;
-        tu = (beta - alpha) / beta;
-        sc = 1.0 / (alpha - beta);
-      }
-      s_tc = tu;
-      s_sc = sc;
-      e[k] = beta;
-      tau[k] = tu;
-    }
-    __syncthreads();
-    const double tk = s_tc, sc = s_sc;
-    for (int r = k1 + tid; r < n; r += NTH) {
-      const double v = (r == k1) ? 1.0 : vk[r] * sc;
-      vk[r] = (tk != 0.0) ? v : 0.0;
-      A[(size_t)k * lda + r] = v;                 // reflector, row storage
-    }
-    for (int t = tid; t < k1; t += NTH) vk[t] = 0.0;
-    __syncthreads();
-    // (c) fused sweep over the lower triangle of the trailing block
-    const int nb = (L + 31) >> 5;
-    const int ntile = nb * (nb + 1) / 2;
-    if (warp < ntw) {
-      double* tb = tiles + (size_t)warp * 32 * 33;
-      for (int tl = warp; tl < ntile; tl += ntw) {
-        int bi = 0;
-        while ((bi + 1) * (bi + 2) / 2 <= tl) bi++;
-        const int bj = tl - bi * (bi + 1) / 2;
-        const int r0 = k1 + 32 * bi, c0 = k1 + 32 * bj;
-        const int c = c0 + lane;
-        const bool cin = c < n;
-        const double vpc = cin ? vp[c] : 0.0, wpc = cin ? wp[c] : 0.0;
-        double colsum = 0.0;
-        for (int i0 = 0; i0 < 32; i0 += 8) {   // eight rows' loads in flight before their arithmetic
-          double av[8];
-#pragma unroll
-          for (int u = 0; u < 8; u++) {
-            const int r = r0 + i0 + u;
-            av[u] = (cin && r < n && r >= c) ? A[(size_t)r * lda + c] : 0.0;
-          }
-#pragma unroll
-          for (int u = 0; u < 8; u++) {
-            const int r = r0 + i0 + u;
-            double a = 0.0;
-            if (cin && r < n && r >= c) {
-              a = av[u];
-              if (k > 0) {
-                a = fma(-wp[r], vpc, fma(-vp[r], wpc, a));
-                A[(size_t)r * lda + c] = a;
-              }
-              colsum = fma(a, vk[r], colsum);
-            }
-            tb[(i0 + u) * 33 + lane] = (r > c) ? a : 0.0;   // the row sums take the strictly lower part
-          }
-        }
-        __syncwarp();
-        double rowsum = 0.0;
-        for (int j = 0; j < 32; j++) rowsum = fma(tb[lane * 33 + j], vk[min(c0 + j, n - 1)], rowsum);   // tb = 0 past n
-        double* gp = gpart + (size_t)tl * 64;
-        gp[lane] = colsum;
-        gp[32 + lane] = rowsum;
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    // (d) p = A_k v_k from the partial sums (fixed order), then w_k
-    double pv = 0.0;
-    for (int c = k1 + tid; c < n; c += NTH) {
-      const int b = (c - k1) >> 5, o = (c - k1) & 31;
-      double s = 0.0;
-      for (int bi = b; bi < nb; bi++) s += gpart[(size_t)(bi * (bi + 1) / 2 + b) * 64 + o];        // column sums
-      for (int bj = 0; bj <= b; bj++) s += gpart[(size_t)(b * (b + 1) / 2 + bj) * 64 + 32 + o];   // row sums
-      s *= tk;
-      p[c] = s;
-      pv += s * vk[c];
-    }
-    const double Kc = 0.5 * tk * cta_sum(pv, red);
-    for (int c = tid; c < n; c += NTH) {
-      const double w = (c >= k1) ? p[c] - Kc * vk[c] : 0.0;
-      wp[c] = w;
-      vp[c] = vk[c];
-    }
-    __syncthreads();
-  }
-  // the trailing 2 x 2 block receives the last update
-  if (tid == 0) {
-    if (n >= 2) {
-      const int a0 = n - 2, a1 = n - 1;
-      double x00 = A[(size_t)a0 * lda + a0], x10 = A[(size_t)a1 * lda + a0], x11 = A[(size_t)a1 * lda + a1];
-      if (n >= 3) {
-        x00 -= 2.0 * vp[a0] * wp[a0];
-        x10 -= vp[a1] * wp[a0] + wp[a1] * vp[a0];
-        x11 -= 2.0 * vp[a1] * wp[a1];
-        tau[n - 2] = 0.0;
-      }
-      d[a0] = x00;
-      e[a0] = x10;
-      d[a1] = x11;
-    } else {
-      d[0] = A[0];
-    }
-    tau[n - 1] = 0.0;
-  }
-  __syncthreads();
-}
-
-// ---------------------------------------------------------------- double-float
-// (arithmetic in common.cuh)
-// CTA sum in double-float (fixed order); red: >= 66 floats of shared memory.
-__device__ inline dfl cta_sum_df(dfl v, float* red) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = df_add(v, df_shfl_xor(v, o));
-  __syncthreads();
-  if (lane == 0) { red[2 * w] = v.h; red[2 * w + 1] = v.l; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    dfl s{0.f, 0.f};
-    for (int k = 0; k < nw; k++) s = df_add(s, dfl{red[2 * k], red[2 * k + 1]});
-    red[64] = s.h;
-    red[65] = s.l;
-  }
-  __syncthreads();
-  return dfl{red[64], red[65]};
-}
-
-// cta_tridiag_sym in double-float arithmetic, for the mixed-form OSV build
-// (whose T_ii carries ~35 significant bits, so the ~48 bits here do not limit
-// it): the same fused sweep over the lower triangle, with A held as (hi, lo)
-// FP32 pairs in place of its FP64 elements (converted on the first step).
-// Outputs in FP64: d, e, tau, and reflector k in row k to the right of the
-// diagonal (A[k][k+1+t] = v_t, v_0 = 1), as cta_tridiag_sym.
-// sm: 4 n + 64 doubles (vp, wp, vk, p as pairs; reductions) + ntw * 16 * 33 doubles of staging
-// tiles (each 32 x 32 tile goes through them in two halves of 16 rows, so that every warp of
-// the CTA fits one).
-// refl_df: reflector k stored as (hi, lo) pairs instead of FP64 (read by k_eig_back_df).
-template <int NTH>
-__device__ inline void cta_tridiag_sym_df(double* A, int n, int lda, double* d, double* e, double* tau, double* sm,
-                                          int ntw, double* gpart_d, bool refl_df) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  dfl* vp = reinterpret_cast<dfl*>(sm);   // previous reflector v_{k-1}
-  dfl* wp = vp + n;                        // previous w_{k-1}
-  dfl* vk = wp + n;                        // current reflector v_k
-  dfl* p = vk + n;                         // A_k v_k, then w_k
-  float* red = reinterpret_cast<float*>(p + n);   // 64 doubles of room
-  dfl* tiles = reinterpret_cast<dfl*>(sm + 4 * n + 64);   // ntw x 16 x 33 pairs
-  dfl* gpart = reinterpret_cast<dfl*>(gpart_d);
-  dfl* Ad = reinterpret_cast<dfl*>(A);     // element (r, c) of the lower triangle at Ad[r * lda + c]
-  __shared__ double s_tc, s_sc;
-  // the lower triangle to (hi, lo) pairs, in place
-  for (int r = warp; r < n; r += NTH / 32)
-    for (int c = lane; c <= r; c += 32) Ad[(size_t)r * lda + c] = df_from(A[(size_t)r * lda + c]);
-  for (int t = tid; t < n; t += NTH) { vp[t] = dfl{0.f, 0.f}; wp[t] = dfl{0.f, 0.f}; }
-  __syncthreads();
-  for (int k = 0; k + 2 < n; k++) {
-    const int L = n - k - 1, k1 = k + 1;
-    // (a) column k (rows k..n-1) receives the previous update
-    dfl part{0.f, 0.f};
-    const dfl vpk = vp[k], wpk = wp[k];
-    for (int r = k + tid; r < n; r += NTH) {
-      dfl a = Ad[(size_t)r * lda + k];
-      if (k > 0) a = df_fma(df_neg(wp[r]), vpk, df_fma(df_neg(vp[r]), wpk, a));
-      if (r == k) d[k] = df_to(a);
-      else {
-        vk[r] = a;
-        if (r > k1) part = df_fma(a, a, part);
-      }
-    }
-    // (b) Householder reflector of column k below the diagonal (scalars in FP64)
-    const double sigma = df_to(cta_sum_df(part, red));
-    if (tid == 0) {
-      const double alpha = df_to(vk[k1]);
-      double tu = 0.0, beta = alpha, sc = 0.0;
-      if (sigma > 0.0) {
-        const double mu = sqrt(alpha * alpha + sigma);
-        beta = alpha <= 0.0 ? mu : -mu;
-        tu = (beta - alpha) / beta;
-        sc = 1.0 / (alpha - beta);
-      }
-      s_tc = tu;
-      s_sc = sc;
-      e[k] = beta;
-      tau[k] = tu;
-    }
-    __syncthreads();
-    const double tk = s_tc;
-    const dfl scd = df_from(s_sc);
-    for (int r = k1 + tid; r < n; r += NTH) {
-      const dfl v = (r == k1) ? dfl{1.f, 0.f} : df_mul(vk[r], scd);
-      vk[r] = (tk != 0.0) ? v : dfl{0.f, 0.f};
-      if (refl_df) Ad[(size_t)k * lda + r] = v;    // reflector, row storage (not read again by this sweep)
-      else A[(size_t)k * lda + r] = df_to(v);
-    }
-    for (int t = tid; t < k1; t += NTH) vk[t] = dfl{0.f, 0.f};
-    __syncthreads();
-    // (c) fused sweep over the lower triangle of the trailing block
-    const int nb = (L + 31) >> 5;
-    const int ntile = nb * (nb + 1) / 2;
-    if (warp < ntw) {
-      dfl* tb = tiles + (size_t)warp * 16 * 33;
-      for (int tl = warp; tl < ntile; tl += ntw) {
-        int bi = 0;
-        while ((bi + 1) * (bi + 2) / 2 <= tl) bi++;
-        const int bj = tl - bi * (bi + 1) / 2;
-        const int r0 = k1 + 32 * bi, c0 = k1 + 32 * bj;
-        const int c = c0 + lane;
-        const bool cin = c < n;
-        const dfl nvpc = cin ? df_neg(vp[c]) : dfl{0.f, 0.f}, nwpc = cin ? df_neg(wp[c]) : dfl{0.f, 0.f};
-        dfl* gp = gpart + (size_t)tl * 64;
-        float csh = 0.f, csl = 0.f;   // column sum, unnormalised pair
-        for (int h = 0; h < 32; h += 16) {
-          for (int i0 = h; i0 < h + 16; i0 += 8) {   // eight rows' loads in flight before their arithmetic
-            dfl av[8];
-#pragma unroll
-            for (int u = 0; u < 8; u++) {
-              const int r = r0 + i0 + u;
-              av[u] = (cin && r < n && r >= c) ? Ad[(size_t)r * lda + c] : dfl{0.f, 0.f};
-            }
-#pragma unroll
-            for (int u = 0; u < 8; u++) {
-              const int r = r0 + i0 + u;
-              dfl a{0.f, 0.f};
-              if (cin && r < n && r >= c) {
-                a = av[u];
-                if (k > 0) {
-                  a = df_fma2(vp[r], nwpc, wp[r], nvpc, a);
-                  Ad[(size_t)r * lda + c] = a;
-                }
-                df_acc(csh, csl, a, vk[r]);
-              }
-              tb[(i0 - h + u) * 33 + lane] = (r > c) ? a : dfl{0.f, 0.f};   // the row sums take the strictly lower part
-            }
-          }
-          __syncwarp();
-          // row sums of these 16 rows: lane (g, rho) sums row rho over column half g, and the
-          // two halves are added in a fixed order
-          const int rho = lane & 15, g = lane >> 4;
-          float rsh = 0.f, rsl = 0.f;
-#pragma unroll 8
-          for (int j = 16 * g; j < 16 * g + 16; j++) df_acc(rsh, rsl, tb[rho * 33 + j], vk[min(c0 + j, n - 1)]);
-          const float oh = __shfl_xor_sync(0xffffffffu, rsh, 16), ol = __shfl_xor_sync(0xffffffffu, rsl, 16);
-          if (g == 0) {
-            float sh, st;
-            two_sum_f(rsh, oh, sh, st);
-            gp[32 + h + rho] = df_norm(sh, (rsl + ol) + st);
-          }
-          __syncwarp();
-        }
-        gp[lane] = df_norm(csh, csl);
-      }
-    }
-    __syncthreads();
-    // (d) p = A_k v_k from the partial sums (fixed order), then w_k
-    const dfl tkd = df_from(tk);
-    dfl pv{0.f, 0.f};
-    for (int c = k1 + tid; c < n; c += NTH) {
-      const int b = (c - k1) >> 5, o = (c - k1) & 31;
-      dfl s2{0.f, 0.f};
-      for (int bi = b; bi < nb; bi++) s2 = df_add(s2, gpart[(size_t)(bi * (bi + 1) / 2 + b) * 64 + o]);
-      for (int bj = 0; bj <= b; bj++) s2 = df_add(s2, gpart[(size_t)(b * (b + 1) / 2 + bj) * 64 + 32 + o]);
-      s2 = df_mul(s2, tkd);
-      p[c] = s2;
-      pv = df_fma(s2, vk[c], pv);
-    }
-    const dfl Kc = df_mul(df_from(0.5 * tk), cta_sum_df(pv, red));
-    const dfl nKc = df_neg(Kc);
-    for (int c = tid; c < n; c += NTH) {
-      const dfl w = (c >= k1) ? df_fma(nKc, vk[c], p[c]) : dfl{0.f, 0.f};
-      wp[c] = w;
-      vp[c] = vk[c];
-    }
-    __syncthreads();
-  }
-  // the trailing 2 x 2 block receives the last update
-  if (tid == 0) {
-    if (n >= 2) {
-      const int a0 = n - 2, a1 = n - 1;
-      double x00 = df_to(Ad[(size_t)a0 * lda + a0]), x10 = df_to(Ad[(size_t)a1 * lda + a0]);
-      double x11 = df_to(Ad[(size_t)a1 * lda + a1]);
-      if (n >= 3) {
-        const double v0 = df_to(vp[a0]), v1 = df_to(vp[a1]), w0 = df_to(wp[a0]), w1 = df_to(wp[a1]);
-        x00 -= 2.0 * v0 * w0;
-        x10 -= v1 * w0 + w1 * v0;
-        x11 -= 2.0 * v1 * w1;
-        tau[n - 2] = 0.0;
-      }
-      d[a0] = x00;
-      e[a0] = x10;
-      d[a1] = x11;
-    } else {
-      d[0] = df_to(Ad[0]);
-    }
-    tau[n - 1] = 0.0;
-  }
-  __syncthreads();
-}
-
 // Z (n x n, row-major, ldz) = H_0 H_1 ... H_{n-3} from the reflectors left in A.
 // y, vs: shared scratch of n doubles each.
 template <int NTH = NT>
@@ -687,7 +248,7 @@ __device__ inline int cta_syev(double* A, int n, int lda, double* w, double* Z, 
 // (Z[r][c] at Z[c * ldz + r]); a warp per column forms the dot products along
 // contiguous memory.  y, vs: shared scratch of n elements each.
 // T = double or float.  ROWV: reflector k in row k to the right of the diagonal
-// (cta_tridiag_sym) instead of below the sub-diagonal of column k (cta_tridiag).
+// (k_eig_tri) instead of below the sub-diagonal of column k (cta_tridiag).
 template <int NTH = NT, class T, bool ROWV = false>
 __device__ inline void cta_form_z_cm(const T* A, int n, int lda, const T* tau, T* Z, int ldz, T* y, T* vs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -880,102 +441,46 @@ __device__ inline void apply_qr_record_cm(T* Z, int ldz, int n, const int* swp, 
   __syncthreads();
 }
 
-// Full symmetric eigen-decomposition as cta_syev_cm (FP64, Z column-major), with the
-// implicit QR split as in the batched routines above: thread 0 chases the tridiagonal
-// and records its rotations into the storage of A (no longer needed once Z is formed;
-// lda == n), and the CTA applies each full record to the rows of Z, so the CTA waits
-// once per record instead of once per rotation.  With ntw >= 2 warps of tiles in sm
-// (after its 4 n + 64 doubles) the tridiagonalisation is the fused sweep cta_tridiag_sym,
-// its partial sums in gpart.  Returns 0 on success, 1 otherwise.
-template <int NTH = NT>
-__device__ inline int cta_syev_cm_rec(double* A, int n, double* w, double* Z, int ldz, double* e, double* tau,
-                                      double* sm, int ntw, double* gpart) {
-  double* v = sm;
-  double* p = sm + n;
-  double* red = sm + 4 * n;
-  __shared__ int s_rc, s_ns;
-  if (n == 1) {
-    if (threadIdx.x == 0) { w[0] = A[0]; Z[0] = 1.0; }
-    __syncthreads();
-    return 0;
-  }
-  if (ntw >= 2) {
-    cta_tridiag_sym<NTH>(A, n, n, w, e, tau, sm, ntw, gpart);
-    cta_form_z_cm<NTH, double, true>(A, n, n, tau, Z, ldz, v, p);
-  } else {
-    cta_tridiag<NTH>(A, n, n, w, e, tau, v, p, red);
-    cta_form_z_cm<NTH>(A, n, n, tau, Z, ldz, v, p);
-  }
-  for (int t = threadIdx.x; t < n; t += NTH) {   // the chase runs on shared copies of d and e
-    v[t] = w[t];
-    p[t] = (t + 1 < n) ? e[t] : 0.0;
-  }
-  __syncthreads();
-  const size_t room = (size_t)n * n;                       // doubles of A
-  const int cap_s = (int)(room / 8 > 16 ? room / 8 : 16);  // sweeps: two ints (one double) each
-  int* swp = reinterpret_cast<int*>(A);
-  double* rot = A + cap_s;
-  const int cap_r = (int)((room - (size_t)cap_s) / 2);     // rotations: (c, s) pairs
-  int rc = 1;
-  for (int chunk = 0; chunk < 64; chunk++) {
-    if (threadIdx.x == 0) {
-      int ns = 0;
-      s_rc = tridiag_qr_record(v, p, n, swp, cap_s, rot, cap_r, &ns, true);
-      s_ns = ns;
-    }
-    __syncthreads();
-    apply_qr_record_cm<NTH>(Z, ldz, n, swp, s_ns, rot);   // ends with a barrier
-    const int r = s_rc;
-    __syncthreads();                                      // every thread has read s_rc
-    if (r != 2) { rc = r; break; }
-  }
-  for (int t = threadIdx.x; t < n; t += NTH) w[t] = v[t];
-  __syncthreads();
-  return rc;
-}
-
 // ---------------------------------------------------------------- top-k
-// Number of eigenvalues of the tridiagonal (d, e) strictly below x
-// (Sturm sequence of the LDL^T pivots).
-__device__ inline int sturm_count(const double* d, const double* e, int n, double x, double pivmin) {
+// Number of eigenvalues of the tridiagonal (d, e) strictly below x: sign changes of the leading principal minors
+// of T - x I by their three-term recurrence, one FMA of chain a row (the LDL^T pivots, the ratios of the minors,
+// take an FP64 division a row, ~10 operations; an FP64 operation of a warp holds its sub-partition's pipe
+// for 64 cycles, so their number is the time).  The rounding is that of a relative change of d - x and e by a few
+// eps, as with the pivots.  ||T|| <= 1 (the caller scales by a power of two), so four rows grow a minor by
+// < 2^7; the two live ones are rescaled every four rows.  e2[i] = e[i]^2, at least 1e-60: no two
+// successive minors vanish, and the sign of a single zero does not change the count.
+__device__ __forceinline__ int sturm_count_minors(const double* d, const double* e2, int n, double x) {
+  double p0 = 0.0, p1 = 1.0;
   int cnt = 0;
-  double q = d[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  cnt += q < 0.0;
-  for (int i = 1; i < n; i++) {
-    q = d[i] - x - e[i - 1] * e[i - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    cnt += q < 0.0;
+  for (int i0 = 0; i0 < n; i0 += 4) {
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const int i = i0 + u;
+      if (i < n) {
+        const double ep = e2[i > 0 ? i - 1 : 0] * p0;
+        const double p = fma(d[i] - x, p1, -ep);
+        cnt += (__double2hiint(p) ^ __double2hiint(p1)) < 0;
+        p0 = p1;
+        p1 = p;
+      }
+    }
+    const int ex = max((__double2hiint(p0) >> 20) & 2047, (__double2hiint(p1) >> 20) & 2047);
+    const double sc = __hiloint2double(min(2046, max(1, 2046 - ex)) << 20, 0);   // 2^(1023 - ex)
+    p0 *= sc;
+    p1 *= sc;
   }
   return cnt;
 }
-
-// sturm_count with the squared off-diagonal e2[i] = e[i]^2 given.
-__device__ inline int sturm_count_sq(const double* d, const double* e2, int n, double x, double pivmin) {
-  int cnt = 0;
-  double q = d[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  cnt += q < 0.0;
-  for (int i = 1; i < n; i++) {
-    q = d[i] - x - e2[i - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    cnt += q < 0.0;
-  }
-  return cnt;
-}
-
 // Eigenvalues with ascending indices n-1-t, t < k, of (d, e) by multisection
-// on the Sturm count, called by one warp that handles t = t0, t0 + tstride, ...
-// (at most tcount of them):
+// on the Sturm count, called by one warp that handles t = t0, t0 + tstride, ...:
 // g = lane / L lanes per eigenvalue split its interval at L points per step
 // (log2(L+1) bits per Sturm sequence instead of one), until the interval is
 // below 2 eps |lambda| or atol (the eigenvalues of the tridiagonal are only
-// determined to ~eps ||T|| by its rounding).  e2 holds the squared
-// off-diagonal.  w[t] receives the eigenvalue.
+// determined to ~eps ||T|| by its rounding).  w[t] receives the eigenvalue times wscale.
 __device__ inline void multisect_eigs(const double* d, const double* e2, int n, int k, int t0, int tstride,
-                                      int tcount, double lo0, double hi0, double pivmin, double atol, double* w) {
+                                      double lo0, double hi0, double atol, double wscale, double* w) {
   const int lane = threadIdx.x & 31;
-  const int ng = min(tcount, (k - t0 + tstride - 1) / tstride);   // eigenvalues of this warp
+  const int ng = (k - t0 + tstride - 1) / tstride;   // eigenvalues of this warp
   if (ng <= 0) return;
   const int L = max(1, 32 / ng);
   const int gmax = 32 / L;                                  // groups per pass
@@ -991,7 +496,7 @@ __device__ inline void multisect_eigs(const double* d, const double* e2, int n, 
       if (!__any_sync(0xffffffffu, !done)) break;
       const double x = lo + (hi - lo) * (double)(q + 1) / (double)(L + 1);
       bool above = false;   // more than j eigenvalues below x: eigenvalue j lies below x
-      if (!done) above = sturm_count_sq(d, e2, n, x, pivmin) > j;
+      if (!done) above = sturm_count_minors(d, e2, n, x) > j;
       const unsigned bal = __ballot_sync(0xffffffffu, above);
       if (!done) {
         const unsigned bits = (bal >> ((lane / L) * L)) & ((L == 32) ? 0xffffffffu : ((1u << L) - 1u));
@@ -1001,10 +506,10 @@ __device__ inline void multisect_eigs(const double* d, const double* e2, int n, 
         if (!(nlo > lo || nhi < hi)) done = true;           // no progress at this precision
         lo = nlo;
         hi = nhi;
-        if (hi - lo <= fmax(2.0 * eps * fmax(fabs(lo), fabs(hi)), atol) + pivmin) done = true;
+        if (hi - lo <= fmax(2.0 * eps * fmax(fabs(lo), fabs(hi)), atol)) done = true;
       }
     }
-    if (mine && q == 0) w[t] = 0.5 * (lo + hi);
+    if (mine && q == 0) w[t] = 0.5 * (lo + hi) * wscale;
   }
   __syncwarp();
 }
@@ -1017,7 +522,7 @@ __device__ __forceinline__ dfl df_div(dfl a, dfl b) {
   const float q2 = __fdividef(r.h, b.h);
   return df_fast2(q1, q2);
 }
-// sturm_count_sq in double-float: d and e^2 as (hi, lo) pairs, x converted once;
+// Sturm count by the LDL^T pivots in double-float: d and e^2 as (hi, lo) pairs, x converted once;
 // pivmin in FP32 range.
 __device__ inline int sturm_count_df(const dfl* d, const dfl* e2, int n, double x, float pivmin) {
   const dfl nx = df_neg(df_from(x));
@@ -1037,7 +542,7 @@ __device__ inline int sturm_count_df(const dfl* d, const dfl* e2, int n, double 
 // warps of a CTA at once (t0 = warp, tstride = warps), so each eigenvalue gets
 // several lanes and rounds are few.
 __device__ inline void multisect_eigs_df(const dfl* d, const dfl* e2, int n, int k, int t0, int tstride,
-                                         double lo0, double hi0, float pivmin, double atol, double* w) {
+                                         double lo0, double hi0, float pivmin, double atol, double wscale, double* w) {
   const int lane = threadIdx.x & 31;
   const int ng = (k - t0 + tstride - 1) / tstride;          // eigenvalues of this warp
   if (ng <= 0) return;
@@ -1068,52 +573,13 @@ __device__ inline void multisect_eigs_df(const dfl* d, const dfl* e2, int n, int
         if (hi - lo <= fmax(2.0 * eps * fmax(fabs(lo), fabs(hi)), atol)) done = true;
       }
     }
-    if (mine && q == 0) w[t] = 0.5 * (lo + hi);
+    if (mine && q == 0) w[t] = 0.5 * (lo + hi) * wscale;
   }
   __syncwarp();
 }
 
-// One solve (T - lam I) x = y by Gaussian elimination with partial pivoting on
-// the tridiagonal; y is overwritten by x.  u0,u1,u2,mul: n doubles; piv: n ints.
-__device__ inline void tri_factor(const double* d, const double* e, int n, double lam, double small,
-                                  double* u0, double* u1, double* u2, double* mul, int* piv) {
-  double wa = d[0] - lam, wb = (n > 1) ? e[0] : 0.0;     // working row (col i, col i+1)
-  for (int i = 0; i + 1 < n; i++) {
-    const double c = e[i], a1 = d[i + 1] - lam, b1 = (i + 2 < n) ? e[i + 1] : 0.0;
-    if (fabs(wa) >= fabs(c)) {
-      double a = wa;
-      if (a == 0.0) a = small;
-      u0[i] = a; u1[i] = wb; u2[i] = 0.0;
-      const double m = c / a;
-      mul[i] = m; piv[i] = 0;
-      wa = a1 - m * wb;
-      wb = b1;
-    } else {
-      u0[i] = c; u1[i] = a1; u2[i] = b1;
-      const double m = wa / c;
-      mul[i] = m; piv[i] = 1;
-      const double na = wb - m * a1, nb = -m * b1;
-      wa = na; wb = nb;
-    }
-  }
-  u0[n - 1] = (wa == 0.0) ? small : wa;
-}
-__device__ inline void tri_solve(int n, const double* u0, const double* u1, const double* u2,
-                                 const double* mul, const int* piv, double* y) {
-  for (int i = 0; i + 1 < n; i++) {
-    if (piv[i]) { const double t = y[i]; y[i] = y[i + 1]; y[i + 1] = t; }
-    y[i + 1] -= mul[i] * y[i];
-  }
-  for (int i = n - 1; i >= 0; i--) {
-    double s = y[i];
-    if (i + 1 < n) s -= u1[i] * y[i + 1];
-    if (i + 2 < n) s -= u2[i] * y[i + 2];
-    y[i] = s / u0[i];
-  }
-}
-
-// The same factorisation and solve for many shifts at once, one per lane of a
-// warp: element i of a lane's arrays at [i * 32] from the lane's base pointer,
+// (T - lam I) x = y by Gaussian elimination with partial pivoting on the tridiagonal, for many
+// shifts at once, one per lane of a warp: element i of a lane's arrays at [i * 32] from the lane's base pointer,
 // so a warp's accesses are coalesced.  Branch-free, one division per row
 // (the inverse pivot ui = 1 / u0 is kept), so the lanes do not diverge.
 __device__ inline void tri_factor_lanes(const double* d, const double* e, int n, double lam, double small,

@@ -61,10 +61,10 @@ int launch_tii_tc(const float* Bt, long long rows, int n_aux, int ldx, const tc:
                   const double* e_vir, int* err, cudaStream_t st);
 // Eigen-decomposition of each T[b] and selection omega >= thr (all if thr <= 0),
 // at most kmax per orbital: V [nb][kmax][nv] (eigenvector-major), w [nb][kmax], k [nb], err |= ERR_*.
-// d, e, tau (3 nv) + Z (nv*nv, full path) or the tridiagonalisation's partial sums,
-// then 4 groups x 176 nv of lane-batched inverse iteration (top-k path)
-// Per-orbital scratch of k_eig_osv: d, e, tau; the work room (Z, partial sums,
-// inverse-iteration factors); the kept vectors as double-float pairs (mixed form).
+// nclu: eig_cluster_table.
+// Per-orbital scratch: d, e, tau (3 nv); the work room (exchange buffers of the tridiagonalisation, Z of a
+// full decomposition, 4 or more groups x 176 nv of lane-batched inverse iteration, the Gram matrix
+// of the kept vectors); the kept vectors of the tridiagonal.
 __host__ __device__ inline size_t eig_osv_work_doubles(int nv) {
   return (size_t)nv * nv > (size_t)4 * 176 * nv ? (size_t)nv * nv : (size_t)4 * 176 * nv;
 }
@@ -74,7 +74,7 @@ __host__ __device__ inline size_t eig_osv_scratch_doubles(int nv, int kmax) {
 // dfl_tridiag: the top-k path tridiagonalises in double-float arithmetic (the
 // mixed-form OSV build, whose T_ii is a split-precision product).
 void launch_eig_osv(double* T, int nb, int nv, double thr, int kmax, double* V, double* w, int* k,
-                    double* scratch, int* err, bool dfl_tridiag, cudaStream_t st);
+                    double* scratch, int* err, bool dfl_tridiag, const int* nclu, cudaStream_t st);
 // Back-transformation of the kept eigenvectors of the top-k path (n_vir above
 // the shared-memory limit, thr > 0) after launch_eig_osv; a no-op otherwise.
 void launch_eig_back(double* T, int nb, int nv, double thr, int kmax, double* V, const int* k, double* scratch,

@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "eig.cuh"
+#include "eig_topk.h"
 #include "internal.h"
 
 namespace osv {
@@ -65,14 +66,10 @@ void launch_tii(const BSrc& src, const double* e_vir, const double* f_occ, int n
 
 // ---------------------------------------------------------------- eigen
 constexpr int ZSMEM_MAX = 160;   // Z kept in shared memory up to this order
-// Orders up to this take the full decomposition also when only the eigenpairs above a threshold are wanted:
-// below it the fixed costs of the top-k path (multisection, inverse iteration) are the larger ones.
+// Orders up to this take one CTA per matrix from start to end: below it the fixed costs of the cluster
+// tridiagonalisation and of the top-k path (multisection, inverse iteration) are the larger ones.
 constexpr int EIG_FULL_MAX = 16;
-// Full decomposition with Z in shared memory: every eigenpair is wanted and Z fits, or the matrix is tiny.  (One
-// thread chases the bulge there: 46 ms at order 160 against 6 ms for the top-k path.)
-static bool eig_in_smem(int nv, double thr) { return thr > 0.0 ? nv <= EIG_FULL_MAX : nv <= ZSMEM_MAX; }
-constexpr int NT_EIG = 1024;     // threads of the OSV eigen kernel (more loads in flight)
-constexpr int INV_GROUPS = 4;    // warps running the lane-batched inverse iteration (176 n doubles each)
+constexpr int NT_EIG = 1024;     // threads of the full decomposition (rows of Z, and one warp that chases)
 constexpr int EB_DF_MAXN = 1536; // double-float back-transformation: the vector in registers up to this order
 
 // Sign eigenvector t (V[t][0..n), eigenvector-major) so that its largest-magnitude
@@ -99,32 +96,25 @@ __device__ inline void sign_vectors(double* V, int n, int k) {
   __syncthreads();
 }
 
-// Full decomposition path (n <= ZSMEM_MAX with Z in shared memory, or any n
-// with Z in global scratch): eigenvalues sorted descending, then selection.
-// zcm: Z column-major (eigenvector-major), for Z in global memory, where the rotations of the
-// QR sweeps then touch contiguous columns; row-major otherwise (Z in shared memory).
-// ntw (zcm only): warps of tiles after the 4 n + 64 doubles of sm for the fused sweep, whose
-// partial sums go to V (written only at the end); 0 for the plain tridiagonalisation.
-__device__ void eig_full_select(double* A, int n, double thr, int kmax, double* V, double* w, int* kout,
-                                double* scr, int* err, double* Zs, int ldz, double* sm, bool zcm, int ntw = 0) {
-  double* e = scr;
-  double* tau = scr + n;
-  double* ww = scr + 2 * n;
-  const int nbt = (n - 1 + 31) / 32;
-  if ((size_t)nbt * (nbt + 1) / 2 * 64 > (size_t)kmax * n) ntw = 0;   // the partial sums must fit V
-  int rc = zcm ? cta_syev_cm_rec<NT_EIG>(A, n, ww, Zs, ldz, e, tau, sm, ntw, V)
-               : cta_syev<NT_EIG>(A, n, n, ww, Zs, ldz, e, tau, sm);
+// The tail of a full decomposition: eigenvalues ww sorted descending, those >= thr (all when thr <= 0) with
+// their vectors, at most kmax.  Z(r, column t) at Zs[r * sr + t * sc]; perm: n ints of shared memory.
+__device__ void eig_select(const double* ww, int n, int rc, double thr, int kmax, double* V, double* w, int* kout,
+                           int* err, const double* Zs, int sr, int sc, int* perm) {
   __shared__ int s_k;
-  int* perm = reinterpret_cast<int*>(sm);   // sm reused: n ints (n <= 4n doubles)
-  if (threadIdx.x == 0) {
-    for (int t = 0; t < n; t++) perm[t] = t;
-    for (int t = 1; t < n; t++) {           // insertion sort, descending, stable
-      const int pv = perm[t];
-      const double x = ww[pv];
-      int u = t - 1;
-      while (u >= 0 && ww[perm[u]] < x) { perm[u + 1] = perm[u]; u--; }
-      perm[u + 1] = pv;
+  __syncthreads();
+  // rank of each eigenvalue (descending, ties by index; NaN after every number)
+  for (int t = threadIdx.x; t < n; t += NT_EIG) {
+    const double x = ww[t];
+    int at = 0;
+    for (int u = 0; u < n; u++) {
+      const double y = ww[u];
+      const bool yn = isnan(y), xn = isnan(x);
+      at += (yn || xn) ? (xn && !yn) || (xn && yn && u < t) : (y > x || (y == x && u < t));
     }
+    perm[at] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
     int k = 0;
     if (thr > 0.0) { while (k < n && ww[perm[k]] >= thr) k++; }
     else k = n;
@@ -140,285 +130,13 @@ __device__ void eig_full_select(double* A, int n, double thr, int kmax, double* 
   const int k = s_k;
   for (int idx = threadIdx.x; idx < n * k; idx += NT_EIG) {
     const int t = idx / n, r = idx % n;
-    V[(size_t)t * n + r] = zcm ? Zs[(size_t)perm[t] * ldz + r] : Zs[(size_t)r * ldz + perm[t]];
+    V[(size_t)t * n + r] = Zs[(size_t)r * sr + (size_t)perm[t] * sc];
   }
   __syncthreads();
   sign_vectors(V, n, k);
 }
 
-// Eigenpairs with eigenvalue >= thr only: tridiagonalise, count by Sturm
-// sequence, multisection for the kept eigenvalues, inverse iteration with
-// Gram-Schmidt inside clusters of close eigenvalues, back-transformation.
-__device__ void eig_topk(double* A, int n, double thr, int kmax, double* V, double* w, int* kout,
-                         double* scr, int* err, double* sm, int ntw, int dfl_tridiag) {
-  double* d = scr;
-  double* e = scr + n;
-  double* tau = scr + 2 * n;
-  double* v = sm;
-  double* p = sm + n;
-  double* red = sm + 2 * n;
-  __shared__ int s_k, s_nclu;
-  __shared__ double s_lo, s_hi, s_piv, s_norm;
-  if (ntw >= 2 && dfl_tridiag)
-    cta_tridiag_sym_df<NT_EIG>(A, n, n, d, e, tau, sm, ntw, scr + 3 * n, n <= EB_DF_MAXN);   // partial sums in the Z room
-  else if (ntw >= 2)
-    cta_tridiag_sym<NT_EIG>(A, n, n, d, e, tau, sm, ntw, scr + 3 * n);
-  else cta_tridiag_col<NT_EIG>(A, n, n, d, e, tau, v, p, red);
-  // Gershgorin bounds and a pivot floor
-  double glo = 1e300, ghi = -1e300, nrm = 0.0, emax = 0.0;
-  for (int t = threadIdx.x; t < n; t += NT_EIG) {
-    const double off = (t > 0 ? fabs(e[t - 1]) : 0.0) + (t + 1 < n ? fabs(e[t]) : 0.0);
-    glo = fmin(glo, d[t] - off);
-    ghi = fmax(ghi, d[t] + off);
-    nrm = fmax(nrm, fabs(d[t]) + off);
-    if (t + 1 < n) emax = fmax(emax, e[t] * e[t]);
-  }
-  glo = -cta_max(-glo, red);
-  ghi = cta_max(ghi, red);
-  nrm = cta_max(nrm, red);
-  emax = cta_max(emax, red);
-  int* clu = reinterpret_cast<int*>(p);     // cluster starts (reuses p)
-  if (threadIdx.x == 0) {
-    const double piv = 1e-290 * fmax(1.0, emax);
-    const double span = ghi - glo;
-    s_lo = glo - 1e-14 * span - piv;
-    s_hi = ghi + 1e-14 * span + piv;
-    s_piv = piv;
-    s_norm = nrm;
-    int k = n - sturm_count(d, e, n, thr, piv);
-    if (k > kmax) { k = kmax; atomicOr(err, ERR_SIZE); }
-    s_k = k;
-    *kout = k;
-  }
-  __syncthreads();
-  const int k = s_k;
-  // kept eigenvalues by multisection: warps 0-3 (one per SM sub-partition, whose
-  // FP64 pipes work in parallel), several lanes per eigenvalue
-  // (shared copies of d and e^2)
-  double* ds = p;
-  double* e2s = v;
-  for (int t = threadIdx.x; t < n; t += NT_EIG) {
-    ds[t] = d[t];
-    e2s[t] = (t + 1 < n) ? e[t] * e[t] : 0.0;
-  }
-  __syncthreads();
-  // Many kept eigenvalues (k >= 64): whole warps of one eigenvalue per lane (pure
-  // bisection, the fewest Sturm counts), so fewer warp instructions feed the FP64
-  // pipe; otherwise four warps, several lanes per eigenvalue.  The mixed-form
-  // build counts in double-float on every warp (its tridiagonal is double-float).
-  const double atol = 4.0 * 2.220446049250313e-16 * s_norm;
-  if (dfl_tridiag) {
-    dfl* dd = reinterpret_cast<dfl*>(ds);
-    dfl* de = reinterpret_cast<dfl*>(e2s);
-    for (int t = threadIdx.x; t < n; t += NT_EIG) {
-      dd[t] = df_from(ds[t]);
-      de[t] = df_from(e2s[t]);
-    }
-    __syncthreads();
-    const float pivf = 1e-30f * (float)fmax(1.0, emax);
-    multisect_eigs_df(dd, de, n, k, threadIdx.x >> 5, NT_EIG / 32, s_lo, s_hi, pivf, 5.7e-14 * s_norm, w);
-  } else if (k >= 64) {
-    const int wv = threadIdx.x >> 5;
-    if (32 * wv < k) multisect_eigs(ds, e2s, n, k, 32 * wv, 1, 32, s_lo, s_hi, s_piv, atol, w);
-  } else if ((threadIdx.x >> 5) < 4) {
-    multisect_eigs(ds, e2s, n, k, threadIdx.x >> 5, 4, k, s_lo, s_hi, s_piv, atol, w);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const double ortol = 1e-3 * s_norm;
-    int nc = 0;
-    for (int t = 0; t < k; t++)
-      if (t == 0 || w[t - 1] - w[t] > ortol) clu[nc++] = t;
-    clu[nc] = k;
-    s_nclu = nc;
-    for (int t = 0; t < k; t++)
-      if (!isfinite(w[t])) atomicOr(err, ERR_NONFINITE);
-  }
-  __syncthreads();
-  // inverse iteration, parallel over the kept vectors, one vector per LANE
-  // (lane-interleaved factorisations, so every instruction of a warp works for 32
-  // vectors): two solves from a seeded start, Gram-Schmidt inside each cluster of
-  // close eigenvalues (FP64: a warp per cluster; mixed form: the whole CTA per
-  // cluster, below), then one more
-  // solve per vector and the Gram-Schmidt again.  With shifts accurate to
-  // ~eps ||T||, one solve leaves a vector contaminated by an eigenvector at
-  // distance g at ~eps ||T|| / g, so the vectors separate without
-  // orthogonalising between every solve; the passes take care of
-  // (near-)degenerate groups.  Warps 0-3 (one per SM sub-partition) take the
-  // groups of 32 vectors; group slot w uses 176 n doubles of the scratch from
-  // scr + 3n (the tridiagonalisation's partial sums are no longer needed).
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const double small = 2.220446049250313e-16 * fmax(s_norm, 1e-300);
-  // The mixed-form build solves in double-float arithmetic (FP32 pipes; its
-  // tridiagonal carries ~48 bits): d and e (and the Gram-Schmidt dots) as pairs in
-  // the tridiagonalisation's tile room, when it holds them and the scales stay
-  // well inside FP32 range.
-  const bool inv_df = dfl_tridiag && ntw >= 2 && 2 * n + k <= ntw * 16 * 33 && s_norm > 1e-12 && s_norm < 1e12;
-  dfl* ddf = reinterpret_cast<dfl*>(sm + 4 * n + 64);
-  dfl* edf = ddf + n;
-  dfl* Vd = reinterpret_cast<dfl*>(scr + 3 * n + eig_osv_work_doubles(n));   // kept vectors, pairs [k][n]
-  dfl* gsd = edf + n;                                                          // -dots of one Gram-Schmidt step [k]
-  if (inv_df) {
-    for (int t = threadIdx.x; t < n; t += NT_EIG) {
-      ddf[t] = df_from(d[t]);
-      edf[t] = (t + 1 < n) ? df_from(e[t]) : dfl{0.f, 0.f};
-    }
-    __syncthreads();
-  }
-  for (int pass = 0; pass < 2; pass++) {
-    if (inv_df && warp < INV_GROUPS) {
-      double* base = scr + 3 * n + (size_t)warp * 176 * n;
-      dfl* ui = reinterpret_cast<dfl*>(base) + lane;
-      dfl* u1 = reinterpret_cast<dfl*>(base + 32 * (size_t)n) + lane;
-      dfl* u2 = reinterpret_cast<dfl*>(base + 64 * (size_t)n) + lane;
-      dfl* mul = reinterpret_cast<dfl*>(base + 96 * (size_t)n) + lane;
-      dfl* y = reinterpret_cast<dfl*>(base + 128 * (size_t)n) + lane;
-      int* piv = reinterpret_cast<int*>(base + 160 * (size_t)n) + lane;
-      for (int g = warp; 32 * g < k; g += INV_GROUPS) {
-        const int t = 32 * g + lane;
-        if (t < k) {
-          if (pass == 0 || k > 32 * INV_GROUPS)
-            tri_factor_lanes_df(ddf, edf, n, df_from(w[t]), (float)small, ui, u1, u2, mul, piv);
-          if (pass == 0) {
-#pragma unroll 4
-            for (int r = 0; r < n; r++) {
-              const uint64_t h = draw(0x5eedull + (uint64_t)t, (uint64_t)r);
-              y[32 * r] = dfl{(float)(uint32_t)(h >> 40) * 0x1p-24f - 0.5f, 0.f};
-            }
-          } else {
-#pragma unroll 4
-            for (int r = 0; r < n; r++) y[32 * r] = Vd[(size_t)t * n + r];
-          }
-          float sc = 1.f;   // scale of the previous solve, applied on the next read
-          for (int it = 0; it < 2 - pass; it++) {
-            const float am = tri_solve_lanes_df(n, sc, ui, u1, u2, mul, piv, y);
-            sc = am > 0.f ? 1.f / am : 0.f;
-          }
-          const dfl s{sc, 0.f};
-#pragma unroll 4
-          for (int r = 0; r < n; r++) Vd[(size_t)t * n + r] = df_mul(y[32 * r], s);
-        }
-      }
-    } else if (warp < INV_GROUPS) {
-      double* base = scr + 3 * n + (size_t)warp * 176 * n;
-      double* ui = base + lane;
-      double* u1 = base + 32 * (size_t)n + lane;
-      double* u2 = base + 64 * (size_t)n + lane;
-      double* mul = base + 96 * (size_t)n + lane;
-      double* y = base + 128 * (size_t)n + lane;
-      int* piv = reinterpret_cast<int*>(base + 160 * (size_t)n) + lane;
-      for (int g = warp; 32 * g < k; g += INV_GROUPS) {
-        const int t = 32 * g + lane;
-        if (t < k) {
-          // the second pass reuses the first pass's factorisation when every group kept its slot
-          if (pass == 0 || k > 32 * INV_GROUPS) tri_factor_lanes(d, e, n, w[t], small, ui, u1, u2, mul, piv);
-          if (pass == 0) {
-#pragma unroll 4
-            for (int r = 0; r < n; r++) {
-              const uint64_t h = draw(0x5eedull + (uint64_t)t, (uint64_t)r);
-              y[32 * r] = (double)(h >> 11) * 0x1p-53 - 0.5;
-            }
-          } else {
-#pragma unroll 8
-            for (int r = 0; r < n; r++) y[32 * r] = V[(size_t)t * n + r];
-          }
-          double sc = 1.0;   // normalisation of the previous solve, applied on the next read
-          for (int it = 0; it < 2 - pass; it++) {
-            const double nn = tri_solve_lanes(n, sc, ui, u1, u2, mul, piv, y);
-            sc = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
-          }
-#pragma unroll 8
-          for (int r = 0; r < n; r++) V[(size_t)t * n + r] = sc * y[32 * r];
-        }
-      }
-    }
-    __syncthreads();
-    if (inv_df) {
-      // Mixed form: the clusters one after another with the whole CTA, each vector
-      // orthogonalised against the earlier ones of its cluster by classical
-      // Gram-Schmidt applied twice (the dots one warp each, the update one thread
-      // per row), so the loads of a cluster's vectors overlap instead of one warp
-      // waiting on each in turn.  Double-float arithmetic on the pairs in Vd.
-      float* redf = reinterpret_cast<float*>(red);
-      for (int c = 0; c < s_nclu; c++) {
-        const int t0 = clu[c], t1 = clu[c + 1];
-        for (int t = t0; t < t1; t++) {
-          dfl* Vt = Vd + (size_t)t * n;
-          for (int rep = 0; rep < 2 && t > t0; rep++) {
-            for (int q = t0 + warp; q < t; q += NT_EIG / 32) {
-              const dfl* Vq = Vd + (size_t)q * n;
-              float dh = 0.f, dl = 0.f;
-              for (int r0 = lane; r0 < n; r0 += 32 * 4) {
-                dfl x[4], y2[4];
-#pragma unroll
-                for (int u = 0; u < 4; u++) {
-                  const int r = r0 + 32 * u;
-                  x[u] = r < n ? Vt[r] : dfl{0.f, 0.f};
-                  y2[u] = r < n ? Vq[r] : dfl{0.f, 0.f};
-                }
-#pragma unroll
-                for (int u = 0; u < 4; u++) df_acc(dh, dl, x[u], y2[u]);
-              }
-              dfl dot = df_norm(dh, dl);
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) dot = df_add(dot, df_shfl_xor(dot, o));
-              if (lane == 0) gsd[q - t0] = df_neg(dot);
-            }
-            __syncthreads();
-            for (int r = threadIdx.x; r < n; r += NT_EIG) {
-              dfl acc = Vt[r];
-              int q = t0;
-              for (; q + 4 <= t; q += 4) {
-                dfl vq[4];
-#pragma unroll
-                for (int u = 0; u < 4; u++) vq[u] = Vd[(size_t)(q + u) * n + r];
-#pragma unroll
-                for (int u = 0; u < 4; u++) acc = df_fma1(gsd[q + u - t0], vq[u], acc);
-              }
-              for (; q < t; q++) acc = df_fma1(gsd[q - t0], Vd[(size_t)q * n + r], acc);
-              Vt[r] = acc;
-            }
-            __syncthreads();
-          }
-          float nh = 0.f, nl = 0.f;
-          for (int r = threadIdx.x; r < n; r += NT_EIG) df_acc(nh, nl, Vt[r], Vt[r]);
-          const double nnd = df_to(cta_sum_df(df_norm(nh, nl), redf));
-          const dfl sc = df_from(nnd > 0.0 ? 1.0 / sqrt(nnd) : 0.0);
-          for (int r = threadIdx.x; r < n; r += NT_EIG) Vt[r] = df_mul(Vt[r], sc);
-          __syncthreads();
-        }
-      }
-    }
-    for (int c = warp; !inv_df && c < s_nclu; c += NT_EIG / 32) {   // Gram-Schmidt within clusters
-      const int t0 = clu[c], t1 = clu[c + 1];
-      for (int t = t0; t < t1; t++) {
-        double* Vt = V + (size_t)t * n;
-        for (int s = t0; s < t; s++) {
-          const double* Vs = V + (size_t)s * n;
-          double dot = 0.0;
-          for (int r = lane; r < n; r += 32) dot += Vt[r] * Vs[r];
-          dot = warp_sum(dot);
-          for (int r = lane; r < n; r += 32) Vt[r] -= dot * Vs[r];
-          __syncwarp();
-        }
-        double nn = 0.0;
-        for (int r = lane; r < n; r += 32) nn += Vt[r] * Vt[r];
-        nn = warp_sum(nn);
-        const double sc = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
-        for (int r = lane; r < n; r += 32) Vt[r] *= sc;
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-  }
-  if (inv_df) {   // the kept vectors to FP64
-    for (size_t idx = threadIdx.x; idx < (size_t)k * n; idx += NT_EIG) V[idx] = df_to(Vd[idx]);
-    __syncthreads();
-  }
-  // the back-transformation to the virtual basis is k_eig_back
-}
-
-// Back-transformation of the kept eigenvectors of eig_topk, one warp per
+// Back-transformation of the kept eigenvectors of the top-k path, one warp per
 // (orbital, vector) over the whole GPU (the vectors are independent, and
 // orbitals keep different numbers of them): x <- H_0 ... H_{n-3} x with the
 // reflectors stored contiguously in the rows of A and tau in the scratch, then
@@ -426,7 +144,7 @@ __device__ void eig_topk(double* A, int n, double thr, int kmax, double* V, doub
 constexpr int EB_WARPS = 8;
 
 // The same back-transformation in double-float for the mixed-form build (its
-// reflectors are stored as (hi, lo) pairs by cta_tridiag_sym_df): the vector
+// reflectors are stored as (hi, lo) pairs by k_eig_tri): the vector
 // lives in registers, NJ elements per lane (n <= 32 NJ), and every reflector
 // costs FP32 instructions only.
 template <int NJ>
@@ -531,63 +249,107 @@ __global__ void __launch_bounds__(EB_WARPS * 32) k_eig_back(const double* T, int
     for (int r = lane; r < n; r += 32) x[r] = -x[r];
 }
 
-__global__ void __launch_bounds__(NT_EIG) k_eig_osv(double* T, int nv, double thr, int kmax, double* V, double* w,
-                                                int* kout, double* scratch, int* err, int zsmem, int ntw,
-                                                int dfl_tridiag) {
+// Orders up to EIG_FULL_MAX: the whole decomposition by one CTA, everything in shared memory.
+__global__ void __launch_bounds__(NT_EIG) k_eig_small(double* T, int n, double thr, int kmax, double* V, double* w,
+                                                  int* kout, double* scratch, int* err) {
   extern __shared__ double dyn[];
-  const int b = blockIdx.x;
-  double* A = T + (size_t)b * nv * nv;
-  double* Vb = V + (size_t)b * nv * kmax;
-  double* wb = w + (size_t)b * kmax;
-  double* scr = scratch + (size_t)b * eig_osv_scratch_doubles(nv, kmax);
-  if (zsmem) {
-    const int ldz = nv + 1;
-    double* Zs = dyn;
-    double* sm = dyn + (size_t)nv * ldz;
-    eig_full_select(A, nv, thr, kmax, Vb, wb, kout + b, scr, err, Zs, ldz, sm, false);
-  } else if (thr > 0.0) {
-    eig_topk(A, nv, thr, kmax, Vb, wb, kout + b, scr, err, dyn, ntw, dfl_tridiag);
-  } else {
-    double* Zg = scr + 3 * nv;
-    eig_full_select(A, nv, thr, kmax, Vb, wb, kout + b, scr, err, Zg, nv, dyn, true, ntw);
-  }
+  const int b = blockIdx.x, ldz = n + 1;
+  double* scr = scratch + (size_t)b * eig_osv_scratch_doubles(n, kmax);
+  double* ww = scr + 2 * n;
+  double* sm = dyn + (size_t)n * ldz;
+  const int rc = cta_syev<NT_EIG>(T + (size_t)b * n * n, n, n, ww, dyn, ldz, scr, scr + n, sm);
+  eig_select(ww, n, rc, thr, kmax, V + (size_t)b * n * kmax, w + (size_t)b * kmax, kout + b, err, dyn, ldz, 1,
+             reinterpret_cast<int*>(sm));
 }
 
-// Warps of rows x 33-double staging tiles in the shared memory of the top-k path's
-// symmetric tridiagonalisation (0 when fewer than two fit): 32 rows in FP64, 16 in
-// double-float (whose sweep stages each tile in two halves).
-static int eig_tile_rows(bool dfl_tridiag) { return dfl_tridiag ? 16 : 32; }
-static int eig_tile_warps(int nv, double thr, int rows) {
-  // the top-k path and the full path with Z in global memory both sweep in tiles
-  if (eig_in_smem(nv, thr)) return 0;
-  const size_t cap = (size_t)224 * 1024 / sizeof(double), base = (size_t)4 * nv + 64, tile = (size_t)rows * 33;
-  const int ntw = cap > base ? (int)std::min<size_t>(NT_EIG / 32, (cap - base) / tile) : 0;
-  return ntw >= 2 ? ntw : 0;
+// Every eigenpair of a tridiagonalised matrix (k_eig_tri): Z from the reflectors, then the implicit QR, one
+// thread chasing and recording rotations into one half of the matrix's storage (free once Z is formed)
+// while the other warps apply the previous record to the rows of Z, one thread a row (column-major, so the accesses of
+// a warp are contiguous; in shared memory up to ZSMEM_MAX).  Bound by the chase (a chain of ~1.6 n^2
+// rotations of ~25 dependent FP64 operations) and, about equally at order 120, by the FP64 pipe of
+// the one SM in the application.  Against a CTA that waits for each rotation: 24 matrices of order 120 27 -> 16 ms,
+// 10 of order 50 6.5 -> 3.9.
+__global__ void __launch_bounds__(NT_EIG) k_eig_full(double* T, int n, double thr, int kmax, double* V, double* w,
+                                                 int* kout, double* scratch, int* err) {
+  extern __shared__ double dyn[];
+  const int b = blockIdx.x, tid = threadIdx.x;
+  double* A = T + (size_t)b * n * n;
+  double* scr = scratch + (size_t)b * eig_osv_scratch_doubles(n, kmax);
+  double* dv = dyn;
+  double* ev = dyn + n;
+  double* Z = n <= ZSMEM_MAX ? dyn + 2 * n : scr + 3 * n;
+  __shared__ int s_rc, s_ns[2];
+  cta_form_z_cm<NT_EIG, double, true>(A, n, n, scr + 2 * n, Z, n, dv, ev);
+  for (int t = tid; t < n; t += NT_EIG) {
+    dv[t] = scr[t];
+    ev[t] = t + 1 < n ? scr[n + t] : 0.0;
+  }
+  __syncthreads();
+  // two records of at most 32 n rotations each (a sweep is below n): sweeps as int pairs, then (c, s) pairs
+  const int half = n * n / 2, cap_s = half / 8, cap_r = min((half - cap_s) / 2, 32 * n);
+  int rc = 2;
+  if (tid == 0) s_rc = 2;
+  for (int c = 0; c <= 40 * n + 100; c++) {   // each record holds at least one sweep
+    double* rec = A + (size_t)(c & 1) * half;
+    const double* old = A + (size_t)((c + 1) & 1) * half;
+    if (tid == 0) {
+      int ns = 0;
+      if (rc == 2) s_rc = tridiag_qr_record(dv, ev, n, reinterpret_cast<int*>(rec), cap_s, rec + cap_s, cap_r, &ns, true);
+      s_ns[c & 1] = ns;
+    } else if (tid >= 32 && c > 0) {
+      const int* swp = reinterpret_cast<const int*>(old);
+      const int ns = s_ns[(c + 1) & 1];
+      for (int row = tid - 32; row < n; row += NT_EIG - 32) {
+        double* zr = Z + row;
+        const double* cs = old + cap_s;
+        for (int q = 0; q < ns; q++) {
+          const int l = swp[2 * q], h = swp[2 * q + 1];
+          double carry = zr[(size_t)l * n];
+          for (int k = l; k < h; k++, cs += 2) {
+            const double co = cs[0], si = cs[1];
+            const double y = zr[(size_t)(k + 1) * n];
+            zr[(size_t)k * n] = co * carry + si * y;
+            carry = -si * carry + co * y;
+          }
+          zr[(size_t)h * n] = carry;
+        }
+      }
+    }
+    __syncthreads();
+    if (rc != 2) break;   // the last record has been applied
+    rc = s_rc;
+    __syncthreads();
+  }
+  double* ww = scr + n;   // the sub-diagonal is no longer needed
+  for (int t = tid; t < n; t += NT_EIG) ww[t] = dv[t];
+  eig_select(ww, n, rc, thr, kmax, V + (size_t)b * n * kmax, w + (size_t)b * kmax, kout + b, err, Z, 1, n,
+             reinterpret_cast<int*>(ev));
 }
 
 void launch_eig_osv(double* T, int nb, int nv, double thr, int kmax, double* V, double* w, int* k,
-                    double* scratch, int* err, bool dfl_tridiag, cudaStream_t st) {
-  const int zsmem = eig_in_smem(nv, thr);
-  if (nv <= ZSMEM_MAX) dfl_tridiag = false;   // FP64 in both forms at these orders
-  size_t smem = (size_t)(4 * nv + 64) * sizeof(double);
-  // the full path (thr <= 0) sweeps in FP64 tiles whatever dfl_tridiag says
-  const int rows = (thr > 0.0) ? eig_tile_rows(dfl_tridiag) : eig_tile_rows(false);
-  const int ntw = eig_tile_warps(nv, thr, rows);
-  if (zsmem) smem += (size_t)nv * (nv + 1) * sizeof(double);
-  else if (ntw >= 2) smem += (size_t)ntw * rows * 33 * sizeof(double);
-  cudaFuncSetAttribute(k_eig_osv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_eig_osv<<<nb, NT_EIG, smem, st>>>(T, nv, thr, kmax, V, w, k, scratch, err, zsmem, ntw, dfl_tridiag ? 1 : 0);
-  note_launch(1);
+                    double* scratch, int* err, bool dfl_tridiag, const int* nclu, cudaStream_t st) {
+  if (nv <= EIG_FULL_MAX) {
+    const size_t smem = ((size_t)nv * (nv + 1) + 4 * nv + 64) * sizeof(double);
+    k_eig_small<<<nb, NT_EIG, smem, st>>>(T, nv, thr, kmax, V, w, k, scratch, err);
+    note_launch(1);
+  } else if (thr > 0.0) {
+    const bool df = dfl_tridiag && nv > ZSMEM_MAX;   // FP64 in both forms below
+    launch_eig_topk(T, nb, nv, thr, kmax, V, w, k, scratch, err, df, df && nv <= EB_DF_MAXN, nclu, st);
+  } else {
+    launch_eig_tridiag(T, nb, nv, kmax, scratch, err, nclu, st);
+    const size_t smem = (2 * (size_t)nv + (nv <= ZSMEM_MAX ? (size_t)nv * nv : 0)) * sizeof(double);
+    cudaFuncSetAttribute(k_eig_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_eig_full<<<nb, NT_EIG, smem, st>>>(T, nv, thr, kmax, V, w, k, scratch, err);
+    note_launch(1);
+  }
 }
 
 void launch_eig_back(double* T, int nb, int nv, double thr, int kmax, double* V, const int* k, double* scratch,
                      bool dfl_tridiag, cudaStream_t st) {
-  if (eig_in_smem(nv, thr) || !(thr > 0.0)) return;   // the other paths form the eigenvectors in k_eig_osv
-  if (nv <= ZSMEM_MAX) dfl_tridiag = false;
-  const int ntw = eig_tile_warps(nv, thr, eig_tile_rows(dfl_tridiag));
+  if (nv <= EIG_FULL_MAX || !(thr > 0.0)) return;   // the other paths form the eigenvectors themselves
   dim3 grid(nb, (std::min(kmax, nv) + EB_WARPS - 1) / EB_WARPS);
   const size_t ss = eig_osv_scratch_doubles(nv, kmax);
-  if (dfl_tridiag && ntw >= 2 && nv <= EB_DF_MAXN) {   // reflectors stored as pairs
+  if (dfl_tridiag && nv > ZSMEM_MAX && nv <= EB_DF_MAXN) {   // reflectors stored as pairs
     if (nv <= 640) k_eig_back_df<20><<<grid, EB_WARPS * 32, 0, st>>>(T, nv, kmax, V, k, scratch, ss);
     else if (nv <= 1280) k_eig_back_df<40><<<grid, EB_WARPS * 32, 0, st>>>(T, nv, kmax, V, k, scratch, ss);
     else k_eig_back_df<48><<<grid, EB_WARPS * 32, 0, st>>>(T, nv, kmax, V, k, scratch, ss);

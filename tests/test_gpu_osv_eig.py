@@ -1,0 +1,67 @@
+"""OSV eigenpairs where the cluster tridiagonalisation and the top-k path can go wrong.
+
+Orders around the tile (32 rows), around the change of path (16 / 17) and with tiles that do not fit shared
+memory; one orbital (the largest clusters) to more orbitals than SMs (none); flat and steep spectra, every eigenvalue
+doubled (Gram-Schmidt inside clusters), all eigenpairs (implicit QR) or those above a threshold.  Tolerances,
+with eps = 2^-53: Householder reduction and back-transformation have a backward error of a few n eps ||T||_F and
+lose a few n eps of orthogonality, bisection stops at 8 eps ||T||; double-float pairs carry 2^-45 in place of
+2^-53, and the mixed form's T_ii itself is good to ~2^-33.
+"""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+EPS = 2.0 ** -53
+
+
+def _system(n_occ, n_vir, seed, spread, twice):
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    m = n_vir // 2 if twice else n_vir
+    n_aux = m + 9
+    B = torch.randn((n_occ, m, n_aux), dtype=torch.float64, device=DEV, generator=g)
+    B *= torch.exp(-spread * torch.rand((n_occ, m, 1), dtype=torch.float64, device=DEV, generator=g))
+    e = 0.1 + 4.9 * torch.rand(m, dtype=torch.float64, device=DEV, generator=g)
+    if twice:
+        z = torch.zeros_like(B)
+        B = torch.cat([torch.cat([B, z], 2), torch.cat([z, B], 2)], 1).contiguous()
+        e = torch.cat([e, e])
+    f = torch.diag(-1.5 + 1.2 * torch.rand(n_occ, dtype=torch.float64, device=DEV, generator=g))
+    return B, e, f
+
+
+@pytest.mark.parametrize("n_occ,n_vir", [(1, 16), (1, 17), (2, 31), (3, 33), (1, 64), (5, 65), (160, 40), (1, 160),
+                                         (7, 161), (20, 200), (160, 96), (50, 243), (1, 300), (3, 520), (30, 520)])
+@pytest.mark.parametrize("spread,twice,cut", [(0.0, False, 0.3), (12.0, False, 1e-6), (3.0, True, 1e-2),
+                                              (6.0, False, 0.0)])
+def test_osv_eigenpairs(n_occ, n_vir, spread, twice, cut):
+    from paper_2603_16575_gb300 import Context
+    if cut == 0.0 and n_vir > 250:
+        pytest.skip("every eigenpair: the implicit QR is covered below this order")
+    n_vir -= n_vir % 2 if twice else 0
+    B, e, f = _system(n_occ, n_vir, 7 * n_vir + n_occ, spread, twice)
+    d = e[:, None] + e[None, :]
+    T = [(B[i] @ B[i].T) / (d - 2.0 * f[i, i]) for i in range(n_occ)]
+    ref = [torch.linalg.eigvalsh(t).flip(0) for t in T]
+    l_osv = 0.0
+    if cut:                                   # a threshold away from every eigenvalue
+        l_osv = cut * float(ref[0][0])
+        ws = torch.cat(ref)
+        while ((ws - l_osv).abs() < 1e-9 * l_osv).any():
+            l_osv *= 1.0 + 1e-7
+    for prec, eps in (("fp64", EPS), ("mixed", 2.0 ** -45 if n_vir > 160 else EPS)):
+        ctx = Context(0, osv_prec=prec)
+        k = ctx.build_osv(f, e, l_osv, B=B)
+        for i in {0, n_occ // 2, n_occ - 1}:
+            Q, w = ctx.get_osv(i)
+            nrm = float(ref[i][0])
+            frob = float(torch.linalg.norm(ref[i]))
+            t_err = 0.0 if prec == "fp64" else 2.0 ** -30 * nrm
+            if prec == "fp64":
+                assert int(k[i]) == int((ref[i] >= l_osv).sum()) if cut else int(k[i]) == n_vir
+            kk = int(k[i])
+            assert (w - ref[i][:kk]).abs().max() <= 8 * n_vir * eps * frob + t_err
+            assert (T[i] @ Q - Q * w).abs().max() <= 8 * n_vir * eps * frob + 4 * t_err
+            assert (Q.T @ Q - torch.eye(kk, dtype=Q.dtype, device=DEV)).abs().max() <= 8 * n_vir * eps
+        ctx.close()
