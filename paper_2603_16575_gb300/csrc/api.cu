@@ -116,10 +116,10 @@ struct osvmp2_ctx {
   std::vector<double*> S_h, F_h, K_h, X_h, et_h, bt_h, Kt_h;
   std::vector<float*> U_h, Gi_h, Gj_h;   // mixed form: per pair U = P X and G = U^T B
   std::vector<float*> Sh_h, Gh_h;        // mixed form: preconditioner leftovers (NULL: exact X)
-  // mixed form: where the TF32 slices of U_p^T live (allocation base, its rows, first row)
-  std::vector<float*> us_base_h;
-  std::vector<long long> us_alloc_rows_h, us_row_h;
-  int us_ldv = 0;
+  // mixed form: digits of U_p (MXSL slices, K = n_vir) of each pair: store of its build and matrix in it
+  std::vector<OzOperand> um_store;
+  std::vector<int> um_of;
+  std::vector<oz::Mat> um_mat;
   // FP64 form: digits of U_p (polished basis) of each pair: store of its build and matrix in it (-1: none)
   std::vector<void*> ud_alloc;
   std::vector<char> pm_basis;        // FP64 form: pair bases from the batched preconditioner
@@ -309,7 +309,7 @@ void free_system(osvmp2_ctx* c) {
   c->sf_id.clear(); c->pair_id.clear(); c->bt_id.clear();
   c->S_h.clear(); c->F_h.clear(); c->K_h.clear(); c->X_h.clear(); c->et_h.clear(); c->bt_h.clear(); c->Kt_h.clear();
   c->U_h.clear(); c->Gi_h.clear(); c->Gj_h.clear(); c->Sh_h.clear(); c->Gh_h.clear();
-  c->us_base_h.clear(); c->us_alloc_rows_h.clear(); c->us_row_h.clear();
+  c->um_store.clear(); c->um_of.clear(); c->um_mat.clear();
   c->ud_store.clear(); c->ud_of.clear(); c->ud_mat.clear();
   c->m_h.clear(); c->pi_h.clear(); c->pj_h.clear();
   c->frags.clear(); c->frag_out.clear(); c->weak.clear(); c->weak_e.clear();
@@ -525,7 +525,7 @@ int reset_pairs(osvmp2_ctx* c) {
   c->bt_id.assign(nn, -1);
   c->S_h.clear(); c->F_h.clear(); c->K_h.clear(); c->X_h.clear(); c->et_h.clear(); c->bt_h.clear(); c->Kt_h.clear();
   c->U_h.clear(); c->Gi_h.clear(); c->Gj_h.clear(); c->Sh_h.clear(); c->Gh_h.clear();
-  c->us_base_h.clear(); c->us_alloc_rows_h.clear(); c->us_row_h.clear();
+  c->um_store.clear(); c->um_of.clear(); c->um_mat.clear();
   c->ud_store.clear(); c->ud_of.clear(); c->ud_mat.clear();
   c->m_h.clear(); c->pi_h.clear(); c->pj_h.clear(); c->r_h.clear();
   TRY(upload(c, c->sf_id_d, c->sf_id));
@@ -605,83 +605,6 @@ double fragment_mixed_flops(const osvmp2_ctx* c, const Frag& f, int iters) {
     }
   return setup + iters * sweep;
 }
-
-// Build S/F blocks, projections, K and preconditioners for every listed pair
-// (and the diagonal pairs of its orbitals) that is not built yet.
-// Mixed form: G_p,x = U_p^T B_x for every G job on the tensor cores.  The
-// orbitals x are processed in batches whose B_x^T slices fit a fixed budget;
-// within a batch the tiles are ordered by (x, aux tile, pair) so that the
-// pairs sharing an aux tile of B_x read it while it is resident in L2.
-int gproj_tensor(osvmp2_ctx* c, const std::vector<GJob>& gj, const std::vector<long long>& usrow, const float* Us,
-                 long long us_rows, int ldv, long long lo_shift) {
-  const int nv = c->sys.n_vir, nx = c->sys.n_aux, n = c->sys.n_occ;
-  if (us_rows + tc::BN >= (long long)INT32_MAX)
-    return fail(c, OSVMP2_E_ARG, "U slice store exceeds the tensor-map row range");
-  std::vector<std::vector<int>> by_x(n);
-  for (size_t q = 0; q < gj.size(); q++) by_x[gj[q].x].push_back((int)q);
-  std::vector<int> xs;
-  for (int x = 0; x < n; x++)
-    if (!by_x[x].empty()) xs.push_back(x);
-  if (xs.empty()) return 0;
-  const size_t slot_bytes = (size_t)tc::NSL * nx * ldv * sizeof(float);
-  const size_t budget = (size_t)4 << 30;
-  const size_t per_batch = std::max<size_t>(1, std::min<size_t>(xs.size(), budget / slot_bytes));
-  if ((long long)per_batch * tc::NSL * nx + tc::BM >= (long long)INT32_MAX)
-    return fail(c, OSVMP2_E_ARG, "B slice batch exceeds the tensor-map row range");
-  Tmp bs, xd;
-  TRY(tmp_alloc(c, bs, per_batch * slot_bytes));
-  TRY(tmp_alloc(c, xd, xs.size() * sizeof(int)));
-  CK(cudaMemcpyAsync(xd.p, xs.data(), xs.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
-  const int n_mt = (nx + tc::BM - 1) / tc::BM;
-  for (size_t b0 = 0; b0 < xs.size(); b0 += per_batch) {
-    const int nb = (int)std::min(per_batch, xs.size() - b0);
-    launch_bslices(bsrc(c), (const int*)xd.p + b0, nb, (float*)bs.p, ldv, c->st);
-    CK(cudaGetLastError());
-    // Tile order: per orbital x, blocks of PB (pair, column tile) jobs, each with all
-    // its aux tiles; a wave of the persistent grid then holds every aux tile of B_x
-    // and only PB tiles of the U slices, so the B_x tiles stay in L2 across the
-    // waves of x and every U tile is read once.
-    const int PB = std::max(1, c->num_sms / std::max(1, n_mt));
-    std::vector<tc::Job> jobs;
-    for (int u = 0; u < nb; u++) {
-      std::vector<std::pair<int, int>> pn;   // (G job, first column)
-      for (int q : by_x[xs[b0 + u]])
-        for (int n0 = 0; n0 < gj[q].r; n0 += tc::BN) pn.push_back({q, n0});
-      for (size_t p0 = 0; p0 < pn.size(); p0 += PB)
-        for (int mt = 0; mt < n_mt; mt++)
-          for (size_t pp = p0; pp < std::min(pn.size(), p0 + (size_t)PB); pp++) {
-            const int q = pn[pp].first, n0 = pn[pp].second;
-            const GJob& g = gj[q];
-            tc::Job jb;
-            jb.a_row = u * tc::NSL * nx + mt * tc::BM;
-            jb.a_sstride = nx;
-            jb.b_row = (int)(usrow[q] + n0);
-            jb.b_sstride = g.r;
-            jb.m_valid = std::min(tc::BM, nx - mt * tc::BM);
-            jb.n_valid = std::min(tc::BN, g.r - n0);
-            jb.out = g.G + (size_t)n0 * nx + mt * tc::BM;
-            jb.ld_out = nx;
-            jb.m0 = mt * tc::BM;
-            jb.n0 = n0;
-            jb.s = 0.0;
-            jobs.push_back(jb);
-          }
-    }
-    Tmp jd;
-    TRY(tmp_alloc(c, jd, jobs.size() * sizeof(tc::Job)));
-    CK(cudaMemcpyAsync(jd.p, jobs.data(), jobs.size() * sizeof(tc::Job), cudaMemcpyHostToDevice, c->st));
-    double fl = 0.0;
-    for (const tc::Job& jb : jobs) fl += 2.0 * (double)jb.m_valid * jb.n_valid * nv;
-    ph_begin(c, OSVMP2_PH_K_GPROJ);
-    if (launch_gproj_tc((const float*)bs.p, (long long)nb * tc::NSL * nx, Us, us_rows, nv, ldv, (const tc::Job*)jd.p,
-                        (int)jobs.size(), lo_shift, c->err_d, c->st))
-      return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the G projection failed");
-    ph_end(c, OSVMP2_PH_K_GPROJ, fl);
-    CK(cudaGetLastError());
-  }
-  return 0;
-}
-
 // ---- FP64 contractions on the tensor cores (tc_oz.cuh) --------------------------------
 // Digit stores are temporaries of a call.  A call that has no room for them (a device-memory
 // cap, a full device) runs the CUDA-core kernels, which need none: the helpers return
@@ -742,11 +665,11 @@ int oz_upload(osvmp2_ctx* c, const OzList& l, OzDev& d) {
   CK(cudaMemcpyAsync(d.s.p, l.segs.data(), l.segs.size() * sizeof(oz::Seg), cudaMemcpyHostToDevice, c->st));
   return 0;
 }
-int oz_run(osvmp2_ctx* c, const OzOperand& A, const OzOperand& B, const OzList& l, int ns = oz::NSL) {
+int oz_run(osvmp2_ctx* c, const OzOperand& A, const OzOperand& B, const OzList& l) {
   if (l.jobs.empty()) return 0;
   OzDev d;
   TRY(oz_upload(c, l, d));
-  if (launch_oz_gemm(A, B, (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, nullptr, ns, c->err_d, c->st))
+  if (launch_oz_gemm(A, B, (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, nullptr, c->err_d, c->st))
     return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for an FP64 contraction failed");
   CK(cudaGetLastError());
   return 0;
@@ -817,6 +740,77 @@ int oz_sf(osvmp2_ctx* c, const std::vector<SFJob>& sfj) {
   }
   TRY(oz_run(c, q.op, q.op, ls));
   return oz_run(c, eq.op, q.op, lf);
+}
+
+// Mixed form: G = U^T B_x of every listed job from the digits of U; the orbitals x in batches whose digits fit a
+// fixed budget.  Remainders of the FP32 pairs lo_shift floats after G.
+struct MxG {
+  int x, r;
+  oz::Mat u;               // digits of U
+  float* G;                // [r][n_aux]
+};
+int mx_project(osvmp2_ctx* c, const std::vector<MxG>& gj, const OzOperand& U, long long lo_shift) {
+  const int nv = c->sys.n_vir, nx = c->sys.n_aux, n = c->sys.n_occ, nch = oz::n_chunks(nv);
+  std::vector<std::vector<int>> by_x(n);
+  for (size_t q = 0; q < gj.size(); q++) by_x[gj[q].x].push_back((int)q);
+  std::vector<int> xs;
+  for (int x = 0; x < n; x++)
+    if (!by_x[x].empty()) xs.push_back(x);
+  if (xs.empty()) return 0;
+  const size_t slot = oz_digit_bytes(nx, nv, oz::MXSL), budget = (size_t)4 << 30;
+  const size_t per = std::max<size_t>(1, std::min<size_t>(xs.size(), budget / slot));
+  if ((long long)per * oz::MXSL * nx + oz::BM >= (long long)INT32_MAX)
+    return fail(c, OSVMP2_E_ARG, "B digit batch exceeds the tensor-map row range");
+  Tmp D, ex, xd;
+  TRY(tmp_alloc(c, D, per * slot));
+  TRY(tmp_alloc(c, ex, oz_exp_bytes(per * nx, nv)));
+  TRY(tmp_alloc(c, xd, xs.size() * sizeof(int)));
+  CK(cudaMemcpyAsync(xd.p, xs.data(), xs.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+  const int n_mt = (nx + oz::BM - 1) / oz::BM;
+  for (size_t b0 = 0; b0 < xs.size(); b0 += per) {
+    const int nb = (int)std::min(per, xs.size() - b0);
+    launch_oz_cols(bsrc(c), (const int*)xd.p + b0, nb, oz::MXSL, (uint16_t*)D.p, (int*)ex.p, c->st);
+    CK(cudaGetLastError());
+    // Tile order: per orbital x, blocks of PB (job, column tile) pairs, each with all its aux tiles; a wave of the
+    // persistent grid then holds every aux tile of B_x and only PB tiles of U, so the B_x tiles stay in L2
+    // across the waves of x and every U tile is read once.
+    const int PB = std::max(1, c->num_sms / std::max(1, n_mt));
+    OzList l;
+    double fl = 0.0;
+    for (int u = 0; u < nb; u++) {
+      std::vector<std::array<int, 3>> pn;   // (G job, segment, first column)
+      for (int q : by_x[xs[b0 + u]]) {
+        l.seg(oz::Mat{u * oz::MXSL * nx, nx, u * nx * nch, nch}, gj[q].u, nv);
+        for (int n0 = 0; n0 < gj[q].r; n0 += oz::BN) pn.push_back({q, (int)l.segs.size() - 1, n0});
+        fl += 2.0 * (double)nx * gj[q].r * nv;
+      }
+      for (size_t p0 = 0; p0 < pn.size(); p0 += PB)
+        for (int mt = 0; mt < n_mt; mt++)
+          for (size_t pp = p0; pp < std::min(pn.size(), p0 + (size_t)PB); pp++) {
+            const MxG& g = gj[pn[pp][0]];
+            oz::Job jb{};
+            jb.seg0 = pn[pp][1];
+            jb.nseg = 1;
+            jb.skip = -1;
+            jb.m0 = mt * oz::BM;
+            jb.n0 = pn[pp][2];
+            jb.m_valid = std::min(oz::BM, nx - jb.m0);
+            jb.n_valid = std::min(oz::BN, g.r - jb.n0);
+            jb.ld_out = nx;
+            jb.out = g.G;
+            l.jobs.push_back(jb);
+          }
+    }
+    OzDev d;
+    if (oz_upload(c, l, d)) return fail(c, OSVMP2_E_NOMEM, "no room for the G projection's tile list");
+    ph_begin(c, OSVMP2_PH_K_GPROJ);
+    if (launch_mx_g(OzOperand{(const uint16_t*)D.p, (long long)per * oz::MXSL * nx, nv, oz::ld_of(nv), (const int*)ex.p}, U,
+                    (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, lo_shift, c->err_d, c->st))
+      return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the G projection failed");
+    ph_end(c, OSVMP2_PH_K_GPROJ, fl);
+    CK(cudaGetLastError());
+  }
+  return 0;
 }
 
 // B~_i^(x) = B_i^T Q_x of every listed job; the orbitals i in batches whose digits fit a fixed budget.
@@ -1022,7 +1016,6 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
 // raw: whether the stored amplitudes are those of the raw basis; otherwise Y (r^2) is left in the slot.
 // df: dE/df of each fragment times its weight (launch_oz_df), NULL if not wanted.
 struct OzWant {
-  int ns = oz::NSL;                 // slices of the products (8: FP64)
   bool raw = true;
   double* df = nullptr;             // device [n][9], by out_id
   const std::vector<Frag>* frags = nullptr;   // by out_id
@@ -1030,7 +1023,7 @@ struct OzWant {
 int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, const std::vector<int>& out_id, size_t f0,
                    size_t f1, const SolveOpts& so, double ulps, FragOut* out, double* tdst, const long long* toff,
                    double* pair_e, const OzWant& want) {
-  const int NS = want.ns;
+  constexpr int NS = oz::NSL;
   const int n = c->sys.n_occ, nv = c->sys.n_vir;
   struct Term { int p, q, ver; double coef; };     // pairs by index in the batch
   std::vector<OzPair> pairs;
@@ -1288,13 +1281,13 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     if (it > 1)
       for (size_t g = 0; g < ng; g++) {
         if (d1[g].n && launch_oz_digits(So, Yo, (const oz::Job*)d1[g].j.p, d1[g].n, (const oz::Seg*)d1[g].s.p,
-                                        (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, NS, c->err_d, c->st))
+                                        (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, c->err_d, c->st))
           return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
         if (d2[g].n && launch_oz_gemm(So, Wo, (const oz::Job*)d2[g].j.p, d2[g].n, (const oz::Seg*)d2[g].s.p,
-                                      (const int*)dn.p, NS, c->err_d, c->st))
+                                      (const int*)dn.p, c->err_d, c->st))
           return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
       }
-    launch_oz_update((const OzPair*)pr.p, np, (const int*)dn.p, it == 1, NS, LD, nch, (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p,
+    launch_oz_update((const OzPair*)pr.p, np, (const int*)dn.p, it == 1, LD, nch, (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p,
                      (double*)pe.p, (double*)pu.p, n_cta, c->st);
     launch_oz_converge((const int*)p0.p, nfb, (const double*)pe.p, (const double*)pu.p, so, ulps, it, (double*)ep.p,
                        (int*)dn.p, (int*)lf.p, out, (const int*)oi.p, c->st);
@@ -1358,7 +1351,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     CK(cudaMemcpyAsync(dfd.p, dfs.data(), dfs.size() * sizeof(OzDf), cudaMemcpyHostToDevice, c->st));
     for (size_t q = 0; q + 1 < cut.size(); q++) {
       if (launch_oz_digits(So, Yo, (const oz::Job*)u1.j.p + cut[q][0], cut[q + 1][0] - cut[q][0], (const oz::Seg*)u1.s.p,
-                           (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, NS, c->err_d, c->st) ||
+                           (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, c->err_d, c->st) ||
           launch_oz_dots(So, Wo, (const oz::Job*)u2.j.p + cut[q][1], cut[q + 1][1] - cut[q][1], (const oz::Seg*)u2.s.p,
                          (double*)parts.p, c->err_d, c->st))
         return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for dE/df failed");
@@ -1438,6 +1431,8 @@ int ensure_pairs(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req, osv
   return rc;
 }
 
+// Build S/F blocks, projections, K and preconditioners for every listed pair
+// (and the diagonal pairs of its orbitals) that is not built yet.
 int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req, osvmp2_prec prec) {
   if (!c->have_osv) return fail(c, OSVMP2_E_STATE, "osvmp2_build_osv has not been called");
   if (prec != OSVMP2_FP64 && prec != OSVMP2_MIXED) return fail(c, OSVMP2_E_ARG, "unknown precision %d", (int)prec);
@@ -1711,123 +1706,148 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
   CK(cudaMemcpyAsync(c->r_h.data(), c->r_d, c->r_h.size() * sizeof(int), cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
   if (mixed) {   // U = P X, G = U^T B, K~ = G_i G_j^T (orthonormal pair basis)
-    size_t ufl = 0, gfl = 0, us_rows = 0;
-    int max_r = 0;
-    const int ldv = (nv + 3) & ~3;     // TMA row stride: a multiple of 16 bytes
-    std::vector<UJob> uj;
-    std::vector<GJob> gj;
-    std::vector<long long> g_usrow;    // row of slice 0 of U_p^T in Us, per G job
-    std::vector<int> g_gsrow;          // row of slice 0 of G_p,x^T in Gs, per G job
-    std::vector<tc::Job> ktj;          // K~ tiles from the slices of G
-    const int ldg = (nx + 3) & ~3;
-    long long gs_rows = 0;
+    // U has entries of order 1 where X reaches lambda_min(S)^(-1/2), so every low-precision product is formed with U.
+    // U itself is an FP64 contraction; G and K~ carry the 39 bits of MXSL slices: an error of U that is the same
+    // for every aux function does not average out in K~, and FP32 products of a rounded G would leave ~1e-8 in
+    // every pair energy.  Against TF32 slices and double-float CTA products for U, at 128 orbitals, 640 virtuals,
+    // 2400 aux: project 66 -> 46 ms, K~ 4.8 -> 4.1, overlaps of the pair bases 9.0 -> 8.4.
+    size_t ufl = 0, gfl = 0;
+    int max_r = 1;
+    long long rows = 0, gs_rows = 0;
     for (auto& p : newp) {
-      const int pid = c->pair_id[(size_t)p.first * n + p.second];
-      const int r = c->r_h[pid];
+      const int r = c->r_h[c->pair_id[(size_t)p.first * n + p.second]];
       max_r = std::max(max_r, r);
       ufl += (size_t)nv * r;
       gfl += (size_t)r * nx * (p.first == p.second ? 1 : 2);
-      us_rows += tc::NSL * (size_t)r;
+      rows += r;
+      gs_rows += (p.first == p.second ? 1 : 2) * (long long)r;
     }
-    float *umem = nullptr, *gmem = nullptr, *usmem = nullptr;
+    const int nchv = oz::n_chunks(nv), nchx = oz::n_chunks(nx), ldv = oz::ld_of(nv), ldx = oz::ld_of(nx);
+    if (std::max(rows, gs_rows) * oz::MXSL + oz::BM >= (long long)INT32_MAX || rows * nchv >= (long long)INT32_MAX ||
+        gs_rows * nchx >= (long long)INT32_MAX)
+      return fail(c, OSVMP2_E_ARG, "pair-basis digit store exceeds the tensor-map row range");
+    float *umem = nullptr, *gmem = nullptr;
+    uint16_t* udig = nullptr;
+    int* uexp = nullptr;
     TRY(palloc(c, reinterpret_cast<double**>(&umem), (ufl + 1) / 2 + 1));
     TRY(palloc(c, reinterpret_cast<double**>(&gmem), (gfl + 1) / 2 + 1));
-    TRY(palloc(c, reinterpret_cast<double**>(&usmem), (us_rows * ldv + 1) / 2 + 1));
-    // rows past a pair's r (read by the fixed-height TMA boxes) must hold finite values
-    CK(cudaMemsetAsync(usmem, 0, us_rows * ldv * sizeof(float), c->st));
+    TRY(palloc(c, reinterpret_cast<double**>(&udig), oz_digit_bytes((size_t)rows, nv, oz::MXSL) / 8 + 1));
+    TRY(palloc(c, reinterpret_cast<double**>(&uexp), oz_exp_bytes((size_t)rows, nv) / 8 + 1));
     c->U_h.resize(c->K_h.size(), nullptr);
     c->Gi_h.resize(c->K_h.size(), nullptr);
     c->Gj_h.resize(c->K_h.size(), nullptr);
-    c->us_base_h.resize(c->K_h.size(), nullptr);
-    c->us_alloc_rows_h.resize(c->K_h.size(), 0);
-    c->us_row_h.resize(c->K_h.size(), 0);
-    c->us_ldv = ldv;
-    size_t uo = 0, go = 0, urow = 0;
+    c->um_of.resize(c->K_h.size(), -1);
+    c->um_mat.resize(c->K_h.size());
+    const OzOperand Uo{udig, rows * oz::MXSL, nv, ldv, uexp};
+    const int sid = (int)c->um_store.size();
+    std::vector<MxG> gj;
+    std::vector<OzMat> gm;             // digits of G
+    OzList lk;
+    size_t uo = 0, go = 0;
+    long long urow = 0, grow = 0;
     double f_u = 0.0, f_g = 0.0, f_kg = 0.0;
     for (auto& p : newp) {
       const int i = p.first, j = p.second, pid = c->pair_id[(size_t)i * n + j];
       const int r = c->r_h[pid], m = pair_dim_h(c, i, j);
-      float* U = umem + uo;
+      c->U_h[pid] = umem + uo;
       uo += (size_t)nv * r;
-      c->U_h[pid] = U;
-      uj.push_back(UJob{i, j, U, usmem + urow * ldv, ldv});
-      c->us_base_h[pid] = usmem;
-      c->us_alloc_rows_h[pid] = (long long)us_rows;
-      c->us_row_h[pid] = (long long)urow;
+      const oz::Mat um{(int)(urow * oz::MXSL), r, (int)(urow * nchv), nchv};
+      urow += r;
+      c->um_of[pid] = sid;
+      c->um_mat[pid] = um;
       f_u += 2.0 * nv * (double)m * r;
-      float* Gi = gmem + go;
-      go += (size_t)r * nx;
-      gj.push_back(GJob{i, r, U, Gi});
-      g_usrow.push_back((long long)urow);
-      const long long gi_row = gs_rows;
-      g_gsrow.push_back((int)gs_rows);
-      gs_rows += tc::NSL * (long long)r;
-      float* Gj = Gi;
-      long long gj_row = gi_row;
-      if (i != j) {
-        Gj = gmem + go;
+      float* G[2];
+      oz::Mat gd[2];
+      const int ng = i == j ? 1 : 2;
+      for (int u = 0; u < ng; u++) {
+        G[u] = gmem + go;
         go += (size_t)r * nx;
-        gj.push_back(GJob{j, r, U, Gj});
-        g_usrow.push_back((long long)urow);
-        gj_row = gs_rows;
-        g_gsrow.push_back((int)gs_rows);
-        gs_rows += tc::NSL * (long long)r;
+        gd[u] = oz::Mat{(int)(grow * oz::MXSL), r, (int)(grow * nchx), nchx};
+        grow += r;
+        gj.push_back(MxG{u ? j : i, r, um, G[u]});
+        gm.push_back(OzMat{(const double*)G[u], r, nx, std::min(ldx, (nx + oz::BK - 1) / oz::BK * oz::BK), nx, gd[u]});
       }
-      urow += tc::NSL * (size_t)r;
-      f_g += (i != j ? 2.0 : 1.0) * 2.0 * r * (double)nv * nx;
-      c->Gi_h[pid] = Gi;
-      c->Gj_h[pid] = Gj;
-      for (int m0 = 0; m0 < r; m0 += tc::BM)
-        for (int n0 = 0; n0 < r; n0 += tc::BN) {
-          tc::Job jb;
-          jb.a_row = (int)(gi_row + m0);
-          jb.a_sstride = r;
-          jb.b_row = (int)(gj_row + n0);
-          jb.b_sstride = r;
-          jb.m_valid = std::min(tc::BM, r - m0);
-          jb.n_valid = std::min(tc::BN, r - n0);
-          jb.out = c->Kt_h[pid] + (size_t)m0 * r + n0;
-          jb.ld_out = r;
-          jb.m0 = m0;
-          jb.n0 = n0;
-          jb.s = 0.0;
-          jb.x_row = jb.x_sstride = 0;
-          ktj.push_back(jb);
-        }
+      c->Gi_h[pid] = G[0];
+      c->Gj_h[pid] = G[ng - 1];
+      lk.product(gd[0], r, gd[ng - 1], r, nx, c->Kt_h[pid], r);
+      f_g += ng * 2.0 * r * (double)nv * nx;
       f_kg += 2.0 * (double)r * r * nx;
     }
     std::vector<float*> uall(c->K_h.size(), nullptr);
     for (size_t q = 0; q < c->U_h.size(); q++) uall[q] = c->U_h[q];
     CK(cudaMemcpyAsync(c->U_d, uall.data(), uall.size() * sizeof(float*), cudaMemcpyHostToDevice, c->st));
-    if (gs_rows + tc::BM >= (long long)INT32_MAX)
-      return fail(c, OSVMP2_E_ARG, "G slice store exceeds the tensor-map row range");
-    Tmp ju, jkt, gsl, glo, jgs;
-    TRY(tmp_alloc(c, ju, uj.size() * sizeof(UJob)));
-    TRY(tmp_alloc(c, glo, (gfl + 1) * sizeof(float)));   // remainders of the G pairs
-    std::vector<GSJob> gsj;
-    for (size_t q = 0; q < gj.size(); q++) gsj.push_back(GSJob{gj[q].G, gj[q].r, g_gsrow[q]});
-    TRY(tmp_alloc(c, jgs, gsj.size() * sizeof(GSJob)));
-    CK(cudaMemcpyAsync(jgs.p, gsj.data(), gsj.size() * sizeof(GSJob), cudaMemcpyHostToDevice, c->st));
-    const long long lo_shift = (long long)((float*)glo.p - gmem);
-    TRY(tmp_alloc(c, jkt, ktj.size() * sizeof(tc::Job)));
-    TRY(tmp_alloc(c, gsl, (size_t)gs_rows * ldg * sizeof(float)));
-    CK(cudaMemcpyAsync(ju.p, uj.data(), uj.size() * sizeof(UJob), cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(jkt.p, ktj.data(), ktj.size() * sizeof(tc::Job), cudaMemcpyHostToDevice, c->st));
-    Tmp uscr;
-    TRY(tmp_alloc(c, uscr, (size_t)n_cta * nv * std::max(max_r, 1) * sizeof(double)));
     ph_begin(c, OSVMP2_PH_PROJECT);
-    launch_ubasis(t, (const UJob*)ju.p, (int)uj.size(), n_cta, (double*)uscr.p, max_r, c->st);
-    CK(cudaGetLastError());
-    TRY(gproj_tensor(c, gj, g_usrow, usmem, (long long)us_rows, ldv, lo_shift));
-    launch_gslices((const GSJob*)jgs.p, (int)gsj.size(), max_r, nx, lo_shift, (float*)gsl.p, ldg, c->st);
+    {   // U = P X: digits of the Q_i with the OSV index innermost, pairs in batches of ~1 GB of U in FP64
+      OzMats q(max_n);
+      std::vector<int> at(n, -1);
+      for (auto& p : newp)
+        for (int x : {p.first, p.second})
+          if (at[x] < 0) at[x] = q.add(c->Qp[x], nv, c->n_osv[x], c->n_osv[x]);
+      auto room = [&](int rc) { return rc == OZ_NO_ROOM ? fail(c, OSVMP2_E_NOMEM, "no room for the pair bases") : rc; };
+      TRY(room(oz_mats_room(c, q)));
+      TRY(oz_mats_fill(c, q, nullptr, true));
+      size_t done = 0;                   // elements of U formed
+      for (size_t b0 = 0; b0 < newp.size();) {
+        size_t b1 = b0, sz = 0;
+        for (; b1 < newp.size() && (b1 == b0 || sz < (size_t)1 << 27); b1++)
+          sz += (size_t)nv * c->r_h[c->pair_id[(size_t)newp[b1].first * n + newp[b1].second]];
+        Tmp u0, mj;
+        TRY(tmp_alloc(c, u0, sz * sizeof(double)));
+        TRY(tmp_alloc(c, mj, (b1 - b0) * sizeof(OzMat)));
+        OzMats xs(max_n);
+        OzList lu;
+        std::vector<OzMat> um;
+        size_t off = 0;
+        for (size_t t2 = b0; t2 < b1; t2++) {
+          const int i = newp[t2].first, j = newp[t2].second, pid = c->pair_id[(size_t)i * n + j];
+          const int r = c->r_h[pid], m = c->m_h[pid], ni = c->n_osv[i], nj = i == j ? 0 : c->n_osv[j];
+          double* U0 = (double*)u0.p + off;
+          off += (size_t)nv * r;
+          oz::Job proto{};
+          proto.skip = -1;
+          const int first = (int)lu.segs.size(), xt = xs.add(c->X_h[pid], r, m, ni);
+          lu.seg(q.mat(at[i]), xs.mat(xt), ni);
+          if (nj) {
+            const int xb = xs.add(c->X_h[pid] + (size_t)ni * m, r, m, nj);
+            lu.seg(q.mat(at[j]), xs.mat(xb), nj);
+          }
+          lu.tiles(first, nv, r, U0, r, proto);
+          um.push_back(OzMat{U0, r, nv, std::min(ldv, (nv + oz::BK - 1) / oz::BK * oz::BK), r, c->um_mat[pid]});
+        }
+        TRY(room(oz_mats_room(c, xs)));
+        TRY(oz_mats_fill(c, xs, nullptr, false));
+        TRY(room(oz_run(c, q.op, xs.op, lu)));
+        launch_oz_float((const double*)u0.p, sz, umem + done, c->st);
+        done += sz;
+        CK(cudaMemcpyAsync(mj.p, um.data(), um.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
+        launch_oz_mats((const OzMat*)mj.p, (int)um.size(), max_r, nv, nullptr, false, oz::MXSL, ldv, udig, uexp, c->st);
+        CK(cudaGetLastError());
+        b0 = b1;
+      }
+    }
+    Tmp glo, gd, ge, gmd;
+    TRY(tmp_alloc(c, glo, (gfl + 1) * sizeof(float)));   // remainders of the G pairs
+    TRY(tmp_alloc(c, gd, oz_digit_bytes((size_t)gs_rows, nx, oz::MXSL)));
+    TRY(tmp_alloc(c, ge, oz_exp_bytes((size_t)gs_rows, nx)));
+    TRY(tmp_alloc(c, gmd, gm.size() * sizeof(OzMat)));
+    CK(cudaMemcpyAsync(gmd.p, gm.data(), gm.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
+    const long long lo_shift = (long long)((float*)glo.p - gmem);
+    TRY(mx_project(c, gj, Uo, lo_shift));
+    launch_mx_pairs((const OzMat*)gmd.p, (int)gm.size(), max_r, nx, lo_shift, ldx, (uint16_t*)gd.p, (int*)ge.p, c->st);
     ph_end(c, OSVMP2_PH_PROJECT, f_u + f_g, c->sys.B ? 8.0 * (double)gj.size() * nx * nv : 0.0);
     CK(cudaGetLastError());
     ph_begin(c, OSVMP2_PH_EXCHANGE);
-    if (launch_kt_tc((const float*)gsl.p, gs_rows, nx, ldg, (const tc::Job*)jkt.p, (int)ktj.size(), c->err_d, c->st))
-      return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for K~ failed");
+    {
+      OzDev d;
+      const OzOperand Go{(const uint16_t*)gd.p, gs_rows * oz::MXSL, nx, ldx, (const int*)ge.p};
+      if (oz_upload(c, lk, d)) return fail(c, OSVMP2_E_NOMEM, "no room for the tile list of K~");
+      if (d.n && launch_mx_gemm(Go, Go, (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, true, c->err_d, c->st))
+        return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for K~ failed");
+    }
     ph_end(c, OSVMP2_PH_EXCHANGE, f_kg);
     CK(cudaGetLastError());
     TRY(check_err_flag(c, "mixed pair build"));
+    c->um_store.push_back(Uo);
   } else {   // polished basis, K~ = X^T K X (used by the preconditioner-basis solver)
     ph_begin(c, OSVMP2_PH_PRECOND);
     oz = oz_pair_basis(c, newp, max_m);
@@ -2033,57 +2053,17 @@ void osvmp2_destroy(osvmp2_ctx* c) {
 
 const char* osvmp2_last_error(const osvmp2_ctx* c) { return c ? c->err.c_str() : "null ctx"; }
 
-// Mixed-form T_i of orbitals [i0, i0+b) on the tensor cores: B_i slices for up
-// to nsl orbitals at a time, then the lower-triangle tiles of each T_i.
-int tii_tensor(osvmp2_ctx* c, int i0, int b, double* T, float* Bt, int nsl, int ldx) {
-  const int nv = c->sys.n_vir, nx = c->sys.n_aux, n = c->sys.n_occ;
-  const int n_mt = (nv + tc::BM - 1) / tc::BM, n_nt = (nv + tc::BN - 1) / tc::BN;
-  for (int u0 = 0; u0 < b; u0 += nsl) {
-    const int nu = std::min(nsl, b - u0);
-    launch_rslices(bsrc(c), i0 + u0, nu, Bt, ldx, c->st);
-    CK(cudaGetLastError());
-    std::vector<tc::Job> jobs;
-    for (int u = 0; u < nu; u++) {
-      const int i = i0 + u0 + u;
-      for (int mt = 0; mt < n_mt; mt++)
-        for (int nt = 0; nt < n_nt && nt * tc::BN < (mt + 1) * tc::BM; nt++) {
-          tc::Job jb;
-          jb.a_row = u * tc::NSL * nv + mt * tc::BM;
-          jb.a_sstride = nv;
-          jb.b_row = u * tc::NSL * nv + nt * tc::BN;
-          jb.b_sstride = nv;
-          jb.m_valid = std::min(tc::BM, nv - mt * tc::BM);
-          jb.n_valid = std::min(tc::BN, nv - nt * tc::BN);
-          jb.out = T + (size_t)(u0 + u) * nv * nv;
-          jb.ld_out = nv;
-          jb.m0 = mt * tc::BM;
-          jb.n0 = nt * tc::BN;
-          jb.s = 2.0 * c->f_h[(size_t)i * n + i];
-          jobs.push_back(jb);
-        }
-    }
-    Tmp jd;
-    TRY(tmp_alloc(c, jd, jobs.size() * sizeof(tc::Job)));
-    CK(cudaMemcpyAsync(jd.p, jobs.data(), jobs.size() * sizeof(tc::Job), cudaMemcpyHostToDevice, c->st));
-    if (launch_tii_tc(Bt, (long long)nu * tc::NSL * nv, nx, ldx, (const tc::Job*)jd.p, (int)jobs.size(),
-                      c->sys.e_vir, c->err_d, c->st))
-      return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for T_ii failed");
-    CK(cudaGetLastError());
-  }
-  return 0;
-}
-
-// FP64 T_i of orbitals [i0, i0+b) on the tensor cores, up to nsl orbitals' digits (D, ex) at a time.
-int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int nsl) {
+// T_i of orbitals [i0, i0+b) on the tensor cores with ns slices, up to nsl orbitals' digits (D, ex) at a time.
+int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int nsl, int ns) {
   const int nv = c->sys.n_vir, nx = c->sys.n_aux, n = c->sys.n_occ, nch = oz::n_chunks(nx);
   for (int u0 = 0; u0 < b; u0 += nsl) {
     const int nu = std::min(nsl, b - u0);
-    launch_oz_rows(bsrc(c), i0 + u0, nu, oz::NSL, D, ex, c->st);
+    launch_oz_rows(bsrc(c), i0 + u0, nu, ns, D, ex, c->st);
     CK(cudaGetLastError());
     OzList all, l;
     for (int u = 0; u < nu; u++) {
       const int i = i0 + u0 + u;
-      const oz::Mat m{u * oz::NSL * nv, nv, u * nv * nch, nch};
+      const oz::Mat m{u * ns * nv, nv, u * nv * nch, nch};
       all.product(m, nv, m, nv, nx, T + (size_t)(u0 + u) * nv * nv, nv);
       for (oz::Job& jb : all.jobs)
         if (jb.n0 < jb.m0 + oz::BM) {          // tiles that touch the lower triangle
@@ -2095,8 +2075,8 @@ int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int ns
     l.segs = all.segs;
     OzDev d;
     if (int rc = oz_upload(c, l, d)) return rc;
-    if (launch_oz_tii(OzOperand{D, (long long)nu * oz::NSL * nv, nx, oz::ld_of(nx), ex}, (const oz::Job*)d.j.p, d.n,
-                      (const oz::Seg*)d.s.p, c->sys.e_vir, oz::NSL, c->err_d, c->st))
+    if (launch_oz_tii(OzOperand{D, (long long)nu * ns * nv, nx, oz::ld_of(nx), ex}, (const oz::Job*)d.j.p, d.n,
+                      (const oz::Seg*)d.s.p, c->sys.e_vir, ns, c->err_d, c->st))
       return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for T_ii failed");
     CK(cudaGetLastError());
   }
@@ -2282,16 +2262,16 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
     nb = (n + nbatch - 1) / nbatch;
   }
   const bool tii_tc = c->opts.osv_prec == OSVMP2_MIXED;
-  const int ldx = (s->n_aux + 3) & ~3;
-  const size_t slot_bytes = (size_t)tc::NSL * nv * ldx * sizeof(float);
-  const int nsl = tii_tc ? (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, ((size_t)1 << 30) / slot_bytes)) : 0;
-  Tmp Tm, Vm, wm, km, sm, Bt;
-  // FP64 form: digits of B for up to 2 GB of orbitals at a time; without room for one orbital's, the
-  // CUDA-core kernel
-  const size_t ozslot = oz_digit_bytes(nv, s->n_aux);
-  const int noz = tii_tc ? 0 : (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, ((size_t)2 << 30) / ozslot));
+  Tmp Tm, Vm, wm, km, sm;
+  // digits of B for up to 2 GB of orbitals at a time; FP64 form without room for one orbital's: the CUDA-core kernel
+  const int tii_ns = tii_tc ? oz::MXSL : oz::NSL;
+  const size_t ozslot = oz_digit_bytes(nv, s->n_aux, tii_ns);
+  const int noz = (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, ((size_t)2 << 30) / ozslot));
   Tmp ozD, ozE;
-  if (tii_tc) TRY(tmp_alloc(c, Bt, (size_t)nsl * slot_bytes));
+  if (tii_tc) {
+    TRY(tmp_alloc(c, ozD, noz * ozslot));
+    TRY(tmp_alloc(c, ozE, oz_exp_bytes((size_t)noz * nv, s->n_aux)));
+  }
   TRY(tmp_alloc(c, Tm, (size_t)nb * nv * nv * sizeof(double)));
   TRY(tmp_alloc(c, Vm, (size_t)nb * nv * kmax * sizeof(double)));
   TRY(tmp_alloc(c, wm, (size_t)nb * kmax * sizeof(double)));
@@ -2306,7 +2286,7 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
   } else {
     TRY(tmp_alloc(c, sm, (size_t)nb * eig_osv_scratch_doubles(nv, kmax) * sizeof(double)));
   }
-  const bool tii_digits = !tii_tc && (double)noz * oz::NSL * nv + oz::BM < (double)INT32_MAX &&
+  const bool tii_digits = !tii_tc && (double)noz * tii_ns * nv + oz::BM < (double)INT32_MAX &&
                           !oz_room(c, ozD, noz * ozslot) && !oz_room(c, ozE, oz_exp_bytes((size_t)noz * nv, s->n_aux));
   std::vector<int> nrows_h(nb);
   const uint64_t rosv_key = mix64((uint64_t)s->seed ^ (7ull * STREAM_MUL));
@@ -2321,8 +2301,8 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
     const int b = std::min(nb, n - i0);
     ph_begin(c, OSVMP2_PH_TII);
     if (tii_tc)
-      TRY(tii_tensor(c, i0, b, (double*)Tm.p, (float*)Bt.p, nsl, ldx));
-    else if (int rc = tii_digits ? tii_oz(c, i0, b, (double*)Tm.p, (uint16_t*)ozD.p, (int*)ozE.p, noz) : OZ_NO_ROOM) {
+      TRY(tii_oz(c, i0, b, (double*)Tm.p, (uint16_t*)ozD.p, (int*)ozE.p, noz, tii_ns));
+    else if (int rc = tii_digits ? tii_oz(c, i0, b, (double*)Tm.p, (uint16_t*)ozD.p, (int*)ozE.p, noz, tii_ns) : OZ_NO_ROOM) {
       if (rc != OZ_NO_ROOM) return rc;
       launch_tii(bsrc(c), s->e_vir, s->f_occ, n, i0, b, (double*)Tm.p, c->st);
     }
@@ -2659,43 +2639,20 @@ int build_sigma_table(osvmp2_ctx* c, SigmaStore& ss) {
     CK(cudaMemcpyAsync(ss.pos.p, pos.data(), pos.size() * sizeof(long long), cudaMemcpyHostToDevice, c->st));
   }
   ss.tab = SigmaTable{(const int*)ss.off.p, (const int*)ss.hi.p, (const long long*)ss.pos.p, (const float*)ss.data.p};
-  // tensor-core tiles, grouped by the U slice stores of the two pairs
-  std::map<std::pair<const float*, const float*>, std::vector<tc::Job>> groups;
+  // tiles, grouped by the digit stores of the two bases
+  std::map<std::pair<int, int>, OzList> groups;
   for (size_t u = 0; u < cps.size(); u++) {
     const int lo = cps[u].first, hq = cps[u].second;
-    const int rl = c->r_h[lo], rh = c->r_h[hq];
-    if (!c->us_base_h[lo] || !c->us_base_h[hq]) return fail(c, OSVMP2_E_STATE, "pair without U slices");
-    auto& js = groups[{c->us_base_h[lo], c->us_base_h[hq]}];
-    for (int m0 = 0; m0 < rl; m0 += tc::BM)
-      for (int n0 = 0; n0 < rh; n0 += tc::BN) {
-        tc::Job jb;
-        jb.a_row = (int)(c->us_row_h[lo] + m0);
-        jb.a_sstride = rl;
-        jb.b_row = (int)(c->us_row_h[hq] + n0);
-        jb.b_sstride = rh;
-        jb.m_valid = std::min(tc::BM, rl - m0);
-        jb.n_valid = std::min(tc::BN, rh - n0);
-        jb.out = (float*)ss.data.p + pos[u] + (size_t)m0 * rh + n0;
-        jb.ld_out = rh;
-        jb.m0 = m0;
-        jb.n0 = n0;
-        jb.s = 0.0;
-        js.push_back(jb);
-      }
+    if (lo >= (int)c->um_of.size() || hq >= (int)c->um_of.size() || c->um_of[lo] < 0 || c->um_of[hq] < 0)
+      return fail(c, OSVMP2_E_STATE, "pair without basis digits");
+    groups[{c->um_of[lo], c->um_of[hq]}].product(c->um_mat[lo], c->r_h[lo], c->um_mat[hq], c->r_h[hq], c->sys.n_vir,
+                                                 reinterpret_cast<double*>((float*)ss.data.p + pos[u]), c->r_h[hq]);
   }
   for (auto& g : groups) {
-    const float* A = g.first.first;
-    const float* B = g.first.second;
-    long long ar = 0, br = 0;
-    for (int q = 0; q < npairs; q++) {
-      if (c->us_base_h[q] == A) ar = c->us_alloc_rows_h[q];
-      if (c->us_base_h[q] == B) br = c->us_alloc_rows_h[q];
-    }
-    Tmp jd;
-    TRY(tmp_alloc(c, jd, g.second.size() * sizeof(tc::Job)));
-    CK(cudaMemcpyAsync(jd.p, g.second.data(), g.second.size() * sizeof(tc::Job), cudaMemcpyHostToDevice, c->st));
-    if (launch_rows_tc(A, ar, B, br, c->sys.n_vir, c->us_ldv, (const tc::Job*)jd.p, (int)g.second.size(), c->err_d,
-                       c->st))
+    OzDev d;
+    if (oz_upload(c, g.second, d)) return fail(c, OSVMP2_E_NOMEM, "no room for the tile list of the pair-couple overlaps");
+    if (d.n && launch_mx_gemm(c->um_store[g.first.first], c->um_store[g.first.second], (const oz::Job*)d.j.p, d.n,
+                              (const oz::Seg*)d.s.p, false, c->err_d, c->st))
       return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the pair-couple overlaps failed");
     CK(cudaGetLastError());
   }

@@ -53,12 +53,6 @@ struct FragOut {
 // T_ii of orbitals [i0, i0+nb) into T [nb][nv][nv].
 void launch_tii(const BSrc& src, const double* e_vir, const double* f_occ, int n_occ, int i0, int nb,
                 double* T, cudaStream_t st);
-// Mixed form (tii_tc.cu): slices of B_i along the aux index for orbitals
-// [i0, i0+nb): slot u, slice s, row a at Bt + ((u * tc::NSL + s) * n_vir + a) * ldx;
-// then the tensor-core tiles of T (jobs built by the host, out = T_i, s = 2 f_ii).
-void launch_rslices(const BSrc& src, int i0, int nb, float* Bt, int ldx, cudaStream_t st);
-int launch_tii_tc(const float* Bt, long long rows, int n_aux, int ldx, const tc::Job* jobs, int n_jobs,
-                  const double* e_vir, int* err, cudaStream_t st);
 // Eigen-decomposition of each T[b] and selection omega >= thr (all if thr <= 0),
 // at most kmax per orbital: V [nb][kmax][nv] (eigenvector-major), w [nb][kmax], k [nb], err |= ERR_*.
 // nclu: eig_cluster_table.
@@ -124,7 +118,7 @@ struct OzMat {           // dense matrix whose digits go to m; row stride ldm (s
   int rows, K, kpad, ldm;  // kpad >= K: digits of k in [K, kpad) are written as zeros
   oz::Mat m;
 };
-// ns: slices (8: FP64; 5 and 4: 39 and 31 bits for the mixed form); operands with more slices serve too.
+// ns: slices (NSL: FP64; MXSL: 39 bits, mixed form).
 // Digits of B: rows B[i0 + u][a][.] (K = aux) or B[xs[u]][.][P] (K = vir); slot u, slice s, row r at
 // row (u ns + s) rows + r of the store, exponent row u rows + r.
 void launch_oz_rows(const BSrc& src, int i0, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st);
@@ -135,12 +129,12 @@ void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const dou
 // out[row][col] per job (row-major); T_ii tiles of the lower triangle (mirrored, with denominators).
 // Return 0, or -1 if a tensor map could not be encoded.
 int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                   const int* skip, int ns, int* err, cudaStream_t st);
+                   const int* skip, int* err, cudaStream_t st);
 int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int ns,
                   int* err, cudaStream_t st);
 // The digits of the output (jobs' o_row, o_ss, o_e) into the store D with row stride ld (a multiple of 32).
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                     const int* skip, uint16_t* D, int ld, const int* exW, int ns, int* err, cudaStream_t st);
+                     const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st);
 // Dot products of (2 Y - Y^T) with the product of every job (see OzEpiDot), 16 partial sums per job.
 int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    double* parts, int* err, cudaStream_t st);
@@ -168,7 +162,7 @@ struct OzPair {          // a pair of a fragment
   double* C;             // [r][r]
   double* T;             // [m][m] raw-basis amplitude (launch_oz_raw) or NULL
 };
-void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ns, int ld, int nch, uint16_t* D,
+void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, int nch, uint16_t* D,
                       int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st);
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
                         double* e_prev, int* done, int* left, FragOut* out, const int* out_id, cudaStream_t st);
@@ -256,36 +250,18 @@ __host__ __device__ inline size_t frag_scratch_doubles(int max_m) { return 26 * 
 void launch_frag_solve(const Tables& t, const int* frag_orbs, const int* order, int n_frag, int max_m,
                        SolveOpts o, double* scratch, int n_cta, int* counter, FragOut* out,
                        double* Tstore, const long long* Toff, cudaStream_t st);
-// Mixed-form pair build (ubasis.cu) in the orthonormal pair basis U = P X.
-struct UJob {
-  int i, j;
-  float* U;            // [n_vir][r]
-  float* Us;           // TF32 slices of U^T (tf32_split.cuh): slice s row mu at Us + (s * r + mu) * ldv
-  int ldv;
-};
-struct GJob {          // G = U^T B_x  [r][n_aux]
-  int x, r;
-  const float* U;
-  float* G;
-};
-void launch_ubasis(const Tables& t, const UJob* jobs, int n_jobs, int n_cta, double* scratch, int max_r,
-                   cudaStream_t st);
-// B_x for the orbitals xs[0..n_x) as TF32 slices (tf32_split.cuh), transposed:
-// slot u, slice s, row P at Bs + ((u * tc::NSL + s) * n_aux + P) * ldv
-void launch_bslices(const BSrc& src, const int* xs, int n_x, float* Bs, int ldv, cudaStream_t st);
-// G tiles with the split-TF32 tensor-core kernel: A = Bs (rows a_rows), B = Us (rows b_rows), K = n_vir;
-// G is written as a normalised FP32 pair: the leading part at job.out, the remainder
-// lo_shift floats further on.  Returns 0, or -1 if a tensor map could not be encoded.
-int launch_gproj_tc(const float* Bs, long long a_rows, const float* Us, long long b_rows, int n_vir, int ldv,
-                    const tc::Job* jobs, int n_jobs, long long lo_shift, int* err, cudaStream_t st);
-// The slices of G^T from the pair (G, lo): slice s of row mu at Gs[(x_row + s r + mu) ldg + P].
-struct GSJob {
-  const float* G;      // [r][n_aux], remainder at G + lo_shift
-  int r, x_row;
-};
-void launch_gslices(const GSJob* jobs, int n_jobs, int max_r, int n_aux, long long lo_shift, float* Gs, int ldg,
-                    cudaStream_t st);
-// K~ = G_i G_j^T tiles from the slices in Gs (rows in total, K = n_aux), FP64 row-major output.
+// Mixed-form pair build in the orthonormal pair basis U = P X: contractions of MXSL slices, summed as FP32 pairs.
+// G = U^T B per job (A rows: aux, B rows: pair basis): out[col][row] of leading parts, remainders lo_shift floats on.
+int launch_mx_g(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                long long lo_shift, int* err, cudaStream_t st);
+// out[row][col] in FP64 or FP32
+int launch_mx_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                   bool fp64_out, int* err, cudaStream_t st);
+// Digits of matrices of FP32 pairs (OzMat.p: the leading parts, [rows][K]).
+void launch_mx_pairs(const OzMat* mats, int n, int max_rows, int K, long long lo_shift, int ld, uint16_t* D, int* ex,
+                     cudaStream_t st);
+void launch_oz_float(const double* x, size_t n, float* y, cudaStream_t st);
+// Products of TF32 slice rows (randomized OSVs): Gs holds `rows` rows of K = n_aux, FP64 row-major output.
 int launch_kt_tc(const float* Gs, long long rows, int n_aux, int ldg, const tc::Job* jobs, int n_jobs, int* err,
                  cudaStream_t st);
 // 2-D FP32 tensor map over rows x n_k (row stride ldk floats, a multiple of 4),
@@ -318,11 +294,6 @@ void launch_frag_solve_mixed(const Tables& t, const int* frag_orbs, const int* o
                              SolveOpts o, const SigmaTable& sgt, double* scratch, int n_cta, int* counter,
                              FragOut* out, double* Tstore, const long long* Toff, int* err, int ctas_per_sm,
                              cudaStream_t st);
-// Row-major tiles of U-slice products (gproj_tc.cu): out[row * ld_out + col] = A_row . B_col,
-// A and B tensor maps over (possibly different) U slice stores with K = n_vir.
-int launch_rows_tc(const float* A, long long a_rows, const float* B, long long b_rows, int n_vir, int ldv,
-                   const tc::Job* jobs, int n_jobs, int* err, cudaStream_t st);
-
 // E = sum_f w_f * E_f in a fixed order -> e_out (device scalar)
 void launch_weighted_sum(const FragOut* out, const int* weights, int n, double* e_out, cudaStream_t st);
 

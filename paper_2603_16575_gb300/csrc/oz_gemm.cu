@@ -110,12 +110,59 @@ __global__ void __launch_bounds__(256) k_oz_rmats(const OzMat* __restrict__ mats
   if (lane == 0) ex[mt.m.eb + (size_t)r * mt.m.es + c] = e;
 }
 
+// Matrices of FP32 pairs with k innermost (mixed form: G and its remainder, lo_shift floats further on): a warp per
+// (row, chunk); the fixed-point numbers without the FP64 pipe, whose conversions would take longer than the reads.
+template <int NS>
+__global__ void __launch_bounds__(256) k_oz_pairs(const OzMat* __restrict__ mats, long long lo_shift, int ld,
+                                                  uint16_t* __restrict__ D, int* __restrict__ ex) {
+  constexpr int T = 7 + 8 * (NS - 1);                  // |x| < 2^e -> |F| < 2^T
+  const OzMat mt = mats[blockIdx.z];
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5), c = blockIdx.y, k0 = c * oz::CHUNK, lane = threadIdx.x & 31;
+  if (r >= mt.rows || k0 >= mt.K) return;
+  const float* g = reinterpret_cast<const float*>(mt.p) + (size_t)r * mt.ldm;
+  float h[8], l[8];
+  unsigned mx = 0;
+#pragma unroll
+  for (int v = 0; v < 8; v++) {
+    const int k = k0 + 64 * (v >> 1) + 2 * lane + (v & 1);
+    h[v] = k < mt.K ? g[k] : 0.f;
+    l[v] = k < mt.K ? g[k + lo_shift] : 0.f;
+    mx = max(mx, (unsigned)__float_as_int(h[v]) & 0x7fffffffu);
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  const int fe = (int)(mx >> 23);                      // below 2^-80: zero
+  const int e = fe == 255 ? oz::EX_NAN : (fe < 47 ? oz::EX_ZERO : fe - 126);
+  const bool live = fe != 255 && fe >= 47;
+  const int sh = live ? T - 16 - e : 0;                // |h 2^sh| < 2^(T - 16) <= 2^23
+  const float s0 = __int_as_float(((sh >> 1) + 127) << 23), s1 = __int_as_float((sh - (sh >> 1) + 127) << 23);
+  uint16_t* dst = D + ((size_t)mt.m.row + r) * ld + k0;
+  const size_t slice = (size_t)mt.m.ss * ld;
+  const int kv = min(oz::CHUNK, mt.kpad - k0);
+#pragma unroll
+  for (int u = 0; u < 4; u++) {
+    const int k = 64 * u + 2 * lane;
+    if (k >= kv) continue;
+    long long f[2];
+#pragma unroll
+    for (int w = 0; w < 2; w++) {
+      const float a = live ? h[2 * u + w] * s0 * s1 : 0.f, b = live ? l[2 * u + w] * s0 * s1 : 0.f;
+      const int top = __float2int_rn(a);
+      f[w] = ((long long)top << 16) + __float2int_rn(fmaf(a - (float)top, 65536.f, b * 65536.f));
+    }
+#pragma unroll
+    for (int s = NS - 1; s >= 0; s--) *reinterpret_cast<uint32_t*>(dst + s * slice + k) = oz::digit_pair(f[0], f[1], s);
+  }
+  if (lane == 0) ex[mt.m.eb + (size_t)r * mt.m.es + c] = e;
+}
+__global__ void k_oz_float(const double* __restrict__ x, size_t n, float* __restrict__ y) {
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) y[i] = (float)x[i];
+}
+
 // One call of f<NS> for the slice counts in use.
-#define OZ_DISPATCH(ns, call)              \
-  do {                                     \
-    if ((ns) == 8) { constexpr int NS = 8; call; } \
-    else if ((ns) == 5) { constexpr int NS = 5; call; } \
-    else { constexpr int NS = 4; call; }   \
+#define OZ_DISPATCH(ns, call)                                  \
+  do {                                                         \
+    if ((ns) == oz::NSL) { constexpr int NS = oz::NSL; call; } \
+    else { constexpr int NS = oz::MXSL; call; }                \
   } while (0)
 
 void launch_oz_rows(const BSrc& src, int i0, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st) {
@@ -143,9 +190,23 @@ void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const dou
   }
 }
 
+void launch_mx_pairs(const OzMat* mats, int n, int max_rows, int K, long long lo_shift, int ld, uint16_t* D, int* ex,
+                     cudaStream_t st) {
+  for (int q = 0; q < n; q += 65535) {     // grid z limit
+    const int nq = n - q < 65535 ? n - q : 65535;
+    k_oz_pairs<oz::MXSL><<<dim3((max_rows + 7) / 8, oz::n_chunks(K), nq), 256, 0, st>>>(mats + q, lo_shift, ld, D, ex);
+    note_launch(1);
+  }
+}
+void launch_oz_float(const double* x, size_t n, float* y, cudaStream_t st) {
+  if (!n) return;
+  k_oz_float<<<1184, 256, 0, st>>>(x, n, y);
+  note_launch(1);
+}
+
 // out[row][col] (row-major), added to what is there when job.s = 1
 struct OzEpiRow {
-  static constexpr bool kWarp = false, kDigits = false;
+  static constexpr bool kWarp = false, kDigits = false, kPair = false;
   __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     double* o = static_cast<double*>(jb.out) + (size_t)(jb.m0 + r) * jb.ld_out + jb.n0 + c0;
 #pragma unroll
@@ -153,9 +214,38 @@ struct OzEpiRow {
       if (c0 + u < jb.n_valid) o[u] = jb.s == 0.0 ? v[u] : o[u] + v[u];
   }
 };
+// Mixed form.  G = U^T B with the row (aux) index innermost, as a normalised FP32 pair: the leading part to
+// out[col][row], the remainder lo_shift floats further on.
+struct OzEpiG {
+  static constexpr bool kWarp = false, kDigits = false, kPair = true;
+  long long lo_shift;
+  __device__ __forceinline__ void pairs(const oz::Job& jb, int r, int c0, const float (&h)[oz::DCOL],
+                                        const float (&l)[oz::DCOL]) const {
+    float* o = static_cast<float*>(jb.out) + (size_t)(jb.n0 + c0) * jb.ld_out + jb.m0 + r;
+#pragma unroll
+    for (int u = 0; u < oz::DCOL; u++)
+      if (c0 + u < jb.n_valid) {
+        const dfl v = df_norm(h[u], l[u]);
+        o[(size_t)u * jb.ld_out] = v.h;
+        o[(size_t)u * jb.ld_out + lo_shift] = v.l;
+      }
+  }
+};
+// out[row][col], FP64 (K~) or FP32 (Sigma)
+template <class T>
+struct OzEpiPair {
+  static constexpr bool kWarp = false, kDigits = false, kPair = true;
+  __device__ __forceinline__ void pairs(const oz::Job& jb, int r, int c0, const float (&h)[oz::DCOL],
+                                        const float (&l)[oz::DCOL]) const {
+    T* o = static_cast<T*>(jb.out) + (size_t)(jb.m0 + r) * jb.ld_out + jb.n0 + c0;
+#pragma unroll
+    for (int u = 0; u < oz::DCOL; u++)
+      if (c0 + u < jb.n_valid) o[u] = (T)h[u] + (T)l[u];
+  }
+};
 // T[a][b] = T[b][a] = v / (e_a + e_b - s) for a >= b; out = T_i, s = 2 f_ii
 struct OzEpiT {
-  static constexpr bool kWarp = false, kDigits = false;
+  static constexpr bool kWarp = false, kDigits = false, kPair = false;
   const double* e_vir;
   __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     const int a = jb.m0 + r;
@@ -173,12 +263,25 @@ struct OzEpiT {
   }
 };
 
+// The same from FP32 pairs (mixed form).
+struct OzEpiTPair {
+  static constexpr bool kWarp = false, kDigits = false, kPair = true;
+  const double* e_vir;
+  __device__ __forceinline__ void pairs(const oz::Job& jb, int r, int c0, const float (&h)[oz::DCOL],
+                                        const float (&l)[oz::DCOL]) const {
+    double v[oz::DCOL];
+#pragma unroll
+    for (int u = 0; u < oz::DCOL; u++) v[u] = (double)h[u] + (double)l[u];
+    OzEpiT{e_vir}(jb, r, c0, v);
+  }
+};
+
 // Digits of the output instead of its values: row m0 + r, k = n0 + c of the matrix at store row o_row (o_ss
 // rows per slice), under the exponent code exW[o_e] (a bound of the whole matrix); columns past n_valid up to the
 // next multiple of 16 are written as zeros (up to 32 by the lanes of the last column group).
 template <int NS>
 struct OzEpiDigits {
-  static constexpr bool kWarp = false, kDigits = true;
+  static constexpr bool kWarp = false, kDigits = true, kPair = false;
   static constexpr int T = 7 + 8 * (NS - 1);
   uint16_t* D;
   int ld;
@@ -210,7 +313,7 @@ struct OzEpiDigits {
 // <2 Y - Y^T, D> of the tile's part of D (never stored): Y = the r x r matrix at job.out (r = ld_out), one
 // partial sum per drain warp at parts + 16 job.o_row.
 struct OzEpiDot {
-  static constexpr bool kWarp = true, kDigits = false;
+  static constexpr bool kWarp = true, kDigits = false, kPair = false;
   double* parts;
   __device__ __forceinline__ void warp(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     const double* Y = static_cast<const double*>(jb.out);
@@ -258,16 +361,21 @@ int run(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs,
 }  // namespace
 
 int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                   const int* skip, int ns, int* err, cudaStream_t st) {
-  int rc = 0;
-  OZ_DISPATCH(ns, (rc = run<NS>(A, B, jobs, n_jobs, segs, skip, err, OzEpiRow{}, st)));
-  return rc;
+                   const int* skip, int* err, cudaStream_t st) {
+  return run<oz::NSL>(A, B, jobs, n_jobs, segs, skip, err, OzEpiRow{}, st);
 }
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                     const int* skip, uint16_t* D, int ld, const int* exW, int ns, int* err, cudaStream_t st) {
-  int rc = 0;
-  OZ_DISPATCH(ns, (rc = run<NS>(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits<NS>{D, ld, exW}, st)));
-  return rc;
+                     const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st) {
+  return run<oz::NSL>(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits<oz::NSL>{D, ld, exW}, st);
+}
+int launch_mx_g(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                long long lo_shift, int* err, cudaStream_t st) {
+  return run<oz::MXSL>(A, B, jobs, n_jobs, segs, nullptr, err, OzEpiG{lo_shift}, st);
+}
+int launch_mx_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                   bool fp64_out, int* err, cudaStream_t st) {
+  return fp64_out ? run<oz::MXSL>(A, B, jobs, n_jobs, segs, nullptr, err, OzEpiPair<double>{}, st)
+                  : run<oz::MXSL>(A, B, jobs, n_jobs, segs, nullptr, err, OzEpiPair<float>{}, st);
 }
 int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    double* parts, int* err, cudaStream_t st) {
@@ -275,9 +383,8 @@ int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, 
 }
 int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int ns,
                   int* err, cudaStream_t st) {
-  int rc = 0;
-  OZ_DISPATCH(ns, (rc = run<NS>(A, A, jobs, n_jobs, segs, nullptr, err, OzEpiT{e_vir}, st)));
-  return rc;
+  return ns == oz::NSL ? run<oz::NSL>(A, A, jobs, n_jobs, segs, nullptr, err, OzEpiT{e_vir}, st)
+                       : run<oz::MXSL>(A, A, jobs, n_jobs, segs, nullptr, err, OzEpiTPair{e_vir}, st);
 }
 
 }  // namespace osv

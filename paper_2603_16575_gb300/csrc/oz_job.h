@@ -9,6 +9,7 @@ constexpr int BM = 128;       // tile rows = TMEM lanes = MMA M
 constexpr int BN = 64;        // max tile columns (MMA N <= 64)
 constexpr int BK = 32;        // k per stage (one 64-byte swizzle row of BF16)
 constexpr int NSL = 8;        // slices per operand
+constexpr int MXSL = 5;       // and in the mixed form's pair build
 constexpr int CHUNK = 256;    // k-extent that shares one power-of-two scale per row
 constexpr int EX_ZERO = -(1 << 20);   // chunk exponent of an all-zero chunk
 constexpr int EX_NAN = 1 << 20;       // and of one that holds a NaN or an Inf

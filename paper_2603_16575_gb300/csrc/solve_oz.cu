@@ -146,7 +146,6 @@ __device__ __forceinline__ int bound_exp(double x) {
 }
 
 // Digits of row m of op(Y) (r x r; v: 0 Y, 1 Y^T, 2 Y + Y^T) under the exponent code e, one warp.
-template <int NS>
 __device__ __forceinline__ void row_digits(const double* Y, int r, int m, int v, int e, int kpad, uint16_t* dst,
                                            size_t slice, int lane) {
   const bool live = e > oz::EX_ZERO / 2 && e < oz::EX_NAN / 2;
@@ -161,15 +160,14 @@ __device__ __forceinline__ void row_digits(const double* Y, int r, int m, int v,
         if (v != 0) x[u] += Y[(size_t)kk * r + m];
       }
     }
-    long long f0 = live ? oz::fixedn<NS>(x[0], (unsigned)(e + 1022)) : 0;
-    long long f1 = live ? oz::fixedn<NS>(x[1], (unsigned)(e + 1022)) : 0;
+    long long f0 = live ? oz::fixed63(x[0], (unsigned)(e + 1022)) : 0;
+    long long f1 = live ? oz::fixed63(x[1], (unsigned)(e + 1022)) : 0;
 #pragma unroll
-    for (int s = NS - 1; s >= 0; s--)
+    for (int s = oz::NSL - 1; s >= 0; s--)
       *reinterpret_cast<uint32_t*>(dst + s * slice + k) = oz::digit_pair(f0, f1, s);
   }
 }
 
-template <int NS>
 __global__ void __launch_bounds__(NT) k_oz_update(const OzPair* __restrict__ pairs, int n_pairs,
                                                   const int* __restrict__ done, int first, int ld, int nch,
                                                   uint16_t* __restrict__ D, int* __restrict__ ex,
@@ -218,7 +216,7 @@ __global__ void __launch_bounds__(NT) k_oz_update(const OzPair* __restrict__ pai
       }
       uint16_t* base = D + (size_t)p.vrow[v] * ld;
       for (int m = warp; m < r; m += NT / 32)
-        row_digits<NS>(p.Y, r, m, v, ey, p.kpad, base + (size_t)m * ld, (size_t)r * ld, lane);
+        row_digits(p.Y, r, m, v, ey, p.kpad, base + (size_t)m * ld, (size_t)r * ld, lane);
     }
     __syncthreads();
   }
@@ -248,12 +246,10 @@ __global__ void k_oz_converge(const int* __restrict__ pair0, int n_frag, const d
   else atomicAdd(left, 1);
 }
 
-void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ns, int ld, int nch, uint16_t* D,
+void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, int nch, uint16_t* D,
                       int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st) {
   if (!n_pairs) return;
-  if (ns == 8) k_oz_update<8><<<n_cta, NT, 0, st>>>(pairs, n_pairs, done, first ? 1 : 0, ld, nch, D, ex, exW, pe, pu);
-  else if (ns == 5) k_oz_update<5><<<n_cta, NT, 0, st>>>(pairs, n_pairs, done, first ? 1 : 0, ld, nch, D, ex, exW, pe, pu);
-  else k_oz_update<4><<<n_cta, NT, 0, st>>>(pairs, n_pairs, done, first ? 1 : 0, ld, nch, D, ex, exW, pe, pu);
+  k_oz_update<<<n_cta, NT, 0, st>>>(pairs, n_pairs, done, first ? 1 : 0, ld, nch, D, ex, exW, pe, pu);
   note_launch(1);
 }
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,

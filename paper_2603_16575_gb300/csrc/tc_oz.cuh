@@ -12,8 +12,7 @@
 //    e_m the smallest exponent with max_k |A[m][k]| < 2^e_m (oz_split.cuh): 63 fractional
 //    bits, ten more than the mantissa, so a value keeps its full mantissa down to 2^-10 of
 //    the row's largest in the chunk and an absolute 2^(e_m - 64) below that.
-//  * Callers that need less take fewer slices (NS = 5: 39 bits, 15 products; NS = 4: 31 bits, 10 products): the leading
-//    ones of the same digits.
+//  * The mixed form takes five slices (39 bits, 15 products).
 //  * A product a_s b_t of level l = s + t is at most 2^14, a chunk sum of one slice pair at
 //    most 2^22, and a sum of up to four pairs (levels 2-5) stays an exact FP32 integer
 //    whatever the accumulator's rounding; levels 6-9 have 5 to 8 pairs, whose sums pass 2^24
@@ -74,7 +73,7 @@ constexpr int ERR_TC_TIMEOUT = 16;           // same bit as ERR_TIMEOUT of the l
 template <int NS>
 struct Cfg {
   static constexpr int STAGE = NS * (A_TILE + B_TILE);
-  static constexpr int NSTAGE = NS == 8 ? 2 : (NS == 5 ? 3 : 4);
+  static constexpr int NSTAGE = NS == 8 ? 2 : 3;
   static constexpr int SMEM = NSTAGE * STAGE + 1024;   // + slack for 1024-byte alignment
   static constexpr int NBUF = NS <= 4 ? 2 : 1;         // sets of NS level accumulators in the 512 TMEM columns
   static constexpr int UNIT = 14 + 8 * (NS < 6 ? NS - 1 : 5);   // the joined integer is in units of 2^(e_m + e_n - UNIT)
@@ -90,10 +89,27 @@ __device__ __forceinline__ double oz_fma(long long v, int x, double coef, double
   return fma(coef, (double)v * pow2(x / 2) * pow2(x - x / 2), acc);
 }
 
+// (ah, al) += (vh, vl) 2^x in FP32 pairs, the error terms gathered in al.
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  const float t = a + b, bb = t - a;
+  e = (a - (t - bb)) + (b - bb);
+  s = t;
+}
+__device__ __forceinline__ void pair_add(float vh, float vl, int x, float& ah, float& al) {
+  if (x < -120) return;                                            // zero rows, and terms below 2^-98
+  float sc = __int_as_float((min(x, 127) + 127) << 23), t;
+  if (x >= EX_NAN / 2) sc = __int_as_float(0x7FC00000);
+  two_sum(ah, vh * sc, ah, t);
+  al += fmaf(vl, sc, t);
+}
+
 // Epi: epi(job, row, col0, acc) stores columns col0 .. col0 + 15 of the tile's row (row < m_valid); or, when
 // Epi::kWarp, epi.warp(job, row, col0, acc) called by every lane of a drain warp, tiles without rows or columns
 // for it included; or, when Epi::kDigits, epi.digits(job, row, col0, F) with F = round(value 2^(T - e)),
-// T = epi.T, e = epi.exponent(job): a tile of one chunk comes there by an integer shift, never as an FP64 number.
+// T = epi.T, e = epi.exponent(job): a tile of one chunk comes there by an integer shift, never as an FP64 number;
+// or, when Epi::kPair (NS <= 5), epi.pairs(job, row, col0, ah, al) with the sum as unnormalised FP32 pairs (the
+// segments' coef is 1): the mixed form's products.  The FP64 drain takes three operations of an FP64 pipe that
+// issues one warp in 64 cycles per element and chunk, more than the 15 products of a chunk; pairs take none.
 template <int NS, class Epi>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_oz(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const int* __restrict__ exA,
@@ -236,13 +252,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const Job jb = jobs[tile];
       if (jb.skip >= 0 && skip[jb.skip]) continue;
       const bool live = col0 < jb.n_valid && 32 * quad < jb.m_valid;   // warp-uniform
-      double acc[Epi::kDigits ? 1 : DCOL];
+      double acc[Epi::kDigits || Epi::kPair ? 1 : DCOL];
+      float ah[Epi::kPair ? DCOL : 1], al[Epi::kPair ? DCOL : 1];
       long long f[Epi::kDigits ? DCOL : 1];
       int eout = 0;
       if constexpr (Epi::kDigits) {
         eout = epi.exponent(jb);
 #pragma unroll
         for (int u = 0; u < DCOL; u++) f[u] = 0;
+      } else if constexpr (Epi::kPair) {
+#pragma unroll
+        for (int u = 0; u < DCOL; u++) ah[u] = al[u] = 0.f;
       } else {
 #pragma unroll
         for (int u = 0; u < DCOL; u++) acc[u] = 0.0;
@@ -257,10 +277,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const int b = (int)(ch % NB) * NS;
           const uint32_t ph = (uint32_t)((ch / NB) & 1);
           const int ea = ea_p[c] - C::UNIT, eb = eb_p[c];
-          long long v[DCOL];
+          long long v[Epi::kPair ? 1 : DCOL];
+          float vh[Epi::kPair ? DCOL : 1], vl[Epi::kPair ? DCOL : 1];
           int lo[NS > 6 ? DCOL : 1];
+          if constexpr (!Epi::kPair) {
 #pragma unroll
-          for (int u = 0; u < DCOL; u++) v[u] = 0;
+            for (int u = 0; u < DCOL; u++) v[u] = 0;
+          }
 #pragma unroll
           for (int l = 0; l < NS; l++) {
             ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::su32(&bar_accf[b + l]), ph));
@@ -277,6 +300,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (!live) continue;
 #pragma unroll
             for (int u = 0; u < DCOL; u++) {
+              if constexpr (Epi::kPair) {                            // levels as an FP32 pair in units of the first
+                const float y = __uint_as_float(x[u]) * __int_as_float((127 - 8 * l) << 23);
+                if (l == 0) { vh[u] = y; vl[u] = 0.f; }
+                else if (l == 1) two_sum(vh[u], y, vh[u], vl[u]);
+                else vl[u] += y;
+                if (l == NS - 1) pair_add(vh[u], vl[u], ea + __shfl_sync(0xffffffffu, eb, u) + C::UNIT - 14, ah[u], al[u]);
+                continue;
+              }
               const int d = __float2int_rn(__uint_as_float(x[u]));
               if (l < 6) v[u] = (v[u] << 8) + d;                   // levels 2 .. 7
               if constexpr (NS > 6) {
@@ -308,6 +339,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (!ok) break;
       if constexpr (Epi::kDigits) {
         if (row < jb.m_valid && live) epi.digits(jb, row, col0, f);
+      } else if constexpr (Epi::kPair) {
+        if (row < jb.m_valid && live) epi.pairs(jb, row, col0, ah, al);
       } else if constexpr (Epi::kWarp) {
         epi.warp(jb, row, col0, acc);
       } else {
