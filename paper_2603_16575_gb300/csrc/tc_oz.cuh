@@ -22,23 +22,17 @@
 //    shifts, 8 and 9 in full where it has room for them and rounded in otherwise), convert it once and add it to the FP64 sum of the element
 //    with one FMA: K / 256 roundings per element where an FP64 dot product makes K.
 //
-// Bound: the shared-memory reads of the MMAs.  An M = 128, N = 64, K = 16 MMA reads 6 KB
-// (48 cycles) for 32 cycles of multiplication; the eight 64-column level accumulators fill
-// the 512 TMEM columns, so N = 64 is the widest tile.  36 products make 128 x 64 x 256
-// cost ~28k cycles an SM; the drain (about 15k, FP64 and integer pipes) runs under the next
-// chunk's MMAs: every level has its own full / empty barrier, so level l of the next chunk
-// starts as soon as level l of this one has been read.
-//
-// The issuing thread's address arithmetic counts too: the 36 products of a K step are unrolled with
-// the slice offsets as constants added to one descriptor each (1.3x on the projections), K steps past
-// the end of a short chunk and quadrants without rows are skipped, and the digit epilogue requantises by
-// integer shifts.  Tensor pipe 50-71% active in the projections, 19-34% in contractions of a length of
-// ~56, which wait on their drain.
+// Bound: the multiplications (36 products: ~18k cycles an SM for 128 x 64 x 256) where K is a chunk or more, and
+// the drain (FP64 and integer pipes; an FP64 operation holds the pipe of its sub-partition for 64 cycles a warp)
+// below.  The eight 64-column level accumulators fill the 512 TMEM columns, so a tile is 64 columns wide (32 when
+// it has no more); the drain of a chunk runs under the next chunk's MMAs: every level has its own full / empty
+// barrier, so level l of the next chunk starts as soon as level l of this one has been read.
 //
 // Measured against the 64 x 64-tile FP64 CTA products (64 orbitals, 320 virtuals, 1200 aux): T_ii 8.5 ->
-// 0.8 ms, projections 53.4 -> 3.2 ms, exchange blocks 16.9 -> 2.6 ms, S and F 2.9 -> 0.44 ms, digits
-// included; at 6 orbitals and 40 virtuals each is still faster or equal (T_ii 0.13 -> 0.05 ms), so there is
-// no size rule.  The CUDA-core kernels remain for calls without room for the digits.
+// 0.72 ms, projections 53.4 -> 3.0 ms, exchange blocks 16.9 -> 2.1 ms, S and F 2.9 -> 0.36 ms, digits
+// included (one MMA a product: 0.80, 3.2, 2.6, 0.44); at 6 orbitals and 40 virtuals each is still faster or equal
+// (T_ii 0.13 -> 0.05 ms), so there is no size rule.  The CUDA-core kernels remain for calls without room
+// for the digits.
 //
 // Persistent CTAs (one per SM) over output tiles of 128 rows (TMEM lanes) x up to 64 columns:
 //   warp 0     TMA producer: the 8 + 8 slice tiles of a 32-wide k-block per stage (64-byte
@@ -75,7 +69,7 @@ struct Cfg {
   static constexpr int STAGE = NS * (A_TILE + B_TILE);
   static constexpr int NSTAGE = NS == 8 ? 2 : 3;
   static constexpr int SMEM = NSTAGE * STAGE + 1024;   // + slack for 1024-byte alignment
-  static constexpr int NBUF = NS <= 4 ? 2 : 1;         // sets of NS level accumulators in the 512 TMEM columns
+  static constexpr int NBUF = 1;                       // sets of NS level accumulators in the 512 TMEM columns
   static constexpr int UNIT = 14 + 8 * (NS < 6 ? NS - 1 : 5);   // the joined integer is in units of 2^(e_m + e_n - UNIT)
 };
 
@@ -87,6 +81,36 @@ __device__ __forceinline__ double oz_fma(long long v, int x, double coef, double
   if (x >= EX_NAN / 2) return __longlong_as_double(0x7FF8000000000000ll);
   if (x < -2040 || x > 2040) return x < 0 ? acc : acc + (double)v * __longlong_as_double(0x7FF0000000000000ll);
   return fma(coef, (double)v * pow2(x / 2) * pow2(x - x / 2), acc);
+}
+
+// Columns of a tile's level accumulators, and rows of its B slices in shared memory: BN, or half of it.
+__device__ __forceinline__ int width(const Job& jb) { return jb.n_valid <= BROWS ? BROWS : BN; }
+
+// The products of one 16-wide k step (ks).  Slice sa of A times the slices 0 .. NS - 1 - sa of B adds to the levels
+// sa .. NS - 1; those slices of B follow one another in shared memory as the levels do in TMEM, so one MMA takes as
+// many of them as N = 256 holds: 12 MMAs for the 36 products of NS = 8, and A is read once for each.  (One MMA a
+// product, N = 64, spent its time on the reads of A: 90 cycles for 32 of multiplication.)  free(l): level l of the
+// last chunk has been read; done: barriers of the levels, committed as they become complete, or NULL.
+template <int NS, int W, class Free>
+__device__ __forceinline__ bool issue(uint64_t da, uint64_t db, uint32_t dcol, int ks, bool zero, const Free& free,
+                                      uint64_t* done) {
+  constexpr int P = 256 / W;                                       // slices of B an MMA takes
+  constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
+#pragma unroll
+  for (int sa = 0; sa < NS; sa++) {
+#pragma unroll
+    for (int j = 0; j < NS - sa; j += P) {
+      const int c = NS - sa - j < P ? NS - sa - j : P;
+      if (sa == 0 && zero)
+        for (int l = j; l < j + c; l++)
+          if (!free(l)) return false;
+      tc::mma_f16(dcol + (uint32_t)((sa + j) * W), da + (uint64_t)((sa * A_TILE + 32 * ks) >> 4),
+                  db + (uint64_t)((j * W * BK * 2 + 32 * ks) >> 4), idesc | ((uint32_t)(c * W >> 3) << 17),
+                  sa == 0 && zero ? 0u : 1u);
+    }
+    if (done) tc::commit(done + sa);
+  }
+  return true;
 }
 
 // (ah, al) += (vh, vl) 2^x in FP32 pairs, the error terms gathered in al.
@@ -157,6 +181,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const Job jb = jobs[tile];
         if (jb.skip >= 0 && skip[jb.skip]) continue;
         const int nbox = (jb.n_valid + BROWS - 1) / BROWS, mbox = (jb.m_valid + AROWS - 1) / AROWS;
+        const int btile = width(jb) * BK * 2;
         const uint32_t bytes = NS * (mbox * AROWS + nbox * BROWS) * BK * 2;
         for (int q = 0; ok && q < jb.nseg; q++) {
           const Seg sg = segs[jb.seg0 + q];
@@ -172,7 +197,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               for (int bx = 0; bx < mbox; bx++)
                 tc::tma_load_2d(st + sl * A_TILE + bx * AROWS * BK * 2, &tmA, fb, c * BK, ra + sl * sg.a.ss + bx * AROWS);
               for (int bx = 0; bx < nbox; bx++)
-                tc::tma_load_2d(st + NS * A_TILE + sl * B_TILE + bx * BROWS * BK * 2, &tmB, fb, c * BK,
+                tc::tma_load_2d(st + NS * A_TILE + sl * btile + bx * BROWS * BK * 2, &tmB, fb, c * BK,
                                 rb + sl * sg.b.ss + bx * BROWS);
             }
           }
@@ -188,12 +213,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   } else if (warp == 1) {
     if (lane == 0) {                                             // ---- MMA issuer
       long long g = 0, ch = 0;
+      bool was_wide = true;
       for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
         const Job jb = jobs[tile];
         if (jb.skip >= 0 && skip[jb.skip]) continue;
-        const int npad = (jb.n_valid + 15) & ~15;
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(npad >> 3) << 17) |
-                               ((uint32_t)(BM >> 4) << 24);
+        const bool wide = width(jb) == BN;
         for (int q = 0; ok && q < jb.nseg; q++) {
           const int K = segs[jb.seg0 + q].K, nkb = (K + BK - 1) / BK;
           for (int c = 0; c < nkb; c++, g++) {
@@ -203,29 +227,27 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             ok = tc::mbar_wait(tc::su32(&bar_full[s]), (uint32_t)((g / NST) & 1));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
-            // one thread issues an MMA every ~50 cycles: descriptors by constant offsets from two bases
             const uint32_t st = sbase + s * C::STAGE;
             const uint64_t da = tc::desc_sw64(st), db = tc::desc_sw64(st + NS * A_TILE);
-            const uint32_t acc0 = first ? 0u : 1u;
-#pragma unroll
-            for (int l = 0; l < NS; l++) {
-              if (first && ch >= NB) {
-                ok = tc::mbar_wait(tc::su32(&bar_acce[b + l]), (uint32_t)((ch / NB - 1) & 1));
-                if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;");
-              }
-              const uint32_t dacc = tmem + (uint32_t)((b + l) * BN);
-#pragma unroll
-              for (int sa = 0; sa <= l; sa++)                    // slices sa + sb = l (counted from 0)
-                tc::mma_f16(dacc, da + (uint64_t)(sa * A_TILE >> 4), db + (uint64_t)((l - sa) * B_TILE >> 4), idesc,
-                            sa == 0 ? acc0 : 1u);
-              if (nks == 2) {
-#pragma unroll
-                for (int sa = 0; sa <= l; sa++)
-                  tc::mma_f16(dacc, da + (uint64_t)((sa * A_TILE + 32) >> 4),
-                              db + (uint64_t)(((l - sa) * B_TILE + 32) >> 4), idesc, 1u);
-              }
-              if (last) tc::commit(&bar_accf[b + l]);
+            const uint32_t dcol = tmem + (uint32_t)(b * BN);
+            auto level_free = [&](int l) {
+              if (ch < NB) return true;
+              const bool f = tc::mbar_wait(tc::su32(&bar_acce[b + l]), (uint32_t)((ch / NB - 1) & 1));
+              asm volatile("tcgen05.fence::after_thread_sync;");
+              return f;
+            };
+            if (first && wide != was_wide) {                     // the levels lie elsewhere: all of the last chunk first
+              for (int l = 0; ok && l < NS; l++) ok = level_free(l);
+              if (!ok) break;
+              was_wide = wide;
+            }
+            for (int ks = 0; ks < nks; ks++) {
+              const bool fin = last && ks == nks - 1;
+              if (wide)
+                ok = issue<NS, BN>(da, db, dcol, ks, first && ks == 0, level_free, fin ? &bar_accf[b] : nullptr);
+              else
+                ok = issue<NS, BROWS>(da, db, dcol, ks, first && ks == 0, level_free, fin ? &bar_accf[b] : nullptr);
+              if (!ok) break;
             }
             if (!ok) break;
             tc::commit(&bar_empty[s]);
@@ -252,6 +274,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const Job jb = jobs[tile];
       if (jb.skip >= 0 && skip[jb.skip]) continue;
       const bool live = col0 < jb.n_valid && 32 * quad < jb.m_valid;   // warp-uniform
+      const int w = width(jb);
       double acc[Epi::kDigits || Epi::kPair ? 1 : DCOL];
       float ah[Epi::kPair ? DCOL : 1], al[Epi::kPair ? DCOL : 1];
       long long f[Epi::kDigits ? DCOL : 1];
@@ -291,7 +314,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             asm volatile("tcgen05.fence::after_thread_sync;");
             uint32_t x[DCOL];
             if (live) {
-              OSV_TMEM_LD16(lcol + (b + l) * BN, x);
+              OSV_TMEM_LD16(lcol + b * BN + l * w, x);
               asm volatile("tcgen05.wait::ld.sync.aligned;");
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
