@@ -681,14 +681,14 @@ struct OzMats {
   OzOperand op{};
   std::vector<OzMat> mats;
   int max_rows = 0, K, ns;
-  long long rows = 0;      // rows of the matrices (the store has ns times as many)
+  long long rows = 0;      // rows of the matrices
   explicit OzMats(int K_, int ns_ = oz::NSL) : K(K_), ns(ns_) {}
   // matrix of r rows and k <= K elements a row at p (row stride ldm); the digits past k are zero up to
   // the next multiple of 32, as far as a tile of K = k reads
   int add(const double* p, int r, int ldm, int k) {
     const int nch = oz::n_chunks(K);
     OzMat m{p, r, k, std::min(oz::ld_of(K), (k + oz::BK - 1) / oz::BK * oz::BK), ldm,
-            oz::Mat{(int)(rows * ns), r, (int)(rows * nch), nch}};
+            oz::Mat{(int)rows, (int)(rows * nch), nch}};
     mats.push_back(m);
     rows += r;
     max_rows = std::max(max_rows, r);
@@ -698,18 +698,17 @@ struct OzMats {
 };
 // Room for the digits of s (OZ_NO_ROOM without), then the digits, scaled by w[k] unless NULL.
 int oz_mats_room(osvmp2_ctx* c, OzMats& s) {
-  if (s.rows * s.ns + oz::BM >= (long long)INT32_MAX || s.rows * oz::n_chunks(s.K) >= (long long)INT32_MAX)
-    return OZ_NO_ROOM;
+  if (s.rows * oz::n_chunks(s.K) + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
   TRY(oz_room(c, s.D, oz_digit_bytes((size_t)s.rows, s.K, s.ns)));
   TRY(oz_room(c, s.ex, oz_exp_bytes((size_t)s.rows, s.K)));
   TRY(oz_room(c, s.md, s.mats.size() * sizeof(OzMat)));
-  s.op = OzOperand{(const uint16_t*)s.D.p, s.rows * s.ns, s.K, oz::ld_of(s.K), (const int*)s.ex.p};
+  s.op = OzOperand{(const uint16_t*)s.D.p, s.rows, s.K, oz::ld_of(s.K), (const int*)s.ex.p};
   return 0;
 }
 int oz_mats_fill(osvmp2_ctx* c, OzMats& s, const double* w, bool k_inner) {
   if (s.mats.empty()) return 0;
   CK(cudaMemcpyAsync(s.md.p, s.mats.data(), s.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
-  launch_oz_mats((const OzMat*)s.md.p, (int)s.mats.size(), s.max_rows, s.K, w, k_inner, s.ns, oz::ld_of(s.K), (uint16_t*)s.D.p,
+  launch_oz_mats((const OzMat*)s.md.p, (int)s.mats.size(), s.max_rows, s.K, w, k_inner, s.ns, oz::ld_of(s.K), s.rows, (uint16_t*)s.D.p,
                  (int*)s.ex.p, c->st);
   CK(cudaGetLastError());
   return 0;
@@ -759,7 +758,7 @@ int mx_project(osvmp2_ctx* c, const std::vector<MxG>& gj, const OzOperand& U, lo
   if (xs.empty()) return 0;
   const size_t slot = oz_digit_bytes(nx, nv, oz::MXSL), budget = (size_t)4 << 30;
   const size_t per = std::max<size_t>(1, std::min<size_t>(xs.size(), budget / slot));
-  if ((long long)per * oz::MXSL * nx + oz::BM >= (long long)INT32_MAX)
+  if ((long long)per * nx * nch + oz::BM >= (long long)INT32_MAX)
     return fail(c, OSVMP2_E_ARG, "B digit batch exceeds the tensor-map row range");
   Tmp D, ex, xd;
   TRY(tmp_alloc(c, D, per * slot));
@@ -780,7 +779,7 @@ int mx_project(osvmp2_ctx* c, const std::vector<MxG>& gj, const OzOperand& U, lo
     for (int u = 0; u < nb; u++) {
       std::vector<std::array<int, 3>> pn;   // (G job, segment, first column)
       for (int q : by_x[xs[b0 + u]]) {
-        l.seg(oz::Mat{u * oz::MXSL * nx, nx, u * nx * nch, nch}, gj[q].u, nv);
+        l.seg(oz::Mat{u * nx, u * nx * nch, nch}, gj[q].u, nv);
         for (int n0 = 0; n0 < gj[q].r; n0 += oz::BN) pn.push_back({q, (int)l.segs.size() - 1, n0});
         fl += 2.0 * (double)nx * gj[q].r * nv;
       }
@@ -804,7 +803,7 @@ int mx_project(osvmp2_ctx* c, const std::vector<MxG>& gj, const OzOperand& U, lo
     OzDev d;
     if (oz_upload(c, l, d)) return fail(c, OSVMP2_E_NOMEM, "no room for the G projection's tile list");
     ph_begin(c, OSVMP2_PH_K_GPROJ);
-    if (launch_mx_g(OzOperand{(const uint16_t*)D.p, (long long)per * oz::MXSL * nx, nv, oz::ld_of(nv), (const int*)ex.p}, U,
+    if (launch_mx_g(OzOperand{(const uint16_t*)D.p, (long long)nb * nx, nv, oz::ld_of(nv), (const int*)ex.p}, U,
                     (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, lo_shift, c->err_d, c->st))
       return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the G projection failed");
     ph_end(c, OSVMP2_PH_K_GPROJ, fl);
@@ -829,7 +828,7 @@ int oz_project(osvmp2_ctx* c, const std::vector<ProjJob>& pj) {
   if (is.empty()) return 0;
   const size_t slot = oz_digit_bytes(nx, nv), budget = (size_t)4 << 30;
   const size_t per = std::max<size_t>(1, std::min<size_t>(is.size(), budget / slot));
-  if ((double)per * oz::NSL * nx + oz::BM >= (double)INT32_MAX) return OZ_NO_ROOM;
+  if ((double)per * nx * nch + oz::BM >= (double)INT32_MAX) return OZ_NO_ROOM;
   Tmp D, ex, xd;
   TRY(oz_mats_room(c, q));
   TRY(oz_room(c, D, per * slot));
@@ -837,7 +836,6 @@ int oz_project(osvmp2_ctx* c, const std::vector<ProjJob>& pj) {
   TRY(oz_room(c, xd, is.size() * sizeof(int)));
   CK(cudaMemcpyAsync(xd.p, is.data(), is.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
   TRY(oz_mats_fill(c, q, nullptr, false));
-  const OzOperand A{(const uint16_t*)D.p, (long long)(per * oz::NSL * nx), nv, oz::ld_of(nv), (const int*)ex.p};
   for (size_t b0 = 0; b0 < is.size(); b0 += per) {
     const int nb = (int)std::min(per, is.size() - b0);
     launch_oz_cols(bsrc(c), (const int*)xd.p + b0, nb, oz::NSL, (uint16_t*)D.p, (int*)ex.p, c->st);
@@ -846,9 +844,9 @@ int oz_project(osvmp2_ctx* c, const std::vector<ProjJob>& pj) {
     for (int u = 0; u < nb; u++)
       for (int t : by_i[is[b0 + u]]) {
         const int k = c->n_osv[pj[t].x];
-        l.product(oz::Mat{u * oz::NSL * nx, nx, u * nx * nch, nch}, nx, q.mat(at[pj[t].x]), k, nv, pj[t].out, k);
+        l.product(oz::Mat{u * nx, u * nx * nch, nch}, nx, q.mat(at[pj[t].x]), k, nv, pj[t].out, k);
       }
-    TRY(oz_run(c, A, q.op, l));
+    TRY(oz_run(c, OzOperand{(const uint16_t*)D.p, (long long)nb * nx, nv, oz::ld_of(nv), (const int*)ex.p}, q.op, l));
   }
   return 0;
 }
@@ -907,7 +905,7 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
     if (c->r_h[id] < 1) return OZ_NO_ROOM;
   }
   const int nch = oz::n_chunks(nv), ld = oz::ld_of(nv);
-  if (rows * oz::NSL + oz::BM >= (long long)INT32_MAX || rows * nch >= (long long)INT32_MAX) return OZ_NO_ROOM;
+  if (rows * nch + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
   // digits of the Q_i with the OSV index innermost (rows of P)
   OzMats q(max_n);
   std::vector<int> at(n, -1);
@@ -919,7 +917,7 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
   TRY(oz_room(c, dmem, oz_digit_bytes((size_t)rows, nv)));
   TRY(oz_room(c, emem, oz_exp_bytes((size_t)rows, nv)));
   TRY(oz_mats_fill(c, q, nullptr, true));
-  const OzOperand store{(const uint16_t*)dmem.p, rows * oz::NSL, nv, ld, (const int*)emem.p};
+  const OzOperand store{(const uint16_t*)dmem.p, rows, nv, ld, (const int*)emem.p};
   const int sid = (int)c->ud_store.size();
   const double budget = 3e9;
   long long row = 0;
@@ -970,7 +968,7 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
       lf.product(ue.mat(a), r, uc.mat(a), r, nv, F1, r);
       pol.push_back(OzPolish{m, r, S1, F1, IE, X, c->et_h[id]});
       lo.product(ur.mat(ur.add(U0, nv, r, r)), nv, ie.mat(ie.add(IE, r, r, r)), r, r, U0, r);
-      const oz::Mat um{(int)(row * oz::NSL), r, (int)(row * nch), nch};
+      const oz::Mat um{(int)row, (int)(row * nch), nch};
       fin.push_back(OzMat{U0, r, nv, nv, r, um});
       c->ud_mat[id] = um;
       row += r;
@@ -995,7 +993,7 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
       TRY(oz_run(c, ur.op, ie.op, lo));
     }
     CK(cudaMemcpyAsync(mj.p, fin.data(), fin.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
-    launch_oz_mats((const OzMat*)mj.p, (int)fin.size(), mr, nv, nullptr, false, oz::NSL, ld, (uint16_t*)dmem.p, (int*)emem.p,
+    launch_oz_mats((const OzMat*)mj.p, (int)fin.size(), mr, nv, nullptr, false, oz::NSL, ld, rows, (uint16_t*)dmem.p, (int*)emem.p,
                    c->st);
     CK(cudaGetLastError());
     b0 = b1;
@@ -1128,7 +1126,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     OzPair& q = pairs[t.q];
     if (q.ver[t.ver] < 0) {
       q.ver[t.ver] = nver++;
-      q.vrow[t.ver] = (int)(yrows * NS);
+      q.vrow[t.ver] = (int)yrows;
       yrows += q.r;
     }
   }
@@ -1154,7 +1152,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   }
   long long srows = 0;
   for (const Couple& k : cps) srows += c->r_h[k.lo] + c->r_h[k.hi];
-  if (yrows * NS + oz::BM >= (long long)INT32_MAX || srows * NS + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
+  if (yrows + oz::BM >= (long long)INT32_MAX || srows * nch + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
   // W: pairs in groups whose digits fit a fixed budget
   const double wbudget = 8e9;
   std::vector<int> grp{0};
@@ -1181,7 +1179,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     wrows = std::max(wrows, wcur);
   }
   dgrp.push_back(nt);
-  if (wrows * NS + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
+  if (wrows + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
   Tmp yc, yd, yx, wx, wd, sd, sx, sgm, pr, p0, pe, pu, ep, dn, lf, oi, smj;
   TRY(oz_room(c, yc, 2 * ysz * sizeof(double)));
   TRY(oz_room(c, yd, (size_t)yrows * NS * LD * 2));
@@ -1223,24 +1221,24 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
       const int lo = cps[u].lo, hi = cps[u].hi, rl = c->r_h[lo], rh = c->r_h[hi];
       double* S = (double*)sgm.p + sgo[u];
       groups[{c->ud_of[lo], c->ud_of[hi]}].product(c->ud_mat[lo], rl, c->ud_mat[hi], rh, nv, S, rh);
-      slo[u] = oz::Mat{(int)(row * NS), rl, (int)(row * nch), nch};
+      slo[u] = oz::Mat{(int)row, (int)(row * nch), nch};
       m1.push_back(OzMat{S, rl, rh, (rh + oz::BK - 1) / oz::BK * oz::BK, rh, slo[u]});
       row += rl;
-      shi[u] = oz::Mat{(int)(row * NS), rh, (int)(row * nch), nch};
+      shi[u] = oz::Mat{(int)row, (int)(row * nch), nch};
       m2.push_back(OzMat{S, rh, rl, (rl + oz::BK - 1) / oz::BK * oz::BK, rh, shi[u]});
       row += rh;
     }
     for (auto& g : groups) TRY(oz_run(c, c->ud_store[g.first.first], c->ud_store[g.first.second], g.second));
     CK(cudaMemcpyAsync(smj.p, m1.data(), m1.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync((OzMat*)smj.p + m1.size(), m2.data(), m2.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
-    launch_oz_mats((const OzMat*)smj.p, (int)m1.size(), max_r, max_r, nullptr, true, NS, LD, (uint16_t*)sd.p, (int*)sx.p, c->st);
-    launch_oz_mats((const OzMat*)smj.p + m1.size(), (int)m2.size(), max_r, max_r, nullptr, false, NS, LD, (uint16_t*)sd.p,
+    launch_oz_mats((const OzMat*)smj.p, (int)m1.size(), max_r, max_r, nullptr, true, NS, LD, srows, (uint16_t*)sd.p, (int*)sx.p, c->st);
+    launch_oz_mats((const OzMat*)smj.p + m1.size(), (int)m2.size(), max_r, max_r, nullptr, false, NS, LD, srows, (uint16_t*)sd.p,
                    (int*)sx.p, c->st);
     CK(cudaGetLastError());
   }
-  const OzOperand So{(const uint16_t*)sd.p, srows * NS, LD, LD, (const int*)sx.p};
-  const OzOperand Yo{(const uint16_t*)yd.p, std::max<long long>(1, yrows) * NS, LD, LD, (const int*)yx.p};
-  const OzOperand Wo{(const uint16_t*)wd.p, std::max<long long>(1, wrows) * NS, LD, LD, (const int*)wx.p};
+  const OzOperand So{(const uint16_t*)sd.p, std::max<long long>(1, srows), LD, LD, (const int*)sx.p};
+  const OzOperand Yo{(const uint16_t*)yd.p, std::max<long long>(1, yrows), LD, LD, (const int*)yx.p};
+  const OzOperand Wo{(const uint16_t*)wd.p, std::max<long long>(1, wrows), LD, LD, (const int*)wx.p};
   // the two products of every group of pairs
   const size_t ng = grp.size() - 1;
   std::vector<OzDev> d1(ng), d2(ng);
@@ -1257,13 +1255,12 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
         const int ve = Q.ver[tm.ver] * nch;
         oz::Job proto{};
         proto.skip = P.frag;
-        proto.o_row = (int)(wrow * NS);
-        proto.o_ss = P.r;
+        proto.o_row = (int)wrow;
         proto.o_e = ve;
         const int f1s = (int)l1.segs.size();
-        l1.seg(S, oz::Mat{Q.vrow[tm.ver], Q.r, ve, 0}, Q.r);
+        l1.seg(S, oz::Mat{Q.vrow[tm.ver], ve, 0}, Q.r);
         l1.tiles(f1s, P.r, Q.r, nullptr, 0, proto);
-        l2.seg(S, oz::Mat{(int)(wrow * NS), P.r, ve, 0}, Q.r, tm.coef);
+        l2.seg(S, oz::Mat{(int)wrow, ve, 0}, Q.r, tm.coef);
         wrow += P.r;
       }
       if ((int)l2.segs.size() > first) {
@@ -1281,13 +1278,13 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     if (it > 1)
       for (size_t g = 0; g < ng; g++) {
         if (d1[g].n && launch_oz_digits(So, Yo, (const oz::Job*)d1[g].j.p, d1[g].n, (const oz::Seg*)d1[g].s.p,
-                                        (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, c->err_d, c->st))
+                                        (const int*)dn.p, (uint16_t*)wd.p, LD, std::max<long long>(1, wrows), (const int*)wx.p, c->err_d, c->st))
           return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
         if (d2[g].n && launch_oz_gemm(So, Wo, (const oz::Job*)d2[g].j.p, d2[g].n, (const oz::Seg*)d2[g].s.p,
                                       (const int*)dn.p, c->err_d, c->st))
           return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
       }
-    launch_oz_update((const OzPair*)pr.p, np, (const int*)dn.p, it == 1, LD, nch, (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p,
+    launch_oz_update((const OzPair*)pr.p, np, (const int*)dn.p, it == 1, LD, std::max<long long>(1, yrows), nch, (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p,
                      (double*)pe.p, (double*)pu.p, n_cta, c->st);
     launch_oz_converge((const int*)p0.p, nfb, (const double*)pe.p, (const double*)pu.p, so, ulps, it, (double*)ep.p,
                        (int*)dn.p, (int*)lf.p, out, (const int*)oi.p, c->st);
@@ -1327,13 +1324,12 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
       const oz::Mat S = pid[tm.p] == cps[tc[t]].lo ? slo[tc[t]] : shi[tc[t]];
       oz::Job proto{};
       proto.skip = -1;
-      proto.o_row = (int)(wrow * NS);
-      proto.o_ss = P.r;
+      proto.o_row = (int)wrow;
       proto.o_e = ve;
       const int f1s = (int)l1.segs.size(), f2s = (int)l2.segs.size();
-      l1.seg(S, oz::Mat{Q.vrow[tm.ver], Q.r, ve, 0}, Q.r);
+      l1.seg(S, oz::Mat{Q.vrow[tm.ver], ve, 0}, Q.r);
       l1.tiles(f1s, P.r, Q.r, nullptr, 0, proto);
-      l2.seg(S, oz::Mat{(int)(wrow * NS), P.r, ve, 0}, Q.r);
+      l2.seg(S, oz::Mat{(int)wrow, ve, 0}, Q.r);
       const size_t j0 = l2.jobs.size();
       l2.tiles(f2s, P.r, P.r, P.Y, P.r, proto);
       dfs[df].tile0[dot] = ntile;
@@ -1351,7 +1347,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     CK(cudaMemcpyAsync(dfd.p, dfs.data(), dfs.size() * sizeof(OzDf), cudaMemcpyHostToDevice, c->st));
     for (size_t q = 0; q + 1 < cut.size(); q++) {
       if (launch_oz_digits(So, Yo, (const oz::Job*)u1.j.p + cut[q][0], cut[q + 1][0] - cut[q][0], (const oz::Seg*)u1.s.p,
-                           (const int*)dn.p, (uint16_t*)wd.p, LD, (const int*)wx.p, c->err_d, c->st) ||
+                           (const int*)dn.p, (uint16_t*)wd.p, LD, std::max<long long>(1, wrows), (const int*)wx.p, c->err_d, c->st) ||
           launch_oz_dots(So, Wo, (const oz::Job*)u2.j.p + cut[q][1], cut[q + 1][1] - cut[q][1], (const oz::Seg*)u2.s.p,
                          (double*)parts.p, c->err_d, c->st))
         return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for dE/df failed");
@@ -1723,8 +1719,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
       gs_rows += (p.first == p.second ? 1 : 2) * (long long)r;
     }
     const int nchv = oz::n_chunks(nv), nchx = oz::n_chunks(nx), ldv = oz::ld_of(nv), ldx = oz::ld_of(nx);
-    if (std::max(rows, gs_rows) * oz::MXSL + oz::BM >= (long long)INT32_MAX || rows * nchv >= (long long)INT32_MAX ||
-        gs_rows * nchx >= (long long)INT32_MAX)
+    if (rows * nchv + oz::BM >= (long long)INT32_MAX || gs_rows * nchx + oz::BM >= (long long)INT32_MAX)
       return fail(c, OSVMP2_E_ARG, "pair-basis digit store exceeds the tensor-map row range");
     float *umem = nullptr, *gmem = nullptr;
     uint16_t* udig = nullptr;
@@ -1738,7 +1733,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     c->Gj_h.resize(c->K_h.size(), nullptr);
     c->um_of.resize(c->K_h.size(), -1);
     c->um_mat.resize(c->K_h.size());
-    const OzOperand Uo{udig, rows * oz::MXSL, nv, ldv, uexp};
+    const OzOperand Uo{udig, rows, nv, ldv, uexp};
     const int sid = (int)c->um_store.size();
     std::vector<MxG> gj;
     std::vector<OzMat> gm;             // digits of G
@@ -1751,7 +1746,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
       const int r = c->r_h[pid], m = pair_dim_h(c, i, j);
       c->U_h[pid] = umem + uo;
       uo += (size_t)nv * r;
-      const oz::Mat um{(int)(urow * oz::MXSL), r, (int)(urow * nchv), nchv};
+      const oz::Mat um{(int)urow, (int)(urow * nchv), nchv};
       urow += r;
       c->um_of[pid] = sid;
       c->um_mat[pid] = um;
@@ -1762,7 +1757,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
       for (int u = 0; u < ng; u++) {
         G[u] = gmem + go;
         go += (size_t)r * nx;
-        gd[u] = oz::Mat{(int)(grow * oz::MXSL), r, (int)(grow * nchx), nchx};
+        gd[u] = oz::Mat{(int)grow, (int)(grow * nchx), nchx};
         grow += r;
         gj.push_back(MxG{u ? j : i, r, um, G[u]});
         gm.push_back(OzMat{(const double*)G[u], r, nx, std::min(ldx, (nx + oz::BK - 1) / oz::BK * oz::BK), nx, gd[u]});
@@ -1820,7 +1815,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
         launch_oz_float((const double*)u0.p, sz, umem + done, c->st);
         done += sz;
         CK(cudaMemcpyAsync(mj.p, um.data(), um.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
-        launch_oz_mats((const OzMat*)mj.p, (int)um.size(), max_r, nv, nullptr, false, oz::MXSL, ldv, udig, uexp, c->st);
+        launch_oz_mats((const OzMat*)mj.p, (int)um.size(), max_r, nv, nullptr, false, oz::MXSL, ldv, rows, udig, uexp, c->st);
         CK(cudaGetLastError());
         b0 = b1;
       }
@@ -1833,13 +1828,13 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     CK(cudaMemcpyAsync(gmd.p, gm.data(), gm.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
     const long long lo_shift = (long long)((float*)glo.p - gmem);
     TRY(mx_project(c, gj, Uo, lo_shift));
-    launch_mx_pairs((const OzMat*)gmd.p, (int)gm.size(), max_r, nx, lo_shift, ldx, (uint16_t*)gd.p, (int*)ge.p, c->st);
+    launch_mx_pairs((const OzMat*)gmd.p, (int)gm.size(), max_r, nx, lo_shift, ldx, gs_rows, (uint16_t*)gd.p, (int*)ge.p, c->st);
     ph_end(c, OSVMP2_PH_PROJECT, f_u + f_g, c->sys.B ? 8.0 * (double)gj.size() * nx * nv : 0.0);
     CK(cudaGetLastError());
     ph_begin(c, OSVMP2_PH_EXCHANGE);
     {
       OzDev d;
-      const OzOperand Go{(const uint16_t*)gd.p, gs_rows * oz::MXSL, nx, ldx, (const int*)ge.p};
+      const OzOperand Go{(const uint16_t*)gd.p, gs_rows, nx, ldx, (const int*)ge.p};
       if (oz_upload(c, lk, d)) return fail(c, OSVMP2_E_NOMEM, "no room for the tile list of K~");
       if (d.n && launch_mx_gemm(Go, Go, (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, true, c->err_d, c->st))
         return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for K~ failed");
@@ -2063,7 +2058,7 @@ int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int ns
     OzList all, l;
     for (int u = 0; u < nu; u++) {
       const int i = i0 + u0 + u;
-      const oz::Mat m{u * ns * nv, nv, u * nv * nch, nch};
+      const oz::Mat m{u * nv, u * nv * nch, nch};
       all.product(m, nv, m, nv, nx, T + (size_t)(u0 + u) * nv * nv, nv);
       for (oz::Job& jb : all.jobs)
         if (jb.n0 < jb.m0 + oz::BM) {          // tiles that touch the lower triangle
@@ -2075,7 +2070,7 @@ int tii_oz(osvmp2_ctx* c, int i0, int b, double* T, uint16_t* D, int* ex, int ns
     l.segs = all.segs;
     OzDev d;
     if (int rc = oz_upload(c, l, d)) return rc;
-    if (launch_oz_tii(OzOperand{D, (long long)nu * ns * nv, nx, oz::ld_of(nx), ex}, (const oz::Job*)d.j.p, d.n,
+    if (launch_oz_tii(OzOperand{D, (long long)nu * nv, nx, oz::ld_of(nx), ex}, (const oz::Job*)d.j.p, d.n,
                       (const oz::Seg*)d.s.p, c->sys.e_vir, ns, c->err_d, c->st))
       return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for T_ii failed");
     CK(cudaGetLastError());
@@ -2286,7 +2281,7 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
   } else {
     TRY(tmp_alloc(c, sm, (size_t)nb * eig_osv_scratch_doubles(nv, kmax) * sizeof(double)));
   }
-  const bool tii_digits = !tii_tc && (double)noz * tii_ns * nv + oz::BM < (double)INT32_MAX &&
+  const bool tii_digits = !tii_tc && (double)noz * nv * oz::n_chunks(s->n_aux) + oz::BM < (double)INT32_MAX &&
                           !oz_room(c, ozD, noz * ozslot) && !oz_room(c, ozE, oz_exp_bytes((size_t)noz * nv, s->n_aux));
   std::vector<int> nrows_h(nb);
   const uint64_t rosv_key = mix64((uint64_t)s->seed ^ (7ull * STREAM_MUL));
@@ -3420,20 +3415,21 @@ static int oz_grad_pairs(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& 
     Tmp D, ex, md;
     const int nch = oz::n_chunks(max_r), ld = oz::ld_of(max_r);
     const long long rows = 2 * yn.rows;
-    if (rows * oz::NSL + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
+    if (rows * nch + oz::BM >= (long long)INT32_MAX) return OZ_NO_ROOM;
     TRY(oz_room(c, D, oz_digit_bytes((size_t)rows, max_r)));
     TRY(oz_room(c, ex, oz_exp_bytes((size_t)rows, max_r)));
     TRY(oz_room(c, md, 2 * yn.mats.size() * sizeof(OzMat)));
     for (OzMat& m : yt.mats) {
-      m.m.row += (int)(yn.rows * oz::NSL);
+      m.m.row += (int)yn.rows;
       m.m.eb += (int)(yn.rows * nch);
     }
     CK(cudaMemcpyAsync(md.p, yn.mats.data(), yn.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
     CK(cudaMemcpyAsync((OzMat*)md.p + yn.mats.size(), yt.mats.data(), yt.mats.size() * sizeof(OzMat), cudaMemcpyHostToDevice,
                        c->st));
-    launch_oz_mats((const OzMat*)md.p, (int)yn.mats.size(), max_r, max_r, nullptr, true, oz::NSL, ld, (uint16_t*)D.p, (int*)ex.p, c->st);
+    launch_oz_mats((const OzMat*)md.p, (int)yn.mats.size(), max_r, max_r, nullptr, true, oz::NSL, ld, rows, (uint16_t*)D.p,
+                   (int*)ex.p, c->st);
     launch_oz_mats((const OzMat*)md.p + yn.mats.size(), (int)yt.mats.size(), max_r, max_r, nullptr, false, oz::NSL, ld,
-                   (uint16_t*)D.p, (int*)ex.p, c->st);
+                   rows, (uint16_t*)D.p, (int*)ex.p, c->st);
     CK(cudaGetLastError());
     size_t k0 = 0;
     for (int q = q0; q < q1; q++) {
@@ -3454,7 +3450,7 @@ static int oz_grad_pairs(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& 
       proto.skip = -1;
       l.tiles(first, g.r, g.r, g.Hy, g.r, proto);
     }
-    const OzOperand op{(const uint16_t*)D.p, rows * oz::NSL, max_r, ld, (const int*)ex.p};
+    const OzOperand op{(const uint16_t*)D.p, rows, max_r, ld, (const int*)ex.p};
     TRY(oz_run(c, op, op, l));
     q0 = q1;
   }

@@ -106,7 +106,7 @@ void launch_pack_q(const double* V, const double* w, int nb, int nv, int kmax, c
                    double* const* Qdst, double* const* wdst, cudaStream_t st);
 
 // ---- FP64 contractions on the tensor cores (oz_gemm.cu, tc_oz.cuh)
-// Digit store of an operand: rows of K BF16 digits with stride ld (a multiple of 8), and chunk exponents.
+// Digit store of an operand: per slice `rows` rows of K BF16 digits with stride ld (a multiple of 8), and chunk exponents.
 struct OzOperand {
   const uint16_t* D;
   long long rows;
@@ -119,22 +119,23 @@ struct OzMat {           // dense matrix whose digits go to m; row stride ldm (s
   oz::Mat m;
 };
 // ns: slices (NSL: FP64; MXSL: 39 bits, mixed form).
-// Digits of B: rows B[i0 + u][a][.] (K = aux) or B[xs[u]][.][P] (K = vir); slot u, slice s, row r at
-// row (u ns + s) rows + r of the store, exponent row u rows + r.
+// Digits of B: rows B[i0 + u][a][.] (K = aux) or B[xs[u]][.][P] (K = vir); slot u, row r at row u rows + r of a store
+// of nb rows per slice.
 void launch_oz_rows(const BSrc& src, int i0, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st);
 void launch_oz_cols(const BSrc& src, const int* xs, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st);
-// Digits of dense matrices: [K][rows] (row index innermost), scaled by w[k] unless NULL; or, k_inner, [rows][K].
+// Digits of dense matrices into a store of `rows` rows: [K][rows] (row index innermost), scaled by w[k] unless
+// NULL; or, k_inner, [rows][K].
 void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const double* w, bool k_inner, int ns, int ld,
-                    uint16_t* D, int* ex, cudaStream_t st);
+                    long long rows, uint16_t* D, int* ex, cudaStream_t st);
 // out[row][col] per job (row-major); T_ii tiles of the lower triangle (mirrored, with denominators).
 // Return 0, or -1 if a tensor map could not be encoded.
 int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    const int* skip, int* err, cudaStream_t st);
 int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int ns,
                   int* err, cudaStream_t st);
-// The digits of the output (jobs' o_row, o_ss, o_e) into the store D with row stride ld (a multiple of 32).
+// The digits of the output (jobs' o_row, o_e) into the store D of `rows` rows with stride ld (a multiple of 32).
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                     const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st);
+                     const int* skip, uint16_t* D, int ld, long long rows, const int* exW, int* err, cudaStream_t st);
 // Dot products of (2 Y - Y^T) with the product of every job (see OzEpiDot), 16 partial sums per job.
 int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    double* parts, int* err, cudaStream_t st);
@@ -162,7 +163,7 @@ struct OzPair {          // a pair of a fragment
   double* C;             // [r][r]
   double* T;             // [m][m] raw-basis amplitude (launch_oz_raw) or NULL
 };
-void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, int nch, uint16_t* D,
+void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, long long rows, int nch, uint16_t* D,
                       int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st);
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
                         double* e_prev, int* done, int* left, FragOut* out, const int* out_id, cudaStream_t st);
@@ -258,8 +259,8 @@ int launch_mx_g(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int
 int launch_mx_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    bool fp64_out, int* err, cudaStream_t st);
 // Digits of matrices of FP32 pairs (OzMat.p: the leading parts, [rows][K]).
-void launch_mx_pairs(const OzMat* mats, int n, int max_rows, int K, long long lo_shift, int ld, uint16_t* D, int* ex,
-                     cudaStream_t st);
+void launch_mx_pairs(const OzMat* mats, int n, int max_rows, int K, long long lo_shift, int ld, long long rows,
+                     uint16_t* D, int* ex, cudaStream_t st);
 void launch_oz_float(const double* x, size_t n, float* y, cudaStream_t st);
 // Products of TF32 slice rows (randomized OSVs): Gs holds `rows` rows of K = n_aux, FP64 row-major output.
 int launch_kt_tc(const float* Gs, long long rows, int n_aux, int ldg, const tc::Job* jobs, int n_jobs, int* err,

@@ -19,8 +19,8 @@ struct OzSrcBT {           // row P of slot u: B[xs[u]][.][P]
 };
 
 template <int NS, class Src>
-__global__ void __launch_bounds__(256) k_oz_rows(Src src, int rows, int K, int ld, uint16_t* __restrict__ D,
-                                                 int* __restrict__ ex) {
+__global__ void __launch_bounds__(256) k_oz_rows(Src src, int rows, int K, int ld, size_t slice,
+                                                 uint16_t* __restrict__ D, int* __restrict__ ex) {
   const int u = blockIdx.y, lane = threadIdx.x & 31;
   const int nch = (K + oz::CHUNK - 1) / oz::CHUNK;
   const long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -32,16 +32,15 @@ __global__ void __launch_bounds__(256) k_oz_rows(Src src, int rows, int K, int l
     const int k = k0 + 64 * (v >> 1) + 2 * lane + (v & 1);
     x[v] = k < K ? src.get(u, r, k) : 0.0;
   }
-  const size_t slice = (size_t)rows * ld;
-  const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, K - k0), D + ((size_t)u * NS * rows + r) * ld + k0, slice, lane);
+  const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, K - k0), D + ((size_t)u * rows + r) * ld + k0, slice, lane);
   if (lane == 0) ex[((size_t)u * rows + r) * nch + c] = e;
 }
 
 // Rows strided in k (their index innermost): one CTA per 16 rows x one chunk, transposed through shared memory so
 // that both the reads (rows innermost) and the digit writes (k innermost) are coalesced.
 template <int NS, class Src>
-__global__ void __launch_bounds__(256) k_oz_cols(Src src, int rows, int K, int ld, uint16_t* __restrict__ D,
-                                                 int* __restrict__ ex) {
+__global__ void __launch_bounds__(256) k_oz_cols(Src src, int rows, int K, int ld, size_t slice,
+                                                 uint16_t* __restrict__ D, int* __restrict__ ex) {
   __shared__ double tile[oz::CHUNK][17];
   const int u = blockIdx.z, r0 = blockIdx.x * 16, c = blockIdx.y, k0 = c * oz::CHUNK;
   const int nch = (K + oz::CHUNK - 1) / oz::CHUNK;
@@ -51,13 +50,12 @@ __global__ void __launch_bounds__(256) k_oz_cols(Src src, int rows, int K, int l
   }
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const size_t slice = (size_t)rows * ld;
   for (int dr = threadIdx.x >> 5; dr < 16 && r0 + dr < rows; dr += 8) {   // warp-uniform
     double x[8];
 #pragma unroll
     for (int v = 0; v < 8; v++) x[v] = tile[64 * (v >> 1) + 2 * lane + (v & 1)][dr];
     const int r = r0 + dr;
-    const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, K - k0), D + ((size_t)u * NS * rows + r) * ld + k0, slice, lane);
+    const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, K - k0), D + ((size_t)u * rows + r) * ld + k0, slice, lane);
     if (lane == 0) ex[((size_t)u * rows + r) * nch + c] = e;
   }
 }
@@ -66,7 +64,7 @@ __global__ void __launch_bounds__(256) k_oz_cols(Src src, int rows, int K, int l
 // digits zero up to kpad.
 template <int NS>
 __global__ void __launch_bounds__(256) k_oz_mats(const OzMat* __restrict__ mats, const double* __restrict__ w,
-                                                 int ld, uint16_t* __restrict__ D, int* __restrict__ ex) {
+                                                 int ld, size_t slice, uint16_t* __restrict__ D, int* __restrict__ ex) {
   __shared__ double tile[oz::CHUNK][17];
   const OzMat mt = mats[blockIdx.z];
   const int r0 = blockIdx.x * 16, c = blockIdx.y, k0 = c * oz::CHUNK, K = mt.K;
@@ -82,7 +80,6 @@ __global__ void __launch_bounds__(256) k_oz_mats(const OzMat* __restrict__ mats,
   }
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const size_t slice = (size_t)mt.m.ss * ld;
   for (int dr = threadIdx.x >> 5; dr < 16 && r0 + dr < mt.rows; dr += 8) {
     double x[8];
 #pragma unroll
@@ -94,8 +91,8 @@ __global__ void __launch_bounds__(256) k_oz_mats(const OzMat* __restrict__ mats,
 }
 // The same for matrices with k innermost ([rows][K], row stride ldm): a warp per (row, chunk).
 template <int NS>
-__global__ void __launch_bounds__(256) k_oz_rmats(const OzMat* __restrict__ mats, int ld, uint16_t* __restrict__ D,
-                                                  int* __restrict__ ex) {
+__global__ void __launch_bounds__(256) k_oz_rmats(const OzMat* __restrict__ mats, int ld, size_t slice,
+                                                  uint16_t* __restrict__ D, int* __restrict__ ex) {
   const OzMat mt = mats[blockIdx.z];
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), c = blockIdx.y, k0 = c * oz::CHUNK, lane = threadIdx.x & 31;
   if (r >= mt.rows || k0 >= mt.K) return;
@@ -106,14 +103,14 @@ __global__ void __launch_bounds__(256) k_oz_rmats(const OzMat* __restrict__ mats
     x[v] = k < mt.K ? mt.p[(size_t)r * mt.ldm + k] : 0.0;
   }
   const int e = oz::warp_slices<NS>(x, min(oz::CHUNK, mt.kpad - k0), D + ((size_t)mt.m.row + r) * ld + k0,
-                                (size_t)mt.m.ss * ld, lane);
+                                slice, lane);
   if (lane == 0) ex[mt.m.eb + (size_t)r * mt.m.es + c] = e;
 }
 
 // Matrices of FP32 pairs with k innermost (mixed form: G and its remainder, lo_shift floats further on): a warp per
 // (row, chunk); the fixed-point numbers without the FP64 pipe, whose conversions would take longer than the reads.
 template <int NS>
-__global__ void __launch_bounds__(256) k_oz_pairs(const OzMat* __restrict__ mats, long long lo_shift, int ld,
+__global__ void __launch_bounds__(256) k_oz_pairs(const OzMat* __restrict__ mats, long long lo_shift, int ld, size_t slice,
                                                   uint16_t* __restrict__ D, int* __restrict__ ex) {
   constexpr int T = 7 + 8 * (NS - 1);                  // |x| < 2^e -> |F| < 2^T
   const OzMat mt = mats[blockIdx.z];
@@ -136,7 +133,6 @@ __global__ void __launch_bounds__(256) k_oz_pairs(const OzMat* __restrict__ mats
   const int sh = live ? T - 16 - e : 0;                // |h 2^sh| < 2^(T - 16) <= 2^23
   const float s0 = __int_as_float(((sh >> 1) + 127) << 23), s1 = __int_as_float((sh - (sh >> 1) + 127) << 23);
   uint16_t* dst = D + ((size_t)mt.m.row + r) * ld + k0;
-  const size_t slice = (size_t)mt.m.ss * ld;
   const int kv = min(oz::CHUNK, mt.kpad - k0);
 #pragma unroll
   for (int u = 0; u < 4; u++) {
@@ -167,34 +163,37 @@ __global__ void k_oz_float(const double* __restrict__ x, size_t n, float* __rest
 
 void launch_oz_rows(const BSrc& src, int i0, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st) {
   if (!nb) return;
+  const size_t slice = (size_t)nb * src.n_vir * oz::ld_of(src.n_aux);
   const long long warps = (long long)src.n_vir * oz::n_chunks(src.n_aux);
   const dim3 grid((unsigned)((warps + 7) / 8), nb);
-  OZ_DISPATCH(ns, (k_oz_rows<NS><<<grid, 256, 0, st>>>(OzSrcB{src, i0}, src.n_vir, src.n_aux, oz::ld_of(src.n_aux), D, ex)));
+  OZ_DISPATCH(ns, (k_oz_rows<NS><<<grid, 256, 0, st>>>(OzSrcB{src, i0}, src.n_vir, src.n_aux, oz::ld_of(src.n_aux), slice, D, ex)));
   note_launch(1);
 }
 void launch_oz_cols(const BSrc& src, const int* xs, int nb, int ns, uint16_t* D, int* ex, cudaStream_t st) {
   if (!nb) return;
+  const size_t slice = (size_t)nb * src.n_aux * oz::ld_of(src.n_vir);
   const dim3 grid((src.n_aux + 15) / 16, oz::n_chunks(src.n_vir), nb);
-  OZ_DISPATCH(ns, (k_oz_cols<NS><<<grid, 256, 0, st>>>(OzSrcBT{src, xs}, src.n_aux, src.n_vir, oz::ld_of(src.n_vir), D, ex)));
+  OZ_DISPATCH(ns, (k_oz_cols<NS><<<grid, 256, 0, st>>>(OzSrcBT{src, xs}, src.n_aux, src.n_vir, oz::ld_of(src.n_vir), slice, D, ex)));
   note_launch(1);
 }
 void launch_oz_mats(const OzMat* mats, int n, int max_rows, int max_K, const double* w, bool k_inner, int ns, int ld,
-                    uint16_t* D, int* ex, cudaStream_t st) {
+                    long long rows, uint16_t* D, int* ex, cudaStream_t st) {
   if (!n) return;
+  const size_t slice = (size_t)rows * ld;
   for (int q = 0; q < n; q += 65535) {     // grid z limit
     const int nq = n - q < 65535 ? n - q : 65535;
     const dim3 gr((max_rows + 7) / 8, oz::n_chunks(max_K), nq), gc((max_rows + 15) / 16, oz::n_chunks(max_K), nq);
-    if (k_inner) OZ_DISPATCH(ns, (k_oz_rmats<NS><<<gr, 256, 0, st>>>(mats + q, ld, D, ex)));
-    else OZ_DISPATCH(ns, (k_oz_mats<NS><<<gc, 256, 0, st>>>(mats + q, w, ld, D, ex)));
+    if (k_inner) OZ_DISPATCH(ns, (k_oz_rmats<NS><<<gr, 256, 0, st>>>(mats + q, ld, slice, D, ex)));
+    else OZ_DISPATCH(ns, (k_oz_mats<NS><<<gc, 256, 0, st>>>(mats + q, w, ld, slice, D, ex)));
     note_launch(1);
   }
 }
 
-void launch_mx_pairs(const OzMat* mats, int n, int max_rows, int K, long long lo_shift, int ld, uint16_t* D, int* ex,
-                     cudaStream_t st) {
+void launch_mx_pairs(const OzMat* mats, int n, int max_rows, int K, long long lo_shift, int ld, long long rows, uint16_t* D,
+                     int* ex, cudaStream_t st) {
   for (int q = 0; q < n; q += 65535) {     // grid z limit
     const int nq = n - q < 65535 ? n - q : 65535;
-    k_oz_pairs<oz::MXSL><<<dim3((max_rows + 7) / 8, oz::n_chunks(K), nq), 256, 0, st>>>(mats + q, lo_shift, ld, D, ex);
+    k_oz_pairs<oz::MXSL><<<dim3((max_rows + 7) / 8, oz::n_chunks(K), nq), 256, 0, st>>>(mats + q, lo_shift, ld, (size_t)rows * ld, D, ex);
     note_launch(1);
   }
 }
@@ -276,8 +275,7 @@ struct OzEpiTPair {
   }
 };
 
-// Digits of the output instead of its values: row m0 + r, k = n0 + c of the matrix at store row o_row (o_ss
-// rows per slice), under the exponent code exW[o_e] (a bound of the whole matrix); columns past n_valid up to the
+// Digits of the output instead of its values: row m0 + r, k = n0 + c of the matrix at store row o_row, under the exponent code exW[o_e] (a bound of the whole matrix); columns past n_valid up to the
 // next multiple of 16 are written as zeros (up to 32 by the lanes of the last column group).
 template <int NS>
 struct OzEpiDigits {
@@ -285,11 +283,11 @@ struct OzEpiDigits {
   static constexpr int T = 7 + 8 * (NS - 1);
   uint16_t* D;
   int ld;
+  size_t slice;
   const int* exW;
   __device__ __forceinline__ int exponent(const oz::Job& jb) const { return exW[jb.o_e]; }
   __device__ __forceinline__ void digits(const oz::Job& jb, int r, int c0, long long (&f)[oz::DCOL]) const {
     uint16_t* o = D + ((size_t)jb.o_row + jb.m0 + r) * ld + jb.n0 + c0;
-    const size_t slice = (size_t)jb.o_ss * ld;
     // the last column group also clears the group after it when that completes a 32-wide k-block
     const bool tail = c0 + oz::DCOL >= jb.n_valid && ((jb.n0 + c0) & 16) == 0;
 #pragma unroll
@@ -332,15 +330,15 @@ struct OzEpiDot {
 };
 
 namespace {
-// 2-D BF16 map over rows x ld, 64-byte swizzle, box 32 x box_rows.  K < ld: k past K reads as 0.
-bool make_digit_map(CUtensorMap* m, const OzOperand& A, int box_rows) {
+// 3-D BF16 map over k x rows x slices, 64-byte swizzle, box 32 x box_rows x ns.  K < ld: k past K reads as 0.
+bool make_digit_map(CUtensorMap* m, const OzOperand& A, int ns, int box_rows) {
   auto enc = tensor_map_encoder();
   if (!enc) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)A.K, (cuuint64_t)A.rows};
-  cuuint64_t strides[1] = {(cuuint64_t)A.ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)oz::BK, (cuuint32_t)box_rows};
-  cuuint32_t es[2] = {1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(A.D), dims, strides, box, es,
+  cuuint64_t dims[3] = {(cuuint64_t)A.K, (cuuint64_t)A.rows, (cuuint64_t)ns};
+  cuuint64_t strides[2] = {(cuuint64_t)A.ld * 2, (cuuint64_t)A.rows * A.ld * 2};
+  cuuint32_t box[3] = {(cuuint32_t)oz::BK, (cuuint32_t)box_rows, (cuuint32_t)ns};
+  cuuint32_t es[3] = {1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<uint16_t*>(A.D), dims, strides, box, es,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -351,9 +349,10 @@ int run(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs,
   if (!n_jobs) return 0;
   constexpr int SMEM = oz::Cfg<NS>::SMEM;
   if (cudaFuncSetAttribute(oz::k_oz<NS, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess) return -1;
-  CUtensorMap ma, mb;
-  if (!make_digit_map(&ma, A, oz::AROWS) || !make_digit_map(&mb, B, oz::BROWS)) return -1;
-  oz::k_oz<NS, Epi><<<tc::persistent_grid(n_jobs), oz::NTHREADS, SMEM, st>>>(ma, mb, A.ex, B.ex, jobs, n_jobs, segs, skip,
+  oz::OzMaps tm;
+  for (int u = 0; u < 2; u++)
+    if (!make_digit_map(&tm.a[u], A, NS, oz::BM >> (1 - u)) || !make_digit_map(&tm.b[u], B, NS, oz::BN >> (1 - u))) return -1;
+  oz::k_oz<NS, Epi><<<tc::persistent_grid(n_jobs), oz::NTHREADS, SMEM, st>>>(tm, A.ex, B.ex, jobs, n_jobs, segs, skip,
                                                                              err, epi);
   note_launch(1);
   return 0;
@@ -365,8 +364,8 @@ int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, 
   return run<oz::NSL>(A, B, jobs, n_jobs, segs, skip, err, OzEpiRow{}, st);
 }
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
-                     const int* skip, uint16_t* D, int ld, const int* exW, int* err, cudaStream_t st) {
-  return run<oz::NSL>(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits<oz::NSL>{D, ld, exW}, st);
+                     const int* skip, uint16_t* D, int ld, long long rows, const int* exW, int* err, cudaStream_t st) {
+  return run<oz::NSL>(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits<oz::NSL>{D, ld, (size_t)rows * ld, exW}, st);
 }
 int launch_mx_g(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                 long long lo_shift, int* err, cudaStream_t st) {

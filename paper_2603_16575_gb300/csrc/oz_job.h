@@ -14,11 +14,11 @@ constexpr int CHUNK = 256;    // k-extent that shares one power-of-two scale per
 constexpr int EX_ZERO = -(1 << 20);   // chunk exponent of an all-zero chunk
 constexpr int EX_NAN = 1 << 20;       // and of one that holds a NaN or an Inf
 
-// An operand matrix: rows with K innermost, BF16 digits at store rows row + s * ss + r (slice s, row r,
-// in units of the store's row stride), exponent of chunk c of row r at ex[eb + r * es + c] (es = 0: one
+// An operand matrix: rows with K innermost, BF16 digits of slice s, row r at store row s * (rows of the store) + row + r
+// (in units of the store's row stride), exponent of chunk c of row r at ex[eb + r * es + c] (es = 0: one
 // exponent for all rows).
 struct Mat {
-  int row, ss, eb, es;
+  int row, eb, es;
 };
 // out += coef * A B^T over K
 struct Seg {
@@ -33,8 +33,7 @@ struct Job {
   int m_valid, n_valid;    // rows (<= 128) and columns (<= 64) to store
   int ld_out;
   int skip;                // index of a flag that makes the kernel leave the tile out, or -1
-  int o_row, o_ss, o_e;    // digit-writing epilogue: output matrix in its store, index of its exponent
-  int pad;
+  int o_row, o_e;          // digit-writing epilogue: output matrix in its store, index of its exponent
   double s;                // epilogue scalar
   void* out;               // the output's first element (not the tile's)
 };

@@ -169,7 +169,7 @@ __device__ __forceinline__ void row_digits(const double* Y, int r, int m, int v,
 }
 
 __global__ void __launch_bounds__(NT) k_oz_update(const OzPair* __restrict__ pairs, int n_pairs,
-                                                  const int* __restrict__ done, int first, int ld, int nch,
+                                                  const int* __restrict__ done, int first, int ld, size_t slice, int nch,
                                                   uint16_t* __restrict__ D, int* __restrict__ ex,
                                                   int* __restrict__ exW, double* __restrict__ pe,
                                                   double* __restrict__ pu) {
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(NT) k_oz_update(const OzPair* __restrict__ pai
       }
       uint16_t* base = D + (size_t)p.vrow[v] * ld;
       for (int m = warp; m < r; m += NT / 32)
-        row_digits(p.Y, r, m, v, ey, p.kpad, base + (size_t)m * ld, (size_t)r * ld, lane);
+        row_digits(p.Y, r, m, v, ey, p.kpad, base + (size_t)m * ld, slice, lane);
     }
     __syncthreads();
   }
@@ -246,10 +246,10 @@ __global__ void k_oz_converge(const int* __restrict__ pair0, int n_frag, const d
   else atomicAdd(left, 1);
 }
 
-void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, int nch, uint16_t* D,
+void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, long long rows, int nch, uint16_t* D,
                       int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st) {
   if (!n_pairs) return;
-  k_oz_update<<<n_cta, NT, 0, st>>>(pairs, n_pairs, done, first ? 1 : 0, ld, nch, D, ex, exW, pe, pu);
+  k_oz_update<<<n_cta, NT, 0, st>>>(pairs, n_pairs, done, first ? 1 : 0, ld, (size_t)rows * ld, nch, D, ex, exW, pe, pu);
   note_launch(1);
 }
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,

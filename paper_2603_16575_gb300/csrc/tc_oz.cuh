@@ -35,7 +35,7 @@
 // for the digits.
 //
 // Persistent CTAs (one per SM) over output tiles of 128 rows (TMEM lanes) x up to 64 columns:
-//   warp 0     TMA producer: the 8 + 8 slice tiles of a 32-wide k-block per stage (64-byte
+//   warp 0     TMA producer: the slices of a 32-wide k-block, one box an operand, per stage (64-byte
 //              swizzle, K-major), two stages of 96 KB
 //   warp 1     TMEM allocation and the single MMA-issuing thread
 //   warps 2-17 drain and epilogue: four warps per TMEM lane quarter, 16 columns each (the 64-bit
@@ -47,6 +47,8 @@
 #include <cuda.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "oz_job.h"
 #include "oz_split.cuh"
 #include "tc_ptx.cuh"
@@ -54,15 +56,21 @@
 namespace osv {
 namespace oz {
 
-constexpr int A_TILE = BM * BK * 2;          // 8 KB per A slice tile (filled up to m rows)
-constexpr int B_TILE = BN * BK * 2;          // 4 KB per B slice tile (filled up to n rows)
-constexpr int AROWS = 64, BROWS = 32;        // rows of one TMA box of the A and B operands
+constexpr int A_TILE = BM * BK * 2;          // 8 KB per A slice tile
+constexpr int B_TILE = BN * BK * 2;          // 4 KB per B slice tile
 constexpr int NDRAIN = 16;                   // drain warps
 constexpr int DCOL = BN * 4 / NDRAIN;        // columns of one: four warps share a TMEM lane quarter
 constexpr int NTHREADS = 64 + 32 * NDRAIN;
 constexpr int KBC = CHUNK / BK;              // k-blocks of a full chunk
 constexpr int TMEM_COLS = 512;
 constexpr int ERR_TC_TIMEOUT = 16;           // same bit as ERR_TIMEOUT of the library
+
+// Tensor maps of the two operands (k, row, slice): boxes of 32 k, every slice, and [0] half of or [1] all of a
+// tile's rows.  One box takes an operand's part of a k-block: a TMA load costs ~95 cycles besides bytes / 80, so
+// boxes of one slice and 64 or 32 rows (2 and 4 KB) fed the SM 17 to 29 bytes a cycle, these feed it 70 and more.
+struct OzMaps {
+  CUtensorMap a[2], b[2];
+};
 
 template <int NS>
 struct Cfg {
@@ -84,14 +92,16 @@ __device__ __forceinline__ double oz_fma(long long v, int x, double coef, double
 }
 
 // Columns of a tile's level accumulators, and rows of its B slices in shared memory: BN, or half of it.
-__device__ __forceinline__ int width(const Job& jb) { return jb.n_valid <= BROWS ? BROWS : BN; }
+__device__ __forceinline__ int width(const Job& jb) { return jb.n_valid <= BN / 2 ? BN / 2 : BN; }
+// Rows of its A slices in shared memory: with half of BM the MMAs read the next slice as the rows past the end.
+__device__ __forceinline__ int height(const Job& jb) { return jb.m_valid <= BM / 2 ? BM / 2 : BM; }
 
 // The products of one 16-wide k step (ks).  Slice sa of A times the slices 0 .. NS - 1 - sa of B adds to the levels
 // sa .. NS - 1; those slices of B follow one another in shared memory as the levels do in TMEM, so one MMA takes as
 // many of them as N = 256 holds: 12 MMAs for the 36 products of NS = 8, and A is read once for each.  (One MMA a
 // product, N = 64, spent its time on the reads of A: 90 cycles for 32 of multiplication.)  free(l): level l of the
 // last chunk has been read; done: barriers of the levels, committed as they become complete, or NULL.
-template <int NS, int W, class Free>
+template <int NS, int W, int H, class Free>
 __device__ __forceinline__ bool issue(uint64_t da, uint64_t db, uint32_t dcol, int ks, bool zero, const Free& free,
                                       uint64_t* done) {
   constexpr int P = 256 / W;                                       // slices of B an MMA takes
@@ -104,7 +114,7 @@ __device__ __forceinline__ bool issue(uint64_t da, uint64_t db, uint32_t dcol, i
       if (sa == 0 && zero)
         for (int l = j; l < j + c; l++)
           if (!free(l)) return false;
-      tc::mma_f16(dcol + (uint32_t)((sa + j) * W), da + (uint64_t)((sa * A_TILE + 32 * ks) >> 4),
+      tc::mma_f16(dcol + (uint32_t)((sa + j) * W), da + (uint64_t)((sa * H * BK * 2 + 32 * ks) >> 4),
                   db + (uint64_t)((j * W * BK * 2 + 32 * ks) >> 4), idesc | ((uint32_t)(c * W >> 3) << 17),
                   sa == 0 && zero ? 0u : 1u);
     }
@@ -136,7 +146,7 @@ __device__ __forceinline__ void pair_add(float vh, float vl, int x, float& ah, f
 // issues one warp in 64 cycles per element and chunk, more than the 15 products of a chunk; pairs take none.
 template <int NS, class Epi>
 __global__ void __launch_bounds__(NTHREADS, 1)
-    k_oz(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const int* __restrict__ exA,
+    k_oz(const __grid_constant__ OzMaps tm, const int* __restrict__ exA,
          const int* __restrict__ exB, const Job* __restrict__ jobs, int n_jobs, const Seg* __restrict__ segs,
          const int* __restrict__ skip, int* err, Epi epi) {
   using C = Cfg<NS>;
@@ -163,8 +173,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       tc::mbar_init(&bar_acce[l], NDRAIN);
     }
     asm volatile("fence.mbarrier_init.release.cluster;");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+    for (int u = 0; u < 2; u++) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm.a[u])) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm.b[u])) : "memory");
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -180,9 +192,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
         const Job jb = jobs[tile];
         if (jb.skip >= 0 && skip[jb.skip]) continue;
-        const int nbox = (jb.n_valid + BROWS - 1) / BROWS, mbox = (jb.m_valid + AROWS - 1) / AROWS;
-        const int btile = width(jb) * BK * 2;
-        const uint32_t bytes = NS * (mbox * AROWS + nbox * BROWS) * BK * 2;
+        const int h = height(jb), w = width(jb);
+        const uint32_t bytes = NS * (h + w) * BK * 2;
+        const CUtensorMap *ma = &tm.a[h == BM], *mb = &tm.b[w == BN];
         for (int q = 0; ok && q < jb.nseg; q++) {
           const Seg sg = segs[jb.seg0 + q];
           const int nkb = (sg.K + BK - 1) / BK, ra = sg.a.row + jb.m0, rb = sg.b.row + jb.n0;
@@ -193,13 +205,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const uint32_t fb = tc::su32(&bar_full[s]);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(bytes) : "memory");
             const uint32_t st = sbase + s * C::STAGE;
-            for (int sl = 0; sl < NS; sl++) {
-              for (int bx = 0; bx < mbox; bx++)
-                tc::tma_load_2d(st + sl * A_TILE + bx * AROWS * BK * 2, &tmA, fb, c * BK, ra + sl * sg.a.ss + bx * AROWS);
-              for (int bx = 0; bx < nbox; bx++)
-                tc::tma_load_2d(st + NS * A_TILE + sl * btile + bx * BROWS * BK * 2, &tmB, fb, c * BK,
-                                rb + sl * sg.b.ss + bx * BROWS);
-            }
+            tc::tma_load_3d(st, ma, fb, c * BK, ra, 0);
+            tc::tma_load_3d(st + NS * A_TILE, mb, fb, c * BK, rb, 0);
           }
         }
       }
@@ -217,7 +224,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
         const Job jb = jobs[tile];
         if (jb.skip >= 0 && skip[jb.skip]) continue;
-        const bool wide = width(jb) == BN;
+        const bool wide = width(jb) == BN, tall = height(jb) == BM;
         for (int q = 0; ok && q < jb.nseg; q++) {
           const int K = segs[jb.seg0 + q].K, nkb = (K + BK - 1) / BK;
           for (int c = 0; c < nkb; c++, g++) {
@@ -243,10 +250,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
             for (int ks = 0; ks < nks; ks++) {
               const bool fin = last && ks == nks - 1;
+              auto go = [&](auto W, auto H) {
+                return issue<NS, W, H>(da, db, dcol, ks, first && ks == 0, level_free, fin ? &bar_accf[b] : nullptr);
+              };
               if (wide)
-                ok = issue<NS, BN>(da, db, dcol, ks, first && ks == 0, level_free, fin ? &bar_accf[b] : nullptr);
+                ok = tall ? go(std::integral_constant<int, BN>{}, std::integral_constant<int, BM>{})
+                          : go(std::integral_constant<int, BN>{}, std::integral_constant<int, BM / 2>{});
               else
-                ok = issue<NS, BROWS>(da, db, dcol, ks, first && ks == 0, level_free, fin ? &bar_accf[b] : nullptr);
+                ok = tall ? go(std::integral_constant<int, BN / 2>{}, std::integral_constant<int, BM>{})
+                          : go(std::integral_constant<int, BN / 2>{}, std::integral_constant<int, BM / 2>{});
               if (!ok) break;
             }
             if (!ok) break;
