@@ -627,16 +627,16 @@ struct OzList {
   std::vector<oz::Seg> segs;
   void seg(const oz::Mat& a, const oz::Mat& b, int K, double coef = 1.0) { segs.push_back(oz::Seg{a, b, K, 0, coef}); }
   // tiles of a rows x cols output that sums the segments added since first
-  void tiles(int first, int rows, int cols, void* out, int ld_out, oz::Job proto = oz::Job{}) {
+  void tiles(int first, int rows, int cols, void* out, int ld_out, oz::Job proto = oz::Job{}, int bn = oz::BN) {
     for (int m0 = 0; m0 < rows; m0 += oz::BM)
-      for (int n0 = 0; n0 < cols; n0 += oz::BN) {
+      for (int n0 = 0; n0 < cols; n0 += bn) {
         oz::Job jb = proto;
         jb.seg0 = first;
         jb.nseg = (int)segs.size() - first;
         jb.m0 = m0;
         jb.n0 = n0;
         jb.m_valid = std::min(oz::BM, rows - m0);
-        jb.n_valid = std::min(oz::BN, cols - n0);
+        jb.n_valid = std::min(bn, cols - n0);
         jb.ld_out = ld_out;
         jb.out = out;
         jobs.push_back(jb);
@@ -1007,6 +1007,17 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
   return 0;
 }
 
+// Overlaps of pair couples of the mixed form (build_sigma_table).
+struct SigmaStore {
+  Tmp data, off, hi, pos;
+  SigmaTable tab{};
+  std::vector<int> off_h, hi_h;          // the table on the host
+  std::vector<long long> pos_h;
+  const float* find(int lo, int h) const {
+    const auto b = hi_h.begin() + off_h[lo], e = hi_h.begin() + off_h[lo + 1], at = std::lower_bound(b, e, h);
+    return at != e && *at == h ? (const float*)data.p + pos_h[at - hi_h.begin()] : nullptr;
+  }
+};
 // Amplitude iterations of a list of fragments in the FP64 form (solve_oz.cu).  orbs: ascending orbitals of
 // each; results to out[out_id[f]]; raw-basis amplitudes (pairs a <= b in order, m^2 each) to tdst + toff[out_id[f]]
 // unless tdst is NULL; pair_e (host, may be NULL; one fragment): the pair energies.  Fragments in batches that
@@ -1017,11 +1028,18 @@ struct OzWant {
   bool raw = true;
   double* df = nullptr;             // device [n][9], by out_id
   const std::vector<Frag>* frags = nullptr;   // by out_id
+  // mixed form (solve_mx.cu): the overlaps, and CTAs per SM of the element-wise update, chosen by timing its first
+  // sweep when *tune (then cleared)
+  const SigmaStore* mx = nullptr;
+  int* ctas_per_sm = nullptr;
+  bool* tune = nullptr;
+  float* tune_ms = nullptr;
 };
 int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, const std::vector<int>& out_id, size_t f0,
                    size_t f1, const SolveOpts& so, double ulps, FragOut* out, double* tdst, const long long* toff,
                    double* pair_e, const OzWant& want) {
-  constexpr int NS = oz::NSL;
+  const bool mx = want.mx != nullptr;
+  const int NS = mx ? oz::MXSOLVE : oz::NSL;
   const int n = c->sys.n_occ, nv = c->sys.n_vir;
   struct Term { int p, q, ver; double coef; };     // pairs by index in the batch
   std::vector<OzPair> pairs;
@@ -1038,7 +1056,8 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     for (int a = 0; a < nc; a++)
       for (int b = a; b < nc; b++) {
         const int i = o[a], j = o[b], id = c->pair_id[(size_t)i * n + j];
-        if (id < 0 || id >= (int)c->ud_of.size() || c->ud_of[id] < 0) return OZ_NO_ROOM;
+        if (!mx && (id < 0 || id >= (int)c->ud_of.size() || c->ud_of[id] < 0)) return OZ_NO_ROOM;
+        if (c->r_h[id] < 1) return OZ_NO_ROOM;
         OzPair p{};
         p.frag = (int)(f - f0);
         p.r = c->r_h[id];
@@ -1118,7 +1137,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
           }
     }
   const int np = (int)pairs.size(), nfb = (int)(f1 - f0), nt = (int)terms.size();
-  const int LD = (max_r + oz::BK - 1) / oz::BK * oz::BK, nch = oz::n_chunks(max_r);
+  const int LD = (max_r + oz::BK - 1) / oz::BK * oz::BK, nch = mx ? 1 : oz::n_chunks(max_r);   // mx: an exponent a matrix
   // digit matrices of the amplitudes
   int nver = 0;
   long long yrows = 0;
@@ -1188,7 +1207,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   TRY(oz_room(c, wd, (size_t)wrows * NS * LD * 2));
   TRY(oz_room(c, sd, (size_t)srows * NS * LD * 2));
   TRY(oz_room(c, sx, (size_t)srows * nch * sizeof(int)));
-  TRY(oz_room(c, sgm, sgsz * sizeof(double)));
+  if (!mx) TRY(oz_room(c, sgm, sgsz * sizeof(double)));
   TRY(oz_room(c, pr, np * sizeof(OzPair)));
   TRY(oz_room(c, p0, pair0.size() * sizeof(int)));
   TRY(oz_room(c, pe, np * sizeof(double)));
@@ -1201,7 +1220,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   {
     size_t off = 0;
     for (OzPair& p : pairs) {
-      p.Y = p.T && !want.raw ? p.T : (double*)yc.p + off;
+      p.Y = p.T && !want.raw && !mx ? p.T : (double*)yc.p + off;
       p.C = (double*)yc.p + ysz + off;
       off += (size_t)p.r * p.r;
     }
@@ -1211,9 +1230,71 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   CK(cudaMemcpyAsync(oi.p, oid.data(), nfb * sizeof(int), cudaMemcpyHostToDevice, c->st));
   CK(cudaMemsetAsync(ep.p, 0, nfb * sizeof(double), c->st));
   CK(cudaMemsetAsync(dn.p, 0, nfb * sizeof(int), c->st));
+  // mixed form: K~ and 1 / D of the pairs in use, P, drift
+  Tmp mt, mp, mtj, mP, dr, scr2, msj, mep, mt0, mtb;
+  const int max_left = std::min(np, 2 * c->num_sms);
+  if (mx) {
+    std::unordered_map<int, size_t> at;
+    std::vector<MxTable> tj;
+    std::vector<MxPair> mpair(np);
+    size_t tsz = 0, off = 0;
+    for (int p = 0; p < np; p++)
+      if (at.emplace(pid[p], tsz).second) tsz += (size_t)pairs[p].r * pairs[p].r;
+    TRY(oz_room(c, mt, 2 * tsz * sizeof(dfl)));
+    TRY(oz_room(c, mP, ysz * sizeof(float)));
+    TRY(oz_room(c, mp, np * sizeof(MxPair)));
+    TRY(oz_room(c, mtj, at.size() * sizeof(MxTable)));
+    TRY(oz_room(c, dr, nfb * (2 * sizeof(double) + sizeof(int))));
+    TRY(oz_room(c, scr2, (size_t)max_left * 2 * max_r * max_r * sizeof(float)));
+    std::vector<char> seen(c->K_h.size(), 0);
+    for (int p = 0; p < np; p++) {
+      const OzPair& P = pairs[p];
+      dfl* Kd = (dfl*)mt.p + at[pid[p]];
+      mpair[p] = MxPair{Kd, Kd + tsz, c->Sh_h[pid[p]], c->Gh_h[pid[p]], (float*)mP.p + off};
+      off += (size_t)P.r * P.r;
+      if (!seen[pid[p]]) {
+        seen[pid[p]] = 1;
+        tj.push_back(MxTable{P.r, 0, P.fij, P.Kt, P.et, Kd, Kd + tsz});
+      }
+    }
+    CK(cudaMemcpyAsync(mp.p, mpair.data(), np * sizeof(MxPair), cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemcpyAsync(mtj.p, tj.data(), tj.size() * sizeof(MxTable), cudaMemcpyHostToDevice, c->st));
+    std::vector<MxBound> mb;
+    for (const Term& t : terms) {
+      int e;
+      std::frexp(t.coef, &e);
+      mb.push_back(MxBound{pairs[t.q].ver[t.ver], e});
+    }
+    TRY(oz_room(c, mep, np * sizeof(int)));
+    TRY(oz_room(c, mt0, term0.size() * sizeof(int)));
+    TRY(oz_room(c, mtb, std::max<size_t>(1, mb.size()) * sizeof(MxBound)));
+    CK(cudaMemcpyAsync(mt0.p, term0.data(), term0.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+    if (!mb.empty()) CK(cudaMemcpyAsync(mtb.p, mb.data(), mb.size() * sizeof(MxBound), cudaMemcpyHostToDevice, c->st));
+    CK(cudaMemsetAsync(mP.p, 0, ysz * sizeof(float), c->st));
+    CK(cudaMemsetAsync(dr.p, 0, nfb * (2 * sizeof(double) + sizeof(int)), c->st));
+    launch_mx_tables((const MxTable*)mtj.p, (int)tj.size(), c->st);
+    CK(cudaGetLastError());
+  }
   // overlaps, grouped by the stores of the two bases, then their digits
   std::vector<oz::Mat> slo(cps.size()), shi(cps.size());
-  if (!cps.empty()) {
+  if (mx && !cps.empty()) {
+    std::vector<MxSigma> sj;
+    long long row = 0;
+    for (size_t u = 0; u < cps.size(); u++) {
+      const int rl = c->r_h[cps[u].lo], rh = c->r_h[cps[u].hi];
+      const float* S = want.mx->find(cps[u].lo, cps[u].hi);
+      if (!S) return fail(c, OSVMP2_E_STATE, "pair couple without an overlap");
+      slo[u] = oz::Mat{(int)row, (int)(row * nch), nch};
+      row += rl;
+      shi[u] = oz::Mat{(int)row, (int)(row * nch), nch};
+      row += rh;
+      sj.push_back(MxSigma{S, rl, rh, slo[u], shi[u]});
+    }
+    TRY(oz_room(c, msj, sj.size() * sizeof(MxSigma)));
+    CK(cudaMemcpyAsync(msj.p, sj.data(), sj.size() * sizeof(MxSigma), cudaMemcpyHostToDevice, c->st));
+    launch_mx_sigma((const MxSigma*)msj.p, (int)sj.size(), max_r, LD, srows, (uint16_t*)sd.p, 6 * c->num_sms, c->st);
+    CK(cudaGetLastError());
+  } else if (!cps.empty()) {
     std::map<std::pair<int, int>, OzList> groups;
     std::vector<OzMat> m1, m2;
     long long row = 0;
@@ -1240,6 +1321,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   const OzOperand Yo{(const uint16_t*)yd.p, std::max<long long>(1, yrows), LD, LD, (const int*)yx.p};
   const OzOperand Wo{(const uint16_t*)wd.p, std::max<long long>(1, wrows), LD, LD, (const int*)wx.p};
   // the two products of every group of pairs
+  const int cols = oz::tile_cols(NS);
   const size_t ng = grp.size() - 1;
   std::vector<OzDev> d1(ng), d2(ng);
   for (size_t g = 0; g < ng; g++) {
@@ -1256,17 +1338,19 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
         oz::Job proto{};
         proto.skip = P.frag;
         proto.o_row = (int)wrow;
-        proto.o_e = ve;
+        proto.o_e = mx ? p : ve;
+        proto.s = mx ? tm.coef : 0.0;
         const int f1s = (int)l1.segs.size();
         l1.seg(S, oz::Mat{Q.vrow[tm.ver], ve, 0}, Q.r);
-        l1.tiles(f1s, P.r, Q.r, nullptr, 0, proto);
+        l1.tiles(f1s, P.r, Q.r, nullptr, mx ? Q.ver[tm.ver] : 0, proto, cols);
         l2.seg(S, oz::Mat{(int)wrow, ve, 0}, Q.r, tm.coef);
         wrow += P.r;
       }
       if ((int)l2.segs.size() > first) {
         oz::Job proto{};
         proto.skip = P.frag;
-        l2.tiles(first, P.r, P.r, P.C, P.r, proto);
+        proto.o_e = p;
+        l2.tiles(first, P.r, P.r, P.C, P.r, proto, cols);
       }
     }
     TRY(oz_upload(c, l1, d1[g]));
@@ -1277,6 +1361,15 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   for (int it = 1; it <= so.max_iter; it++) {
     if (it > 1)
       for (size_t g = 0; g < ng; g++) {
+        if (mx) {
+          if ((d1[g].n && launch_mx_w(So, Yo, (const oz::Job*)d1[g].j.p, d1[g].n, (const oz::Seg*)d1[g].s.p, (const int*)dn.p,
+                                      (uint16_t*)wd.p, LD, std::max<long long>(1, wrows), (const int*)yx.p,
+                                      (const int*)mep.p, c->err_d, c->st)) ||
+              (d2[g].n && launch_mx_c(So, Wo, (const oz::Job*)d2[g].j.p, d2[g].n, (const oz::Seg*)d2[g].s.p, (const int*)dn.p,
+                                      (const int*)mep.p, c->err_d, c->st)))
+            return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
+          continue;
+        }
         if (d1[g].n && launch_oz_digits(So, Yo, (const oz::Job*)d1[g].j.p, d1[g].n, (const oz::Seg*)d1[g].s.p,
                                         (const int*)dn.p, (uint16_t*)wd.p, LD, std::max<long long>(1, wrows), (const int*)wx.p, c->err_d, c->st))
           return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
@@ -1284,10 +1377,52 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
                                       (const int*)dn.p, c->err_d, c->st))
           return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the amplitude products failed");
       }
+    if (mx) {
+      double* scale = (double*)dr.p;
+      double* drift = scale + nfb;
+      int* refresh = (int*)(drift + nfb);
+      auto update = [&](int per_sm) {
+        launch_mx_update((const OzPair*)pr.p, (const MxPair*)mp.p, np, (const int*)dn.p, it == 1, max_r, LD,
+                         std::max<long long>(1, yrows), (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p, (double*)pe.p,
+                         (double*)pu.p, std::min(np, per_sm * c->num_sms), c->st);
+      };
+      if (it > 1)
+        launch_mx_leftover((const OzPair*)pr.p, (const MxPair*)mp.p, np, (const int*)dn.p, refresh, max_r, (float*)scr2.p,
+                           max_left, c->st);
+      if (it == 1 && want.tune && *want.tune) {   // the first sweep starts from Y = 0 and can be repeated
+        cudaEvent_t e0, e1;
+        CK(cudaEventCreate(&e0));
+        CK(cudaEventCreate(&e1));
+        update(1);
+        float best = 1e30f;
+        for (int k = 1; k <= 3; k++) {
+          CK(cudaEventRecord(e0, c->st));
+          update(k);
+          CK(cudaEventRecord(e1, c->st));
+          CK(cudaEventSynchronize(e1));
+          float ms = 0.f;
+          CK(cudaEventElapsedTime(&ms, e0, e1));
+          if (ms < best) {
+            best = ms;
+            *want.ctas_per_sm = k;
+          }
+        }
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        *want.tune = false;
+        *want.tune_ms = best;
+      } else {
+        update(*want.ctas_per_sm);
+      }
+      launch_mx_bounds((const int*)mt0.p, (const MxBound*)mtb.p, np, (const int*)wx.p, (int*)mep.p, c->st);
+      launch_mx_converge((const int*)p0.p, nfb, (const double*)pe.p, (const double*)pu.p, so, it, (double*)ep.p, scale, drift,
+                         refresh, (int*)dn.p, (int*)lf.p, out, (const int*)oi.p, c->st);
+    } else {
     launch_oz_update((const OzPair*)pr.p, np, (const int*)dn.p, it == 1, LD, std::max<long long>(1, yrows), nch, (uint16_t*)yd.p, (int*)yx.p, (int*)wx.p,
                      (double*)pe.p, (double*)pu.p, n_cta, c->st);
     launch_oz_converge((const int*)p0.p, nfb, (const double*)pe.p, (const double*)pu.p, so, ulps, it, (double*)ep.p,
                        (int*)dn.p, (int*)lf.p, out, (const int*)oi.p, c->st);
+    }
     CK(cudaGetLastError());
     if (it >= 4 || it == so.max_iter) {      // (a finished fragment's sweeps are skipped on the device, few finish before the fourth)
       int left = 0;
@@ -1356,7 +1491,10 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
                  c->st);
     CK(cudaGetLastError());
   }
-  if (tdst && want.raw) {
+  if (tdst && mx) {
+    launch_mx_store((const OzPair*)pr.p, np, c->st);
+    CK(cudaGetLastError());
+  } else if (tdst && want.raw) {
     Tmp scr;
     TRY(oz_room(c, scr, (size_t)n_cta * max_m * max_m * sizeof(double)));
     launch_oz_raw((const OzPair*)pr.p, np, max_m, (double*)scr.p, n_cta, c->st);
@@ -2588,10 +2726,6 @@ int osvmp2_mbe3_fragments(const double* r_occ, int32_t n_occ, double r2, double 
 // Mixed form: the overlaps Sigma_(lo,hi) = U_lo^T U_hi of every pair couple that
 // a coupling term of some fragment uses (pair p with the pairs (a,c), (c,b) of
 // its fragment), each computed once on the tensor cores from the U slices.
-struct SigmaStore {
-  Tmp data, off, hi, pos;
-  SigmaTable tab{};
-};
 int build_sigma_table(osvmp2_ctx* c, SigmaStore& ss) {
   const int n = c->sys.n_occ, npairs = (int)c->K_h.size();
   std::vector<std::pair<int, int>> cps;
@@ -2624,6 +2758,9 @@ int build_sigma_table(osvmp2_ctx* c, SigmaStore& ss) {
     tot += (long long)c->r_h[cps[u].first] * c->r_h[cps[u].second];
   }
   for (int q = 0; q < npairs; q++) off[q + 1] += off[q];
+  ss.off_h = off;
+  ss.hi_h = hi;
+  ss.pos_h = pos;
   TRY(tmp_alloc(c, ss.data, (size_t)std::max<long long>(tot, 1) * sizeof(float)));
   TRY(tmp_alloc(c, ss.off, off.size() * sizeof(int)));
   TRY(tmp_alloc(c, ss.hi, std::max<size_t>(hi.size(), 1) * sizeof(int)));
@@ -2717,7 +2854,6 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
   TRY(tmp_alloc(c, d_out, nf * sizeof(FragOut)));
   TRY(tmp_alloc(c, d_cnt, sizeof(int)));
   const size_t per_cta = (prec == OSVMP2_MIXED) ? frag_mixed_scratch_doubles(max_m) : frag_scratch_doubles(max_m);
-  if (prec == OSVMP2_MIXED) TRY(tmp_alloc(c, d_scr, (size_t)n_cta * per_cta * sizeof(double)));
   CK(cudaMemcpyAsync(d_orbs.p, orbs_h.data(), orbs_h.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(d_order.p, order.data(), nf * sizeof(int), cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(d_w.p, w_h.data(), nf * sizeof(int), cudaMemcpyHostToDevice, c->st));
@@ -2749,6 +2885,38 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
     ph_begin(c, OSVMP2_PH_SIGMA);
     TRY(build_sigma_table(c, sig));
     ph_end(c, OSVMP2_PH_SIGMA, 0.0);
+    const std::pair<int, int> key{nf, max_m};
+    auto it = c->plans.find(key);
+    const bool known = it != c->plans.end();
+    SolvePlan plan;
+    if (known) plan = it->second;
+    else if (c->opts.no_autotune == 2) plan.ctas_per_sm = 3;
+    bool tune = !known && !c->opts.no_autotune;
+    std::vector<std::vector<int>> fo(nf);
+    for (int f = 0; f < nf; f++)
+      for (int u = 0; u < 3; u++)
+        if (c->frags[order[f]].orbs[u] >= 0) fo[f].push_back(c->frags[order[f]].orbs[u]);
+    OzWant want;
+    want.raw = false;
+    want.mx = &sig;
+    want.ctas_per_sm = &plan.ctas_per_sm;
+    want.tune = &tune;
+    want.tune_ms = &plan.ms;
+    ph_begin(c, OSVMP2_PH_K_FRAGSOLVE);
+    const int mx = oz_solve(c, fo, order, so, 0.0, (FragOut*)d_out.p, tdst, tstore ? toff->data() : nullptr, nullptr, want);
+    if (mx && mx != OZ_NO_ROOM) return mx;
+    if (!mx) {
+      if (!known) {
+        plan.tuned = !c->opts.no_autotune;
+        it = c->plans.emplace(key, plan).first;
+      }
+      c->last_plan = it->second;
+      launch_weighted_sum((const FragOut*)d_out.p, (const int*)d_w.p, nf, c->scal_d, c->st);
+      ph_end(c, OSVMP2_PH_K_FRAGSOLVE, 0.0);
+    } else {                // without room for the batch: one CTA per fragment
+    ph_end(c, OSVMP2_PH_K_FRAGSOLVE, 0.0);
+    CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
+    TRY(tmp_alloc(c, d_scr, (size_t)n_cta * per_cta * sizeof(double)));
     const Tables tb = tables(c);
     auto solve = [&](const SolvePlan& pl, cudaStream_t st) {
       SolveOpts o = so;
@@ -2760,8 +2928,6 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
     };
     // autotuner: the first call for a (fragment count, largest pair order) times
     // every candidate plan on the full solve and keeps the fastest
-    const std::pair<int, int> key{nf, max_m};
-    auto it = c->plans.find(key);
     if (it == c->plans.end()) {
       SolvePlan best;
       if (c->opts.no_autotune == 2) best.ctas_per_sm = 3;
@@ -2828,6 +2994,7 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
       launch_weighted_sum((const FragOut*)d_out.p, (const int*)d_w.p, nf, c->scal_d, c->st);
     }
     ph_end(c, OSVMP2_PH_K_FRAGSOLVE, 0.0);
+    }
   } else {
     ph_begin(c, OSVMP2_PH_K_FRAGSOLVE);
     std::vector<std::vector<int>> fo(nf);

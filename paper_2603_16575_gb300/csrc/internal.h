@@ -168,6 +168,49 @@ void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool fi
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
                         double* e_prev, int* done, int* left, FragOut* out, const int* out_id, cudaStream_t st);
 void launch_oz_raw(const OzPair* pairs, int n_pairs, int max_m, double* scratch, int n_cta, cudaStream_t st);
+// Mixed form (solve_mx.cu): Y and C are double-float pairs in the same storage, coef of a segment the bits of a pair.
+struct MxPair {          // beside OzPair
+  const dfl* Kd;         // K~ and 1 / D [r][r]
+  const dfl* iD;
+  const float* Sh;
+  const float* Gh;
+  float* P;              // [r][r], zero until first formed
+};
+struct MxSigma {         // digits of S (rl x rh) and of its transpose
+  const float* S;
+  int rl, rh;
+  oz::Mat lo, hi;
+};
+struct MxTable {
+  int r, pad;
+  double fij;
+  const double* Kt;
+  const double* et;
+  dfl* Kd;
+  dfl* iD;
+};
+void launch_mx_sigma(const MxSigma* jobs, int n, int max_r, int ld, long long rows, uint16_t* D, int n_cta,
+                     cudaStream_t st);
+void launch_mx_tables(const MxTable* jobs, int n, cudaStream_t st);
+void launch_mx_leftover(const OzPair* pairs, const MxPair* mp, int n, const int* done, const int* refresh, int max_r,
+                        float* scratch, int n_cta, cudaStream_t st);
+void launch_mx_update(const OzPair* pairs, const MxPair* mp, int n, const int* done, bool first, int max_r, int ld,
+                      long long rows, uint16_t* D, int* ex, int* exW, double* pe, double* pu, int n_cta,
+                      cudaStream_t st);
+void launch_mx_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, int it,
+                        double* e_prev, double* scale, double* drift, int* refresh, int* done, int* left, FragOut* out,
+                        const int* out_id, cudaStream_t st);
+void launch_mx_store(const OzPair* pairs, int n, cudaStream_t st);
+// W digits under the codes eP of the pairs (job.o_e; Y's code eY[job.ld_out], coefficient job.s), and C from them.
+int launch_mx_w(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                const int* skip, uint16_t* D, int ld, long long rows, const int* eY, const int* eP, int* err,
+                cudaStream_t st);
+int launch_mx_c(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                const int* skip, const int* eP, int* err, cudaStream_t st);
+struct MxBound {         // a term of a pair: id of its Y matrix, exponent of its coefficient (|c| < 2^e)
+  int ver, e;
+};
+void launch_mx_bounds(const int* term0, const MxBound* terms, int n_pairs, const int* exW, int* eP, cudaStream_t st);
 struct OzDf {            // dE/df of a fragment of nc <= 3 orbitals
   int nc, pair0, out;    // its pairs; fragment index of the result
   int pad;

@@ -205,7 +205,7 @@ void launch_oz_float(const double* x, size_t n, float* y, cudaStream_t st) {
 
 // out[row][col] (row-major), added to what is there when job.s = 1
 struct OzEpiRow {
-  static constexpr bool kWarp = false, kDigits = false, kPair = false;
+  static constexpr bool kWarp = false, kDigits = false, kPair = false, kLong = false;
   __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     double* o = static_cast<double*>(jb.out) + (size_t)(jb.m0 + r) * jb.ld_out + jb.n0 + c0;
 #pragma unroll
@@ -216,7 +216,7 @@ struct OzEpiRow {
 // Mixed form.  G = U^T B with the row (aux) index innermost, as a normalised FP32 pair: the leading part to
 // out[col][row], the remainder lo_shift floats further on.
 struct OzEpiG {
-  static constexpr bool kWarp = false, kDigits = false, kPair = true;
+  static constexpr bool kWarp = false, kDigits = false, kPair = true, kLong = false;
   long long lo_shift;
   __device__ __forceinline__ void pairs(const oz::Job& jb, int r, int c0, const float (&h)[oz::DCOL],
                                         const float (&l)[oz::DCOL]) const {
@@ -233,7 +233,7 @@ struct OzEpiG {
 // out[row][col], FP64 (K~) or FP32 (Sigma)
 template <class T>
 struct OzEpiPair {
-  static constexpr bool kWarp = false, kDigits = false, kPair = true;
+  static constexpr bool kWarp = false, kDigits = false, kPair = true, kLong = false;
   __device__ __forceinline__ void pairs(const oz::Job& jb, int r, int c0, const float (&h)[oz::DCOL],
                                         const float (&l)[oz::DCOL]) const {
     T* o = static_cast<T*>(jb.out) + (size_t)(jb.m0 + r) * jb.ld_out + jb.n0 + c0;
@@ -244,7 +244,7 @@ struct OzEpiPair {
 };
 // T[a][b] = T[b][a] = v / (e_a + e_b - s) for a >= b; out = T_i, s = 2 f_ii
 struct OzEpiT {
-  static constexpr bool kWarp = false, kDigits = false, kPair = false;
+  static constexpr bool kWarp = false, kDigits = false, kPair = false, kLong = false;
   const double* e_vir;
   __device__ __forceinline__ void operator()(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     const int a = jb.m0 + r;
@@ -262,9 +262,75 @@ struct OzEpiT {
   }
 };
 
-// The same from FP32 pairs (mixed form).
+// Mixed amplitude iterations.  Sigma has the exponent 1 (|x| <= 1 + rounding), Y and W one exponent a matrix.
+// W: the digits of c Sigma op(Y)^T under the exponent code eP[o_e] of its pair; c = job.s, Y's code eY[job.ld_out].
+struct OzEpiW {
+  static constexpr bool kWarp = false, kDigits = false, kPair = true, kLong = true;
+  static constexpr int NS = oz::MXSOLVE, T = 7 + 8 * (NS - 1);
+  uint16_t* D;
+  int ld;
+  size_t slice;
+  const int *eY, *eP;
+  struct Scale {
+    float ch, cl;          // c 2^(exponents) as a pair: the fixed-point number per unit of the first level
+  };
+  __device__ __forceinline__ Scale scale(const oz::Job& jb) const {
+    const int ey = eY[jb.ld_out], ep = eP[jb.o_e];
+    if (ey < oz::EX_ZERO / 2 || ep < oz::EX_ZERO / 2 || ey > oz::EX_NAN / 2 || ep > oz::EX_NAN / 2) return Scale{0.f, 0.f};
+    const int x = T - ep + 1 + ey - 14;                // |c v| 2^x < 2^T
+    const float h = (float)jb.s, l = (float)(jb.s - (double)h);
+    const float s0 = __int_as_float(((x >> 1) + 127) << 23), s1 = __int_as_float((x - (x >> 1) + 127) << 23);
+    return Scale{h * s0 * s1, l * s0 * s1};
+  }
+  __device__ __forceinline__ void tile(const oz::Job& jb, const Scale& sc, int r, int c0, const float (&vh)[oz::DCOL],
+                                       const float (&vl)[oz::DCOL]) const {
+    uint16_t* o = D + ((size_t)jb.o_row + jb.m0 + r) * ld + jb.n0 + c0;
+    const bool tail = c0 + oz::DCOL >= jb.n_valid && ((jb.n0 + c0) & 16) == 0;   // also clears the rest of a k-block
+    int f[oz::DCOL];
+#pragma unroll
+    for (int u = 0; u < oz::DCOL; u++) {
+      const float p = vh[u] * sc.ch;
+      float e = fmaf(vh[u], sc.ch, -p);
+      e = fmaf(vh[u], sc.cl, e);
+      e = fmaf(vl[u], sc.ch, e);
+      const int top = __float2int_rn(p);
+      f[u] = c0 + u < jb.n_valid ? top + __float2int_rn((p - (float)top) + e) : 0;
+    }
+#pragma unroll
+    for (int h = 0; h < oz::DCOL / 8; h++)
+#pragma unroll
+      for (int s = NS - 1; s >= 0; s--) {
+        uint4 w;
+        w.x = oz::digit_pair32(f[8 * h], f[8 * h + 1], s);
+        w.y = oz::digit_pair32(f[8 * h + 2], f[8 * h + 3], s);
+        w.z = oz::digit_pair32(f[8 * h + 4], f[8 * h + 5], s);
+        w.w = oz::digit_pair32(f[8 * h + 6], f[8 * h + 7], s);
+        *reinterpret_cast<uint4*>(o + s * slice + 8 * h) = w;
+        if (tail) *reinterpret_cast<uint4*>(o + s * slice + 16 + 8 * h) = make_uint4(0, 0, 0, 0);
+      }
+  }
+};
+// C = sum Sigma W as double-float pairs, out[row][col].
+struct OzEpiC {
+  static constexpr bool kWarp = false, kDigits = false, kPair = true, kLong = true;
+  const int* eP;
+  using Scale = float;
+  __device__ __forceinline__ float scale(const oz::Job& jb) const {
+    const int ep = eP[jb.o_e];
+    if (ep > oz::EX_NAN / 2) return __int_as_float(0x7FC00000);
+    return ep < -100 ? 0.f : __int_as_float((1 + ep - 14 + 127) << 23);
+  }
+  __device__ __forceinline__ void tile(const oz::Job& jb, float sc, int r, int c0, const float (&vh)[oz::DCOL],
+                                       const float (&vl)[oz::DCOL]) const {
+    dfl* o = static_cast<dfl*>(jb.out) + (size_t)(jb.m0 + r) * jb.ld_out + jb.n0 + c0;
+#pragma unroll
+    for (int u = 0; u < oz::DCOL; u++)
+      if (c0 + u < jb.n_valid) o[u] = df_norm(vh[u] * sc, vl[u] * sc);
+  }
+};
+// T_ii from FP32 pairs (mixed form).
 struct OzEpiTPair {
-  static constexpr bool kWarp = false, kDigits = false, kPair = true;
+  static constexpr bool kWarp = false, kDigits = false, kPair = true, kLong = false;
   const double* e_vir;
   __device__ __forceinline__ void pairs(const oz::Job& jb, int r, int c0, const float (&h)[oz::DCOL],
                                         const float (&l)[oz::DCOL]) const {
@@ -279,7 +345,7 @@ struct OzEpiTPair {
 // next multiple of 16 are written as zeros (up to 32 by the lanes of the last column group).
 template <int NS>
 struct OzEpiDigits {
-  static constexpr bool kWarp = false, kDigits = true, kPair = false;
+  static constexpr bool kWarp = false, kDigits = true, kPair = false, kLong = false;
   static constexpr int T = 7 + 8 * (NS - 1);
   uint16_t* D;
   int ld;
@@ -311,7 +377,7 @@ struct OzEpiDigits {
 // <2 Y - Y^T, D> of the tile's part of D (never stored): Y = the r x r matrix at job.out (r = ld_out), one
 // partial sum per drain warp at parts + 16 job.o_row.
 struct OzEpiDot {
-  static constexpr bool kWarp = true, kDigits = false, kPair = false;
+  static constexpr bool kWarp = true, kDigits = false, kPair = false, kLong = false;
   double* parts;
   __device__ __forceinline__ void warp(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
     const double* Y = static_cast<const double*>(jb.out);
@@ -351,7 +417,7 @@ int run(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs,
   if (cudaFuncSetAttribute(oz::k_oz<NS, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess) return -1;
   oz::OzMaps tm;
   for (int u = 0; u < 2; u++)
-    if (!make_digit_map(&tm.a[u], A, NS, oz::BM >> (1 - u)) || !make_digit_map(&tm.b[u], B, NS, oz::BN >> (1 - u))) return -1;
+    if (!make_digit_map(&tm.a[u], A, NS, oz::BM >> (1 - u)) || !make_digit_map(&tm.b[u], B, NS, oz::tile_cols(NS) >> (1 - u))) return -1;
   oz::k_oz<NS, Epi><<<tc::persistent_grid(n_jobs), oz::NTHREADS, SMEM, st>>>(tm, A.ex, B.ex, jobs, n_jobs, segs, skip,
                                                                              err, epi);
   note_launch(1);
@@ -366,6 +432,15 @@ int launch_oz_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, 
 int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                      const int* skip, uint16_t* D, int ld, long long rows, const int* exW, int* err, cudaStream_t st) {
   return run<oz::NSL>(A, B, jobs, n_jobs, segs, skip, err, OzEpiDigits<oz::NSL>{D, ld, (size_t)rows * ld, exW}, st);
+}
+int launch_mx_w(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                const int* skip, uint16_t* D, int ld, long long rows, const int* eY, const int* eP, int* err,
+                cudaStream_t st) {
+  return run<oz::MXSOLVE>(A, B, jobs, n_jobs, segs, skip, err, OzEpiW{D, ld, (size_t)rows * ld, eY, eP}, st);
+}
+int launch_mx_c(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                const int* skip, const int* eP, int* err, cudaStream_t st) {
+  return run<oz::MXSOLVE>(A, B, jobs, n_jobs, segs, skip, err, OzEpiC{eP}, st);
 }
 int launch_mx_g(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                 long long lo_shift, int* err, cudaStream_t st) {

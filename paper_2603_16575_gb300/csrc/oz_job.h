@@ -6,10 +6,13 @@ namespace osv {
 namespace oz {
 
 constexpr int BM = 128;       // tile rows = TMEM lanes = MMA M
-constexpr int BN = 64;        // max tile columns (MMA N <= 64)
+constexpr int BN = 64;        // most columns of a tile with eight or five slices (level accumulators: 512 columns)
+constexpr int BN4 = 128;      // and with four
+constexpr __host__ __device__ int tile_cols(int ns) { return ns == 4 ? BN4 : BN; }
 constexpr int BK = 32;        // k per stage (one 64-byte swizzle row of BF16)
 constexpr int NSL = 8;        // slices per operand
-constexpr int MXSL = 5;       // and in the mixed form's pair build
+constexpr int MXSL = 5;       // in the mixed form's pair build
+constexpr int MXSOLVE = 4;    // and in its amplitude iterations
 constexpr int CHUNK = 256;    // k-extent that shares one power-of-two scale per row
 constexpr int EX_ZERO = -(1 << 20);   // chunk exponent of an all-zero chunk
 constexpr int EX_NAN = 1 << 20;       // and of one that holds a NaN or an Inf

@@ -57,6 +57,14 @@ __device__ __forceinline__ uint32_t digit_pair(long long& f0, long long& f1, int
   return bf16_of_int(d0) | (bf16_of_int(d1) << 16);
 }
 
+// The same for 32-bit fixed-point numbers (four slices).
+__device__ __forceinline__ uint32_t digit_pair32(int& f0, int& f1, int s) {
+  const int d0 = s ? (int)(signed char)(f0 & 255) : f0, d1 = s ? (int)(signed char)(f1 & 255) : f1;
+  f0 = (f0 >> 8) + ((f0 >> 7) & 1);
+  f1 = (f1 >> 8) + ((f1 >> 7) & 1);
+  return bf16_of_int(d0) | (bf16_of_int(d1) << 16);
+}
+
 // One row-chunk held by a warp: lane l has elements k = 64 u + 2 l + {0, 1}, u = 0 .. 3 (zero past the
 // end).  Writes the digits at dst + s * slice + k for k < kv and returns the exponent code.
 template <int NS>

@@ -12,7 +12,7 @@
 //    e_m the smallest exponent with max_k |A[m][k]| < 2^e_m (oz_split.cuh): 63 fractional
 //    bits, ten more than the mantissa, so a value keeps its full mantissa down to 2^-10 of
 //    the row's largest in the chunk and an absolute 2^(e_m - 64) below that.
-//  * The mixed form takes five slices (39 bits, 15 products).
+//  * The mixed form takes five slices (39 bits, 15 products) or four (31 bits, 10 products).
 //  * A product a_s b_t of level l = s + t is at most 2^14, a chunk sum of one slice pair at
 //    most 2^22, and a sum of up to four pairs (levels 2-5) stays an exact FP32 integer
 //    whatever the accumulator's rounding; levels 6-9 have 5 to 8 pairs, whose sums pass 2^24
@@ -57,9 +57,8 @@ namespace osv {
 namespace oz {
 
 constexpr int A_TILE = BM * BK * 2;          // 8 KB per A slice tile
-constexpr int B_TILE = BN * BK * 2;          // 4 KB per B slice tile
 constexpr int NDRAIN = 16;                   // drain warps
-constexpr int DCOL = BN * 4 / NDRAIN;        // columns of one: four warps share a TMEM lane quarter
+constexpr int DCOL = 16;                     // columns read at a time; four warps share a TMEM lane quarter
 constexpr int NTHREADS = 64 + 32 * NDRAIN;
 constexpr int KBC = CHUNK / BK;              // k-blocks of a full chunk
 constexpr int TMEM_COLS = 512;
@@ -74,10 +73,10 @@ struct OzMaps {
 
 template <int NS>
 struct Cfg {
-  static constexpr int STAGE = NS * (A_TILE + B_TILE);
+  static constexpr int BN = tile_cols(NS);
+  static constexpr int STAGE = NS * (A_TILE + BN * BK * 2);
   static constexpr int NSTAGE = NS == 8 ? 2 : 3;
   static constexpr int SMEM = NSTAGE * STAGE + 1024;   // + slack for 1024-byte alignment
-  static constexpr int NBUF = 1;                       // sets of NS level accumulators in the 512 TMEM columns
   static constexpr int UNIT = 14 + 8 * (NS < 6 ? NS - 1 : 5);   // the joined integer is in units of 2^(e_m + e_n - UNIT)
 };
 
@@ -91,8 +90,11 @@ __device__ __forceinline__ double oz_fma(long long v, int x, double coef, double
   return fma(coef, (double)v * pow2(x / 2) * pow2(x - x / 2), acc);
 }
 
-// Columns of a tile's level accumulators, and rows of its B slices in shared memory: BN, or half of it.
-__device__ __forceinline__ int width(const Job& jb) { return jb.n_valid <= BN / 2 ? BN / 2 : BN; }
+// Columns of a tile's level accumulators, and rows of its B slices in shared memory: those of the widest, or half.
+template <int NS>
+__device__ __forceinline__ int width(const Job& jb) {
+  return jb.n_valid <= tile_cols(NS) / 2 ? tile_cols(NS) / 2 : tile_cols(NS);
+}
 // Rows of its A slices in shared memory: with half of BM the MMAs read the next slice as the rows past the end.
 __device__ __forceinline__ int height(const Job& jb) { return jb.m_valid <= BM / 2 ? BM / 2 : BM; }
 
@@ -144,15 +146,18 @@ __device__ __forceinline__ void pair_add(float vh, float vl, int x, float& ah, f
 // or, when Epi::kPair (NS <= 5), epi.pairs(job, row, col0, ah, al) with the sum as unnormalised FP32 pairs (the
 // segments' coef is 1): the mixed form's products.  The FP64 drain takes three operations of an FP64 pipe that
 // issues one warp in 64 cycles per element and chunk, more than the 15 products of a chunk; pairs take none.
+// Epi::kLong: exponents are the epilogue's (one for each operand matrix), all segments add up in tensor memory (K up to
+// ~1000: exact but for roundings at 2^-24 of a level in the later ones) and are read once, as pairs in units of the
+// first level: epi.tile(job, epi.scale(job), row, col0, vh, vl) for the rows and columns of the tile.
 template <int NS, class Epi>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_oz(const __grid_constant__ OzMaps tm, const int* __restrict__ exA,
          const int* __restrict__ exB, const Job* __restrict__ jobs, int n_jobs, const Seg* __restrict__ segs,
          const int* __restrict__ skip, int* err, Epi epi) {
   using C = Cfg<NS>;
-  constexpr int NST = C::NSTAGE, NB = C::NBUF;
+  constexpr int NST = C::NSTAGE, BN = C::BN;
   extern __shared__ uint8_t dsm[];
-  __shared__ __align__(8) uint64_t bar_full[NST], bar_empty[NST], bar_accf[NB * NS], bar_acce[NB * NS];
+  __shared__ __align__(8) uint64_t bar_full[NST], bar_empty[NST], bar_accf[NS], bar_acce[NS];
   __shared__ uint32_t s_tmem;
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = tc::su32(sm);
@@ -168,7 +173,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       tc::mbar_init(&bar_full[s], 1);
       tc::mbar_init(&bar_empty[s], 1);
     }
-    for (int l = 0; l < NB * NS; l++) {
+    for (int l = 0; l < NS; l++) {
       tc::mbar_init(&bar_accf[l], 1);
       tc::mbar_init(&bar_acce[l], NDRAIN);
     }
@@ -192,7 +197,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
         const Job jb = jobs[tile];
         if (jb.skip >= 0 && skip[jb.skip]) continue;
-        const int h = height(jb), w = width(jb);
+        const int h = height(jb), w = width<NS>(jb);
         const uint32_t bytes = NS * (h + w) * BK * 2;
         const CUtensorMap *ma = &tm.a[h == BM], *mb = &tm.b[w == BN];
         for (int q = 0; ok && q < jb.nseg; q++) {
@@ -224,22 +229,25 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int tile = blockIdx.x; ok && tile < n_jobs; tile += gridDim.x) {
         const Job jb = jobs[tile];
         if (jb.skip >= 0 && skip[jb.skip]) continue;
-        const bool wide = width(jb) == BN, tall = height(jb) == BM;
+        const bool wide = width<NS>(jb) == BN, tall = height(jb) == BM;
         for (int q = 0; ok && q < jb.nseg; q++) {
           const int K = segs[jb.seg0 + q].K, nkb = (K + BK - 1) / BK;
           for (int c = 0; c < nkb; c++, g++) {
-            const int s = (int)(g % NST), b = (int)(ch % NB) * NS;
-            const bool first = (c % KBC) == 0, last = (c % KBC) == KBC - 1 || c == nkb - 1;
+            const int s = (int)(g % NST);
+            bool first = (c % KBC) == 0, last = (c % KBC) == KBC - 1 || c == nkb - 1;
+            if constexpr (Epi::kLong) {
+              first = q == 0 && c == 0;
+              last = q == jb.nseg - 1 && c == nkb - 1;
+            }
             const int nks = K - c * BK > 16 ? 2 : 1;             // 16-wide steps that hold elements
             ok = tc::mbar_wait(tc::su32(&bar_full[s]), (uint32_t)((g / NST) & 1));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
             const uint32_t st = sbase + s * C::STAGE;
             const uint64_t da = tc::desc_sw64(st), db = tc::desc_sw64(st + NS * A_TILE);
-            const uint32_t dcol = tmem + (uint32_t)(b * BN);
             auto level_free = [&](int l) {
-              if (ch < NB) return true;
-              const bool f = tc::mbar_wait(tc::su32(&bar_acce[b + l]), (uint32_t)((ch / NB - 1) & 1));
+              if (ch < 1) return true;
+              const bool f = tc::mbar_wait(tc::su32(&bar_acce[l]), (uint32_t)((ch - 1) & 1));
               asm volatile("tcgen05.fence::after_thread_sync;");
               return f;
             };
@@ -251,7 +259,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             for (int ks = 0; ks < nks; ks++) {
               const bool fin = last && ks == nks - 1;
               auto go = [&](auto W, auto H) {
-                return issue<NS, W, H>(da, db, dcol, ks, first && ks == 0, level_free, fin ? &bar_accf[b] : nullptr);
+                return issue<NS, W, H>(da, db, tmem, ks, first && ks == 0, level_free, fin ? bar_accf : nullptr);
               };
               if (wide)
                 ok = tall ? go(std::integral_constant<int, BN>{}, std::integral_constant<int, BM>{})
@@ -278,7 +286,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
   } else {                                                       // ---- drain + epilogue
     const int quad = warp & 3;                                   // TMEM lane quarter of this warp
-    const int col0 = ((warp - 2) >> 2) * DCOL;                   // and its columns
+    const int col0 = ((warp - 2) >> 2) * (BN / 4);               // and its columns
     const uint32_t lcol = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)col0;
     const int row = 32 * quad + lane;
     long long ch = 0;
@@ -286,7 +294,47 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const Job jb = jobs[tile];
       if (jb.skip >= 0 && skip[jb.skip]) continue;
       const bool live = col0 < jb.n_valid && 32 * quad < jb.m_valid;   // warp-uniform
-      const int w = width(jb);
+      const int w = width<NS>(jb);
+      if constexpr (Epi::kLong) {
+        // one sum over all segments, read DCOL columns at a time
+        typename Epi::Scale sc = epi.scale(jb);
+#pragma unroll
+        for (int g = 0; g < BN / 4; g += DCOL) {
+          const bool here = col0 + g < jb.n_valid && 32 * quad < jb.m_valid;   // warp-uniform
+          float vh[DCOL], vl[DCOL];
+#pragma unroll
+          for (int l = 0; l < NS; l++) {
+            if (g == 0) {
+              ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::su32(&bar_accf[l]), (uint32_t)(ch & 1)));
+              if (!ok) break;
+              asm volatile("tcgen05.fence::after_thread_sync;");
+            }
+            uint32_t x[DCOL];
+            if (here) {
+              OSV_TMEM_LD16(lcol + l * w + g, x);
+              asm volatile("tcgen05.wait::ld.sync.aligned;");
+            }
+            if (g == BN / 4 - DCOL) {
+              asm volatile("tcgen05.fence::before_thread_sync;");
+              __syncwarp();
+              if (lane == 0) tc::mbar_arrive(&bar_acce[l]);
+            }
+            if (!here) continue;
+#pragma unroll
+            for (int u = 0; u < DCOL; u++) {
+              const float y = __uint_as_float(x[u]) * __int_as_float((127 - 8 * l) << 23);
+              if (l == 0) { vh[u] = y; vl[u] = 0.f; }
+              else if (l == 1) two_sum(vh[u], y, vh[u], vl[u]);
+              else vl[u] += y;
+            }
+          }
+          if (!ok) break;
+          if (here && row < jb.m_valid) epi.tile(jb, sc, row, col0 + g, vh, vl);
+        }
+        if (!ok) break;
+        ch++;
+        continue;
+      }
       double acc[Epi::kDigits || Epi::kPair ? 1 : DCOL];
       float ah[Epi::kPair ? DCOL : 1], al[Epi::kPair ? DCOL : 1];
       long long f[Epi::kDigits ? DCOL : 1];
@@ -309,8 +357,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int* eb_p = exB + sg->b.eb + (long long)(jb.n0 + min(col0 + (lane & (DCOL - 1)), jb.n_valid - 1)) * sg->b.es;
         const double coef = sg->coef;
         for (int c = 0; ok && c < nch; c++, ch++) {
-          const int b = (int)(ch % NB) * NS;
-          const uint32_t ph = (uint32_t)((ch / NB) & 1);
+          const uint32_t ph = (uint32_t)(ch & 1);
           const int ea = ea_p[c] - C::UNIT, eb = eb_p[c];
           long long v[Epi::kPair ? 1 : DCOL];
           float vh[Epi::kPair ? DCOL : 1], vl[Epi::kPair ? DCOL : 1];
@@ -321,17 +368,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           }
 #pragma unroll
           for (int l = 0; l < NS; l++) {
-            ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::su32(&bar_accf[b + l]), ph));
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::su32(&bar_accf[l]), ph));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
             uint32_t x[DCOL];
             if (live) {
-              OSV_TMEM_LD16(lcol + b * BN + l * w, x);
+              OSV_TMEM_LD16(lcol + l * w, x);
               asm volatile("tcgen05.wait::ld.sync.aligned;");
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&bar_acce[b + l]);
+            if (lane == 0) tc::mbar_arrive(&bar_acce[l]);
             if (!live) continue;
 #pragma unroll
             for (int u = 0; u < DCOL; u++) {
@@ -374,6 +421,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (!ok) break;
       if constexpr (Epi::kDigits) {
         if (row < jb.m_valid && live) epi.digits(jb, row, col0, f);
+      } else if constexpr (Epi::kLong) {                            // (stored above)
       } else if constexpr (Epi::kPair) {
         if (row < jb.m_valid && live) epi.pairs(jb, row, col0, ah, al);
       } else if constexpr (Epi::kWarp) {
