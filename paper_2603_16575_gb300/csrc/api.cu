@@ -934,11 +934,11 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
     Tmp u0, sq, scr, pj, mj;
     TRY(oz_room(c, u0, u0sz * sizeof(double)));
     TRY(oz_room(c, sq, 3 * sqsz * sizeof(double)));
-    TRY(oz_room(c, scr, (size_t)n_cta * max_m * max_m * sizeof(double)));
+    TRY(oz_room(c, scr, (size_t)n_cta * max_r * max_r * sizeof(double)));
     TRY(oz_room(c, pj, (b1 - b0) * sizeof(OzPolish)));
     TRY(oz_room(c, mj, (b1 - b0) * sizeof(OzMat)));
-    OzMats xs(max_n), uc(nv), ue(nv), ur(max_r), ie(max_r);
-    OzList lu, ls, lf, lo;
+    OzMats xs(max_n), uc(nv), ue(nv), ur(max_r), ie(max_r), xm(max_r);
+    OzList lu, ls, lf, lo, lx;
     std::vector<OzPolish> pol;
     std::vector<OzMat> fin;
     size_t uo = 0, so = 0;
@@ -966,8 +966,10 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
       ue.add(U0, r, r, nv);
       ls.product(uc.mat(a), r, uc.mat(a), r, nv, S1, r);
       lf.product(ue.mat(a), r, uc.mat(a), r, nv, F1, r);
-      pol.push_back(OzPolish{m, r, S1, F1, IE, X, c->et_h[id]});
-      lo.product(ur.mat(ur.add(U0, nv, r, r)), nv, ie.mat(ie.add(IE, r, r, r)), r, r, U0, r);
+      pol.push_back(OzPolish{r, 0, S1, F1, IE, c->et_h[id]});
+      const int ix = ie.add(IE, r, r, r);
+      lo.product(ur.mat(ur.add(U0, nv, r, r)), nv, ie.mat(ix), r, r, U0, r);
+      lx.product(xm.mat(xm.add(X, m, m, r)), m, ie.mat(ix), r, r, X, m);
       const oz::Mat um{(int)row, (int)(row * nch), nch};
       fin.push_back(OzMat{U0, r, nv, nv, r, um});
       c->ud_mat[id] = um;
@@ -978,6 +980,7 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
     TRY(oz_mats_room(c, ue));
     TRY(oz_mats_room(c, ur));
     TRY(oz_mats_room(c, ie));
+    TRY(oz_mats_room(c, xm));
     TRY(oz_mats_fill(c, xs, nullptr, false));
     TRY(oz_run(c, q.op, xs.op, lu));
     CK(cudaMemcpyAsync(pj.p, pol.data(), pol.size() * sizeof(OzPolish), cudaMemcpyHostToDevice, c->st));
@@ -987,10 +990,12 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
       TRY(oz_mats_fill(c, ur, nullptr, true));
       TRY(oz_run(c, uc.op, uc.op, ls));
       TRY(oz_run(c, ue.op, uc.op, lf));
-      launch_oz_polish((const OzPolish*)pj.p, (int)pol.size(), max_m, (double*)scr.p, n_cta, c->st);
+      TRY(oz_mats_fill(c, xm, nullptr, true));
+      launch_oz_polish((const OzPolish*)pj.p, (int)pol.size(), max_r, (double*)scr.p, n_cta, c->st);
       CK(cudaGetLastError());
       TRY(oz_mats_fill(c, ie, nullptr, false));
       TRY(oz_run(c, ur.op, ie.op, lo));
+      TRY(oz_run(c, xm.op, ie.op, lx));
     }
     CK(cudaMemcpyAsync(mj.p, fin.data(), fin.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
     launch_oz_mats((const OzMat*)mj.p, (int)fin.size(), mr, nv, nullptr, false, oz::NSL, ld, rows, (uint16_t*)dmem.p, (int*)emem.p,
@@ -1003,6 +1008,42 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
   for (Tmp* t : {&dmem, &emem}) {
     c->ud_alloc.push_back(t->p);
     t->p = nullptr;
+  }
+  return 0;
+}
+
+// FP64 form: K~ = X^T (K X) of the listed pairs, in batches whose temporaries fit a fixed budget.
+int oz_ktilde(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, int max_m) {
+  const int n = c->sys.n_occ;
+  for (size_t b0 = 0; b0 < newp.size();) {
+    OzMats ks(max_m), xs(max_m), ws(max_m);
+    OzList l1, l2;
+    size_t b1 = b0, wsz = 0;
+    for (size_t held = 0; b1 < newp.size() && (b1 == b0 || held < ((size_t)2 << 30)); b1++) {
+      const size_t m = pair_dim_h(c, newp[b1].first, newp[b1].second);
+      held += 3 * oz_digit_bytes(m, max_m);
+      wsz += m * m;
+    }
+    Tmp w;
+    TRY(oz_room(c, w, std::max<size_t>(1, wsz) * sizeof(double)));
+    size_t off = 0;
+    for (size_t t = b0; t < b1; t++) {
+      const int id = c->pair_id[(size_t)newp[t].first * n + newp[t].second], m = c->m_h[id], r = c->r_h[id];
+      double* W = (double*)w.p + off;       // [m][r]
+      off += (size_t)m * m;
+      const int x = xs.add(c->X_h[id], r, m, m);
+      l1.product(ks.mat(ks.add(c->K_h[id], m, m, m)), m, xs.mat(x), r, m, W, r);
+      l2.product(xs.mat(x), r, ws.mat(ws.add(W, r, r, m)), r, m, c->Kt_h[id], r);
+    }
+    TRY(oz_mats_room(c, ks));
+    TRY(oz_mats_room(c, xs));
+    TRY(oz_mats_room(c, ws));
+    TRY(oz_mats_fill(c, ks, nullptr, true));
+    TRY(oz_mats_fill(c, xs, nullptr, false));
+    TRY(oz_run(c, ks.op, xs.op, l1));
+    TRY(oz_mats_fill(c, ws, nullptr, false));
+    TRY(oz_run(c, xs.op, ws.op, l2));
+    b0 = b1;
   }
   return 0;
 }
@@ -1067,6 +1108,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
         p.ver[0] = p.ver[1] = p.ver[2] = -1;
         p.fij = c->f_h[(size_t)i * n + i] + c->f_h[(size_t)j * n + j];
         p.Kt = c->Kt_h[id];
+        p.iD = nullptr;
         p.et = c->et_h[id];
         p.X = c->X_h[id];
         p.T = tdst ? tdst + toff[out_id[f]] + toff_p : nullptr;
@@ -1224,6 +1266,28 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
       p.C = (double*)yc.p + ysz + off;
       off += (size_t)p.r * p.r;
     }
+  }
+  Tmp idm, idj;
+  if (!mx) {                             // 1 / D of the pairs in use
+    std::unordered_map<int, size_t> at;
+    std::vector<OzTable> tj;
+    size_t tsz = 0;
+    for (int p = 0; p < np; p++)
+      if (at.emplace(pid[p], tsz).second) {
+        tj.push_back(OzTable{pairs[p].r, 0, pairs[p].fij, pairs[p].et, nullptr});
+        tsz += (size_t)pairs[p].r * pairs[p].r;
+      }
+    TRY(oz_room(c, idm, tsz * sizeof(double)));
+    TRY(oz_room(c, idj, tj.size() * sizeof(OzTable)));
+    size_t off = 0;
+    for (OzTable& t : tj) {
+      t.iD = (double*)idm.p + off;
+      off += (size_t)t.r * t.r;
+    }
+    for (int p = 0; p < np; p++) pairs[p].iD = (double*)idm.p + at[pid[p]];
+    CK(cudaMemcpyAsync(idj.p, tj.data(), tj.size() * sizeof(OzTable), cudaMemcpyHostToDevice, c->st));
+    launch_oz_tables((const OzTable*)idj.p, (int)tj.size(), c->st);
+    CK(cudaGetLastError());
   }
   CK(cudaMemcpyAsync(pr.p, pairs.data(), np * sizeof(OzPair), cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(p0.p, pair0.data(), pair0.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
@@ -1999,8 +2063,10 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
       CK(cudaStreamSynchronize(c->st));
     }
     ph_end(c, OSVMP2_PH_PRECOND, 0.0);
+    oz = oz_ktilde(c, newp, max_m);
+    if (oz && oz != OZ_NO_ROOM) return oz;
     std::vector<KtJob> ktj;
-    for (size_t q = 0; q < kj.size(); q++) ktj.push_back(KtJob{kj[q].i, kj[q].j, c->Kt_h[c->pair_id[(size_t)kj[q].i * n + kj[q].j]]});
+    for (size_t q = 0; oz == OZ_NO_ROOM && q < kj.size(); q++) ktj.push_back(KtJob{kj[q].i, kj[q].j, c->Kt_h[c->pair_id[(size_t)kj[q].i * n + kj[q].j]]});
     Tmp jkt;
     TRY(tmp_alloc(c, jkt, ktj.size() * sizeof(KtJob)));
     CK(cudaMemcpyAsync(jkt.p, ktj.data(), ktj.size() * sizeof(KtJob), cudaMemcpyHostToDevice, c->st));
@@ -3388,15 +3454,22 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
   if (np) CK(cudaMemcpyAsync(d_kj.p, kj.data(), kj.size() * sizeof(RelaxKJob), cudaMemcpyHostToDevice, c->st));
   launch_relax_kpart(t, bs, (const RelaxKJob*)d_kj.p, np, (double*)kscr.p, n_cta_k, max_m, c->st);
   CK(cudaGetLastError());
-  // the rest per fragment, into one slot per (fragment, orbital)
+  // the rest per pair of a fragment (without room for that many slots: per fragment), into one slot per (job, orbital)
   std::vector<std::vector<RelaxGTerm>> gt(n);
-  size_t slot_total = 0;
+  size_t slot_total = 0, slot_pairs = 0;
   for (int f = 0; f < nf; f++)
     if (c->frags[f].weight != 0)
       for (int u = 0; u < 3; u++)
-        if (c->frags[f].orbs[u] >= 0) slot_total += (size_t)nv * c->n_osv[c->frags[f].orbs[u]];
+        if (c->frags[f].orbs[u] >= 0) {
+          const size_t one = (size_t)nv * c->n_osv[c->frags[f].orbs[u]];
+          const int no = c->frags[f].orbs[1] < 0 ? 1 : (c->frags[f].orbs[2] < 0 ? 2 : 3);
+          slot_total += one;
+          slot_pairs += no * one;
+        }
   Tmp slots, fscr, d_fj;
-  TRY(tmp_alloc(c, slots, std::max<size_t>(1, slot_total) * sizeof(double)));
+  const size_t most = c->opts.mem_cap_mib > 0 ? (size_t)c->opts.mem_cap_mib << 17 : (size_t)4 << 30;   // an eighth of a cap
+  const bool by_pair = slot_pairs * sizeof(double) <= most && !oz_room(c, slots, std::max<size_t>(1, slot_pairs) * sizeof(double));
+  if (!by_pair) TRY(tmp_alloc(c, slots, std::max<size_t>(1, slot_total) * sizeof(double)));
   std::vector<RelaxFragJob> fj;
   size_t so = 0;
   for (int f = 0; f < nf; f++) {
@@ -3407,14 +3480,27 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
     jb.c = (double)fr.weight;
     jb.T = tstore + toff[f];
     for (int u = 0; u < 3; u++)
-      if (fr.orbs[u] >= 0) {
-        const int x = fr.orbs[u];
-        jb.orbs[jb.no] = x;
-        jb.slot[jb.no] = (double*)slots.p + so;
-        gt[x].push_back(RelaxGTerm{jb.slot[jb.no], c->n_osv[x], 0});
-        so += (size_t)nv * c->n_osv[x];
-        jb.no++;
+      if (fr.orbs[u] >= 0) jb.orbs[jb.no++] = fr.orbs[u];
+    const int n_pair = jb.no * (jb.no + 1) / 2;
+    auto add_job = [&](int u0, int u1) {
+      RelaxFragJob p = jb;
+      p.u0 = u0;
+      p.u1 = u1;
+      for (int a = 0; a < jb.no; a++) {
+        bool has = false;
+        for (int x = 0, u = 0; x < jb.no; x++)
+          for (int y = x; y < jb.no; y++, u++) has |= u >= u0 && u < u1 && (x == a || y == a);
+        if (!has) continue;
+        p.slot[a] = (double*)slots.p + so;
+        gt[jb.orbs[a]].push_back(RelaxGTerm{p.slot[a], c->n_osv[jb.orbs[a]], 0});
+        so += (size_t)nv * c->n_osv[jb.orbs[a]];
       }
+      fj.push_back(p);
+    };
+    if (by_pair)
+      for (int u = 0; u < n_pair; u++) add_job(u, u + 1);
+    else
+      add_job(0, n_pair);
     double rows = 0.0;
     for (int a = 0; a < jb.no; a++) rows += c->n_osv[jb.orbs[a]];
     for (int a = 0; a < jb.no; a++)
@@ -3428,9 +3514,8 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
             fl += 4.0 * (mq * mq * m + mq * m * m);
           }
       }
-    fj.push_back(jb);
   }
-  // one CTA per fragment in flight, two per SM (112 registers x 256 threads each), their scratch
+  // one CTA per job in flight, two per SM (112 registers x 256 threads each), their scratch
   // within a quarter of the free memory
   const size_t scr_per = 8 * (size_t)std::max(max_m, 1) * std::max(max_m, 1) + (size_t)nv * std::max(max_m, 1);
   int n_cta_f = std::max(1, std::min((int)fj.size(), 2 * c->num_sms));

@@ -101,6 +101,8 @@ __device__ __forceinline__ void tile_mma_t(int M, int N, int K, int m0, int n0, 
   V* As = sm;             // [TK][TM]
   V* Bs = sm + TK * TM;   // [TK][TN]
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  // FP64: rows and columns of 16 past the end are skipped (an FMA holds the pipe for 64 cycles a warp)
+  const int mi = sizeof(V) == 8 ? (min(M - m0, TM) + 15) / 16 : 4, nj = sizeof(V) == 8 ? (min(N - n0, TN) + 15) / 16 : 4;
   for (int k0 = 0; k0 < K; k0 += TK) {
 #pragma unroll
     for (int t = 0; t < TM * TK / NT; t++) {
@@ -124,8 +126,11 @@ __device__ __forceinline__ void tile_mma_t(int M, int N, int K, int m0, int n0, 
       for (int j = 0; j < 4; j++) b[j] = Bs[k * TN + tx + 16 * j];
 #pragma unroll
       for (int i = 0; i < 4; i++)
+        if (sizeof(V) == 4 || i < mi) {
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+          for (int j = 0; j < 4; j++)
+            if (sizeof(V) == 4 || j < nj) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        }
     }
     __syncthreads();
   }
@@ -388,6 +393,7 @@ __device__ void cta_gemm_r(int M, int N, int K, double alpha, const VA& A, const
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int m0 = 0; m0 < M; m0 += TMR)
     for (int n0 = 0; n0 < N; n0 += TMR) {
+      const int mi = (min(M - m0, TMR) + 15) / 16, nj = (min(N - n0, TMR) + 15) / 16;   // 16s with elements
       double acc[R][R];
 #pragma unroll
       for (int i = 0; i < R; i++)
@@ -416,8 +422,11 @@ __device__ void cta_gemm_r(int M, int N, int K, double alpha, const VA& A, const
           for (int j = 0; j < R; j++) b[j] = Bs[k * TMR + tx + 16 * j];
 #pragma unroll
           for (int i = 0; i < R; i++)
+            if (i < mi) {
 #pragma unroll
-            for (int j = 0; j < R; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+              for (int j = 0; j < R; j++)
+                if (j < nj) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+            }
         }
         __syncthreads();
       }

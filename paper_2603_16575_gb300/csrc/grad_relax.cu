@@ -62,15 +62,16 @@ __global__ void __launch_bounds__(NT) k_relax_kpart(Tables t, BSrc bs, const Rel
   }
 }
 
-// ---- the rest, one CTA per fragment, in the OSV bases: with T~ = 2T - T^T,
+// ---- the rest, one CTA per pair of a fragment (or per fragment: pairs [u0, u1) of the job), in the OSV bases: with T~ = 2T - T^T,
 //   dP_u = c alpha [R_L P T~^T + R_L^T P T~]   (R_L: the residual without exchange)
 //        = diag(e) P_u (T S_uu T~^T + T^T S_uu T~) + P_u (T F_uu T~^T + T^T F_uu T~)
 //          + sum over (x, y) in {(k, j), (i, k)} of coef P_q (op(T_q) S_qu T~^T + op(T_q)^T S_qu T~)
 // (coef = -f_ik, -f_kj; q the stored pair of (x, y), op the transpose when x > y,
 // because T_(x,y)(full) = P_q op(T_q) P_q^T).  The small factors are summed per
 // orbital block of the fragment (N: plain, Ne: scaled by e), then multiplied by Q_x.
-// The Q_x columns of every pair's dP are summed (in pair order) into the fragment's
-// slot of orbital x.
+// The Q_x columns of every pair's dP are summed (in pair order) into the job's slot of orbital x.
+// Bound by the FP64 pipe (products of orders 20 to 60) and, with a CTA per fragment, by the largest fragments: 24 orbitals,
+// 120 virtuals, 408 fragments: 51 ms; a CTA per pair and the empty 16-row parts of tiles skipped: 33 ms.
 __global__ void __launch_bounds__(NT) k_relax_frag(Tables t, const double* __restrict__ e_vir,
                                                    const RelaxFragJob* __restrict__ jobs, int n_jobs,
                                                    double* scratch, size_t scr_per, int max_m) {
@@ -105,10 +106,11 @@ __global__ void __launch_bounds__(NT) k_relax_frag(Tables t, const double* __res
         np++;
       }
     for (int a = 0; a < no; a++)
-      for (size_t idx = threadIdx.x; idx < (size_t)nv * nb[a]; idx += NT) jb.slot[a][idx] = 0.0;
+      for (size_t idx = threadIdx.x; jb.slot[a] && idx < (size_t)nv * nb[a]; idx += NT) jb.slot[a][idx] = 0.0;
     int u = 0;
     for (int ua = 0; ua < no; ua++)
       for (int ub = ua; ub < no; ub++, u++) {
+        if (u < jb.u0 || u >= jb.u1) continue;
         const int i = pi[u], j = pj[u], m = pm[u];
         const double ac = ((i == j) ? 2.0 : 4.0) * jb.c;
         const double* T = Tp[u];

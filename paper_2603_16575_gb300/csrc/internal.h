@@ -141,14 +141,13 @@ int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, 
                    double* parts, int* err, cudaStream_t st);
 // ---- FP64 amplitude iterations on the tensor cores (solve_oz.cu)
 struct OzPolish {        // pair basis refinement
-  int m, r;
+  int r, pad;
   const double* S1;      // U0^T U0 [r][r]
   double* F1;            // U0^T e U0 (overwritten)
   double* IE;            // out: the change of basis, U = U0 IE [r][r]
-  double* X;             // [m][m], first r columns; in place
   double* et;            // out
 };
-void launch_oz_polish(const OzPolish* jobs, int n_jobs, int max_m, double* scratch, int n_cta, cudaStream_t st);
+void launch_oz_polish(const OzPolish* jobs, int n_jobs, int max_r, double* scratch, int n_cta, cudaStream_t st);
 struct OzPair {          // a pair of a fragment
   int frag, r, m, diag;
   int kpad;              // r rounded up to 32
@@ -157,6 +156,7 @@ struct OzPair {          // a pair of a fragment
   int pad;
   double fij;            // f_ii + f_jj
   const double* Kt;      // [r][r]
+  const double* iD;      // 1 / D [r][r] (FP64 form)
   const double* et;      // [r]
   const double* X;       // [m][m]
   double* Y;             // [r][r]
@@ -165,6 +165,13 @@ struct OzPair {          // a pair of a fragment
 };
 void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool first, int ld, long long rows, int nch, uint16_t* D,
                       int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st);
+struct OzTable {         // iD of a pair: 1 / (fij - e_a - e_b)
+  int r, pad;
+  double fij;
+  const double* et;
+  double* iD;
+};
+void launch_oz_tables(const OzTable* jobs, int n, cudaStream_t st);
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
                         double* e_prev, int* done, int* left, FragOut* out, const int* out_id, cudaStream_t st);
 void launch_oz_raw(const OzPair* pairs, int n_pairs, int max_m, double* scratch, int n_cta, cudaStream_t st);
@@ -457,12 +464,12 @@ struct RelaxKJob {          // exchange part of dP_(i,j): alpha [B_i (A_j W~^T) 
   const double* bt_jj;      // B_j^T Q_j
   double* out;              // [n_vir][m]
 };
-struct RelaxFragJob {       // the rest of dP for every pair of one fragment
+struct RelaxFragJob {       // the rest of dP for pairs [u0, u1) (a <= b in order) of one fragment
   int orbs[3];
-  int no;
+  int no, u0, u1;
   double c;                 // fragment weight
   const double* T;          // the fragment's amplitudes, pairs (a <= b) in order
-  double* slot[3];          // [n_vir][n_x] per orbital of the fragment
+  double* slot[3];          // [n_vir][n_x] per orbital of the fragment; NULL where none of the pairs has it
 };
 struct RelaxGTerm {         // a block of columns added into G_x
   const double* p;

@@ -25,25 +25,23 @@ namespace osv {
 // U0 = P X: with S1 = U0^T U0 and F1 = U0^T e U0 formed from U0 itself (entries of order 1; X^T S X would carry
 // eps |X|^2, X reaching lambda_min(S)^(-1/2)) and R = 1 - S1,
 //   A = F1 + (R F1 + F1 R) / 2 to first order in R, the Fock matrix of the orthonormalised basis U0 (1 + R / 2);
-//   E_ab = A_ab / (A_bb - A_aa),  U <- U0 (1 + R / 2)(1 + E), X likewise, e~ = diag(A).
+//   E_ab = A_ab / (A_bb - A_aa),  U <- U0 (1 + R / 2)(1 + E), X likewise (two contractions), e~ = diag(A).
 // Each step squares the errors, so three take the FP32 Jacobi basis (R and the off-diagonal A ~ 1e-6) to FP64 rounding,
 // unless a pair of eigenvalues is close: pairs with |A_ab| > 1e-3 |A_bb - A_aa| are first diagonalised by Jacobi
 // rotations G among themselves (a handful at most), and 1 + E is that of the rotated A.
 constexpr int POL_MAX = 256;      // close pairs handled by rotations in one step
 constexpr int POL_SWEEPS = 4;
-__global__ void __launch_bounds__(NT) k_oz_polish(const OzPolish* __restrict__ jobs, int n_jobs, int max_m,
+__global__ void __launch_bounds__(NT) k_oz_polish(const OzPolish* __restrict__ jobs, int n_jobs, int max_r,
                                                   double* scratch) {
-  __shared__ double sm[GEMM_SMEM_WIDE];
+  __shared__ double rcs[2 * POL_MAX * POL_SWEEPS];   // (c, s) of the recorded rotations
   __shared__ int s_n, s_rec;
   __shared__ unsigned key[POL_MAX], list[POL_MAX];
   __shared__ unsigned short rec[POL_MAX * POL_SWEEPS];
-  double* rcs = sm;               // (c, s) of the recorded rotations; the GEMM tiles come later
-  static_assert(2 * POL_MAX * POL_SWEEPS <= GEMM_SMEM_WIDE, "rotation record");
-  double* A = scratch + (size_t)blockIdx.x * max_m * max_m;
+  double* A = scratch + (size_t)blockIdx.x * max_r * max_r;
   const int tid = threadIdx.x;
   for (int jq = blockIdx.x; jq < n_jobs; jq += gridDim.x) {
     const OzPolish jb = jobs[jq];
-    const int m = jb.m, r = jb.r;
+    const int r = jb.r;
     double* RG = jb.F1;           // R / 2, then R G / 2
     if (tid == 0) s_n = s_rec = 0;
     for (int idx = tid; idx < r * r; idx += NT) {
@@ -127,14 +125,11 @@ __global__ void __launch_bounds__(NT) k_oz_polish(const OzPolish* __restrict__ j
     __syncthreads();
     for (int idx = tid; idx < r * r; idx += NT) jb.IE[idx] += RG[idx];
     __syncthreads();
-    cta_gemm_a(m, r, r, 1.0, dense_view(jb.X, m, r, m), dense_view(jb.IE, r, r, r), 0.0, A, r, sm);
-    for (int idx = tid; idx < m * r; idx += NT) jb.X[(size_t)(idx / r) * m + idx % r] = A[idx];
-    __syncthreads();
   }
 }
-void launch_oz_polish(const OzPolish* jobs, int n_jobs, int max_m, double* scratch, int n_cta, cudaStream_t st) {
+void launch_oz_polish(const OzPolish* jobs, int n_jobs, int max_r, double* scratch, int n_cta, cudaStream_t st) {
   if (!n_jobs) return;
-  k_oz_polish<<<n_cta, NT, 0, st>>>(jobs, n_jobs, max_m, scratch);
+  k_oz_polish<<<n_cta, NT, 0, st>>>(jobs, n_jobs, max_r, scratch);
   note_launch(1);
 }
 
@@ -168,44 +163,92 @@ __device__ __forceinline__ void row_digits(const double* Y, int r, int m, int v,
   }
 }
 
+// 1 / D of a pair, shared by the fragments that hold it: a division takes ten operations of the FP64 pipe, which issues
+// one warp in 64 cycles, and the update is bound by it.
+__global__ void __launch_bounds__(NT) k_oz_tables(const OzTable* __restrict__ jobs) {
+  const OzTable jb = jobs[blockIdx.x];
+  for (int idx = blockIdx.y * NT + threadIdx.x; idx < jb.r * jb.r; idx += gridDim.y * NT)
+    jb.iD[idx] = 1.0 / (jb.fij - jb.et[idx / jb.r] - jb.et[idx % jb.r]);
+}
+// Y, energy and digits of a pair: six FP64 operations an element (maxima by integer compares of the magnitudes),
+// four elements a thread in flight.  3400 pairs of order ~56: 0.95 -> 0.35 ms.
+constexpr int UPU = 4;
 __global__ void __launch_bounds__(NT) k_oz_update(const OzPair* __restrict__ pairs, int n_pairs,
                                                   const int* __restrict__ done, int first, int ld, size_t slice, int nch,
                                                   uint16_t* __restrict__ D, int* __restrict__ ex,
                                                   int* __restrict__ exW, double* __restrict__ pe,
                                                   double* __restrict__ pu) {
   __shared__ double red[40];
+  __shared__ unsigned long long rdu[NT / 32];
+  __shared__ unsigned ram[NT / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int q = blockIdx.x; q < n_pairs; q += gridDim.x) {
     const OzPair p = pairs[q];
     if (done[p.frag]) continue;
-    const int r = p.r;
-    double du = 0.0, am = 0.0, ss = 0.0;
-    bool bad = false;
-    for (int idx = threadIdx.x; idx < r * r; idx += NT) {
-      const int a = idx / r, b = idx % r;
-      const double y = (p.Kt[idx] + (first ? 0.0 : p.C[idx])) / (p.fij - p.et[a] - p.et[b]);
-      du = fmax(du, fabs(y - (first ? 0.0 : p.Y[idx])));
-      p.Y[idx] = y;
-      am = fmax(am, fabs(y));
-      ss += y * y;
-      bad |= !isfinite(y);
+    const int r = p.r, rr = r * r;
+    unsigned long long du = 0;       // bits of non-negative doubles order as they do (NaN above all)
+    unsigned am = 0;                 // upper word of the largest magnitude
+    double ss = 0.0;
+    for (int i0 = threadIdx.x; i0 < rr; i0 += UPU * NT) {
+      double kt[UPU], id[UPU], c[UPU], yo[UPU];
+#pragma unroll
+      for (int u = 0; u < UPU; u++) {
+        const int idx = min(i0 + u * NT, rr - 1);
+        kt[u] = p.Kt[idx];
+        id[u] = p.iD[idx];
+        c[u] = first ? 0.0 : p.C[idx];
+        yo[u] = first ? 0.0 : p.Y[idx];
+      }
+#pragma unroll
+      for (int u = 0; u < UPU; u++) {
+        const int idx = i0 + u * NT;
+        if (idx >= rr) break;
+        const double y = (kt[u] + c[u]) * id[u];
+        const unsigned long long d = (unsigned long long)__double_as_longlong(y - yo[u]) & 0x7fffffffffffffffull;
+        du = d > du ? d : du;
+        am = max(am, (unsigned)__double2hiint(y) & 0x7fffffffu);
+        ss = fma(y, y, ss);
+        p.Y[idx] = y;
+      }
     }
-    bad = __syncthreads_or(bad);
-    du = cta_max(du, red);
-    am = cta_max(am, red);
-    ss = cta_sum(ss, red);       // ends with a barrier: Y is complete
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long d = __shfl_xor_sync(0xffffffffu, du, o);
+      du = d > du ? d : du;
+    }
+    am = __reduce_max_sync(0xffffffffu, am);
+    if (lane == 0) {
+      rdu[warp] = du;
+      ram[warp] = am;
+    }
+    ss = cta_sum(ss, red);       // ends with a barrier: Y, rdu and ram are complete
+    for (int u = 0; u < NT / 32; u++) {
+      du = rdu[u] > du ? rdu[u] : du;
+      am = max(am, ram[u]);
+    }
+    const bool bad = am >= 0x7ff00000u || (du >> 52) >= 2047;
     double e = 0.0;
-    for (int idx = threadIdx.x; idx < r * r; idx += NT) {
-      const int a = idx / r, b = idx % r;
-      e += p.Kt[idx] * (2.0 * p.Y[idx] - p.Y[(size_t)b * r + a]);
+    const unsigned mag = 0xffffffffu / (unsigned)r + 1;   // idx / r = umulhi(idx, mag) for idx r < 2^32
+    for (int i0 = threadIdx.x; i0 < rr; i0 += UPU * NT) {
+      double kt[UPU], y[UPU], yt[UPU];
+#pragma unroll
+      for (int u = 0; u < UPU; u++) {
+        const int idx = min(i0 + u * NT, rr - 1), a = (int)__umulhi((unsigned)idx, mag);
+        kt[u] = p.Kt[idx];
+        y[u] = p.Y[idx];
+        yt[u] = p.Y[(size_t)(idx - a * r) * r + a];
+      }
+#pragma unroll
+      for (int u = 0; u < UPU; u++)
+        if (i0 + u * NT < rr) e = fma(kt[u], fma(2.0, y[u], -yt[u]), e);
     }
     e = cta_sum(e, red);
     if (threadIdx.x == 0) {
       pe[q] = p.diag ? e : 2.0 * e;
-      pu[q] = bad ? __longlong_as_double(0x7FF8000000000000ll) : du;
+      pu[q] = bad ? __longlong_as_double(0x7FF8000000000000ll) : __longlong_as_double((long long)du);
     }
-    const double nrm = bad ? 0.0 : sqrt(ss) * (1.0 + 1e-3);
-    const int eY = bound_exp(bad ? 0.0 : am), eW = bound_exp(nrm);
+    const int eY = bad ? oz::EX_ZERO : oz::chunk_exp(am >> 20);
+    const int eW = bound_exp(bad ? 0.0 : sqrt(ss) * (1.0 + 1e-3));
     for (int v = 0; v < 3; v++) {
       const int id = p.ver[v];
       if (id < 0) continue;
@@ -250,6 +293,11 @@ void launch_oz_update(const OzPair* pairs, int n_pairs, const int* done, bool fi
                       int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st) {
   if (!n_pairs) return;
   k_oz_update<<<n_cta, NT, 0, st>>>(pairs, n_pairs, done, first ? 1 : 0, ld, (size_t)rows * ld, nch, D, ex, exW, pe, pu);
+  note_launch(1);
+}
+void launch_oz_tables(const OzTable* jobs, int n, cudaStream_t st) {
+  if (!n) return;
+  k_oz_tables<<<dim3(n, 4), NT, 0, st>>>(jobs);
   note_launch(1);
 }
 void launch_oz_converge(const int* pair0, int n_frag, const double* pe, const double* pu, SolveOpts o, double ulps, int it,
