@@ -1089,6 +1089,9 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   std::vector<int> term0{0};
   int max_r = 1, max_m = 1;
   size_t ysz = 0;
+  std::vector<std::array<double, 3>> tq;
+  pairs.reserve(6 * (f1 - f0));
+  terms.reserve(18 * (f1 - f0));
   for (size_t f = f0; f < f1; f++) {
     const std::vector<int>& o = orbs[f];
     const int nc = (int)o.size(), base = (int)pairs.size();
@@ -1122,7 +1125,7 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     for (int a = 0; a < nc; a++)
       for (int b = a; b < nc; b++) {
         const int P = lp(a, b), i = o[a], j = o[b];
-        std::vector<std::array<double, 3>> tq;   // pair, coefficient of Y_q, of Y_q^T
+        tq.clear();                              // pair, coefficient of Y_q, of Y_q^T
         auto put = [&](int x, int y, double coef) {
           if (coef == 0.0) return;
           const int Q = lp(std::min(x, y), std::max(x, y));
@@ -1194,7 +1197,10 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   // pair-couple overlaps Sigma_(lo,hi), in both orientations
   struct Couple { int lo, hi; };
   std::vector<Couple> cps;
-  std::unordered_map<uint64_t, int> cid;
+  // open-addressed table of the couples (a node per couple of a hash map took longer than the rest of the lists)
+  size_t hsz = 64;
+  while (hsz < 2 * (size_t)nt) hsz *= 2;
+  std::vector<std::pair<uint64_t, int>> cid(hsz, {~0ull, -1});
   std::vector<int> tc(nt);
   size_t sgsz = 0;
   std::vector<size_t> sgo;
@@ -1202,14 +1208,15 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
     const int P = pid[terms[t].p], Q = pid[terms[t].q];
     const int lo = std::min(P, Q), hi = std::max(P, Q);
     const uint64_t key = ((uint64_t)lo << 32) | (unsigned)hi;
-    auto it = cid.find(key);
-    if (it == cid.end()) {
-      it = cid.emplace(key, (int)cps.size()).first;
+    size_t h = (size_t)(key * 0x9E3779B97F4A7C15ull >> 20) & (hsz - 1);
+    while (cid[h].second >= 0 && cid[h].first != key) h = (h + 1) & (hsz - 1);
+    if (cid[h].second < 0) {
+      cid[h] = {key, (int)cps.size()};
       cps.push_back(Couple{lo, hi});
       sgo.push_back(sgsz);
       sgsz += (size_t)c->r_h[lo] * c->r_h[hi];
     }
-    tc[t] = it->second;
+    tc[t] = cid[h].second;
   }
   long long srows = 0;
   for (const Couple& k : cps) srows += c->r_h[k.lo] + c->r_h[k.hi];
@@ -1269,11 +1276,12 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   }
   Tmp idm, idj;
   if (!mx) {                             // 1 / D of the pairs in use
-    std::unordered_map<int, size_t> at;
+    std::vector<long long> at(c->K_h.size(), -1);
     std::vector<OzTable> tj;
     size_t tsz = 0;
     for (int p = 0; p < np; p++)
-      if (at.emplace(pid[p], tsz).second) {
+      if (at[pid[p]] < 0) {
+        at[pid[p]] = (long long)tsz;
         tj.push_back(OzTable{pairs[p].r, 0, pairs[p].fij, pairs[p].et, nullptr});
         tsz += (size_t)pairs[p].r * pairs[p].r;
       }
@@ -1298,16 +1306,19 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   Tmp mt, mp, mtj, mP, dr, scr2, msj, mep, mt0, mtb;
   const int max_left = std::min(np, 2 * c->num_sms);
   if (mx) {
-    std::unordered_map<int, size_t> at;
+    std::vector<long long> at(c->K_h.size(), -1);
     std::vector<MxTable> tj;
     std::vector<MxPair> mpair(np);
     size_t tsz = 0, off = 0;
     for (int p = 0; p < np; p++)
-      if (at.emplace(pid[p], tsz).second) tsz += (size_t)pairs[p].r * pairs[p].r;
+      if (at[pid[p]] < 0) {
+        at[pid[p]] = (long long)tsz;
+        tsz += (size_t)pairs[p].r * pairs[p].r;
+      }
     TRY(oz_room(c, mt, 2 * tsz * sizeof(dfl)));
     TRY(oz_room(c, mP, ysz * sizeof(float)));
     TRY(oz_room(c, mp, np * sizeof(MxPair)));
-    TRY(oz_room(c, mtj, at.size() * sizeof(MxTable)));
+    TRY(oz_room(c, mtj, c->K_h.size() * sizeof(MxTable)));
     TRY(oz_room(c, dr, nfb * (2 * sizeof(double) + sizeof(int))));
     TRY(oz_room(c, scr2, (size_t)max_left * 2 * max_r * max_r * sizeof(float)));
     std::vector<char> seen(c->K_h.size(), 0);
@@ -1390,6 +1401,10 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
   std::vector<OzDev> d1(ng), d2(ng);
   for (size_t g = 0; g < ng; g++) {
     OzList l1, l2;
+    const size_t tg = term0[grp[g + 1]] - term0[grp[g]];
+    l1.jobs.reserve(tg * (1 + (max_r > cols)));
+    l1.segs.reserve(tg);
+    l2.segs.reserve(tg);
     long long wrow = 0;
     for (int p = grp[g]; p < grp[g + 1]; p++) {
       const OzPair& P = pairs[p];
@@ -2153,8 +2168,38 @@ int compute_s2b(osvmp2_ctx* c, std::vector<double>& s2b) {
   TRY(tmp_alloc(c, vd, pl.size() * sizeof(double)));
   CK(cudaMemcpyAsync(pd.p, pl.data(), pl.size() * sizeof(int2), cudaMemcpyHostToDevice, c->st));
   ph_begin(c, OSVMP2_PH_SCREEN);
-  launch_s2b(tables(c), (const int2*)pd.p, (int)pl.size(), (double*)vd.p,
-             (int)std::min<size_t>(pl.size(), 4 * (size_t)c->num_sms), c->st);
+  // the overlaps as sliced contractions, their squares summed in the epilogue
+  auto sliced = [&]() -> int {
+    const int nv = c->sys.n_vir;
+    OzMats q(nv);
+    std::vector<int> at(n), tile0{0};
+    for (int i = 0; i < n; i++) at[i] = q.add(c->Qp[i], c->n_osv[i], c->n_osv[i], nv);
+    OzList l;
+    for (const int2& p : pl) {
+      l.product(q.mat(at[p.x]), c->n_osv[p.x], q.mat(at[p.y]), c->n_osv[p.y], nv, nullptr, 0);
+      tile0.push_back((int)l.jobs.size());
+    }
+    for (size_t j = 0; j < l.jobs.size(); j++) l.jobs[j].o_row = (int)j;
+    Tmp parts, t0;
+    OzDev d;
+    TRY(oz_mats_room(c, q));
+    TRY(oz_room(c, parts, std::max<size_t>(1, l.jobs.size()) * 16 * sizeof(double)));
+    TRY(oz_room(c, t0, tile0.size() * sizeof(int)));
+    TRY(oz_upload(c, l, d));
+    CK(cudaMemcpyAsync(t0.p, tile0.data(), tile0.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+    TRY(oz_mats_fill(c, q, nullptr, false));
+    CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
+    if (d.n && launch_oz_squares(q.op, q.op, (const oz::Job*)d.j.p, d.n, (const oz::Seg*)d.s.p, (double*)parts.p, c->err_d, c->st))
+      return fail(c, OSVMP2_E_CUDA, "tensor-map encoding for the pair screening failed");
+    launch_s2b_sum(tables(c), (const int2*)pd.p, (int)pl.size(), (const int*)t0.p, (const double*)parts.p, (double*)vd.p, c->st);
+    CK(cudaGetLastError());
+    return check_err_flag(c, "pair screening");
+  };
+  const int rc = sliced();
+  if (rc && rc != OZ_NO_ROOM) return rc;
+  if (rc)
+    launch_s2b(tables(c), (const int2*)pd.p, (int)pl.size(), (double*)vd.p,
+               (int)std::min<size_t>(pl.size(), 4 * (size_t)c->num_sms), c->st);
   ph_end(c, OSVMP2_PH_SCREEN, fl);
   CK(cudaGetLastError());
   std::vector<double> v(pl.size());
@@ -3429,8 +3474,11 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
   // exchange part per stored pair
   std::vector<size_t> koff(np + 1, 0);
   for (int q = 0; q < np; q++) koff[q + 1] = koff[q] + (size_t)nv * pair_dim_h(c, plist[q].first, plist[q].second);
-  Tmp dk, kscr, d_kj;
+  Tmp dk, dk2, kscr, d_kj;
   TRY(tmp_alloc(c, dk, std::max<size_t>(1, koff[np]) * sizeof(double)));
+  // the two terms of a pair side by side where a second buffer fits
+  const size_t k_most = c->opts.mem_cap_mib > 0 ? (size_t)c->opts.mem_cap_mib << 17 : (size_t)4 << 30;
+  const bool both = koff[np] * sizeof(double) <= k_most && !oz_room(c, dk2, std::max<size_t>(1, koff[np]) * sizeof(double));
   std::vector<RelaxKJob> kj(np);
   for (int q = 0; q < np; q++) {
     const int i = plist[q].first, j = plist[q].second;
@@ -3445,14 +3493,15 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
     if (!k.bt_ii || (i != j && (!k.bt_ij || !k.bt_ji || !k.bt_jj)))
       return fail(c, OSVMP2_E_STATE, "relaxed gradient: the projections of pair (%d, %d) are missing", i, j);
     k.out = (double*)dk.p + koff[q];
+    k.out2 = both ? (double*)dk2.p + koff[q] : k.out;
     const double m = pair_dim_h(c, i, j);
     fl += 4.0 * nx * m * m + 4.0 * nv * (double)nx * m;
   }
-  const int n_cta_k = std::max(1, std::min(np, 2 * c->num_sms));
-  TRY(tmp_alloc(c, kscr, (size_t)n_cta_k * 2 * nx * std::max(max_m, 1) * sizeof(double)));
+  const int n_cta_k = std::max(1, std::min((both ? 2 : 1) * np, 2 * c->num_sms));
+  TRY(tmp_alloc(c, kscr, (size_t)n_cta_k * nx * std::max(max_m, 1) * sizeof(double)));
   TRY(tmp_alloc(c, d_kj, std::max<size_t>(1, kj.size()) * sizeof(RelaxKJob)));
   if (np) CK(cudaMemcpyAsync(d_kj.p, kj.data(), kj.size() * sizeof(RelaxKJob), cudaMemcpyHostToDevice, c->st));
-  launch_relax_kpart(t, bs, (const RelaxKJob*)d_kj.p, np, (double*)kscr.p, n_cta_k, max_m, c->st);
+  launch_relax_kpart(t, bs, (const RelaxKJob*)d_kj.p, np, (double*)kscr.p, n_cta_k, max_m, both, c->st);
   CK(cudaGetLastError());
   // the rest per pair of a fragment (without room for that many slots: per fragment), into one slot per (job, orbital)
   std::vector<std::vector<RelaxGTerm>> gt(n);
@@ -3538,6 +3587,10 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
     const int i = plist[q].first, j = plist[q].second, m = pair_dim_h(c, i, j);
     gt[i].push_back(RelaxGTerm{(const double*)dk.p + koff[q], m, 0});
     if (i != j) gt[j].push_back(RelaxGTerm{(const double*)dk.p + koff[q], m, c->n_osv[i]});
+    if (both) {
+      gt[i].push_back(RelaxGTerm{(const double*)dk2.p + koff[q], m, 0});
+      if (i != j) gt[j].push_back(RelaxGTerm{(const double*)dk2.p + koff[q], m, c->n_osv[i]});
+    }
   }
   std::vector<RelaxGJob> gj(n);
   std::vector<RelaxGTerm> gflat;

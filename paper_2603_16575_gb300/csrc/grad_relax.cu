@@ -43,22 +43,22 @@ __device__ inline View proj_view(const RelaxKJob& jb, int side, int ni, int nj, 
 
 }  // namespace
 
-// ---- exchange part, one CTA per stored pair: out = alpha [B_i (A_j W~^T) + B_j (A_i W~)]
+// ---- exchange part, a CTA for each term of a stored pair: out = alpha B_i (A_j W~^T), out2 = alpha B_j (A_i W~)
 __global__ void __launch_bounds__(NT) k_relax_kpart(Tables t, BSrc bs, const RelaxKJob* __restrict__ jobs,
-                                                    int n_jobs, double* scratch, int max_m) {
+                                                    int n_jobs, double* scratch, int max_m, int s0, int ns) {
   __shared__ double sm[GEMM_SMEM_DOUBLES];
   const int nx = bs.n_aux, nv = t.n_vir;
-  double* M1 = scratch + (size_t)blockIdx.x * 2 * nx * max_m;
-  double* M2 = M1 + (size_t)nx * max_m;
-  for (int jid = blockIdx.x; jid < n_jobs; jid += gridDim.x) {
-    const RelaxKJob jb = jobs[jid];
+  double* M1 = scratch + (size_t)blockIdx.x * nx * max_m;
+  for (int q = blockIdx.x; q < ns * n_jobs; q += gridDim.x) {   // terms s0 .. s0 + ns - 1 of every pair
+    const RelaxKJob jb = jobs[q / ns];
+    const int side = s0 + q % ns;
     const int i = jb.i, j = jb.j, ni = t.n_osv[i], nj = (i == j) ? 0 : t.n_osv[j], m = ni + nj;
     const double alpha = (i == j) ? 2.0 : 4.0;
     const View W = dense_view(jb.W, m, m, m);
-    cta_gemm(nx, m, m, 1.0, proj_view(jb, 1, ni, nj, nx), transpose(W), 0.0, M1, m, sm);   // A_j W~^T
-    cta_gemm(nx, m, m, 1.0, proj_view(jb, 0, ni, nj, nx), W, 0.0, M2, m, sm);              // A_i W~
-    cta_gemm(nv, m, nx, alpha, BRows{bs, i}, dense_view(M1, nx, m, m), 0.0, jb.out, m, sm);
-    cta_gemm(nv, m, nx, alpha, BRows{bs, j}, dense_view(M2, nx, m, m), 1.0, jb.out, m, sm);
+    // side 0: B_i (A_j W~^T), side 1: B_j (A_i W~)
+    cta_gemm(nx, m, m, 1.0, proj_view(jb, 1 - side, ni, nj, nx), side ? W : transpose(W), 0.0, M1, m, sm);
+    cta_gemm(nv, m, nx, alpha, BRows{bs, side ? j : i}, dense_view(M1, nx, m, m),
+             side && jb.out2 == jb.out ? 1.0 : 0.0, side ? jb.out2 : jb.out, m, sm);
   }
 }
 
@@ -274,10 +274,12 @@ __global__ void k_relax_de_df(int n_vir, int n_occ, const RelaxRJob* __restrict_
 
 // ---------------------------------------------------------------- launchers
 void launch_relax_kpart(const Tables& t, const BSrc& bs, const RelaxKJob* jobs, int n_jobs, double* scratch,
-                        int n_cta, int max_m, cudaStream_t st) {
+                        int n_cta, int max_m, bool both, cudaStream_t st) {
   if (!n_jobs) return;
-  k_relax_kpart<<<n_cta, NT, 0, st>>>(t, bs, jobs, n_jobs, scratch, max_m);
-  note_launch(1);
+  for (int s0 = 0; s0 < (both ? 1 : 2); s0++) {
+    k_relax_kpart<<<n_cta, NT, 0, st>>>(t, bs, jobs, n_jobs, scratch, max_m, s0, both ? 2 : 1);
+    note_launch(1);
+  }
 }
 void launch_relax_frag(const Tables& t, const double* e_vir, const RelaxFragJob* jobs, int n_jobs, double* scratch,
                        size_t scr_per, int n_cta, int max_m, cudaStream_t st) {

@@ -139,6 +139,9 @@ int launch_oz_digits(const OzOperand& A, const OzOperand& B, const oz::Job* jobs
 // Dot products of (2 Y - Y^T) with the product of every job (see OzEpiDot), 16 partial sums per job.
 int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    double* parts, int* err, cudaStream_t st);
+// Sums of the squares of the product of every job (see OzEpiSquares), 16 partial sums per job.
+int launch_oz_squares(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                      double* parts, int* err, cudaStream_t st);
 // ---- FP64 amplitude iterations on the tensor cores (solve_oz.cu)
 struct OzPolish {        // pair basis refinement
   int r, pad;
@@ -385,6 +388,9 @@ bool launch_pm_localize_grid(const double* C, int n, const int* atom_ao, int n_a
 
 // ---- pair screening and weak pairs (screen.cu), FP64 in both forms
 // s2b[p] of the pairs (i, j) = pairs[p] (Eq. s2b), grid-stride over n_cta CTAs.
+// s2b of a pair from the partial sums [tile0[p], tile0[p + 1]) of launch_oz_squares.
+void launch_s2b_sum(const Tables& t, const int2* pairs, int n_pairs, const int* tile0, const double* parts, double* s2b,
+                    cudaStream_t st);
 void launch_s2b(const Tables& t, const int2* pairs, int n_pairs, double* s2b, int n_cta, cudaStream_t st);
 struct DiagJob {           // T_ii (raw basis, [n_i][n_i]) = sum of contributions [c0, c1)
   int i, pid;              // orbital, id of the pair (i, i)
@@ -462,7 +468,8 @@ struct RelaxKJob {          // exchange part of dP_(i,j): alpha [B_i (A_j W~^T) 
   const double* bt_ij;      // B_i^T Q_j (unused for i = j)
   const double* bt_ji;      // B_j^T Q_i
   const double* bt_jj;      // B_j^T Q_j
-  double* out;              // [n_vir][m]
+  double* out;              // [n_vir][m]: first term
+  double* out2;             // second term; may be out (then added, by a launch of its own)
 };
 struct RelaxFragJob {       // the rest of dP for pairs [u0, u1) (a <= b in order) of one fragment
   int orbs[3];
@@ -493,7 +500,7 @@ struct RelaxRJob {          // eigenvector response of orbital x
   double* df;               // [1]
 };
 void launch_relax_kpart(const Tables& t, const BSrc& bs, const RelaxKJob* jobs, int n_jobs, double* scratch,
-                        int n_cta, int max_m, cudaStream_t st);
+                        int n_cta, int max_m, bool both, cudaStream_t st);
 void launch_relax_frag(const Tables& t, const double* e_vir, const RelaxFragJob* jobs, int n_jobs, double* scratch,
                        size_t scr_per, int n_cta, int max_m, cudaStream_t st);
 void launch_relax_gather(int n_vir, const int* n_osv, const RelaxGJob* jobs, int n_jobs, const RelaxGTerm* terms,

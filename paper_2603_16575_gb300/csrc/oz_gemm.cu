@@ -395,6 +395,22 @@ struct OzEpiDot {
   }
 };
 
+// Sum of the squares of the tile's part of D (never stored), one partial sum per drain warp at parts + 16 job.o_row.
+struct OzEpiSquares {
+  static constexpr bool kWarp = true, kDigits = false, kPair = false, kLong = false;
+  double* parts;
+  __device__ __forceinline__ void warp(const oz::Job& jb, int r, int c0, const double (&v)[oz::DCOL]) const {
+    double s = 0.0;
+    if (r < jb.m_valid) {
+#pragma unroll
+      for (int u = 0; u < oz::DCOL; u++)
+        if (c0 + u < jb.n_valid) s = fma(v[u], v[u], s);
+    }
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) parts[(size_t)oz::NDRAIN * jb.o_row + (threadIdx.x >> 5) - 2] = s;
+  }
+};
+
 namespace {
 // 3-D BF16 map over k x rows x slices, 64-byte swizzle, box 32 x box_rows x ns.  K < ld: k past K reads as 0.
 bool make_digit_map(CUtensorMap* m, const OzOperand& A, int ns, int box_rows) {
@@ -454,6 +470,10 @@ int launch_mx_gemm(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, 
 int launch_oz_dots(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
                    double* parts, int* err, cudaStream_t st) {
   return run<8>(A, B, jobs, n_jobs, segs, nullptr, err, OzEpiDot{parts}, st);
+}
+int launch_oz_squares(const OzOperand& A, const OzOperand& B, const oz::Job* jobs, int n_jobs, const oz::Seg* segs,
+                      double* parts, int* err, cudaStream_t st) {
+  return run<oz::NSL>(A, B, jobs, n_jobs, segs, nullptr, err, OzEpiSquares{parts}, st);
 }
 int launch_oz_tii(const OzOperand& A, const oz::Job* jobs, int n_jobs, const oz::Seg* segs, const double* e_vir, int ns,
                   int* err, cudaStream_t st) {

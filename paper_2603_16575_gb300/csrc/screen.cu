@@ -12,7 +12,8 @@
 namespace osv {
 
 // S = Q_i^T Q_j tile by tile (16R x 16R outputs), summing the squares of the
-// finished tile entries; one CTA per pair.
+// finished tile entries; one CTA per pair.  For calls without room for the digits of Q: the sliced
+// contraction (launch_oz_squares) takes 0.8 ms for 276 pairs of 188 OSVs in 760 virtuals, this 30.
 template <int R>
 __device__ double s2b_tiles(int ni, int nj, int nv, const double* __restrict__ qi, const double* __restrict__ qj,
                             double* sm) {
@@ -76,6 +77,21 @@ __global__ void __launch_bounds__(NT) k_s2b(Tables t, const int2* __restrict__ p
 void launch_s2b(const Tables& t, const int2* pairs, int n_pairs, double* s2b, int n_cta, cudaStream_t st) {
   if (n_pairs == 0) return;
   k_s2b<<<n_cta, NT, 0, st>>>(t, pairs, n_pairs, s2b);
+  note_launch(1);
+}
+
+__global__ void k_s2b_sum(Tables t, const int2* __restrict__ pairs, int n_pairs, const int* __restrict__ tile0,
+                          const double* __restrict__ parts, double* __restrict__ s2b) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n_pairs) return;
+  double s = 0.0;
+  for (int u = 16 * tile0[p]; u < 16 * tile0[p + 1]; u++) s += parts[u];
+  s2b[p] = s / sqrt((double)t.n_osv[pairs[p].x] * (double)t.n_osv[pairs[p].y]);
+}
+void launch_s2b_sum(const Tables& t, const int2* pairs, int n_pairs, const int* tile0, const double* parts, double* s2b,
+                    cudaStream_t st) {
+  if (n_pairs == 0) return;
+  k_s2b_sum<<<(n_pairs + 127) / 128, 128, 0, st>>>(t, pairs, n_pairs, tile0, parts, s2b);
   note_launch(1);
 }
 
