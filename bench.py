@@ -37,12 +37,9 @@ R2_CUT, R3_CUT, L_OSV = 8.0, 6.0, 1e-4
 MEASURED_GEMM_PEAKS = {"fp64_tflops": 1.099, "tf32_tflops": 1037.8, "fp32_tflops": 69.86,
                        "source": "torch.matmul 8192^3 on a GB300 of this pool, best of 10"}
 FP32_SIMT_PEAK = 152 * 128 * 2 * 2.070e9 / 1e12    # 128 FFMA/clk/SM at the 2070 MHz maximum -> 80.5
-# dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel,
-# from one single-pass ncu capture of the bench workload
-# (profiles/traffic_k_eig_osv_mbe3_n128.md); kernels without a capture of their
-# current code report null.
-KERNEL_TRAFFIC = {"k_eig_osv": 34.27e9 + 43.22e9,          # 128-orbital workload itself (1 pass), bytes per launch
-                  "k_frag_solve_mixed": 20.24e9 + 12.24e9}   # the autotuner's plan (2 CTAs per SM)
+# dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from a single-pass ncu capture of
+# the bench workload; kernels without a capture of their current code report null.
+KERNEL_TRAFFIC = {}
 
 
 def load_peaks():
@@ -315,21 +312,24 @@ def run_gpu(args):
     gemm = MEASURED_GEMM_PEAKS
     peak_fp64 = gemm["fp64_tflops"]
     peak_fp32 = gemm["fp32_tflops"] or FP32_SIMT_PEAK
-    peak_split = gemm["tf32_tflops"] / 10.0       # split-TF32: 10 TF32 slice products per product
+    bf16 = load_peaks().get("bf16_tflops") or 1900.0
+    peak_split = bf16 / 15.0                      # five BF16 slices: 15 slice products per product
+    peak_solve = bf16 / (10.0 if args.prec == "mixed" else 36.0)   # four slices: 10; eight (FP64): 36
     a1_flops = projection_flops(ctx, s, n_osv) * args.steps   # algorithmic A1: 2 n_aux n_vir N_i per orbital
     kern = {
         # phase key: (kernel, bound, peak TFLOP/s, peak source, algorithmic flops in the timed region)
-        "k_eig": ("k_eig_osv", "alu",
+        "k_eig": ("k_eig_tri", "alu",
                   peak_fp32 / 16.0 if args.prec == "mixed" else peak_fp64,
                   ("double-float on the FP32 pipes: FP32 peak / 16 instructions per double-float FMA"
                    if args.prec == "mixed" else "FP64 DGEMM measured"),
                   prof.get("k_eig", (0, 0))[1]),
-        "k_gproj": ("k_tf32x3<EpiG2>", "tensor", peak_split,
-                    f"split-TF32 on tcgen05: measured TF32 {gemm['tf32_tflops']:.0f} TF/s / 10 slice products",
+        "k_gproj": ("k_oz<5, OzEpiG>", "tensor", peak_split,
+                    f"BF16 slices on tcgen05: measured BF16 {bf16:.0f} TF/s / 15 slice products",
                     a1_flops),
-        "k_fragsolve": ("k_frag_solve_mixed" if args.prec == "mixed" else "k_frag_solve", "alu",
-                        peak_fp32 if args.prec == "mixed" else peak_fp64,
-                        "FP32 SIMT" if args.prec == "mixed" else "FP64 DGEMM measured",
+        "k_fragsolve": ("amplitude iterations (k_oz<4>, k_mx_*)" if args.prec == "mixed" else
+                        "amplitude iterations (k_oz<8>, k_oz_update)", "tensor", peak_solve,
+                        f"BF16 slices on tcgen05: measured BF16 {bf16:.0f} TF/s / "
+                        f"{10 if args.prec == 'mixed' else 36} slice products",
                         prof.get("k_fragsolve", (0, 0))[1]),
     }
     kernels = {}
@@ -378,7 +378,7 @@ def run_gpu(args):
         "higher_is_better": True,
         "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "f64" if args.prec == "fp64" else "split-tf32+f32+f64",
+        "dtype": "f64" if args.prec == "fp64" else "split-bf16+f32+f64",
         "data": "synthetic",
         "config": {"workload": f"{args.workload} (n_occ={s.n_occ}, n_vir={s.n_vir}, n_aux={s.n_aux}, "
                                f"lambda={s.lam} A, l_osv={L_OSV}, " +
@@ -516,7 +516,7 @@ def run_osv_only(args, ctx, s, env, f_occ, e_vir, stream, flush, dev, pkg, torch
     out = {"metric": "OSV build orbitals/s", "value": s.n_occ * args.steps / t_tot, "unit": "orbitals/s",
            "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * t_tot / args.steps,
            "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-           "dtype": "split-tf32+f64" if args.prec == "mixed" else "f64", "data": "synthetic",
+           "dtype": "split-bf16+f64" if args.prec == "mixed" else "f64", "data": "synthetic",
            "config": {"workload": f"{args.workload} (n_occ={s.n_occ}, n_vir={s.n_vir}, n_aux={s.n_aux}, "
                                   f"{s.geometry}, lambda={s.lam} A, l_osv={L_OSV}), A0 only",
                       "osv_method": args.osv_method, "osv_prec": args.prec, "b_mode": "regen",

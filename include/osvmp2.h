@@ -63,8 +63,8 @@ typedef enum {
  * products (A4).  OSV eigen-decomposition, preconditioner, update denominators
  * and every energy accumulation are FP64 in all forms. */
 typedef enum {
-  OSVMP2_FP64 = 0,   /* all FP64 on the CUDA cores */
-  OSVMP2_MIXED = 1   /* split-precision products with FP32 accumulation, FP64 elsewhere */
+  OSVMP2_FP64 = 0,   /* FP64 throughout (contractions by exact integer slices on the tensor cores) */
+  OSVMP2_MIXED = 1   /* split-precision products summed as FP32 pairs, FP64 elsewhere */
 } osvmp2_prec;
 
 typedef struct {
@@ -78,12 +78,12 @@ typedef struct {
   int32_t max_iter;   /* amplitude iterations per fragment                    (default 100) */
   int32_t osv_prec;   /* arithmetic of the T_ii contraction B_i B_i^T in osvmp2_build_osv
                          (an osvmp2_prec; default OSVMP2_FP64).  OSVMP2_MIXED runs it on
-                         the tensor cores with split-precision operands (~35 significant
+                         the tensor cores with split-precision operands (~39 significant
                          bits); the eigen-decomposition stays FP64 in both.  Library
                          extension: the paper forms T_ii in one precision only. */
   int32_t no_autotune; /* 0 (default): the first osvmp2_mbe3_energy for a given fragment count and
                           largest pair order times the candidate launch shapes of the mixed
-                          fragment solve and keeps the fastest (osvmp2_get_solve_plan); 1: fixed
+                          amplitude update and keeps the fastest (osvmp2_get_solve_plan); 1: fixed
                           default shape (2 CTAs per SM); 2: fixed shape of 3 CTAs per SM.  The
                           energies are identical either way. */
   int32_t mem_cap_mib; /* 0 (default): no limit.  Otherwise the device memory this ctx may hold at
@@ -150,12 +150,11 @@ void osvmp2_default_opts(osvmp2_opts *opts);
  * unchanged).  Takes effect for the next call; built OSVs and pair blocks are
  * kept. */
 int osvmp2_set_opts(osvmp2_ctx *ctx, const osvmp2_opts *opts);
-/* Launch shape of the last mixed MBE(3) fragment solve: out[0] CTAs per SM (1-3; 3 runs the
- * solver built for 80 registers per thread), out[1] tile set
- * of its FP32 contractions (0: 64/96-wide tiles, 1: also 80-wide), out[2] 1 if chosen by the
- * autotuner, out[3] number of tuned (fragment count, largest pair order) keys.  out: 4 ints
- * (host).  The solve and the MBE(3) sum run as one CUDA graph, replayed with updated
- * arguments on later calls.  Library extension (the paper does not batch this way). */
+/* Launch shape of the last mixed MBE(3) amplitude iterations: out[0] CTAs per SM of the element-wise
+ * update (1-3), out[1] tile set of the FP32 contractions of the per-fragment solver that runs when
+ * device memory has no room for the batch (0: 64/96-wide tiles, 1: also 80-wide), out[2] 1 if chosen
+ * by the autotuner, out[3] number of tuned (fragment count, largest pair order) keys.  out: 4 ints
+ * (host).  Library extension (the paper does not batch this way). */
 int osvmp2_get_solve_plan(const osvmp2_ctx *ctx, int32_t *out);
 /* Number of CUDA kernels this library has launched in this process (all ctxs). */
 int64_t osvmp2_kernel_launches(void);
