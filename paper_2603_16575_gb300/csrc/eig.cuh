@@ -17,6 +17,27 @@
 
 namespace osv {
 
+// FP32 seeds of FP64 reciprocals and roots by integer operations (a conversion holds the FP64 pipe as an FMA does).
+__device__ __forceinline__ float mant_f(int hi, int lo) {          // the float below a double in [1, 4)
+  return __int_as_float((((hi >> 20) - 1023 + 127) << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
+}
+__device__ __forceinline__ double widen(float f, int de) {         // f 2^de, f normal and positive, by integer operations
+  const int b = __float_as_int(f);
+  return __hiloint2double(((b >> 23) - 127 + 1023 + de) << 20 | (b & 0x7fffff) >> 3, b << 29);
+}
+// s^(-1/2) for s > 0: the FP32 reciprocal root of the mantissa refined by one step of third order (Halley; error
+// ~2^-60 before rounding), six FP64 operations; near the ends of the range by the library's function.
+__device__ __forceinline__ double rsqrt_halley(double s) {
+  const int hi = __double2hiint(s), lo = __double2loint(s), ex = (hi >> 20) & 2047;
+  if (ex < 64 || ex > 1983) return rsqrt(s);
+  const int q = (ex - 1023) >> 1;                                  // s = m 4^q, m in [1, 4)
+  const double m = __hiloint2double(hi - (q << 21), lo);
+  const double r0 = widen(rsqrtf(mant_f(hi - (q << 21), lo)), 0);
+  const double e = fma(-m * r0, r0, 1.0);
+  const double r = fma(r0 * e, fma(e, 0.375, 0.5), r0);
+  return __hiloint2double(__double2hiint(r) - (q << 20), __double2loint(r));
+}
+
 // Householder tridiagonalisation of the symmetric n x n matrix A (row-major,
 // lda; global or shared memory), in place.  Outputs d[n], e[n-1] (any memory)
 // and tau[n]; v and p are shared scratch of n elements each, red >= 33.
@@ -316,7 +337,9 @@ __device__ inline int cta_syev_cm(T* A, int n, int lda, T* w, T* Z, int ldz, T* 
 // problems per warp, recording the sweeps (l, h) and their rotations, and (b)
 // the application of the recorded rotations to the rows of Z by a CTA.  The
 // sweeps are those of cta_tridiag_qr; the rotations are formed with fewer
-// FP64 operations (chase_rotation).
+// FP64 operations, since each holds the pipe 64 cycles however few lanes work:
+// ~20 a rotation in place of ~28 (chase_rotation by rsqrt_halley, a shared
+// term in the update, exponents in the tests for zero).
 
 // (a) One thread: chase (d[n], e[n-1]) to diagonal form, appending each sweep
 // to swp (l, h pairs, capacity cap_s sweeps) and its rotations (c, s pairs,
@@ -331,9 +354,10 @@ __device__ inline int cta_syev_cm(T* A, int n, int lda, T* w, T* Z, int ldz, T* 
 // to the FP32 rounding level).  hypot and two divisions where x^2 + z^2 could
 // leave the normal range.
 __device__ __forceinline__ void chase_rotation(double x, double z, double& c, double& s, double& r) {
-  const double q = x * x + z * z;
-  if (q > 1e-280 && q < 1e280) {
-    const double inv = rsqrt(q);
+  const double q = fma(z, z, x * x);
+  const int ex = (__double2hiint(q) >> 20) & 2047;
+  if (ex > 93 && ex < 1953) {     // 1e-280 .. 1e280
+    const double inv = rsqrt_halley(q);
     c = x * inv;
     s = z * inv;
     r = q * inv;
@@ -359,6 +383,18 @@ __device__ __forceinline__ void chase_rotation(float x, float z, float& c, float
   }
 }
 
+// |e| <= eps (|d0| + |d1|); in FP64 the exponents decide for the entries far above it (eps = 2^-52, so
+// |e| >= 2^-49 max |d| is not; no FP64 operation); zeros take the comparison.
+template <class T>
+__device__ __forceinline__ bool off_negligible(T e, T d0, T d1, T eps) {
+  if constexpr (sizeof(T) == 8) {
+    const int xe = (__double2hiint(e) >> 20) & 2047;
+    const int xd = max((__double2hiint(d0) >> 20) & 2047, (__double2hiint(d1) >> 20) & 2047);
+    if (xe > 0 && xe > xd - 50) return false;
+  }
+  return fabs(e) <= eps * (fabs(d0) + fabs(d1));
+}
+
 // S: stride of d and e (one tridiagonal per lane, interleaved in shared memory).
 template <int S = 1, class T>
 __device__ inline int tridiag_qr_record(T* __restrict__ d, T* __restrict__ e, int n, int* __restrict__ swp, int cap_s,
@@ -370,14 +406,14 @@ __device__ inline int tridiag_qr_record(T* __restrict__ d, T* __restrict__ e, in
   for (int sweeps = 0;; sweeps++) {
     int h = n - 1;
     while (h > 0) {
-      if (fabs(e[(h - 1) * S]) <= eps * (fabs(d[(h - 1) * S]) + fabs(d[(h) * S]))) { e[(h - 1) * S] = T(0.0); h--; }
+      if (off_negligible(e[(h - 1) * S], d[(h - 1) * S], d[(h) * S], eps)) { e[(h - 1) * S] = T(0.0); h--; }
       else break;
     }
     if (h == 0) { *n_sw = ns; return 0; }
     if (sweeps >= max_sweeps) return 1;
     int l = h - 1;
     while (l > 0) {
-      if (fabs(e[(l - 1) * S]) <= eps * (fabs(d[(l - 1) * S]) + fabs(d[(l) * S]))) { e[(l - 1) * S] = T(0.0); break; }
+      if (off_negligible(e[(l - 1) * S], d[(l - 1) * S], d[(l) * S], eps)) { e[(l - 1) * S] = T(0.0); break; }
       l--;
     }
     if (ns >= cap_s || nr + (h - l) > cap_r) {
@@ -402,10 +438,12 @@ __device__ inline int tridiag_qr_record(T* __restrict__ d, T* __restrict__ e, in
       T c, s, r;
       chase_rotation(x, z, c, s, r);
       if (k > l) e[(k - 1) * S] = r;
-      const T a = dk, b = ek;
-      d[(k) * S] = c * c * a + T(2.0) * c * s * b + s * s * cc;
-      dk = s * s * a - T(2.0) * c * s * b + c * c * cc;
-      const T ekn = c * s * (cc - a) + (c * c - s * s) * b;
+      // c^2 a + 2 c s b + s^2 cc = a + s h, s^2 a - 2 c s b + c^2 cc = cc - s h, c s (cc - a) + (c^2 - s^2) b = c h - b
+      // with h = s (cc - a) + 2 c b: eight operations of a chain that one thread walks
+      const T a = dk, b = ek, h2 = fma(s, cc - a, (c + c) * b), p = s * h2;
+      d[(k) * S] = a + p;
+      dk = cc - p;
+      const T ekn = fma(c, h2, -b);
       e[(k) * S] = ekn;
       if (k + 1 < h) {
         x = ekn;

@@ -120,13 +120,6 @@ __device__ __forceinline__ void cluster_sync() {
 // tu = (beta - alpha) / beta, sc = 1 / (alpha - beta).  An FP64 operation holds the pipe for 64 cycles, a
 // square root or division ten of them, on the critical path of every step: the FP32 reciprocal (root) of the
 // mantissa refined by one step of third order (Halley; error ~2^-60 before rounding) takes six.
-__device__ __forceinline__ float mant_f(int hi, int lo) {          // the float below a double in [1, 4)
-  return __int_as_float((((hi >> 20) - 1023 + 127) << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
-}
-__device__ __forceinline__ double widen(float f, int de) {         // f 2^de, f normal and positive, by integer operations
-  const int b = __float_as_int(f);
-  return __hiloint2double(((b >> 23) - 127 + 1023 + de) << 20 | (b & 0x7fffff) >> 3, b << 29);
-}
 __device__ __forceinline__ void reflector(double alpha, double sigma, double& beta, double& tu, double& sc) {
   const double s = fma(alpha, alpha, sigma);
   const int hi = __double2hiint(s), lo = __double2loint(s), ex = (hi >> 20) & 2047;

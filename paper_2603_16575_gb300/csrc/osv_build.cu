@@ -266,9 +266,9 @@ __global__ void __launch_bounds__(NT_EIG) k_eig_small(double* T, int n, double t
 // thread chasing and recording rotations into one half of the matrix's storage (free once Z is formed)
 // while the other warps apply the previous record to the rows of Z, one thread a row (column-major, so the accesses of
 // a warp are contiguous; in shared memory up to ZSMEM_MAX).  Bound by the chase (a chain of ~1.6 n^2
-// rotations of ~25 dependent FP64 operations) and, about equally at order 120, by the FP64 pipe of
-// the one SM in the application.  Against a CTA that waits for each rotation: 24 matrices of order 120 27 -> 16 ms,
-// 10 of order 50 6.5 -> 3.9.
+// rotations of ~20 dependent FP64 operations; the application keeps clear of it: with its rows off the
+// chase's sub-partition the time is the same).  Against a CTA that waits for each rotation and ~28 operations a
+// rotation: 24 matrices of order 120 27 -> 13.1 ms (15.4 with the longer rotation), 10 of order 50 6.5 -> 3.0 (3.6).
 __global__ void __launch_bounds__(NT_EIG) k_eig_full(double* T, int n, double thr, int kmax, double* V, double* w,
                                                  int* kout, double* scratch, int* err) {
   extern __shared__ double dyn[];

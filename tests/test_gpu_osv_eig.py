@@ -65,3 +65,21 @@ def test_osv_eigenpairs(n_occ, n_vir, spread, twice, cut):
             assert (T[i] @ Q - Q * w).abs().max() <= 8 * n_vir * eps * frob + 4 * t_err
             assert (Q.T @ Q - torch.eye(kk, dtype=Q.dtype, device=DEV)).abs().max() <= 8 * n_vir * eps
         ctx.close()
+
+
+@pytest.mark.parametrize("n_vir,zero", [(17, 16), (24, 23), (40, 15), (65, 33), (120, 60)])
+def test_osv_rank_deficient_full_spectrum(n_vir, zero):
+    """Virtuals without amplitudes: zero rows, so exact zeros on and off the diagonal of the tridiagonal."""
+    from paper_2603_16575_gb300 import Context
+    B, e, f = _system(3, n_vir, 11 * n_vir, 2.0, False)
+    B[:, n_vir - zero:] = 0.0
+    d = e[:, None] + e[None, :]
+    ctx = Context(0)
+    ctx.build_osv(f, e, 0.0, B=B)
+    for i in range(3):
+        T = (B[i] @ B[i].T) / (d - 2.0 * f[i, i])
+        Q, w = ctx.get_osv(i)
+        frob = float(torch.linalg.norm(T))
+        bound = 8.0 * n_vir * EPS
+        assert float(torch.linalg.norm(Q * w @ Q.T - T)) <= bound * frob
+        assert float((Q.T @ Q - torch.eye(Q.shape[1], dtype=Q.dtype, device=Q.device)).abs().max()) <= bound
