@@ -3566,7 +3566,7 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
   }
   // one CTA per job in flight, two per SM (112 registers x 256 threads each), their scratch
   // within a quarter of the free memory
-  const size_t scr_per = 8 * (size_t)std::max(max_m, 1) * std::max(max_m, 1) + (size_t)nv * std::max(max_m, 1);
+  const size_t scr_per = 9 * (size_t)std::max(max_m, 1) * std::max(max_m, 1) + (size_t)nv * std::max(max_m, 1);
   int n_cta_f = std::max(1, std::min((int)fj.size(), 2 * c->num_sms));
   {
     size_t fr = 0, tot = 0;

@@ -71,7 +71,9 @@ __global__ void __launch_bounds__(NT) k_relax_kpart(Tables t, BSrc bs, const Rel
 // orbital block of the fragment (N: plain, Ne: scaled by e), then multiplied by Q_x.
 // The Q_x columns of every pair's dP are summed (in pair order) into the job's slot of orbital x.
 // Bound by the FP64 pipe (products of orders 20 to 60) and, with a CTA per fragment, by the largest fragments: 24 orbitals,
-// 120 virtuals, 408 fragments: 51 ms; a CTA per pair and the empty 16-row parts of tiles skipped: 33 ms.
+// 120 virtuals, 408 fragments: 51 ms; a CTA per pair and the empty 16-row parts of tiles skipped: 33 ms; the products
+// op(T_q) S_qu of all terms summed per orbital block before the one product with T~ (a product with T~ for every term
+// before), those with the diagonal couplings taken from T S_uu: 14 m^3 in place of 27, 19.6 ms.
 __global__ void __launch_bounds__(NT) k_relax_frag(Tables t, const double* __restrict__ e_vir,
                                                    const RelaxFragJob* __restrict__ jobs, int n_jobs,
                                                    double* scratch, size_t scr_per, int max_m) {
@@ -79,10 +81,11 @@ __global__ void __launch_bounds__(NT) k_relax_frag(Tables t, const double* __res
   const int nv = t.n_vir, n = t.n_occ;
   const size_t M2 = (size_t)max_m * max_m;
   double* Tt = scratch + (size_t)blockIdx.x * scr_per;   // T~ of the pair   [m][m]
-  double* W1 = Tt + M2;                                   // op(T_q) S_qu     [m_q][m]
-  double* N = W1 + M2;                                    // per-block factors [sum n_x][m]
-  double* Ne = N + 3 * M2;
-  double* Dt = Ne + 3 * M2;                               // dP               [nv][m]
+  double* W1 = Tt + M2;                                   // T S_uu           [m][m]
+  double* Ne = W1 + M2;                                   // factors of i, j  [m][m]
+  double* Acc = Ne + M2;                                  // sum op(T_q) S_qu [sum n_x][m]
+  double* N = Acc + 3 * M2;                               // per-block factors [sum n_x][m]
+  double* Dt = N + 3 * M2;                                // dP               [nv][m]
   for (int jid = blockIdx.x; jid < n_jobs; jid += gridDim.x) {
     const RelaxFragJob jb = jobs[jid];
     const int no = jb.no;
@@ -118,52 +121,50 @@ __global__ void __launch_bounds__(NT) k_relax_frag(Tables t, const double* __res
           const int r = idx / m, c = idx % m;
           Tt[idx] = 2.0 * T[idx] - T[(size_t)c * m + r];
         }
-        for (size_t idx = threadIdx.x; idx < (size_t)rows * m; idx += NT) { N[idx] = 0.0; Ne[idx] = 0.0; }
+        const int ra = off[ua] * m, na = nb[ua] * m, rb = off[ub] * m;   // the rows of orbitals i and j in Acc
+        const double fd = -(t.f_occ[(size_t)i * n + i] + t.f_occ[(size_t)j * n + j]);
         __syncthreads();
         const View Ttv = dense_view(Tt, m, m, m);
-        // W1 (m_q x m) times T~^T and times T~ into the rows of the blocks (qa, qb) of Acc
-        auto add_rows = [&](int mq, int qa, int qb, double coef, const View& Wop, const View& Tside, double* Acc) {
-          const int n1 = nb[qa];
-          cta_gemm(n1, m, m, coef, Wop, Tside, 1.0, Acc + (size_t)off[qa] * m, m, sm);
-          if (qa != qb) {
-            View w2 = Wop;   // rows [n1, mq) of a dense row-major view
-            w2.b[0][0].p += (size_t)n1 * w2.b[0][0].ld;
-            w2.b[0][1] = w2.b[1][0] = w2.b[1][1] = w2.b[0][0];
-            w2.rows = w2.rs = mq - n1;
-            cta_gemm(mq - n1, m, m, coef, w2, Tside, 1.0, Acc + (size_t)off[qb] * m, m, sm);
+        for (int tr = 0; tr < 2; tr++) {   // the terms in T T~^T, then those in T^T T~
+          const View Tside = tr ? Ttv : transpose(Ttv);
+          // Acc += coef op(T_q) R, the rows of block qa and those of block qb
+          auto add_rows = [&](int qa, int qb, double coef, const double* Tq, int mq, int trq, const View& R) {
+            const int n1 = qb - qa > 1 ? nb[qa] : mq;   // neighbouring blocks: one product
+            cta_gemm(n1, m, mq, coef, dense_view(Tq, n1, mq, mq, trq), R, 1.0, Acc + (size_t)off[qa] * m, m, sm);
+            if (n1 < mq)
+              cta_gemm(mq - n1, m, mq, coef, dense_view(Tq + (trq ? n1 : (size_t)n1 * mq), mq - n1, mq, mq, trq), R, 1.0,
+                       Acc + (size_t)off[qb] * m, m, sm);
+          };
+          // self terms: diag(e) P T S T~^T (also with the diagonal couplings -f_ii, -f_jj) and P T F T~^T
+          cta_gemm(m, m, m, 1.0, dense_view(T, m, m, m, tr), pair_view(t, t.S, i, j, i, j), 0.0, W1, m, sm);
+          cta_gemm(m, m, m, ac, dense_view(W1, m, m, m), Tside, (double)tr, Ne, m, sm);
+          for (int idx = threadIdx.x; idx < rows * m; idx += NT) {
+            double v = 0.0;
+            if (idx >= ra && idx < ra + na) v = fd * W1[idx - ra];
+            else if (ub != ua && idx >= rb && idx < rb + nb[ub] * m) v = fd * W1[idx - rb + na];
+            Acc[idx] = v;
           }
-        };
-        // self terms: diag(e) P (T S T~^T + T^T S T~) and P (T F T~^T + T^T F T~)
-        for (int s2 = 0; s2 < 2; s2++) {
-          const View Mu = pair_view(t, s2 ? t.F : t.S, i, j, i, j);
-          double* Acc = s2 ? N : Ne;
-          for (int tr = 0; tr < 2; tr++) {
-            cta_gemm(m, m, m, 1.0, dense_view(T, m, m, m, tr), Mu, 0.0, W1, m, sm);
-            add_rows(m, ua, ub, ac, dense_view(W1, m, m, m), tr ? Ttv : transpose(Ttv), Acc);
-          }
-        }
-        // couplings: -f_ik T_(k,j) and -f_kj T_(i,k) for every k of the fragment
-        for (int kc = 0; kc < no; kc++) {
-          const int k = jb.orbs[kc];
-          for (int s2 = 0; s2 < 2; s2++) {
-            const int x = s2 ? ua : kc, y = s2 ? kc : ub;
-            const double coef = s2 ? -t.f_occ[(size_t)k * n + j] : -t.f_occ[(size_t)i * n + k];
-            if (coef == 0.0) continue;
-            const int qa = min(x, y), qb = max(x, y), trq = x > y;
-            const int q = uid[qa * 3 + qb], mq = pm[q];
-            const View Squ = pair_view(t, t.S, jb.orbs[qa], jb.orbs[qb], i, j);
-            for (int tr = 0; tr < 2; tr++) {
-              cta_gemm(mq, m, mq, 1.0, dense_view(Tp[q], mq, mq, mq, trq ^ tr), Squ, 0.0, W1, m, sm);
-              add_rows(mq, qa, qb, ac * coef, dense_view(W1, mq, m, m), tr ? Ttv : transpose(Ttv), N);
+          __syncthreads();
+          add_rows(ua, ub, 1.0, T, m, tr, pair_view(t, t.F, i, j, i, j));
+          // the other couplings: -f_ik T_(k,j) and -f_kj T_(i,k) for every k of the fragment
+          for (int kc = 0; kc < no; kc++) {
+            const int k = jb.orbs[kc];
+            for (int s2 = 0; s2 < 2; s2++) {
+              const int x = s2 ? ua : kc, y = s2 ? kc : ub;
+              const double coef = s2 ? -t.f_occ[(size_t)k * n + j] : -t.f_occ[(size_t)i * n + k];
+              if (coef == 0.0 || (x == ua && y == ub)) continue;
+              const int qa = min(x, y), qb = max(x, y), q = uid[qa * 3 + qb];
+              add_rows(qa, qb, coef, Tp[q], pm[q], (x > y) ^ tr, pair_view(t, t.S, jb.orbs[qa], jb.orbs[qb], i, j));
             }
           }
+          cta_gemm(rows, m, m, ac, dense_view(Acc, rows, m, m), Tside, (double)tr, N, m, sm);
         }
         // dP = diag(e) (Q_i Ne_i + Q_j Ne_j) + sum_x Q_x N_x
         cta_gemm(nv, m, nb[ua], 1.0, dense_view(t.Q[i], nv, nb[ua], nb[ua]),
-                 dense_view(Ne + (size_t)off[ua] * m, nb[ua], m, m), 0.0, Dt, m, sm);
+                 dense_view(Ne, nb[ua], m, m), 0.0, Dt, m, sm);
         if (ub != ua)
           cta_gemm(nv, m, nb[ub], 1.0, dense_view(t.Q[j], nv, nb[ub], nb[ub]),
-                   dense_view(Ne + (size_t)off[ub] * m, nb[ub], m, m), 1.0, Dt, m, sm);
+                   dense_view(Ne + na, nb[ub], m, m), 1.0, Dt, m, sm);
         for (size_t idx = threadIdx.x; idx < (size_t)nv * m; idx += NT) Dt[idx] *= e_vir[idx / m];
         __syncthreads();
         for (int a = 0; a < no; a++)
