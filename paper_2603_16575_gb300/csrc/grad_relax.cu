@@ -73,10 +73,11 @@ __global__ void __launch_bounds__(NT) k_relax_kpart(Tables t, BSrc bs, const Rel
 // Bound by the FP64 pipe (products of orders 20 to 60) and, with a CTA per fragment, by the largest fragments: 24 orbitals,
 // 120 virtuals, 408 fragments: 51 ms; a CTA per pair and the empty 16-row parts of tiles skipped: 33 ms; the products
 // op(T_q) S_qu of all terms summed per orbital block before the one product with T~ (a product with T~ for every term
-// before), those with the diagonal couplings taken from T S_uu: 14 m^3 in place of 27, 19.6 ms.
+// before), those with the diagonal couplings taken from T S_uu: 14 m^3 in place of 27, 19.6 ms.  CTAs take jobs from a
+// counter: the implicit QR of T_xx holds some of the SMs meanwhile.
 __global__ void __launch_bounds__(NT) k_relax_frag(Tables t, const double* __restrict__ e_vir,
                                                    const RelaxFragJob* __restrict__ jobs, int n_jobs,
-                                                   double* scratch, size_t scr_per, int max_m) {
+                                                   double* scratch, size_t scr_per, int max_m, int* next) {
   __shared__ double sm[GEMM_SMEM_DOUBLES];
   const int nv = t.n_vir, n = t.n_occ;
   const size_t M2 = (size_t)max_m * max_m;
@@ -86,7 +87,13 @@ __global__ void __launch_bounds__(NT) k_relax_frag(Tables t, const double* __res
   double* Acc = Ne + M2;                                  // sum op(T_q) S_qu [sum n_x][m]
   double* N = Acc + 3 * M2;                               // per-block factors [sum n_x][m]
   double* Dt = N + 3 * M2;                                // dP               [nv][m]
-  for (int jid = blockIdx.x; jid < n_jobs; jid += gridDim.x) {
+  __shared__ int s_jid;
+  for (;;) {   // jobs as CTAs become free: some SMs may first finish other work
+    if (threadIdx.x == 0) s_jid = atomicAdd(next, 1);
+    __syncthreads();
+    const int jid = s_jid;
+    __syncthreads();
+    if (jid >= n_jobs) break;
     const RelaxFragJob jb = jobs[jid];
     const int no = jb.no;
     int pi[6], pj[6], pm[6], uid[9], off[3], nb[3];
@@ -283,9 +290,10 @@ void launch_relax_kpart(const Tables& t, const BSrc& bs, const RelaxKJob* jobs, 
   }
 }
 void launch_relax_frag(const Tables& t, const double* e_vir, const RelaxFragJob* jobs, int n_jobs, double* scratch,
-                       size_t scr_per, int n_cta, int max_m, cudaStream_t st) {
+                       size_t scr_per, int n_cta, int max_m, int* next, cudaStream_t st) {
   if (!n_jobs) return;
-  k_relax_frag<<<n_cta, NT, 0, st>>>(t, e_vir, jobs, n_jobs, scratch, scr_per, max_m);
+  cudaMemsetAsync(next, 0, sizeof(int), st);
+  k_relax_frag<<<n_cta, NT, 0, st>>>(t, e_vir, jobs, n_jobs, scratch, scr_per, max_m, next);
   note_launch(1);
 }
 void launch_relax_gather(int n_vir, const int* n_osv, const RelaxGJob* jobs, int n_jobs, const RelaxGTerm* terms,

@@ -68,7 +68,8 @@ __host__ __device__ inline size_t eig_osv_scratch_doubles(int nv, int kmax) {
 // dfl_tridiag: the top-k path tridiagonalises in double-float arithmetic (the
 // mixed-form OSV build, whose T_ii is a split-precision product).
 void launch_eig_osv(double* T, int nb, int nv, double thr, int kmax, double* V, double* w, int* k,
-                    double* scratch, int* err, bool dfl_tridiag, const int* nclu, cudaStream_t st);
+                    double* scratch, int* err, bool dfl_tridiag, const int* nclu, cudaStream_t st,
+                    cudaStream_t st_qr = nullptr, cudaEvent_t fork = nullptr);   // fork: the implicit QR on st_qr, after st so far
 // Back-transformation of the kept eigenvectors of the top-k path (n_vir above
 // the shared-memory limit, thr > 0) after launch_eig_osv; a no-op otherwise.
 void launch_eig_back(double* T, int nb, int nv, double thr, int kmax, double* V, const int* k, double* scratch,
@@ -502,7 +503,7 @@ struct RelaxRJob {          // eigenvector response of orbital x
 void launch_relax_kpart(const Tables& t, const BSrc& bs, const RelaxKJob* jobs, int n_jobs, double* scratch,
                         int n_cta, int max_m, bool both, cudaStream_t st);
 void launch_relax_frag(const Tables& t, const double* e_vir, const RelaxFragJob* jobs, int n_jobs, double* scratch,
-                       size_t scr_per, int n_cta, int max_m, cudaStream_t st);
+                       size_t scr_per, int n_cta, int max_m, int* next, cudaStream_t st);
 void launch_relax_gather(int n_vir, const int* n_osv, const RelaxGJob* jobs, int n_jobs, const RelaxGTerm* terms,
                          cudaStream_t st);
 void launch_relax_resp(const Tables& t, const BSrc& bs, const double* e_vir, const RelaxRJob* jobs, int nb,

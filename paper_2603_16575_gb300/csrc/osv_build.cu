@@ -327,7 +327,8 @@ __global__ void __launch_bounds__(NT_EIG) k_eig_full(double* T, int n, double th
 }
 
 void launch_eig_osv(double* T, int nb, int nv, double thr, int kmax, double* V, double* w, int* k,
-                    double* scratch, int* err, bool dfl_tridiag, const int* nclu, cudaStream_t st) {
+                    double* scratch, int* err, bool dfl_tridiag, const int* nclu, cudaStream_t st, cudaStream_t st_qr,
+                    cudaEvent_t fork) {
   if (nv <= EIG_FULL_MAX) {
     const size_t smem = ((size_t)nv * (nv + 1) + 4 * nv + 64) * sizeof(double);
     k_eig_small<<<nb, NT_EIG, smem, st>>>(T, nv, thr, kmax, V, w, k, scratch, err);
@@ -339,6 +340,7 @@ void launch_eig_osv(double* T, int nb, int nv, double thr, int kmax, double* V, 
     launch_eig_tridiag(T, nb, nv, kmax, scratch, err, nclu, st);
     const size_t smem = (2 * (size_t)nv + (nv <= ZSMEM_MAX ? (size_t)nv * nv : 0)) * sizeof(double);
     cudaFuncSetAttribute(k_eig_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (fork && cudaEventRecord(fork, st) == cudaSuccess && cudaStreamWaitEvent(st_qr, fork, 0) == cudaSuccess) st = st_qr;
     k_eig_full<<<nb, NT_EIG, smem, st>>>(T, nv, thr, kmax, V, w, k, scratch, err);
     note_launch(1);
   }
