@@ -41,12 +41,13 @@ __device__ __forceinline__ int chunk_exp(unsigned emax) {
   return emax == 0 ? EX_ZERO : (emax == 2047 ? EX_NAN : (int)emax - 1022);
 }
 
-// round(x 2^(T - e)) for NS slices, T = 7 + 8 (NS - 1) (63 for eight).
+// round(x 2^(T - e)) for NS slices, T = 7 + 8 (NS - 1) (63 for eight).  One place is left for the rounding before half
+// a unit is added: F itself reaches 2^63 - 2^10, where that sum has no room.  The result 2^T has the top digit 128.
 template <int NS>
 __device__ __forceinline__ long long fixedn(double x, unsigned emax) {
   const long long F = fixed63(x, emax);
   constexpr int D = 8 * (NSL - NS);
-  return D ? (F + (1ll << (D > 0 ? D - 1 : 0))) >> D : F;
+  return D ? ((F >> (D > 0 ? D - 1 : 0)) + 1) >> 1 : F;
 }
 
 // Digit s (taken in the order s = NS - 1 .. 0) of two values, as a BF16 pair.
