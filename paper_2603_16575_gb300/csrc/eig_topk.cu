@@ -528,7 +528,8 @@ __global__ void __launch_bounds__(R::NTH, 1) k_eig_tri(double* T, int n, double 
   __syncthreads();
   E* VE = reinterpret_cast<E*>(work + eig_osv_work_doubles(n));   // [k][n]
   const double small = 2.220446049250313e-16 * fmax(norm, 1e-300);
-  const int nslot = (int)(eig_osv_work_doubles(n) / ((size_t)176 * n));   // >= 4
+  // factorisation slots, at most one a warp: above order 16 x 176 the room holds more of them than one CTA has warps
+  const int nslot = min((int)(eig_osv_work_doubles(n) / ((size_t)176 * n)), tw);   // >= 4
   const int slot = gw;
   for (int pass = 0; pass < 2; pass++) {
     if (slot < nslot) {
