@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "pairview.cuh"
+#include "row_index.h"
 
 namespace osv {
 namespace {
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(MXT) k_mx_update(const OzPair* __restrict__ pa
     const dfl* C = reinterpret_cast<const dfl*>(p.C);
     dfl* Ys = in ? ysm : Y;
     const int ys = in ? pitch : r;
-    const unsigned rr = (unsigned)(r * r), mag = 0xffffffffu / (unsigned)r + 1;   // idx / r = umulhi(idx, mag), idx r < 2^32
+    const unsigned rr = (unsigned)(r * r), mag = row_magic((unsigned)r);
     float du = 0.f, am = 0.f, ss = 0.f;
     float sh = 0.f, sl = 0.f;              // <K~, 2 Y>
     for (unsigned i0 = threadIdx.x; i0 < rr; i0 += MU * MXT) {   // MU elements' loads in flight
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(MXT) k_mx_update(const OzPair* __restrict__ pa
         df_acc(sh, sl, kd[u], dfl{2.f * y.h, 2.f * y.l});
         Y[idx] = y;
         if (in) {
-          const unsigned a = __umulhi(idx, mag);
+          const unsigned a = row_of(idx, (unsigned)r, mag);
           ysm[a * pitch + (idx - a * r)] = y;
         }
       }
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(MXT) k_mx_update(const OzPair* __restrict__ pa
       for (int u = 0; u < MU; u++) {
         const unsigned idx = i0 + u * MXT;
         if (idx >= rr) break;
-        const unsigned a = __umulhi(idx, mag);
+        const unsigned a = row_of(idx, (unsigned)r, mag);
         df_acc(sh, sl, kd[u], df_neg(Ys[(idx - a * r) * ys + a]));
       }
     }

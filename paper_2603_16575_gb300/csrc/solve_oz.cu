@@ -17,6 +17,7 @@
 // bound, ten more than the mantissa.
 #include "oz_split.cuh"
 #include "pairview.cuh"
+#include "row_index.h"
 
 namespace osv {
 
@@ -228,12 +229,12 @@ __global__ void __launch_bounds__(NT) k_oz_update(const OzPair* __restrict__ pai
     }
     const bool bad = am >= 0x7ff00000u || (du >> 52) >= 2047;
     double e = 0.0;
-    const unsigned mag = 0xffffffffu / (unsigned)r + 1;   // idx / r = umulhi(idx, mag) for idx r < 2^32
+    const unsigned mag = row_magic((unsigned)r);
     for (int i0 = threadIdx.x; i0 < rr; i0 += UPU * NT) {
       double kt[UPU], y[UPU], yt[UPU];
 #pragma unroll
       for (int u = 0; u < UPU; u++) {
-        const int idx = min(i0 + u * NT, rr - 1), a = (int)__umulhi((unsigned)idx, mag);
+        const int idx = min(i0 + u * NT, rr - 1), a = (int)row_of((unsigned)idx, (unsigned)r, mag);
         kt[u] = p.Kt[idx];
         y[u] = p.Y[idx];
         yt[u] = p.Y[(size_t)(idx - a * r) * r + a];
