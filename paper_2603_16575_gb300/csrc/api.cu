@@ -612,6 +612,7 @@ double fragment_mixed_flops(const osvmp2_ctx* c, const Frag& f, int iters) {
 // cap, a full device) runs the CUDA-core kernels, which need none: the helpers return
 // OZ_NO_ROOM then, with nothing launched that the caller would have to undo.
 constexpr int OZ_NO_ROOM = -100;
+constexpr int OZ_NO_BASIS = -101;   // oz_pair_basis
 
 // Bytes of the digits of `rows` operand rows with K elements each, and of their exponents.
 size_t oz_digit_bytes(size_t rows, int K, int ns = oz::NSL) { return rows * ns * oz::ld_of(K) * sizeof(uint16_t); }
@@ -890,8 +891,10 @@ int oz_exchange(osvmp2_ctx* c, const std::vector<KJob>& kj) {
 
 // FP64 form: U_p = P_p X_p of the new pairs with the basis polished (solve_oz.cu), kept as digits for the
 // pair-couple overlaps.  X and e~ become those of the polished basis.  Pairs in batches whose temporaries
-// fit a fixed budget.
-int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, int max_m) {
+// fit a fixed budget.  OZ_NO_BASIS: a basis still has something left after POLISH_STEPS steps.  *touched: X of some
+// pairs may be that of an unfinished polish (when it does not return 0).
+constexpr int POLISH_FIRST = 3, POLISH_STEPS = 17;
+int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, bool* touched) {
   const int n = c->sys.n_occ, nv = c->sys.n_vir;
   c->ud_of.resize(c->K_h.size(), -1);
   c->ud_mat.resize(c->K_h.size());
@@ -933,71 +936,100 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, i
       u0sz += r * nv;
       sqsz += r * r;
     }
-    Tmp u0, sq, scr, pj, mj;
+    Tmp u0, sq, scr, pj, mj, okd;
     TRY(oz_room(c, u0, u0sz * sizeof(double)));
     TRY(oz_room(c, sq, 3 * sqsz * sizeof(double)));
     TRY(oz_room(c, scr, (size_t)n_cta * max_r * max_r * sizeof(double)));
     TRY(oz_room(c, pj, (b1 - b0) * sizeof(OzPolish)));
     TRY(oz_room(c, mj, (b1 - b0) * sizeof(OzMat)));
-    OzMats xs(max_n), uc(nv), ue(nv), ur(max_r), ie(max_r), xm(max_r);
-    OzList lu, ls, lf, lo, lx;
+    TRY(oz_room(c, okd, (b1 - b0) * sizeof(int)));
     std::vector<OzPolish> pol;
     std::vector<OzMat> fin;
-    size_t uo = 0, so = 0;
     int mr = 0;
-    for (size_t t = b0; t < b1; t++) {
-      const int i = newp[t].first, j = newp[t].second, id = pid[t], r = c->r_h[id], m = c->m_h[id];
-      const int ni = c->n_osv[i], nj = i == j ? 0 : c->n_osv[j];
-      double* X = c->X_h[id];
-      double* U0 = (double*)u0.p + uo;
-      double* S1 = (double*)sq.p + so;
-      double *F1 = S1 + sqsz, *IE = F1 + sqsz;
-      uo += (size_t)r * nv;
-      so += (size_t)r * r;
-      mr = std::max(mr, r);
-      oz::Job proto{};
-      proto.skip = -1;
-      const int first = (int)lu.segs.size(), xt = xs.add(X, r, m, ni);
-      lu.seg(q.mat(at[i]), xs.mat(xt), ni);
-      if (nj) {
-        const int xb = xs.add(X + (size_t)ni * m, r, m, nj);
-        lu.seg(q.mat(at[j]), xs.mat(xb), nj);
+    {   // U0 = P X
+      OzMats xs(max_n);
+      OzList lu;
+      size_t uo = 0, so = 0;
+      for (size_t t = b0; t < b1; t++) {
+        const int i = newp[t].first, j = newp[t].second, id = pid[t], r = c->r_h[id], m = c->m_h[id];
+        const int ni = c->n_osv[i], nj = i == j ? 0 : c->n_osv[j];
+        const double* X = c->X_h[id];
+        double* U0 = (double*)u0.p + uo;
+        double* S1 = (double*)sq.p + so;
+        uo += (size_t)r * nv;
+        so += (size_t)r * r;
+        mr = std::max(mr, r);
+        oz::Job proto{};
+        proto.skip = -1;
+        const int first = (int)lu.segs.size(), xt = xs.add(X, r, m, ni);
+        lu.seg(q.mat(at[i]), xs.mat(xt), ni);
+        if (nj) {
+          const int xb = xs.add(X + (size_t)ni * m, r, m, nj);
+          lu.seg(q.mat(at[j]), xs.mat(xb), nj);
+        }
+        lu.tiles(first, nv, r, U0, r, proto);
+        pol.push_back(OzPolish{r, 0, S1, S1 + sqsz, S1 + 2 * sqsz, c->et_h[id], (int*)okd.p + (t - b0)});
+        const oz::Mat um{(int)row, (int)(row * nch), nch};
+        fin.push_back(OzMat{U0, r, nv, nv, r, um});
+        c->ud_mat[id] = um;
+        row += r;
       }
-      lu.tiles(first, nv, r, U0, r, proto);
-      const int a = uc.add(U0, r, r, nv);
-      ue.add(U0, r, r, nv);
-      ls.product(uc.mat(a), r, uc.mat(a), r, nv, S1, r);
-      lf.product(ue.mat(a), r, uc.mat(a), r, nv, F1, r);
-      pol.push_back(OzPolish{r, 0, S1, F1, IE, c->et_h[id]});
-      const int ix = ie.add(IE, r, r, r);
-      lo.product(ur.mat(ur.add(U0, nv, r, r)), nv, ie.mat(ix), r, r, U0, r);
-      lx.product(xm.mat(xm.add(X, m, m, r)), m, ie.mat(ix), r, r, X, m);
-      const oz::Mat um{(int)row, (int)(row * nch), nch};
-      fin.push_back(OzMat{U0, r, nv, nv, r, um});
-      c->ud_mat[id] = um;
-      row += r;
+      TRY(oz_mats_room(c, xs));
+      TRY(oz_mats_fill(c, xs, nullptr, false));
+      TRY(oz_run(c, q.op, xs.op, lu));
     }
-    TRY(oz_mats_room(c, xs));
-    TRY(oz_mats_room(c, uc));
-    TRY(oz_mats_room(c, ue));
-    TRY(oz_mats_room(c, ur));
-    TRY(oz_mats_room(c, ie));
-    TRY(oz_mats_room(c, xm));
-    TRY(oz_mats_fill(c, xs, nullptr, false));
-    TRY(oz_run(c, q.op, xs.op, lu));
-    CK(cudaMemcpyAsync(pj.p, pol.data(), pol.size() * sizeof(OzPolish), cudaMemcpyHostToDevice, c->st));
-    for (int step = 0; step < 3; step++) {
-      TRY(oz_mats_fill(c, uc, nullptr, false));
-      TRY(oz_mats_fill(c, ue, c->sys.e_vir, false));
-      TRY(oz_mats_fill(c, ur, nullptr, true));
-      TRY(oz_run(c, uc.op, uc.op, ls));
-      TRY(oz_run(c, ue.op, uc.op, lf));
-      TRY(oz_mats_fill(c, xm, nullptr, true));
-      launch_oz_polish((const OzPolish*)pj.p, (int)pol.size(), max_r, (double*)scr.p, n_cta, c->st);
-      CK(cudaGetLastError());
-      TRY(oz_mats_fill(c, ie, nullptr, false));
-      TRY(oz_run(c, ur.op, ie.op, lo));
-      TRY(oz_run(c, xm.op, ie.op, lx));
+    // steps on the pairs `todo` of the batch
+    auto polish = [&](const std::vector<int>& todo, int steps) -> int {
+      OzMats uc(nv), ue(nv), ur(max_r), ie(max_r), xm(max_r);
+      OzList ls, lf, lo, lx;
+      std::vector<OzPolish> jobs;
+      for (int t : todo) {
+        const int id = pid[b0 + t], m = c->m_h[id], r = pol[t].r;
+        double* X = c->X_h[id];
+        double* U0 = const_cast<double*>(fin[t].p);
+        const int a = uc.add(U0, r, r, nv);
+        ue.add(U0, r, r, nv);
+        ls.product(uc.mat(a), r, uc.mat(a), r, nv, const_cast<double*>(pol[t].S1), r);
+        lf.product(ue.mat(a), r, uc.mat(a), r, nv, pol[t].F1, r);
+        jobs.push_back(pol[t]);
+        const int ix = ie.add(pol[t].IE, r, r, r);
+        lo.product(ur.mat(ur.add(U0, nv, r, r)), nv, ie.mat(ix), r, r, U0, r);
+        lx.product(xm.mat(xm.add(X, m, m, r)), m, ie.mat(ix), r, r, X, m);
+      }
+      TRY(oz_mats_room(c, uc));
+      TRY(oz_mats_room(c, ue));
+      TRY(oz_mats_room(c, ur));
+      TRY(oz_mats_room(c, ie));
+      TRY(oz_mats_room(c, xm));
+      CK(cudaMemcpyAsync(pj.p, jobs.data(), jobs.size() * sizeof(OzPolish), cudaMemcpyHostToDevice, c->st));
+      *touched = true;
+      for (int step = 0; step < steps; step++) {
+        TRY(oz_mats_fill(c, uc, nullptr, false));
+        TRY(oz_mats_fill(c, ue, c->sys.e_vir, false));
+        TRY(oz_mats_fill(c, ur, nullptr, true));
+        TRY(oz_run(c, uc.op, uc.op, ls));
+        TRY(oz_run(c, ue.op, uc.op, lf));
+        TRY(oz_mats_fill(c, xm, nullptr, true));
+        launch_oz_polish((const OzPolish*)pj.p, (int)jobs.size(), max_r, (double*)scr.p, n_cta, c->st);
+        CK(cudaGetLastError());
+        TRY(oz_mats_fill(c, ie, nullptr, false));
+        TRY(oz_run(c, ur.op, ie.op, lo));
+        TRY(oz_run(c, xm.op, ie.op, lx));
+      }
+      return 0;
+    };
+    std::vector<int> todo(b1 - b0), ok(b1 - b0);
+    for (size_t t = 0; t < todo.size(); t++) todo[t] = (int)t;
+    for (int done = 0, steps = POLISH_FIRST; !todo.empty(); steps = 2) {
+      if (done >= POLISH_STEPS) return OZ_NO_BASIS;
+      TRY(polish(todo, steps));
+      done += steps;
+      CK(cudaMemcpyAsync(ok.data(), okd.p, ok.size() * sizeof(int), cudaMemcpyDeviceToHost, c->st));
+      CK(cudaStreamSynchronize(c->st));
+      std::vector<int> rest;
+      for (int t : todo)
+        if (!ok[t]) rest.push_back(t);
+      todo.swap(rest);
     }
     CK(cudaMemcpyAsync(mj.p, fin.data(), fin.size() * sizeof(OzMat), cudaMemcpyHostToDevice, c->st));
     launch_oz_mats((const OzMat*)mj.p, (int)fin.size(), mr, nv, nullptr, false, oz::NSL, ld, rows, (uint16_t*)dmem.p, (int*)emem.p,
@@ -2064,13 +2096,14 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     c->um_store.push_back(Uo);
   } else {   // polished basis, K~ = X^T K X (used by the preconditioner-basis solver)
     ph_begin(c, OSVMP2_PH_PRECOND);
-    oz = oz_pair_basis(c, newp, max_m);
-    if (oz && oz != OZ_NO_ROOM) return oz;
-    if (pm && oz != OZ_NO_ROOM) {
+    bool touched = false;
+    oz = oz_pair_basis(c, newp, &touched);
+    if (oz && oz != OZ_NO_ROOM && oz != OZ_NO_BASIS) return oz;
+    if (oz == 0 && pm) {
       c->pm_basis.resize(c->K_h.size(), 0);
       for (auto& p : newp) c->pm_basis[c->pair_id[(size_t)p.first * n + p.second]] = 1;
     }
-    if (oz == OZ_NO_ROOM && pm) {   // no room to polish: bases accurate to FP64 without it
+    if (oz && (pm || touched)) {    // no room to polish, or no end to it: bases accurate to FP64 without it
       tmp_free(pm_slots);
       TRY(tmp_alloc(c, scr, scr_old * sizeof(double)));
       precond64();

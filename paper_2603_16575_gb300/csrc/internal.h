@@ -150,6 +150,7 @@ struct OzPolish {        // pair basis refinement
   double* F1;            // U0^T e U0 (overwritten)
   double* IE;            // out: the change of basis, U = U0 IE [r][r]
   double* et;            // out
+  int* ok;               // out: this step was the last one the basis needed
 };
 void launch_oz_polish(const OzPolish* jobs, int n_jobs, int max_r, double* scratch, int n_cta, cudaStream_t st);
 struct OzPair {          // a pair of a fragment

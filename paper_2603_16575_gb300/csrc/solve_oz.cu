@@ -26,105 +26,180 @@ namespace osv {
 // U0 = P X: with S1 = U0^T U0 and F1 = U0^T e U0 formed from U0 itself (entries of order 1; X^T S X would carry
 // eps |X|^2, X reaching lambda_min(S)^(-1/2)) and R = 1 - S1,
 //   A = F1 + (R F1 + F1 R) / 2 to first order in R, the Fock matrix of the orthonormalised basis U0 (1 + R / 2);
-//   E_ab = A_ab / (A_bb - A_aa),  U <- U0 (1 + R / 2)(1 + E), X likewise (two contractions), e~ = diag(A).
-// Each step squares the errors, so three take the FP32 Jacobi basis (R and the off-diagonal A ~ 1e-6) to FP64 rounding,
-// unless a pair of eigenvalues is close: pairs with |A_ab| > 1e-3 |A_bb - A_aa| are first diagonalised by Jacobi
-// rotations G among themselves (a handful at most), and 1 + E is that of the rotated A.
-constexpr int POL_MAX = 256;      // close pairs handled by rotations in one step
-constexpr int POL_SWEEPS = 4;
+//   U <- U0 (1 + R / 2) G (1 + E), X likewise (two contractions), e~ = diag(A),
+// G the Jacobi rotations of the pairs of levels with |A_ab| > 1e-3 |A_bb - A_aa|, E_ab = A_ab / (A_bb - A_aa) of the
+// rotated A for the others.  A step squares the errors, so two or three take the FP32 basis (R and the off-diagonal A ~
+// 1e-6) to FP64 rounding, groups of close levels four to eleven.  What it takes for these:
+//  * an entry of A is known to 8 eps (|A_aa| + |A_bb|) (rounding) and |R|_F^2 max|A| (the second order in R); entries below
+//    are left alone, since E or a rotation of what is not known would scramble equal or close levels in every step
+//    (E up to 1e-8 is harmless: 1 + E is orthogonal to E^2);
+//  * every pair of close levels is rotated, a list at a time in index order, whatever their number: sums over a list do not
+//    depend on timing.  Above POL_MAX pairs (a group of 24 and more) the rotations act on a G kept in IE and E = 0.
+// The last step is one that finds nothing left to do: |R| < 1e-9 and every |A_ab| either below 1e-8 of its gap or
+// within rounding (16 eps max|A|); *ok says whether this one was, and the caller repeats the step for the others.
+constexpr int POL_MAX = 256;      // close pairs listed at a time
+constexpr int POL_REC = 1024;     // recorded rotations (lists of up to POL_MAX pairs)
+constexpr int POL_SWEEPS = 12;
+constexpr double POL_EPS = 2.220446049250313e-16;
 __global__ void __launch_bounds__(NT) k_oz_polish(const OzPolish* __restrict__ jobs, int n_jobs, int max_r,
                                                   double* scratch) {
-  __shared__ double rcs[2 * POL_MAX * POL_SWEEPS];   // (c, s) of the recorded rotations
-  __shared__ int s_n, s_rec;
+  __shared__ double red[40];
+  __shared__ double rcs[2 * POL_REC];                // (c, s) of the recorded rotations
+  __shared__ unsigned rec[POL_REC];                  // and their elements of A
   __shared__ unsigned key[POL_MAX], list[POL_MAX];
-  __shared__ unsigned short rec[POL_MAX * POL_SWEEPS];
+  __shared__ int s_n, s_rec, wcnt[NT / 32];
   double* A = scratch + (size_t)blockIdx.x * max_r * max_r;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int jq = blockIdx.x; jq < n_jobs; jq += gridDim.x) {
     const OzPolish jb = jobs[jq];
-    const int r = jb.r;
+    const int r = jb.r, rr = r * r;
     double* RG = jb.F1;           // R / 2, then R G / 2
-    if (tid == 0) s_n = s_rec = 0;
-    for (int idx = tid; idx < r * r; idx += NT) {
+    double r2 = 0.0;
+    unsigned rm = 0;              // upper word of max|R|
+    for (int idx = tid; idx < rr; idx += NT) {
       const int a = idx / r, b = idx % r;
       const double R = (a == b ? 1.0 : 0.0) - 0.5 * (jb.S1[idx] + jb.S1[b * r + a]);
+      r2 = fma(R, R, r2);
+      rm = max(rm, (unsigned)__double2hiint(R) & 0x7fffffffu);
       A[idx] = 0.5 * (jb.F1[idx] + jb.F1[b * r + a]) + 0.5 * R * (jb.F1[(size_t)a * r + a] + jb.F1[(size_t)b * r + b]);
     }
-    __syncthreads();
-    for (int idx = tid; idx < r * r; idx += NT) {
+    if (tid == 0) s_n = s_rec = 0;
+    r2 = cta_sum(r2, red);        // ends with a barrier: A is complete
+    double em = 0.0;
+    for (int a = tid; a < r; a += NT) em = fmax(em, fabs(A[(size_t)a * r + a]));
+    em = cta_max(em, red);
+    const double second = r2 * em, round_max = 16.0 * POL_EPS * em;
+    // |x| of the pair of levels da, db: known to `known`
+    auto known = [&](double da, double db) { return fmax(second, 8.0 * POL_EPS * (fabs(da) + fabs(db))); };
+    auto close = [&](int idx) {
+      const int a = idx / r, b = idx % r;
+      if (a >= b) return false;
+      const double x = fabs(A[idx]), da = A[(size_t)a * r + a], db = A[(size_t)b * r + b];
+      return x > 1e-3 * fabs(db - da) && x > known(da, db);
+    };
+    bool left = __double2hiint(1e-9) <= (int)rm || !(r2 < 1.0);
+    for (int idx = tid; idx < rr; idx += NT) {
       const int a = idx / r, b = idx % r;
       RG[idx] = 0.5 * ((a == b ? 1.0 : 0.0) - 0.5 * (jb.S1[idx] + jb.S1[b * r + a]));
       if (a < b) {
         const double x = fabs(A[idx]), da = A[(size_t)a * r + a], db = A[(size_t)b * r + b];
-        if (x > 1e-3 * fabs(db - da) && x > 1e-15 * (fabs(da) + fabs(db))) {
+        if (!(x <= 1e-8 * fabs(db - da))) left |= !(x <= fmax(round_max, known(da, db)));
+      }
+    }
+    left = __syncthreads_or(left);
+    if (tid == 0) *jb.ok = !left;
+    bool many = false;
+    for (int sw = 0; left && sw < POL_SWEEPS; sw++) {
+      for (int idx = tid; idx < rr; idx += NT)
+        if (close(idx)) {
           const int k = atomicAdd(&s_n, 1);
           if (k < POL_MAX) key[k] = (unsigned)idx;
         }
-      }
-    }
-    __syncthreads();
-    const int n = min(s_n, POL_MAX);
-    for (int k = tid; k < n; k += NT) {            // in index order, whatever order they were found in
-      int rank = 0;
-      for (int u = 0; u < n; u++) rank += key[u] < key[k];
-      list[rank] = key[k];
-    }
-    __syncthreads();
-    for (int sw = 0; sw < POL_SWEEPS && n > 0; sw++)
-      for (int k = 0; k < n; k++) {
-        const int p = list[k] / r, q = list[k] % r;
-        const double app = A[(size_t)p * r + p], aqq = A[(size_t)q * r + q], apq = A[(size_t)p * r + q];
+      __syncthreads();
+      const int n = s_n;
+      __syncthreads();
+      if (tid == 0) s_n = 0;
+      if (n == 0) break;
+      if (n > POL_MAX && !many) {
+        if (sw > 0) break;          // the next step takes them
+        many = true;
+        for (int idx = tid; idx < rr; idx += NT) jb.IE[idx] = idx / r == idx % r ? 1.0 : 0.0;
         __syncthreads();
-        if (!(fabs(apq) > 1e-6 * fabs(aqq - app) && fabs(apq) > 1e-16 * (fabs(app) + fabs(aqq)))) continue;   // uniform
-        const double th = (aqq - app) / (2.0 * apq);
-        const double tt = copysign(1.0, th) / (fabs(th) + sqrt(1.0 + th * th));
-        const double c = 1.0 / sqrt(1.0 + tt * tt), s = tt * c;
-        for (int u = tid; u < r; u += NT) {
-          if (u != p && u != q) {
-            const double x = A[(size_t)p * r + u], y = A[(size_t)q * r + u];
-            const double nx = c * x - s * y, ny = s * x + c * y;
-            A[(size_t)p * r + u] = A[(size_t)u * r + p] = nx;
-            A[(size_t)q * r + u] = A[(size_t)u * r + q] = ny;
+      }
+      for (int pos = 0; pos < rr;) {
+        int cnt = 0;
+        if (n <= POL_MAX) {          // all of them, in index order whatever order they were found in
+          for (int k = tid; k < n; k += NT) {
+            int rank = 0;
+            for (int u = 0; u < n; u++) rank += key[u] < key[k];
+            list[rank] = key[k];
           }
-          const double x = RG[(size_t)u * r + p], y = RG[(size_t)u * r + q];
-          RG[(size_t)u * r + p] = c * x - s * y;
-          RG[(size_t)u * r + q] = s * x + c * y;
-        }
-        if (tid == 0) {
-          A[(size_t)p * r + p] = app - tt * apq;
-          A[(size_t)q * r + q] = aqq + tt * apq;
-          A[(size_t)p * r + q] = A[(size_t)q * r + p] = 0.0;
-          rec[s_rec] = (unsigned short)k;
-          rcs[2 * s_rec] = c;
-          rcs[2 * s_rec + 1] = s;
-          s_rec++;
+          cnt = n;
+          pos = rr;
+        } else {                     // the next POL_MAX in index order
+          while (pos < rr && cnt < POL_MAX) {
+            const bool f = pos + tid < rr && close(pos + tid);
+            const unsigned bal = __ballot_sync(0xffffffffu, f);
+            if (lane == 0) wcnt[warp] = __popc(bal);
+            __syncthreads();
+            int at = cnt + __popc(bal & ((1u << lane) - 1u)), all = cnt;
+            for (int w = 0; w < NT / 32; w++) {
+              at += w < warp ? wcnt[w] : 0;
+              all += wcnt[w];
+            }
+            if (f && at < POL_MAX) list[at] = (unsigned)(pos + tid);
+            __syncthreads();
+            pos = all > POL_MAX ? (int)list[POL_MAX - 1] + 1 : pos + NT;
+            cnt = min(all, POL_MAX);
+          }
         }
         __syncthreads();
+        for (int k = 0; k < cnt && (many || s_rec < POL_REC); k++) {
+          const int p = list[k] / r, q = list[k] % r;
+          const double app = A[(size_t)p * r + p], aqq = A[(size_t)q * r + q], apq = A[(size_t)p * r + q];
+          __syncthreads();
+          if (!(fabs(apq) > 1e-6 * fabs(aqq - app) && fabs(apq) > known(app, aqq))) continue;   // uniform
+          const double th = (aqq - app) / (2.0 * apq);
+          const double tt = copysign(1.0, th) / (fabs(th) + sqrt(1.0 + th * th));
+          const double c = 1.0 / sqrt(1.0 + tt * tt), s = tt * c;
+          for (int u = tid; u < r; u += NT) {
+            if (u != p && u != q) {
+              const double x = A[(size_t)p * r + u], y = A[(size_t)q * r + u];
+              const double nx = c * x - s * y, ny = s * x + c * y;
+              A[(size_t)p * r + u] = A[(size_t)u * r + p] = nx;
+              A[(size_t)q * r + u] = A[(size_t)u * r + q] = ny;
+            }
+            const double x = RG[(size_t)u * r + p], y = RG[(size_t)u * r + q];
+            RG[(size_t)u * r + p] = c * x - s * y;
+            RG[(size_t)u * r + q] = s * x + c * y;
+            if (many) {
+              const double gx = jb.IE[(size_t)u * r + p], gy = jb.IE[(size_t)u * r + q];
+              jb.IE[(size_t)u * r + p] = c * gx - s * gy;
+              jb.IE[(size_t)u * r + q] = s * gx + c * gy;
+            }
+          }
+          if (tid == 0) {
+            A[(size_t)p * r + p] = app - tt * apq;
+            A[(size_t)q * r + q] = aqq + tt * apq;
+            A[(size_t)p * r + q] = A[(size_t)q * r + p] = 0.0;
+            if (!many) {
+              rec[s_rec] = list[k];
+              rcs[2 * s_rec] = c;
+              rcs[2 * s_rec + 1] = s;
+              s_rec++;
+            }
+          }
+          __syncthreads();
+        }
       }
-    __syncthreads();
-    for (int idx = tid; idx < r * r; idx += NT) {
-      const int a = idx / r, b = idx % r;
-      double e = a == b ? 1.0 : 0.0;
-      if (a != b) {
-        const double x = A[idx], gap = A[(size_t)b * r + b] - A[(size_t)a * r + a];
-        if (fabs(x) < 1e-2 * fabs(gap)) e = x / gap;
-      }
-      jb.IE[idx] = e;
+      if (!many && s_rec >= POL_REC) break;
     }
-    for (int a = tid; a < r; a += NT) jb.et[a] = A[(size_t)a * r + a];
     __syncthreads();
-    for (int k = s_rec - 1; k >= 0; k--) {         // G (1 + E): the rotations on the rows, last one first
-      const int p = list[rec[k]] / r, q = list[rec[k]] % r;
-      const double c = rcs[2 * k], s = rcs[2 * k + 1];
-      for (int u = tid; u < r; u += NT) {
-        const double x = jb.IE[(size_t)p * r + u], y = jb.IE[(size_t)q * r + u];
-        jb.IE[(size_t)p * r + u] = c * x + s * y;
-        jb.IE[(size_t)q * r + u] = c * y - s * x;
+    for (int a = tid; a < r; a += NT) jb.et[a] = A[(size_t)a * r + a];
+    if (!many) {
+      for (int idx = tid; idx < rr; idx += NT) {
+        const int a = idx / r, b = idx % r;
+        double e = a == b ? 1.0 : 0.0;
+        if (a != b) {
+          const double da = A[(size_t)a * r + a], db = A[(size_t)b * r + b], gap = db - da, x = fabs(A[idx]), g = fabs(gap);
+          if (g > 0.0 && (x <= 1e-8 * g || (left && x <= 1e-3 * g && x > known(da, db)))) e = A[idx] / gap;
+        }
+        jb.IE[idx] = e;
       }
       __syncthreads();
+      for (int k = s_rec - 1; k >= 0; k--) {         // G (1 + E): the rotations on the rows, last one first
+        const int p = rec[k] / r, q = rec[k] % r;
+        const double c = rcs[2 * k], s = rcs[2 * k + 1];
+        for (int u = tid; u < r; u += NT) {
+          const double x = jb.IE[(size_t)p * r + u], y = jb.IE[(size_t)q * r + u];
+          jb.IE[(size_t)p * r + u] = c * x + s * y;
+          jb.IE[(size_t)q * r + u] = c * y - s * x;
+        }
+        __syncthreads();
+      }
     }
     __syncthreads();
-    for (int idx = tid; idx < r * r; idx += NT) jb.IE[idx] += RG[idx];
+    for (int idx = tid; idx < rr; idx += NT) jb.IE[idx] += RG[idx];
     __syncthreads();
   }
 }
