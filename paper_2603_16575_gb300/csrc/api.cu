@@ -2436,6 +2436,7 @@ static int rosv_batch(osvmp2_ctx* c, double* T, int b, int i0, double l_osv, int
   // go through the OSV eigen-kernel with the cut l_osv^2, then Q = Z^T Q~.
   int ldm = 1;
   for (int u = 0; u < b; u++) ldm = std::max(ldm, nrows_h[u]);
+  if (!eig_order_fits(ldm)) return fail(c, OSVMP2_E_ARG, "randomized OSVs: %d rows exceed the eigen-solver's shared memory", ldm);
   double* M = scr + rl.svd;
   double* Vs = M + (size_t)b * ldm * ldm;
   double* ws = Vs + (size_t)b * ldm * ldm;
@@ -2488,6 +2489,8 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
   if ((int64_t)s->n_occ * s->n_occ > (int64_t)1 << 30) return fail(c, OSVMP2_E_ARG, "n_occ too large");
   if (c->opts.osv_method == 1 && !(l_osv > 0.0))
     return fail(c, OSVMP2_E_ARG, "randomized OSVs need l_osv > 0 (the range finder stops on it)");
+  if (c->opts.osv_method == 0 && !eig_order_fits(s->n_vir))
+    return fail(c, OSVMP2_E_ARG, "n_vir = %d exceeds the exact OSV eigen-solver's shared memory", s->n_vir);
   CK(cudaSetDevice(c->device));
   free_system(c);
   c->sys = *s;
@@ -4283,6 +4286,8 @@ int osvmp2_energy_grad_relaxed(osvmp2_ctx* c, double r2, double r3, double* e_ou
   if (!c->have_osv) return fail(c, OSVMP2_E_STATE, "no OSVs built");
   if (c->opts.osv_method != 0)
     return fail(c, OSVMP2_E_ARG, "the relaxed gradient needs exact OSVs (opts.osv_method 0)");
+  if (!eig_order_fits(c->sys.n_vir))
+    return fail(c, OSVMP2_E_ARG, "n_vir = %d exceeds the eigen-solver's shared memory", c->sys.n_vir);
   return energy_grad_impl(c, r2, r3, OSVMP2_FP64, e_out, dE_dB, dE_df, dE_de, stats, true, min_gap_out);
 }
 

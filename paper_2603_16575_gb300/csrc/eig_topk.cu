@@ -719,6 +719,12 @@ void launch_tri(double* T, int nb, int n, double thr, int kmax, double* w, int* 
 
 }  // namespace
 
+bool eig_order_fits(int n) {
+  int cap, nsw;
+  td_layout(n, 8, ArD::NWS, &cap, &nsw);
+  return nsw > 0;
+}
+
 void eig_cluster_table(int* nclu) {
   cudaFuncSetAttribute(k_eig_tri<ArD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TD_SMEM);
   for (int C = 1; C <= 8; C++) {

@@ -4,6 +4,9 @@
 
 namespace osv {
 
+// Whether the vectors of a step and one warp's staging rows of the reduction fit shared memory (orders up to 9536);
+// larger matrices must not be given to the calls below.
+bool eig_order_fits(int n);
 // nclu[C], C = 1..8: clusters of C CTAs of the tridiagonalisation that the GPU holds at a time.
 void eig_cluster_table(int* nclu);
 // T (nb matrices of order n >= 3, lower triangles): d, e, tau at the start of each matrix's scratch
