@@ -2171,8 +2171,7 @@ int ensure_sf_blocks_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>&
   else TRY(oz);
   ph_end(c, OSVMP2_PH_SF, fl);
   CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(c->st));
-  return 0;
+  return check_err_flag(c, "overlap blocks");   // a stuck wait of the contraction shows only there
 }
 int ensure_sf_blocks(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& blocks) {
   const int rc = ensure_sf_blocks_impl(c, blocks);
