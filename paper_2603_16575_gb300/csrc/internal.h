@@ -35,6 +35,15 @@ struct Tables {
 // Process-wide count of kernel launches issued by the library.
 void note_launch(int n);
 
+// Lets kernel fn ask for all the dynamic shared memory that its static part leaves of a CTA's 227 KB.  The limit belongs
+// to the process, so it is this one in every call: set to the size of the call at hand, another thread's smaller
+// system could lower it before the launch.
+inline cudaError_t allow_dynamic_smem(const void* fn) {
+  cudaFuncAttributes a;
+  const cudaError_t e = cudaFuncGetAttributes(&a, fn);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)a.sharedSizeBytes);
+}
+
 struct SolveOpts {
   double tol_update, tol_energy;
   int max_iter;

@@ -414,7 +414,7 @@ bool launch_pm_localize_grid(const double* C, int n, const int* atom_ao, int n_a
   const bool use_smem = smem <= 200 * 1024;
   void* fn = use_smem ? (void*)k_pm_grid<true> : (void*)k_pm_grid<false>;
   const size_t dsm = use_smem ? smem : ang;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm) != cudaSuccess) {
+  if (allow_dynamic_smem(fn) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

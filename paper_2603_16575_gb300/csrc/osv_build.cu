@@ -339,7 +339,7 @@ void launch_eig_osv(double* T, int nb, int nv, double thr, int kmax, double* V, 
   } else {
     launch_eig_tridiag(T, nb, nv, kmax, scratch, err, nclu, st);
     const size_t smem = (2 * (size_t)nv + (nv <= ZSMEM_MAX ? (size_t)nv * nv : 0)) * sizeof(double);
-    cudaFuncSetAttribute(k_eig_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem((const void*)k_eig_full);
     if (fork && cudaEventRecord(fork, st) == cudaSuccess && cudaStreamWaitEvent(st_qr, fork, 0) == cudaSuccess) st = st_qr;
     k_eig_full<<<nb, NT_EIG, smem, st>>>(T, nv, thr, kmax, V, w, k, scratch, err);
     note_launch(1);

@@ -701,15 +701,10 @@ int launch_precond_mixed(const Tables& t, double tau_s, const PJob* jobs, const 
   while (((size_t)nmax * (nmax + 1) + nmax) * sizeof(double) > PM_SMEM) nmax--;
   while (2 * (size_t)jmax * (jmax | 1) * sizeof(float) > PM_SMEM) jmax--;
   const size_t sm_c = ((size_t)nmax * (nmax + 1) + nmax) * sizeof(double);
-  if (cudaFuncSetAttribute(k_pm_overlap_a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_d) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_overlap_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_d) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_c) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, PM_SMEM) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_eig_a<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_t) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_chase<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * nsm * 8) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_chase<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * nsm * 4) != cudaSuccess ||
-      cudaFuncSetAttribute(k_pm_eig_c<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_t) != cudaSuccess)
-    return -1;
+  for (const void* fn : {(const void*)k_pm_overlap_a, (const void*)k_pm_overlap_c, (const void*)k_pm_chol, (const void*)k_pm_jacobi,
+                         (const void*)k_pm_eig_a<float>, (const void*)k_pm_chase<double>, (const void*)k_pm_chase<float>,
+                         (const void*)k_pm_eig_c<float>})
+    if (allow_dynamic_smem(fn) != cudaSuccess) return -1;
   const int lpw = std::min(32, std::max(1, (n_jobs + 4 * num_sms - 1) / (4 * num_sms)));
   const int n_chase = (n_jobs + lpw - 1) / lpw;
   // Jacobi costs ~2.5 ns per r^3 and SM, the three-step QR a serial ~3 ms and ~1.3 ns: Jacobi below their crossing

@@ -292,7 +292,7 @@ void launch_rosv_finder(double* Y, int nb, int nv, int r, int n_max, double l_os
                         double* wmax, int* err, cudaStream_t st) {
   const double thr = l_osv / (10.0 * 0.7978845608028654);   // l_osv / (10 sqrt(2/pi))
   const size_t smem = (size_t)(nv + n_max + r) * sizeof(double);
-  cudaFuncSetAttribute(k_rosv_finder, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem((const void*)k_rosv_finder);
   k_rosv_finder<<<nb, NT_F, smem, st>>>(Y, nv, r, n_max, thr, Z, nrows, wmax, err);
   note_launch(1);
 }

@@ -323,7 +323,7 @@ void launch_mx_sigma(const MxSigma* jobs, int n, int max_r, int ld, long long ro
                      cudaStream_t st) {
   if (!n) return;
   const int cap = mx_cap(max_r, sizeof(float));
-  cudaFuncSetAttribute(k_mx_sigma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(cap * sizeof(float)));
+  allow_dynamic_smem((const void*)k_mx_sigma);
   k_mx_sigma<<<std::min(n, n_cta), NT, cap * sizeof(float), st>>>(jobs, n, ld, (size_t)rows * ld, cap, D);
   note_launch(1);
 }
@@ -347,7 +347,7 @@ void launch_mx_update(const OzPair* pairs, const MxPair* mp, int n, const int* d
                       long long rows, uint16_t* D, int* ex, int* exW, double* pe, double* pu, int n_cta, cudaStream_t st) {
   if (!n) return;
   const int cap = mx_cap(max_r, sizeof(dfl));
-  cudaFuncSetAttribute(k_mx_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(cap * sizeof(dfl)));
+  allow_dynamic_smem((const void*)k_mx_update);
   k_mx_update<<<n_cta, MXT, cap * sizeof(dfl), st>>>(pairs, mp, n, done, first ? 1 : 0, ld, (size_t)rows * ld, cap, D, ex, exW,
                                                              pe, pu);
   note_launch(1);
