@@ -124,7 +124,7 @@ struct osvmp2_ctx {
   std::vector<oz::Mat> um_mat;
   // FP64 form: digits of U_p (polished basis) of each pair: store of its build and matrix in it (-1: none)
   std::vector<void*> ud_alloc;
-  std::vector<char> pm_basis;        // FP64 form: pair bases from the batched preconditioner
+  std::vector<double> pm_tau;        // FP64 form: cut of the pair bases from the batched preconditioner (else negative)
   std::vector<OzOperand> ud_store;
   std::vector<int> ud_of;
   std::vector<oz::Mat> ud_mat;
@@ -304,7 +304,7 @@ void free_system(osvmp2_ctx* c) {
   for (void* p : c->pair_allocs) pool_put(c, p);
   c->pair_allocs.clear();
   drop_basis_digits(c);
-  c->pm_basis.clear();
+  c->pm_tau.clear();
   c->pair_prec = -1;
   c->have_sys = c->have_osv = false;
   c->n_osv.clear(); c->Qp.clear(); c->Wp.clear();
@@ -520,7 +520,7 @@ int reset_pairs(osvmp2_ctx* c) {
   for (void* p : c->pair_allocs) pool_put(c, p);
   c->pair_allocs.clear();
   drop_basis_digits(c);
-  c->pm_basis.clear();
+  c->pm_tau.clear();
   const size_t nn = (size_t)c->sys.n_occ * c->sys.n_occ;
   c->sf_id.assign(nn, -1);
   c->pair_id.assign(nn, -1);
@@ -2100,8 +2100,8 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     oz = oz_pair_basis(c, newp, &touched);
     if (oz && oz != OZ_NO_ROOM && oz != OZ_NO_BASIS) return oz;
     if (oz == 0 && pm) {
-      c->pm_basis.resize(c->K_h.size(), 0);
-      for (auto& p : newp) c->pm_basis[c->pair_id[(size_t)p.first * n + p.second]] = 1;
+      c->pm_tau.resize(c->K_h.size(), -1.0);
+      for (auto& p : newp) c->pm_tau[c->pair_id[(size_t)p.first * n + p.second]] = c->opts.tau_s;
     }
     if (oz && (pm || touched)) {    // no room to polish, or no end to it: bases accurate to FP64 without it
       tmp_free(pm_slots);
@@ -2726,27 +2726,31 @@ int osvmp2_get_precond(osvmp2_ctx* c, int32_t i, int32_t j, double* X, double* e
   const int pid = c->pair_id[(size_t)i * n + j];
   if (pid < 0) return fail(c, OSVMP2_E_STATE, "pair (%d,%d) not built", i, j);
   const int m = c->m_h[pid];
-  if (c->pair_prec == OSVMP2_FP64 && c->r_h[pid] < m && pid < (int)c->pm_basis.size() && c->pm_basis[pid]) {
-    // A dependent pair space: the coefficients of a basis are not unique, and the batched preconditioner's are
-    // not the shortest ones.  Hand out those of the canonical orthogonalisation of S.
+  if (X && c->pair_prec == OSVMP2_FP64 && c->r_h[pid] < m && pid < (int)c->pm_tau.size() && c->pm_tau[pid] >= 0.0) {
+    // A dependent pair space: the coefficients of a basis are not unique, and the batched preconditioner's are not the
+    // shortest ones.  The solver's basis is handed out in those of the canonical orthogonalisation of S.
+    const int r = c->r_h[pid];
     Tmp xb, scr, jd;
-    TRY(tmp_alloc(c, xb, ((size_t)m * m + m + 1) * sizeof(double)));
-    TRY(tmp_alloc(c, scr, precond_scratch_doubles(m) * sizeof(double)));
+    TRY(tmp_alloc(c, xb, ((size_t)2 * m * m + m + 1) * sizeof(double)));
+    TRY(tmp_alloc(c, scr, std::max(precond_scratch_doubles(m), (size_t)2 * m * r) * sizeof(double)));
     TRY(tmp_alloc(c, jd, sizeof(PJob)));
-    double* xp = (double*)xb.p;
-    const PJob job{i, j, xp, xp + (size_t)m * m, (int*)(xp + (size_t)m * m + m), nullptr, nullptr};
+    double* xc = (double*)xb.p;
+    double* out = xc + (size_t)m * m;
+    const PJob job{i, j, xc, out + (size_t)m * m, (int*)(out + (size_t)m * m + m), nullptr, nullptr};
     CK(cudaMemcpyAsync(jd.p, &job, sizeof job, cudaMemcpyHostToDevice, c->st));
     CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
-    CK(cudaMemsetAsync(xb.p, 0, ((size_t)m * m + m + 1) * sizeof(double), c->st));
-    launch_precond(tables(c), c->opts.tau_s, (const PJob*)jd.p, 1, m, (double*)scr.p, 1, c->err_d, c->st);
+    CK(cudaMemsetAsync(xb.p, 0, ((size_t)2 * m * m + m + 1) * sizeof(double), c->st));
+    launch_precond(tables(c), c->pm_tau[pid], (const PJob*)jd.p, 1, m, (double*)scr.p, 1, c->err_d, c->st);
     CK(cudaGetLastError());
-    int r = 0;
-    CK(cudaMemcpyAsync(&r, job.r, sizeof r, cudaMemcpyDeviceToHost, c->st));
-    if (X) CK(cudaMemcpyAsync(X, job.X, (size_t)m * m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    if (et) CK(cudaMemcpyAsync(et, job.et, (size_t)m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
+    int rc = 0;
+    CK(cudaMemcpyAsync(&rc, job.r, sizeof rc, cudaMemcpyDeviceToHost, c->st));
     TRY(check_err_flag(c, "preconditioner"));
-    if (r_out) *r_out = r;
-    return OSVMP2_OK;
+    if (rc == r) {                // (a direction at the cut itself: the stored coefficients)
+      launch_precond_rewrite(tables(c), i, j, xc, c->X_h[pid], r, (double*)scr.p, out, c->st);
+      CK(cudaGetLastError());
+      CK(cudaMemcpyAsync(X, out, (size_t)m * m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
+      X = nullptr;
+    }
   }
   if (X) CK(cudaMemcpyAsync(X, c->X_h[pid], (size_t)m * m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
   if (et) CK(cudaMemcpyAsync(et, c->et_h[pid], (size_t)m * sizeof(double), cudaMemcpyDeviceToDevice, c->st));

@@ -290,6 +290,9 @@ __host__ __device__ inline size_t precond_scratch_doubles(int max_m) {
 }
 void launch_precond(const Tables& t, double tau_s, const PJob* jobs, int n_jobs, int max_m, double* scratch,
                     int n_cta, int* err, cudaStream_t st);
+// out = Xc (Xc^T S X) of the pair (i, j), W: 2 m r doubles.
+void launch_precond_rewrite(const Tables& t, int i, int j, const double* Xc, const double* X, int r, double* W,
+                            double* out, cudaStream_t st);
 // One warp per pair (pair order <= 192); returns -1 if max_m is too large.
 size_t precond_w_scratch_doubles(int max_m, int n_warps);
 int launch_precond_w(const Tables& t, double tau_s, const PJob* jobs, int n_jobs, int max_m, double* scratch,

@@ -85,4 +85,21 @@ void launch_precond(const Tables& t, double tau_s, const PJob* jobs, int n_jobs,
   note_launch(1);
 }
 
+// out = Xc (Xc^T S X): the basis of X written in the coefficients of Xc, another basis of the same space (both [m][m],
+// r columns); one CTA.  W: 2 m r doubles.
+__global__ void __launch_bounds__(NT) k_precond_rewrite(Tables t, int i, int j, const double* Xc, const double* X, int r,
+                                                        double* W, double* out) {
+  __shared__ double sm[GEMM_SMEM_DOUBLES];
+  const int m = pair_dim(t, i, j);
+  double* M = W + (size_t)m * r;
+  cta_gemm(m, r, m, 1.0, pair_view(t, t.S, i, j, i, j), dense_view(X, m, r, m), 0.0, W, r, sm);
+  cta_gemm(r, r, m, 1.0, transpose(dense_view(Xc, m, r, m)), dense_view(W, m, r, r), 0.0, M, r, sm);
+  cta_gemm(m, r, r, 1.0, dense_view(Xc, m, r, m), dense_view(M, r, r, r), 0.0, out, m, sm);
+}
+void launch_precond_rewrite(const Tables& t, int i, int j, const double* Xc, const double* X, int r, double* W,
+                            double* out, cudaStream_t st) {
+  k_precond_rewrite<<<1, NT, 0, st>>>(t, i, j, Xc, X, r, W, out);
+  note_launch(1);
+}
+
 }  // namespace osv
