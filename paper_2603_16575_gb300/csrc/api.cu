@@ -128,6 +128,7 @@ struct osvmp2_ctx {
   std::vector<OzOperand> ud_store;
   std::vector<int> ud_of;
   std::vector<oz::Mat> ud_mat;
+  bool no_polish = false;            // FP64 form: a pair basis of this system did not come out of the polish
   std::vector<int> m_h;
   std::vector<int> pi_h, pj_h;       // pair id -> (i, j)
   // last MBE call
@@ -307,6 +308,7 @@ void free_system(osvmp2_ctx* c) {
   c->pm_tau.clear();
   c->pair_prec = -1;
   c->have_sys = c->have_osv = false;
+  c->no_polish = false;
   c->n_osv.clear(); c->Qp.clear(); c->Wp.clear();
   c->sf_id.clear(); c->pair_id.clear(); c->bt_id.clear();
   c->S_h.clear(); c->F_h.clear(); c->K_h.clear(); c->X_h.clear(); c->et_h.clear(); c->bt_h.clear(); c->Kt_h.clear();
@@ -891,11 +893,12 @@ int oz_exchange(osvmp2_ctx* c, const std::vector<KJob>& kj) {
 
 // FP64 form: U_p = P_p X_p of the new pairs with the basis polished (solve_oz.cu), kept as digits for the
 // pair-couple overlaps.  X and e~ become those of the polished basis.  Pairs in batches whose temporaries
-// fit a fixed budget.  OZ_NO_BASIS: a basis still has something left after POLISH_STEPS steps.  *touched: X of some
+// fit a fixed budget.  OZ_NO_BASIS: a basis still has something left after POLISH_STEPS steps (then c->no_polish).  *touched: X of some
 // pairs may be that of an unfinished polish (when it does not return 0).
 constexpr int POLISH_FIRST = 3, POLISH_STEPS = 17;
 int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, bool* touched) {
   const int n = c->sys.n_occ, nv = c->sys.n_vir;
+  if (c->no_polish) return OZ_NO_ROOM;
   c->ud_of.resize(c->K_h.size(), -1);
   c->ud_mat.resize(c->K_h.size());
   int max_n = 1, max_r = 1;
@@ -1021,7 +1024,10 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, b
     std::vector<int> todo(b1 - b0), ok(b1 - b0);
     for (size_t t = 0; t < todo.size(); t++) todo[t] = (int)t;
     for (int done = 0, steps = POLISH_FIRST; !todo.empty(); steps = 2) {
-      if (done >= POLISH_STEPS) return OZ_NO_BASIS;
+      if (done >= POLISH_STEPS) {
+        c->no_polish = true;
+        return OZ_NO_BASIS;
+      }
       TRY(polish(todo, steps));
       done += steps;
       CK(cudaMemcpyAsync(ok.data(), okd.p, ok.size() * sizeof(int), cudaMemcpyDeviceToHost, c->st));
@@ -1080,6 +1086,63 @@ int oz_ktilde(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, int m
     b0 = b1;
   }
   return 0;
+}
+
+// The same, on the CUDA cores without room for the digits.
+int form_ktilde(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& pairs, int max_m) {
+  const int oz = oz_ktilde(c, pairs, max_m);
+  if (oz != OZ_NO_ROOM) return oz;
+  std::vector<KtJob> jobs;
+  for (auto& p : pairs) jobs.push_back(KtJob{p.first, p.second, c->Kt_h[c->pair_id[(size_t)p.first * c->sys.n_occ + p.second]]});
+  const int n_cta = std::min<int>((int)jobs.size(), 2 * c->num_sms);
+  Tmp jd, scr;
+  TRY(tmp_alloc(c, jd, jobs.size() * sizeof(KtJob)));
+  TRY(tmp_alloc(c, scr, (size_t)n_cta * max_m * max_m * sizeof(double)));
+  CK(cudaMemcpyAsync(jd.p, jobs.data(), jobs.size() * sizeof(KtJob), cudaMemcpyHostToDevice, c->st));
+  launch_ktilde(tables(c), (const KtJob*)jd.p, (int)jobs.size(), (double*)scr.p, n_cta, max_m, c->st);
+  CK(cudaGetLastError());
+  return 0;
+}
+
+// FP64 form: built pairs of the list whose basis digits were given up, or that were built without room for them, get them
+// now if there is room (half of what is free at least): without them the CUDA-core solver runs, ten times slower.
+int restore_bases(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req) {
+  const int n = c->sys.n_occ, nv = c->sys.n_vir;
+  std::vector<std::pair<int, int>> list;
+  for (auto& p : req)
+    for (auto q : {std::pair<int, int>{p.first, p.first}, {p.second, p.second}, p}) {
+      const int id = c->pair_id[(size_t)q.first * n + q.second];
+      if (id >= 0 && (id >= (int)c->ud_of.size() || c->ud_of[id] < 0)) list.push_back(q);
+    }
+  if (list.empty() || c->no_polish) return 0;
+  std::sort(list.begin(), list.end());
+  list.erase(std::unique(list.begin(), list.end()), list.end());
+  double need = 0.0, tmp = 0.0, have = 0.0;
+  int max_m = 1;
+  for (auto& p : list) {
+    const int id = c->pair_id[(size_t)p.first * n + p.second], r = c->r_h[id];
+    need += (double)oz_digit_bytes(r, nv);
+    tmp += 56.0 * r * (nv + r);
+    max_m = std::max(max_m, c->m_h[id]);
+  }
+  need += std::min(tmp, 3e9);
+  for (auto& b : c->pool.free_blocks) have += (double)b.first;
+  size_t fr = 0, tot = 0;
+  if (c->opts.mem_cap_mib > 0) have += std::max(0.0, (double)c->opts.mem_cap_mib * 1048576.0 - (double)c->held);
+  else if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) have += (double)fr;
+  else cudaGetLastError();
+  if (need > 0.5 * have) return 0;
+  CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
+  ph_begin(c, OSVMP2_PH_PRECOND);
+  bool touched = false;
+  const int rc = oz_pair_basis(c, list, &touched);
+  if (rc) {
+    ph_end(c, OSVMP2_PH_PRECOND, 0.0);
+    return rc == OZ_NO_ROOM ? 0 : rc;
+  }
+  TRY(form_ktilde(c, list, max_m));      // X has moved within its rounding
+  ph_end(c, OSVMP2_PH_PRECOND, 0.0);
+  return check_err_flag(c, "pair bases");
 }
 
 // Overlaps of pair couples of the mixed form (build_sigma_table).
@@ -1668,7 +1731,14 @@ int ensure_pairs(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req, osv
   for (auto& p : req)
     if (p.first < 0 || p.second < 0 || p.first >= c->sys.n_occ || p.second >= c->sys.n_occ || p.first > p.second)
       return fail(c, OSVMP2_E_ARG, "pair (%d,%d) invalid: need 0 <= i <= j < n_occ", p.first, p.second);
-  const int rc = ensure_pairs_impl(c, req, prec);
+  int rc = ensure_pairs_impl(c, req, prec);
+  if (rc == 0 && prec == OSVMP2_FP64) {
+    rc = restore_bases(c, req);
+    if (rc == OZ_NO_BASIS) {       // (not seen) rebuild the pairs without the polish
+      TRY(reset_pairs(c));
+      rc = ensure_pairs_impl(c, req, prec);
+    }
+  }
   if (rc != 0 && rc != OSVMP2_E_STATE && c->have_osv) {
     const std::string msg = c->err;
     cudaGetLastError();
@@ -2113,21 +2183,12 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
       CK(cudaStreamSynchronize(c->st));
     }
     ph_end(c, OSVMP2_PH_PRECOND, 0.0);
-    oz = oz_ktilde(c, newp, max_m);
-    if (oz && oz != OZ_NO_ROOM) return oz;
-    std::vector<KtJob> ktj;
-    for (size_t q = 0; oz == OZ_NO_ROOM && q < kj.size(); q++) ktj.push_back(KtJob{kj[q].i, kj[q].j, c->Kt_h[c->pair_id[(size_t)kj[q].i * n + kj[q].j]]});
-    Tmp jkt;
-    TRY(tmp_alloc(c, jkt, ktj.size() * sizeof(KtJob)));
-    CK(cudaMemcpyAsync(jkt.p, ktj.data(), ktj.size() * sizeof(KtJob), cudaMemcpyHostToDevice, c->st));
-    launch_ktilde(t, (const KtJob*)jkt.p, (int)ktj.size(), (double*)scr.p, n_cta, max_m, c->st);
-    CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(c->st));
+    tmp_free(scr);
+    tmp_free(pm_slots);
+    TRY(form_ktilde(c, newp, max_m));
   }
-  (void)prec;
   CK(cudaStreamSynchronize(c->st));
-  TRY(check_err_flag(c, "pair integrals"));
-  return 0;
+  return check_err_flag(c, "pair integrals");
 }
 
 // S/F blocks (x < y) that are not built yet, without the pair data around them
