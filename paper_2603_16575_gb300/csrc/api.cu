@@ -1939,8 +1939,8 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     ph_end(c, OSVMP2_PH_EXCHANGE, f_k);
     CK(cudaGetLastError());
   }
-  const int n_cta = std::min<int>((int)pjb.size(), 2 * c->num_sms);
-  const int n_warps = std::min<int>((int)pjb.size(), 16 * c->num_sms);
+  int n_cta = std::min<int>((int)pjb.size(), 2 * c->num_sms);
+  int n_warps = std::min<int>((int)pjb.size(), 16 * c->num_sms);
   const int n_cta_pm = std::min<int>((int)pjb.size(), 3 * c->num_sms);
   const bool warp_pc = max_m <= PW_MAX_ORDER;
   // Batched preconditioner (precond_mixed.cu): always in the mixed form; in the FP64 form when its work
@@ -1968,6 +1968,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     } else {
       pm = !oz_room(c, pm_slots, (size_t)tot * sizeof(double)) && !oz_room(c, pm_off, off.size() * sizeof(long long)) &&
            !oz_room(c, pm_m, md.size() * sizeof(int)) && !oz_room(c, pm_order, ord.size() * sizeof(int));
+      if (!pm) tmp_free(pm_slots);
     }
     if (pm) {
       CK(cudaMemcpyAsync(pm_off.p, off.data(), off.size() * sizeof(long long), cudaMemcpyHostToDevice, c->st));
@@ -1976,12 +1977,19 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     }
   }
   const size_t scr_pm = precond_mixed_scratch_doubles(max_m, n_cta_pm);
-  const size_t scr_old = std::max((size_t)n_cta * precond_scratch_doubles(max_m),
-                                  warp_pc ? precond_w_scratch_doubles(max_m, n_warps) : (size_t)0);
-  if (mixed_pc || !pm) TRY(tmp_alloc(c, scr, std::max(scr_old, mixed_pc ? scr_pm : (size_t)0) * sizeof(double)));
-  else if (oz_room(c, scr, std::max(scr_pm, (size_t)n_cta * max_m * max_m) * sizeof(double))) {
+  // work areas of the FP64 preconditioner without the batched one's, for fewer CTAs or warps where not all have room
+  auto room64 = [&]() -> int {
+    for (;; n_cta = (n_cta + 1) / 2, n_warps = (n_warps + 1) / 2) {
+      const size_t dbl = warp_pc ? precond_w_scratch_doubles(max_m, n_warps) : (size_t)n_cta * precond_scratch_doubles(max_m);
+      const int rc = tmp_alloc(c, scr, dbl * sizeof(double));
+      if (!rc) c->err.clear();
+      if (!rc || (n_cta == 1 && n_warps == 1)) return rc;
+    }
+  };
+  if (mixed_pc) TRY(tmp_alloc(c, scr, scr_pm * sizeof(double)));
+  else if (pm && oz_room(c, scr, scr_pm * sizeof(double))) {
     pm = false;
-    TRY(tmp_alloc(c, scr, scr_old * sizeof(double)));
+    tmp_free(pm_slots);
   }
   // the FP64 preconditioner without the batched one's work areas
   auto precond64 = [&]() {
@@ -2010,10 +2018,13 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
                                         (double*)scr.p, n_cta_pm, c->num_sms, c->err_d, c->st);
     if (rc && mixed_pc)
       return fail(c, OSVMP2_E_ARG, "pair order %d exceeds the mixed preconditioner's shared scratch", max_m);
-    if (rc) pm = false;
+    if (rc) {
+      pm = false;
+      tmp_free(pm_slots);
+    }
   }
   if (!pm) {
-    if (!mixed_pc) TRY(tmp_alloc(c, scr, scr_old * sizeof(double)));
+    TRY(room64());
     precond64();
   }
   ph_end(c, OSVMP2_PH_PRECOND, f_pc);
@@ -2175,7 +2186,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
     }
     if (oz && (pm || touched)) {    // no room to polish, or no end to it: bases accurate to FP64 without it
       tmp_free(pm_slots);
-      TRY(tmp_alloc(c, scr, scr_old * sizeof(double)));
+      TRY(room64());
       precond64();
       CK(cudaGetLastError());
       TRY(check_err_flag(c, "pair integrals"));
@@ -2608,10 +2619,11 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
   }
   const bool tii_tc = c->opts.osv_prec == OSVMP2_MIXED;
   Tmp Tm, Vm, wm, km, sm;
-  // digits of B for up to 2 GB of orbitals at a time; FP64 form without room for one orbital's: the CUDA-core kernel
+  // digits of B for up to 2 GB (a quarter of a cap) of orbitals at a time; FP64 form without room for one orbital's: the CUDA-core kernel
   const int tii_ns = tii_tc ? oz::MXSL : oz::NSL;
   const size_t ozslot = oz_digit_bytes(nv, s->n_aux, tii_ns);
-  const int noz = (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, ((size_t)2 << 30) / ozslot));
+  const size_t ozmost = c->opts.mem_cap_mib > 0 ? std::min((size_t)2 << 30, (size_t)c->opts.mem_cap_mib << 18) : (size_t)2 << 30;
+  const int noz = (int)std::max<size_t>(1, std::min<size_t>((size_t)nb, ozmost / ozslot));
   Tmp ozD, ozE;
   if (tii_tc) {
     TRY(tmp_alloc(c, ozD, noz * ozslot));
@@ -2631,7 +2643,7 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
   } else {
     TRY(tmp_alloc(c, sm, (size_t)nb * eig_osv_scratch_doubles(nv, kmax) * sizeof(double)));
   }
-  const bool tii_digits = !tii_tc && (double)noz * nv * oz::n_chunks(s->n_aux) + oz::BM < (double)INT32_MAX &&
+  bool tii_digits = !tii_tc && (double)noz * nv * oz::n_chunks(s->n_aux) + oz::BM < (double)INT32_MAX &&
                           !oz_room(c, ozD, noz * ozslot) && !oz_room(c, ozE, oz_exp_bytes((size_t)noz * nv, s->n_aux));
   std::vector<int> nrows_h(nb);
   const uint64_t rosv_key = mix64((uint64_t)s->seed ^ (7ull * STREAM_MUL));
@@ -2684,7 +2696,16 @@ int osvmp2_build_osv(osvmp2_ctx* c, const osvmp2_system* s, double l_osv, int32_
     size_t tot = 0;
     for (int u = 0; u < b; u++) tot += (size_t)kh[u] * (nv + 1);
     double* mem = nullptr;
-    TRY(dalloc_t(c, &mem, tot));
+    int rc = dalloc_t(c, &mem, tot);
+    if (rc == OSVMP2_E_NOMEM && !tii_tc && ozD.p) {   // the digits of B are dispensable in the FP64 form
+      tmp_free(ozD);
+      tmp_free(ozE);
+      tii_digits = false;
+      pool_trim(c);
+      c->err.clear();
+      rc = dalloc_t(c, &mem, tot);
+    }
+    TRY(rc);
     std::vector<double*> qd(2 * b);
     size_t off = 0;
     for (int u = 0; u < b; u++) {
@@ -3585,10 +3606,11 @@ struct OverlapQr {
 
 // OSV response of the relaxed gradient (FP64 form), added to the frozen outputs:
 // dE/dQ_x from the exchange part per pair and the rest per fragment, then per batch
-// of orbitals T_xx again, all its eigenpairs, the response Z_x and its chain rule.
+// of orbitals T_xx again, all its eigenpairs, the response Z_x and its chain rule.  lean: without the buffers that only
+// serve more CTAs at a time.  All memory is taken before an output is touched, so a call that found none can be repeated.
 static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plist,
                      const std::vector<GradPairJob>& pjobs, const double* tstore, const std::vector<long long>& toff,
-                     int max_m, double* dE_dB, double* dE_df, double* dE_de, double* gap_out) {
+                     int max_m, bool lean, double* dE_dB, double* dE_df, double* dE_de, double* gap_out) {
   const int n = c->sys.n_occ, nv = c->sys.n_vir, nx = c->sys.n_aux;
   const int np = (int)plist.size(), nf = (int)c->frags.size();
   const Tables t = tables(c);
@@ -3639,7 +3661,7 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
   TRY(tmp_alloc(c, dk, std::max<size_t>(1, koff[np]) * sizeof(double)));
   // the two terms of a pair side by side where a second buffer fits
   const size_t k_most = c->opts.mem_cap_mib > 0 ? (size_t)c->opts.mem_cap_mib << 17 : (size_t)4 << 30;
-  const bool both = koff[np] * sizeof(double) <= k_most && !oz_room(c, dk2, std::max<size_t>(1, koff[np]) * sizeof(double));
+  const bool both = !lean && koff[np] * sizeof(double) <= k_most && !oz_room(c, dk2, std::max<size_t>(1, koff[np]) * sizeof(double));
   std::vector<RelaxKJob> kj(np);
   for (int q = 0; q < np; q++) {
     const int i = plist[q].first, j = plist[q].second;
@@ -3678,7 +3700,7 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
         }
   Tmp slots, fscr, d_fj, d_next;
   const size_t most = c->opts.mem_cap_mib > 0 ? (size_t)c->opts.mem_cap_mib << 17 : (size_t)4 << 30;   // an eighth of a cap
-  const bool by_pair = slot_pairs * sizeof(double) <= most && !oz_room(c, slots, std::max<size_t>(1, slot_pairs) * sizeof(double));
+  const bool by_pair = !lean && slot_pairs * sizeof(double) <= most && !oz_room(c, slots, std::max<size_t>(1, slot_pairs) * sizeof(double));
   if (!by_pair) TRY(tmp_alloc(c, slots, std::max<size_t>(1, slot_total) * sizeof(double)));
   std::vector<RelaxFragJob> fj;
   size_t so = 0;
@@ -3736,7 +3758,9 @@ static int relax_osv(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& plis
     else
       cudaGetLastError();
   }
-  TRY(tmp_alloc(c, fscr, (size_t)n_cta_f * scr_per * sizeof(double)));
+  int frc = tmp_alloc(c, fscr, (size_t)n_cta_f * scr_per * sizeof(double));
+  for (; frc && lean && n_cta_f > 1; frc = tmp_alloc(c, fscr, (size_t)n_cta_f * scr_per * sizeof(double))) n_cta_f = (n_cta_f + 1) / 2;
+  TRY(frc);
   TRY(tmp_alloc(c, d_fj, std::max<size_t>(1, fj.size()) * sizeof(RelaxFragJob)));
   TRY(tmp_alloc(c, d_next, sizeof(int)));
   if (!fj.empty())
@@ -4332,7 +4356,14 @@ static int energy_grad_impl(osvmp2_ctx* c, double r2, double r3, osvmp2_prec pre
     CK(cudaGetLastError());
   }
   ph_end(c, OSVMP2_PH_GRAD, fl);
-  if (relaxed) TRY(relax_osv(c, plist, pjobs, (const double*)tstore.p, toff, max_m, dE_dB, dE_df, dE_de, gap_out));
+  if (relaxed) {
+    int rc = OSVMP2_E_NOMEM;
+    for (int lean = 0; lean < 2 && rc == OSVMP2_E_NOMEM; lean++) {
+      c->err.clear();
+      rc = relax_osv(c, plist, pjobs, (const double*)tstore.p, toff, max_m, lean != 0, dE_dB, dE_df, dE_de, gap_out);
+    }
+    TRY(rc);
+  }
   CK(cudaStreamSynchronize(c->st));
   ph_collect(c);
   return check_err_flag(c, "gradient");
