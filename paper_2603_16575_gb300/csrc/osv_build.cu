@@ -287,14 +287,17 @@ __global__ void __launch_bounds__(NT_EIG) k_eig_full(double* T, int n, double th
   __syncthreads();
   // two records of at most 32 n rotations each (a sweep is below n): sweeps as int pairs, then (c, s) pairs
   const int half = n * n / 2, cap_s = half / 8, cap_r = min((half - cap_s) / 2, 32 * n);
-  int rc = 2;
+  const int max_sweeps = 40 * n + 100;        // of all records: a matrix that never deflates (NaN) ends here
+  int rc = 2, total = 0;
   if (tid == 0) s_rc = 2;
-  for (int c = 0; c <= 40 * n + 100; c++) {   // each record holds at least one sweep
+  for (int c = 0; c <= max_sweeps; c++) {     // each record holds at least one sweep
     double* rec = A + (size_t)(c & 1) * half;
     const double* old = A + (size_t)((c + 1) & 1) * half;
     if (tid == 0) {
       int ns = 0;
       if (rc == 2) s_rc = tridiag_qr_record(dv, ev, n, reinterpret_cast<int*>(rec), cap_s, rec + cap_s, cap_r, &ns, true);
+      total += ns;
+      if (rc == 2 && s_rc == 2 && total > max_sweeps) s_rc = 1;
       s_ns[c & 1] = ns;
     } else if (tid >= 32 && c > 0) {
       const int* swp = reinterpret_cast<const int*>(old);
