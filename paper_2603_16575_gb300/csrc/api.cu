@@ -55,10 +55,9 @@ struct DevPool {
   std::unordered_map<void*, size_t> size_of;  // every block the pool handed out
 };
 
-// Launch shape of the mixed fragment solve, chosen per (fragment count, largest
-// pair order) by the autotuner of mbe3_core: CTAs per SM and the tile set of
-// the solver's FP32 contractions.  Every candidate computes the same numbers
-// (one CTA per fragment, the same FMA order), so the choice changes time only.
+// Launch shape of the mixed amplitude iterations, chosen per (fragment count, largest pair order) by the autotuners of
+// mbe3_core: CTAs per SM of the element-wise update, or CTAs per SM and the tile set of the FP32 contractions of
+// the per-fragment solver.  Every candidate computes the same numbers, so the choice changes time only.
 struct SolvePlan {
   int ctas_per_sm = 2;
   int tiles = 0;
@@ -70,7 +69,8 @@ struct osvmp2_ctx {
   DevPool pool;
   size_t held = 0;                                  // device bytes this ctx holds from the driver
   std::unordered_map<void*, size_t> raw_size;       // every driver block it holds, with its size
-  std::map<std::pair<int, int>, SolvePlan> plans;   // mixed solve plans by (n_frag, max_m)
+  std::map<std::pair<int, int>, SolvePlan> plans;       // plans of the mixed amplitude update by (n_frag, max_m)
+  std::map<std::pair<int, int>, SolvePlan> cta_plans;   // and of the per-fragment solver that runs without room for the batch
   SolvePlan last_plan;
   cudaStream_t cap_st = nullptr;      // private stream used only to record the solve graph
   cudaStream_t qr_st = nullptr;       // beside st: the implicit QR of the relaxed gradient (high priority)
@@ -1686,7 +1686,6 @@ int oz_solve_batch(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, con
 int oz_solve(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, const std::vector<int>& out_id, const SolveOpts& so,
              double ulps, FragOut* out, double* tdst, const long long* toff, double* pair_e,
              const OzWant& want = OzWant{}) {
-  const int n = c->sys.n_occ;
   // device memory of a fragment: amplitudes and their digits, W and the overlaps
   std::vector<double> mem(orbs.size(), 0.0);
   for (size_t f = 0; f < orbs.size(); f++) {
@@ -1697,7 +1696,6 @@ int oz_solve(osvmp2_ctx* c, const std::vector<std::vector<int>>& orbs, const std
         mem[f] += m * (m + 32.0) * 16.0 * (4.0 + 3.0 * 4.0 * (o.size() - 1) / 2.0);
       }
   }
-  (void)n;
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
     cudaGetLastError();
@@ -1798,7 +1796,7 @@ int ensure_pairs_impl(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& req
   };
   const bool mixed = prec == OSVMP2_MIXED;
   for (auto& p : newp) {
-    if (mixed) break;    // the mixed form projects onto U = P X instead (ubasis.cu)
+    if (mixed) break;    // the mixed form projects onto U = P X instead
     want_bt(p.first, p.first);
     if (p.first != p.second) {
       want_bt(p.first, p.second);
@@ -2350,7 +2348,7 @@ int osvmp2_get_solve_plan(const osvmp2_ctx* c, int32_t* out) {
   out[0] = c->last_plan.ctas_per_sm;
   out[1] = c->last_plan.tiles;
   out[2] = c->last_plan.tuned ? 1 : 0;
-  out[3] = (int32_t)c->plans.size();
+  out[3] = (int32_t)(c->plans.size() + c->cta_plans.size());
   return OSVMP2_OK;
 }
 
@@ -2962,7 +2960,7 @@ int osvmp2_mbe3_fragments(const double* r_occ, int32_t n_occ, double r2, double 
 
 // Mixed form: the overlaps Sigma_(lo,hi) = U_lo^T U_hi of every pair couple that
 // a coupling term of some fragment uses (pair p with the pairs (a,c), (c,b) of
-// its fragment), each computed once on the tensor cores from the U slices.
+// its fragment), each computed once on the tensor cores from the digits of U.
 int build_sigma_table(osvmp2_ctx* c, SigmaStore& ss) {
   const int n = c->sys.n_occ, npairs = (int)c->K_h.size();
   std::vector<std::pair<int, int>> cps;
@@ -3165,7 +3163,8 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
     };
     // autotuner: the first call for a (fragment count, largest pair order) times
     // every candidate plan on the full solve and keeps the fastest
-    if (it == c->plans.end()) {
+    it = c->cta_plans.find(key);
+    if (it == c->cta_plans.end()) {
       SolvePlan best;
       if (c->opts.no_autotune == 2) best.ctas_per_sm = 3;
       if (!c->opts.no_autotune) {
@@ -3195,7 +3194,7 @@ static int mbe3_core(osvmp2_ctx* c, osvmp2_prec prec, double* e_out, osvmp2_mbe_
         best.ms = best_ms;
         CK(cudaMemsetAsync(c->err_d, 0, sizeof(int), c->st));
       }
-      it = c->plans.emplace(key, best).first;
+      it = c->cta_plans.emplace(key, best).first;
     }
     c->last_plan = it->second;
     // the solve and the MBE(3) sum replayed as one CUDA graph (recorded on a

@@ -126,16 +126,11 @@ __device__ __forceinline__ bool issue(uint64_t da, uint64_t db, uint32_t dcol, i
 }
 
 // (ah, al) += (vh, vl) 2^x in FP32 pairs, the error terms gathered in al.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  const float t = a + b, bb = t - a;
-  e = (a - (t - bb)) + (b - bb);
-  s = t;
-}
 __device__ __forceinline__ void pair_add(float vh, float vl, int x, float& ah, float& al) {
   if (x < -120) return;                                            // zero rows, and terms below 2^-98
   float sc = __int_as_float((min(x, 127) + 127) << 23), t;
   if (x >= EX_NAN / 2) sc = __int_as_float(0x7FC00000);
-  two_sum(ah, vh * sc, ah, t);
+  tc::two_sum(ah, vh * sc, ah, t);
   al += fmaf(vl, sc, t);
 }
 
@@ -324,7 +319,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             for (int u = 0; u < DCOL; u++) {
               const float y = __uint_as_float(x[u]) * __int_as_float((127 - 8 * l) << 23);
               if (l == 0) { vh[u] = y; vl[u] = 0.f; }
-              else if (l == 1) two_sum(vh[u], y, vh[u], vl[u]);
+              else if (l == 1) tc::two_sum(vh[u], y, vh[u], vl[u]);
               else vl[u] += y;
             }
           }
@@ -385,7 +380,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               if constexpr (Epi::kPair) {                            // levels as an FP32 pair in units of the first
                 const float y = __uint_as_float(x[u]) * __int_as_float((127 - 8 * l) << 23);
                 if (l == 0) { vh[u] = y; vl[u] = 0.f; }
-                else if (l == 1) two_sum(vh[u], y, vh[u], vl[u]);
+                else if (l == 1) tc::two_sum(vh[u], y, vh[u], vl[u]);
                 else vl[u] += y;
                 if (l == NS - 1) pair_add(vh[u], vl[u], ea + __shfl_sync(0xffffffffu, eb, u) + C::UNIT - 14, ah[u], al[u]);
                 continue;
