@@ -1023,7 +1023,7 @@ int oz_pair_basis(osvmp2_ctx* c, const std::vector<std::pair<int, int>>& newp, b
     };
     std::vector<int> todo(b1 - b0), ok(b1 - b0);
     for (size_t t = 0; t < todo.size(); t++) todo[t] = (int)t;
-    for (int done = 0, steps = POLISH_FIRST; !todo.empty(); steps = 2) {
+    for (int done = 0, steps = POLISH_FIRST; !todo.empty(); steps = 1) {
       if (done >= POLISH_STEPS) {
         c->no_polish = true;
         return OZ_NO_BASIS;
