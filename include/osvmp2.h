@@ -59,12 +59,17 @@ typedef enum {
                             flagged the call; the call's results are invalid */
 } osvmp2_status;
 
-/* Arithmetic of the projection/exchange contractions (A1-A2) and of the residual
- * products (A4).  OSV eigen-decomposition, preconditioner, update denominators
- * and every energy accumulation are FP64 in all forms. */
+/* Arithmetic of the contractions (A1-A2) and of the residual products (A4).
+ * OSVMP2_FP64: results to FP64 rounding.  The large contractions take their operands as 63-bit integers below the power
+ * of two of a row's largest element in 256 consecutive ones (of the whole matrix for the amplitudes), whose
+ * products are exact, and sum them in FP64: elements below 2^-10 of that largest one keep fewer bits than an
+ * FP64 operand has, with an absolute error of 2^-64 of it.  The pair bases are formed in double-float and FP32 and
+ * refined in FP64 until they are orthonormal with F diagonal to FP64 rounding.  The rest is FP64.
+ * OSVMP2_MIXED: 39- and 31-bit operands, products summed as FP32 pairs; double-float updates and basis products; FP64
+ * for overlaps, Cholesky factors and the sums of energies over fragments. */
 typedef enum {
-  OSVMP2_FP64 = 0,   /* FP64 throughout (contractions by exact integer slices on the tensor cores) */
-  OSVMP2_MIXED = 1   /* split-precision products summed as FP32 pairs, FP64 elsewhere */
+  OSVMP2_FP64 = 0,
+  OSVMP2_MIXED = 1
 } osvmp2_prec;
 
 typedef struct {
@@ -185,10 +190,11 @@ int osvmp2_pair_integrals(osvmp2_ctx *ctx, const int32_t *pairs, int64_t n_pairs
 int osvmp2_get_pair_blocks(osvmp2_ctx *ctx, int32_t i, int32_t j, double *K_dev, double *S_dev,
                            double *F_dev);
 
-/* Preconditioner of built pair (i,j) (Eq. prec_eig): X (device [m][m], row-major;
- * columns 0..r-1 valid) with X^T S X = 1 and X^T F X = diag(e~), e~ (device [m],
- * first r valid), r (host scalar) = number of S_(ij,ij) eigenvalues above
- * tau_s * max.  Any output may be NULL. */
+/* Preconditioner of built pair (i,j) (Eq. prec_eig), the basis that the solver uses: X (device
+ * [m][m], row-major; columns 0..r-1 valid) with X^T S X = 1 and X^T F X = diag(e~), e~ (device
+ * [m], first r valid), r (host scalar) = number of S_(ij,ij) eigenvalues above tau_s * max.  The
+ * coefficients X of a basis are not unique when r < m; the FP64 form hands out the shortest ones.
+ * Any output may be NULL. */
 int osvmp2_get_precond(osvmp2_ctx *ctx, int32_t i, int32_t j, double *X_dev, double *et_dev, int32_t *r_out);
 
 /* ---- A3-A4: OSV-MP2 solve of one subsystem (Eq. res_close, Algorithm 7) ----

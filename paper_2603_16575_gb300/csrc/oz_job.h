@@ -33,7 +33,7 @@ struct Seg {
 struct Job {
   int seg0, nseg;          // the tile sums segments [seg0, seg0 + nseg)
   int m0, n0;              // first row / column of the tile in the output
-  int m_valid, n_valid;    // rows (<= 128) and columns (<= 64) to store
+  int m_valid, n_valid;    // rows (<= 128) and columns (<= tile_cols) to store
   int ld_out;
   int skip;                // index of a flag that makes the kernel leave the tile out, or -1
   int o_row, o_e;          // digit-writing epilogue: output matrix in its store, index of its exponent
